@@ -1,6 +1,6 @@
 // Plain CUDA-core kernels (fp32 arithmetic, any head_dim that is a multiple of 8 up to 256, bf16
 // or fp32 inputs).  They serve the fp32 configuration and every shape the tensor-core kernels do
-// not cover, and are the on-device cross-check for those kernels.  One warp per query row.
+// not cover, and are the on-device cross-check for those kernels.
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -32,16 +32,45 @@ template <> struct Ld8<__nv_bfloat16> {
   static __device__ __forceinline__ void store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
+// The keys a block works on at a time sit in shared memory as fp32 rows.  A K row is padded by four floats: the lanes of
+// a warp read four consecutive floats of 32 different rows, and since d is a multiple of 8 the row pitch in 16-byte units
+// is odd, so the eight rows of a quarter warp fall into eight different bank groups.
+constexpr int kStageKeys = 64;
+__host__ __device__ inline int k_pitch(int d) { return d + 4; }
+
+// rows [j0, j0 + kStageKeys) of a [tokens][d] matrix (row stride `st` elements) into fp32 rows of `pitch` floats; rows
+// from `n` on are zero
 template <typename T>
-__device__ __forceinline__ float dot_row(const float* __restrict__ q_s, const T* __restrict__ k, int d) {
-  float acc = 0.f;
-  for (int t = 0; t < d; t += 8) {
-    float kv[8];
-    Ld8<T>::load(k + t, kv);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) acc = fmaf(q_s[t + u], kv[u], acc);
+__device__ __forceinline__ void load_stage(float* dst, int pitch, const T* __restrict__ src, int64_t st, int j0, int n, int d) {
+  const int ppr = d >> 3;                                       // pieces of 8 elements per row
+  for (int x = threadIdx.x; x < kStageKeys * ppr; x += blockDim.x) {
+    const int r = x / ppr, piece = x % ppr;
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (j0 + r < n) Ld8<T>::load(src + (int64_t)(j0 + r) * st + piece * 8, v);
+    float4* o = reinterpret_cast<float4*>(dst + r * pitch + piece * 8);
+    o[0] = make_float4(v[0], v[1], v[2], v[3]);
+    o[1] = make_float4(v[4], v[5], v[6], v[7]);
   }
-  return acc;
+}
+
+// Dot products of R query rows (fp32, shared memory, d floats apart) with the keys of rows k0 and k1: one fused
+// multiply-add per dimension in ascending order.
+template <int R>
+__device__ __forceinline__ void dot_rows(const float* q_s, const float* k0, const float* k1, int d, float (&s)[R][2]) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) s[r][0] = s[r][1] = 0.f;
+#pragma unroll 4
+  for (int t = 0; t < d; t += 4) {
+    const float4 a = *reinterpret_cast<const float4*>(k0 + t), b = *reinterpret_cast<const float4*>(k1 + t);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float4 q = *reinterpret_cast<const float4*>(q_s + r * d + t);
+      s[r][0] = fmaf(q.x, a.x, s[r][0]); s[r][1] = fmaf(q.x, b.x, s[r][1]);
+      s[r][0] = fmaf(q.y, a.y, s[r][0]); s[r][1] = fmaf(q.y, b.y, s[r][1]);
+      s[r][0] = fmaf(q.z, a.z, s[r][0]); s[r][1] = fmaf(q.z, b.z, s[r][1]);
+      s[r][0] = fmaf(q.w, a.w, s[r][0]); s[r][1] = fmaf(q.w, b.w, s[r][1]);
+    }
+  }
 }
 
 __device__ __forceinline__ float warp_max(float v) {
@@ -60,58 +89,101 @@ __device__ __forceinline__ float warp_sum(float v) {
 // Two sweeps over the keys of a row (max / sum, then probabilities); the fp32 probability that is
 // compared with p* is the very value written to the dump.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void scores_ref_kernel(unsigned char* blob, const T* __restrict__ Q, const T* __restrict__ K,
-                                  int Hq, int group, int d, int64_t qst, int64_t qsh, int64_t kst, int64_t ksh,
-                                  float scale, float pstar, float* __restrict__ dump) {
+// Bound by latency at the sizes this path serves.  A block takes 8 R adjacent rows (R per warp) of one map and walks
+// the keys in stages of 64 held in shared memory, so that a key row is read from memory once per block and not once per
+// row.  R = 1 while that leaves SMs idle, 4 otherwise (a stage then feeds four times the multiply-adds).
+template <typename T, int R>
+__global__ void __launch_bounds__(256)
+scores_ref_kernel(unsigned char* blob, const T* __restrict__ Q, const T* __restrict__ K,
+                  int Hq, int group, int d, int64_t qst, int64_t qsh, int64_t kst, int64_t ksh,
+                  float scale, float pstar, float* __restrict__ dump) {
   extern __shared__ float smem[];
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   const int sh = blockIdx.y;
   const int b = sh / Hq, h = sh % Hq;
   const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[b];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int i = blockIdx.x * nw + warp;
-  if (i >= sq.L) return;
-  float* q_s = smem + warp * d;
-  const T* qrow = Q + (int64_t)(sq.tok_start + i) * qst + (int64_t)h * qsh;
-  for (int t = lane; t < d; t += 32) q_s[t] = Ld8<T>::one(qrow + t);
-  __syncwarp();
-  const T* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
-  float m = -CUDART_INF_F, l = 0.f;
-  for (int j = lane; j <= i; j += 32) {
-    float s = dot_row<T>(q_s, Kh + (int64_t)j * kst, d) * scale;
-    float mn = fmaxf(m, s);
-    l = l * expf(m - mn) + expf(s - mn);
-    m = mn;
+  const int i_block = blockIdx.x * nw * R;
+  if (i_block >= sq.L) return;
+  const int i_end = min(i_block + nw * R, sq.L);                // keys 0 .. i_end - 1 matter to the block
+  const int i0 = i_block + warp * R;
+  float* k_s = smem;
+  float* q_s = smem + kStageKeys * k_pitch(d) + warp * R * d;
+  for (int x = lane; x < R * d; x += 32) {
+    const int i = i0 + x / d;
+    q_s[x] = i < sq.L ? Ld8<T>::one(Q + (int64_t)(sq.tok_start + i) * qst + (int64_t)h * qsh + x % d) : 0.f;
   }
-  float mw = warp_max(m);
-  l = (m == -CUDART_INF_F) ? 0.f : l * expf(m - mw);
-  l = warp_sum(l);
+  const T* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
   uint32_t* M = reinterpret_cast<uint32_t*>(blob + H->off_true) + sq.true_off + (uint64_t)h * sq.L * sq.W;
-  float* Ph = dump ? dump + sq.p_off + (uint64_t)h * sq.L * sq.L + (uint64_t)i * sq.L : nullptr;
-  for (int w = 0; w < sq.W; ++w) {
-    int j = w * 32 + lane;
-    float p = 0.f;
-    if (j <= i) {
-      float s = dot_row<T>(q_s, Kh + (int64_t)j * kst, d) * scale;
-      p = expf(s - mw) / l;
+  float* Ph = dump ? dump + sq.p_off + (uint64_t)h * sq.L * sq.L : nullptr;
+  float m[R], l[R], mw[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) { m[r] = -CUDART_INF_F; l[r] = 0.f; mw[r] = 0.f; }
+  const float* k0 = k_s + lane * k_pitch(d);
+  const float* k1 = k0 + 32 * k_pitch(d);
+  const int nstage = (i_end + kStageKeys - 1) / kStageKeys;
+  for (int sweep = 0; sweep < 2; ++sweep) {
+    for (int t = 0; t < nstage; ++t) {
+      const int j0 = t * kStageKeys;
+      if (nstage > 1 || sweep == 0) {                           // a single stage is still there in the second sweep
+        __syncthreads();
+        load_stage<T>(k_s, k_pitch(d), Kh, kst, j0, sq.L, d);
+        __syncthreads();
+      }
+      float s[R][2];
+      dot_rows<R>(q_s, k0, k1, d, s);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int j = j0 + c * 32 + lane;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int i = i0 + r;
+          const float x = s[r][c] * scale;
+          if (sweep == 0) {
+            if (j <= i) {
+              const float mn = fmaxf(m[r], x);
+              l[r] = l[r] * expf(m[r] - mn) + expf(x - mn);
+              m[r] = mn;
+            }
+          } else {
+            const float p = j <= i ? expf(x - mw[r]) / l[r] : 0.f;
+            if (Ph && i < sq.L && j < sq.L) Ph[(uint64_t)i * sq.L + j] = p;
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, p >= pstar);
+            if (lane == 0 && i < sq.L && (j0 >> 5) + c < sq.W) M[(size_t)i * sq.W + (j0 >> 5) + c] = word;
+          }
+        }
+      }
     }
-    if (Ph && j < sq.L) Ph[j] = p;
-    uint32_t word = __ballot_sync(0xFFFFFFFFu, p >= pstar);
-    if (lane == 0) M[(size_t)i * sq.W + w] = word;
+    if (sweep == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        mw[r] = warp_max(m[r]);
+        l[r] = warp_sum((m[r] == -CUDART_INF_F) ? 0.f : l[r] * expf(m[r] - mw[r]));
+      }
+    }
+  }
+  // words (and map cells) to the right of the stages the block visited lie above the diagonal
+  for (int r = 0; r < R; ++r) {
+    const int i = i0 + r;
+    if (i >= sq.L) break;
+    for (int w = nstage * (kStageKeys / 32) + lane; w < sq.W; w += 32) M[(size_t)i * sq.W + w] = 0u;
+    if (Ph) for (int j = nstage * kStageKeys + lane; j < sq.L; j += 32) Ph[(uint64_t)i * sq.L + j] = 0.f;
   }
 }
 
 // ---------------------------------------------------------------------------------------------
-// Masked attention over the listed tiles.  Block = 4 warps = one (head, q-block) row of the tile
-// list; each warp walks 32 of its 128 query rows.  Online softmax in fp32.
+// Masked attention over the listed tiles, online softmax in fp32.  A block takes 8 R adjacent rows (R per warp) of one
+// (head, q-block) row of the tile list and walks its tiles in stages of 64 keys whose K and V rows sit in shared memory;
+// a stage without an active cell in the block's rows is not loaded.  The lanes of a warp are keys for the scores and
+// dimensions for the output.  Latency bound at the sizes this path serves: R = 1 while that leaves SMs idle, 4 otherwise.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __restrict__ K,
-                                const T* __restrict__ V, int Hq, int group, int d, int64_t qst, int64_t qsh,
-                                int64_t kst, int64_t ksh, int64_t vst, int64_t vsh, int64_t ost, int64_t osh,
-                                int causal, float scale, T* __restrict__ O, float* __restrict__ lse, int total_tokens,
-                                const int32_t* __restrict__ ranges) {
+template <typename T, int R, int ND>
+__global__ void __launch_bounds__(256)
+attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __restrict__ K,
+                const T* __restrict__ V, int Hq, int group, int d, int64_t qst, int64_t qsh,
+                int64_t kst, int64_t ksh, int64_t vst, int64_t vsh, int64_t ost, int64_t osh,
+                int causal, float scale, T* __restrict__ O, float* __restrict__ lse, int total_tokens,
+                const int32_t* __restrict__ ranges) {
   extern __shared__ float smem[];
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   const int row = blockIdx.x;
@@ -123,70 +195,151 @@ __global__ void attn_ref_kernel(const unsigned char* blob, const T* __restrict__
     const int r0 = (qb & ~1) * DAM_TILE;
     if (r0 < ranges[2 * b] || r0 >= ranges[2 * b + 1]) return;
   }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int i_block = qb * DAM_TILE + blockIdx.y * nw * R;
+  if (i_block >= sq.S) return;
+  const int i0 = i_block + warp * R;
   const uint32_t* tile_ptr = reinterpret_cast<const uint32_t*>(blob + H->off_tile_ptr);
   const uint32_t* tiles = reinterpret_cast<const uint32_t*>(blob + H->off_tiles);
   const uint32_t t0 = tile_ptr[row], t1 = tile_ptr[row + 1];
   const DamHeadBits hb = dam_head_bits(blob, H, sq, h);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  float* q_s = smem + warp * d;
+  const int pitch = k_pitch(d);
+  float* k_s = smem;
+  float* v_s = k_s + kStageKeys * pitch;
+  float* q_s = v_s + kStageKeys * d + warp * R * d;
+  float* p_s = v_s + kStageKeys * d + nw * R * d + warp * R * kStageKeys;       // the warp's probabilities of a stage
+  for (int x = lane; x < R * d; x += 32) {
+    const int i = i0 + x / d;
+    q_s[x] = i < sq.S ? Ld8<T>::one(Q + (int64_t)(sq.tok_start + i) * qst + (int64_t)h * qsh + x % d) : 0.f;
+  }
   const T* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
   const T* Vh = V + (int64_t)sq.tok_start * vst + (int64_t)(h / group) * vsh;
-  const int nd = d / 32 + ((d % 32) ? 1 : 0);
-
-  for (int r = warp; r < DAM_TILE; r += nw) {
-    const int i = qb * DAM_TILE + r;
-    if (i >= sq.S) break;
-    const T* qrow = Q + (int64_t)(sq.tok_start + i) * qst + (int64_t)h * qsh;
-    __syncwarp();
-    for (int t = lane; t < d; t += 32) q_s[t] = Ld8<T>::one(qrow + t);
-    __syncwarp();
-    float acc[8];
+  const float* k0 = k_s + lane * pitch;
+  const float* k1 = k0 + 32 * pitch;
+  float acc[R][ND], m[R], l[R];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) acc[u] = 0.f;
-    float m = -CUDART_INF_F, l = 0.f;
-    for (uint32_t t = t0; t < t1; ++t) {
-      const uint32_t e = __ldg(tiles + t);
-      if ((e >> 28) == 0u) continue;                    // padding behind the row's entries
-      const int kb = (int)(e & 0x0FFFFFFFu);
-      const uint4 bits = dam_apply_bits(hb, e >> 28, i, kb, causal);
-      const uint32_t w4[4] = {bits.x, bits.y, bits.z, bits.w};
+  for (int r = 0; r < R; ++r) {
+    m[r] = -CUDART_INF_F; l[r] = 0.f;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        uint32_t word = w4[c];
-        if (!word) continue;
-        const int jb = kb * DAM_TILE + c * 32;
-        const bool act = (word >> lane) & 1u;
-        float s = -CUDART_INF_F;
-        if (act) s = dot_row<T>(q_s, Kh + (int64_t)(jb + lane) * kst, d) * scale;
-        float mn = fmaxf(m, warp_max(s));
-        float corr = (m == -CUDART_INF_F) ? 0.f : expf(m - mn);
-        float p = act ? expf(s - mn) : 0.f;
-        l = l * corr + warp_sum(p);
+    for (int u = 0; u < ND; ++u) acc[r][u] = 0.f;
+  }
+  for (uint32_t t = t0; t < t1; ++t) {
+    const uint32_t e = __ldg(tiles + t);
+    if ((e >> 28) == 0u) continue;                      // padding behind the row's entries
+    const int kb = (int)(e & 0x0FFFFFFFu);
+    uint4 bits[R];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) acc[u] *= corr;
-        m = mn;
-        while (word) {
-          int kk = __ffs(word) - 1;
-          word &= word - 1;
-          float pj = __shfl_sync(0xFFFFFFFFu, p, kk);
-          const T* vrow = Vh + (int64_t)(jb + kk) * vst;
+    for (int r = 0; r < R; ++r) bits[r] = dam_apply_bits(hb, e >> 28, i0 + r, kb, causal);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            int t_ = lane + 32 * u;
-            if (u < nd && t_ < d) acc[u] = fmaf(pj, Ld8<T>::one(vrow + t_), acc[u]);
+    for (int half = 0; half < 2; ++half) {
+      uint32_t any = 0u;
+#pragma unroll
+      for (int r = 0; r < R; ++r) any |= half ? (bits[r].z | bits[r].w) : (bits[r].x | bits[r].y);
+      if (!__syncthreads_or(any != 0u)) continue;       // (the previous stage is no longer read)
+      const int j0 = kb * DAM_TILE + half * kStageKeys;
+      load_stage<T>(k_s, pitch, Kh, kst, j0, sq.S, d);
+      load_stage<T>(v_s, d, Vh, vst, j0, sq.S, d);
+      __syncthreads();
+      if (!any) continue;                               // (the same in all lanes: the words are the row's)
+      float s[R][2];
+      dot_rows<R>(q_s, k0, k1, d, s);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint32_t w0 = half ? bits[r].z : bits[r].x, w1 = half ? bits[r].w : bits[r].y;
+        const bool a0 = (w0 >> lane) & 1u, a1 = (w1 >> lane) & 1u;
+        const float x0 = a0 ? s[r][0] * scale : -CUDART_INF_F, x1 = a1 ? s[r][1] * scale : -CUDART_INF_F;
+        const float mn = fmaxf(m[r], warp_max(fmaxf(x0, x1)));
+        const float corr = (m[r] == -CUDART_INF_F) ? 0.f : expf(m[r] - mn);
+        const float p0 = a0 ? expf(x0 - mn) : 0.f, p1 = a1 ? expf(x1 - mn) : 0.f;
+        l[r] = l[r] * corr + warp_sum(p0 + p1);
+        m[r] = mn;
+#pragma unroll
+        for (int u = 0; u < ND; ++u) acc[r][u] *= corr;
+        p_s[r * kStageKeys + lane] = p0;
+        p_s[r * kStageKeys + 32 + lane] = p1;
+      }
+      __syncwarp();
+#pragma unroll 2
+      for (int k = 0; k < kStageKeys; k += 4) {
+        float4 p[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) p[r] = *reinterpret_cast<const float4*>(p_s + r * kStageKeys + k);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+          for (int u = 0; u < ND; ++u) {
+            const int t_ = lane + 32 * u;
+            const float v = t_ < d ? v_s[(k + q) * d + t_] : 0.f;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              // (a key the row does not keep is left out, whatever its V row holds)
+              const float pk = q == 0 ? p[r].x : q == 1 ? p[r].y : q == 2 ? p[r].z : p[r].w;
+              if (pk != 0.f) acc[r][u] = fmaf(pk, v, acc[r][u]);
+            }
           }
         }
       }
+      __syncwarp();
     }
-    T* orow = O + (int64_t)(sq.tok_start + i) * ost + (int64_t)h * osh;
-    const float inv = l > 0.f ? 1.0f / l : 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      int t_ = lane + 32 * u;
-      if (u < nd && t_ < d) Ld8<T>::store(orow + t_, acc[u] * inv);
-    }
-    if (lane == 0) lse[(int64_t)h * total_tokens + sq.tok_start + i] = l > 0.f ? m + logf(l) : -CUDART_INF_F;
   }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int i = i0 + r;
+    if (i >= sq.S) break;
+    T* orow = O + (int64_t)(sq.tok_start + i) * ost + (int64_t)h * osh;
+    const float inv = l[r] > 0.f ? 1.0f / l[r] : 0.f;
+#pragma unroll
+    for (int u = 0; u < ND; ++u) {
+      const int t_ = lane + 32 * u;
+      if (t_ < d) Ld8<T>::store(orow + t_, acc[r][u] * inv);
+    }
+    if (lane == 0) lse[(int64_t)h * total_tokens + sq.tok_start + i] = l[r] > 0.f ? m[r] + logf(l[r]) : -CUDART_INF_F;
+  }
+}
+
+// R rows per warp: 4 where that still gives every SM a block of 8 warps, otherwise 1 (so that a short prompt's rows are
+// spread over the whole chip).
+constexpr int kRefWarps = 8;
+inline bool four_rows(long long rows, int sm_count) { return rows >= (long long)sm_count * kRefWarps * 4; }
+
+size_t score_smem(int d, int R) { return ((size_t)kStageKeys * k_pitch(d) + (size_t)kRefWarps * R * d) * sizeof(float); }
+size_t attn_smem(int d, int R) {
+  return ((size_t)kStageKeys * (k_pitch(d) + d) + (size_t)kRefWarps * R * (d + kStageKeys)) * sizeof(float);
+}
+
+template <typename T, int R>
+cudaError_t launch_scores(const void* Q, const void* K, const dam_shape_t* s, const DamBuildCtx& c, float* dump, cudaStream_t st) {
+  const size_t sm = score_smem(c.d, R);
+  cudaError_t e = cudaFuncSetAttribute(scores_ref_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((c.max_L + kRefWarps * R - 1) / (kRefWarps * R), c.num_seqs * c.Hq);
+  scores_ref_kernel<T, R><<<grid, kRefWarps * 32, sm, st>>>(c.blob, (const T*)Q, (const T*)K, c.Hq, c.Hq / c.Hkv, c.d, s->q_stride_tok,
+                                                            s->q_stride_head, s->k_stride_tok, s->k_stride_head, c.scale,
+                                                            c.pstar, dump);
+  return cudaGetLastError();
+}
+
+template <typename T, int R, int ND>
+cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
+                        float scale, void* O, float* lse, const int32_t* ranges, int rows, cudaStream_t st) {
+  const size_t sm = attn_smem(s->head_dim, R);
+  cudaError_t e = cudaFuncSetAttribute(attn_ref_kernel<T, R, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const dim3 grid(rows, DAM_TILE / (kRefWarps * R));
+  attn_ref_kernel<T, R, ND><<<grid, kRefWarps * 32, sm, st>>>(
+      (const unsigned char*)blob, (const T*)Q, (const T*)K, (const T*)V, s->num_q_heads, s->num_q_heads / s->num_kv_heads, s->head_dim,
+      s->q_stride_tok, s->q_stride_head, s->k_stride_tok, s->k_stride_head, s->v_stride_tok, s->v_stride_head, s->o_stride_tok,
+      s->o_stride_head, causal, scale, (T*)O, lse, s->total_tokens, ranges);
+  return cudaGetLastError();
+}
+
+template <typename T, int R>
+cudaError_t launch_attn_dims(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
+                             float scale, void* O, float* lse, const int32_t* ranges, int rows, cudaStream_t st) {
+  const int nd = (s->head_dim + 31) / 32;
+  if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
+  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
+  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
 }
 
 }  // namespace
@@ -194,20 +347,14 @@ __global__ void attn_ref_kernel(const unsigned char* blob, const T* __restrict__
 cudaError_t dam_launch_scores_ref(const void* Q, const void* K, const dam_shape_t* s, const DamBuildCtx& c,
                                   float* dump, cudaStream_t st) {
   if (c.max_L == 0) return cudaSuccess;
-  const int nw = 8;
-  dim3 grid((c.max_L + nw - 1) / nw, c.num_seqs * c.Hq);
-  size_t sm = (size_t)nw * c.d * sizeof(float);
-  int group = c.Hq / c.Hkv;
+  int dev = 0;
+  DamDeviceInfo di;
+  cudaError_t e = dam_current_device(&dev, &di);
+  if (e != cudaSuccess) return e;
+  const bool four = four_rows((long long)c.max_L * c.num_seqs * c.Hq, di.sm_count);
   if (c.dtype == DAM_F32)
-    scores_ref_kernel<float><<<grid, nw * 32, sm, st>>>(c.blob, (const float*)Q, (const float*)K, c.Hq, group, c.d,
-                                                        s->q_stride_tok, s->q_stride_head, s->k_stride_tok,
-                                                        s->k_stride_head, c.scale, c.pstar, dump);
-  else
-    scores_ref_kernel<__nv_bfloat16><<<grid, nw * 32, sm, st>>>(c.blob, (const __nv_bfloat16*)Q,
-                                                                (const __nv_bfloat16*)K, c.Hq, group, c.d,
-                                                                s->q_stride_tok, s->q_stride_head, s->k_stride_tok,
-                                                                s->k_stride_head, c.scale, c.pstar, dump);
-  return cudaGetLastError();
+    return four ? launch_scores<float, 4>(Q, K, s, c, dump, st) : launch_scores<float, 1>(Q, K, s, c, dump, st);
+  return four ? launch_scores<__nv_bfloat16, 4>(Q, K, s, c, dump, st) : launch_scores<__nv_bfloat16, 1>(Q, K, s, c, dump, st);
 }
 
 cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s,
@@ -219,18 +366,14 @@ cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, con
     rows += (s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b] + DAM_TILE - 1) / DAM_TILE;
   rows *= s->num_q_heads;
   if (rows == 0) return cudaSuccess;
-  const int nw = 4;
-  size_t sm = (size_t)nw * s->head_dim * sizeof(float);
-  int group = s->num_q_heads / s->num_kv_heads;
+  int dev = 0;
+  DamDeviceInfo di;
+  cudaError_t e = dam_current_device(&dev, &di);
+  if (e != cudaSuccess) return e;
+  const bool four = four_rows((long long)rows * DAM_TILE, di.sm_count);
   if (s->dtype == DAM_F32)
-    attn_ref_kernel<float><<<rows, nw * 32, sm, st>>>((const unsigned char*)blob, (const float*)Q, (const float*)K,
-        (const float*)V, s->num_q_heads, group, s->head_dim, s->q_stride_tok, s->q_stride_head, s->k_stride_tok,
-        s->k_stride_head, s->v_stride_tok, s->v_stride_head, s->o_stride_tok, s->o_stride_head, causal, scale,
-        (float*)O, lse, s->total_tokens, ranges);
-  else
-    attn_ref_kernel<__nv_bfloat16><<<rows, nw * 32, sm, st>>>((const unsigned char*)blob, (const __nv_bfloat16*)Q,
-        (const __nv_bfloat16*)K, (const __nv_bfloat16*)V, s->num_q_heads, group, s->head_dim, s->q_stride_tok,
-        s->q_stride_head, s->k_stride_tok, s->k_stride_head, s->v_stride_tok, s->v_stride_head, s->o_stride_tok,
-        s->o_stride_head, causal, scale, (__nv_bfloat16*)O, lse, s->total_tokens, ranges);
-  return cudaGetLastError();
+    return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st)
+                : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
+  return four ? launch_attn_dims<__nv_bfloat16, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st)
+              : launch_attn_dims<__nv_bfloat16, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
 }
