@@ -207,6 +207,7 @@ dam_status_t fill_ctx(const dam_shape_t* s, const dam_rule_t* r, void* mask, siz
   c->num_seqs = s->num_seqs; c->Hq = s->num_q_heads; c->Hkv = s->num_kv_heads; c->d = s->head_dim; c->dtype = s->dtype;
   c->total_qblocks = y->hdr.total_qblocks; c->rows = y->hdr.rows; c->prows = y->hdr.prows;
   c->max_L = y->max_L; c->max_W = y->max_W; c->max_nL = y->max_nL; c->max_nq = y->max_nq;
+  c->pcl_max = r->pcl_max;
   c->per_map = (r->transform == DAM_TRANSFORM_ZSCORE || r->transform == DAM_TRANSFORM_MINMAX) ? r->transform : 0;
   c->tau = r->tau; c->eps = r->eps;
   c->pstar = c->per_map ? INFINITY : find_pstar(r);

@@ -87,26 +87,46 @@ __global__ void init_blob_kernel(unsigned char* blob, DamHeader hdr, const int32
 
 // ---------------------------------------------------------------------------------------------
 // True-mask bits from an fp32 map P ([L][L] per (seq, head)): bit = [P >= p*], forced to 0 above
-// the diagonal.  One warp per (row, 32-column word); coalesced reads, one word written per warp.
+// the diagonal.  One warp per row; eight coalesced 128-byte reads in flight, one 32-bit word each, stored 16 bytes at a
+// time; nothing is read above the diagonal.  Bound by the read of the lower triangle: 32 maps of 512 x 512 57 -> 10.4 us (a warp per
+// word before, with two divisions each).  `active(p)` decides a cell of it.
 // ---------------------------------------------------------------------------------------------
+template <typename F>
+__device__ __forceinline__ void row_bits(uint32_t* __restrict__ Mrow, const float* __restrict__ Prow, int i, int W, int lane, F active) {
+  constexpr int kWords = 8;
+  for (int w0 = 0; w0 < W; w0 += kWords) {
+    uint32_t word = 0u;                          // lane k keeps word w0 + k
+    if (w0 * 32 <= i) {
+      float p[kWords];
+#pragma unroll
+      for (int k = 0; k < kWords; ++k) {
+        const int j = (w0 + k) * 32 + lane;
+        p[k] = j <= i ? __ldg(Prow + j) : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < kWords; ++k) {
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, (w0 + k) * 32 + lane <= i && active(p[k]));
+        if (lane == k) word = bal;
+      }
+    }
+    // W is a multiple of 4, so the eight words are one or two 16-byte pieces
+    const int src = 4 * (lane & 1);
+    const uint32_t x = __shfl_sync(0xFFFFFFFFu, word, src), y = __shfl_sync(0xFFFFFFFFu, word, src + 1),
+                   z = __shfl_sync(0xFFFFFFFFu, word, src + 2), w = __shfl_sync(0xFFFFFFFFu, word, src + 3);
+    if (lane < 2 && w0 + 4 * lane < W) *reinterpret_cast<uint4*>(Mrow + w0 + 4 * lane) = make_uint4(x, y, z, w);
+  }
+}
+
 __global__ void bits_from_scores_kernel(unsigned char* blob, const float* __restrict__ P, float pstar) {
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   const int sh = blockIdx.y;
   const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
   const DamSeq sq = blob_seqs(blob, H)[b];
-  if (sq.L == 0) return;
   uint32_t* M = reinterpret_cast<uint32_t*>(blob + H->off_true) + sq.true_off + (uint64_t)h * sq.L * sq.W;
   const float* Ph = P + sq.p_off + (uint64_t)h * sq.L * sq.L;
-  const int lane = threadIdx.x & 31;
-  const long long nitems = (long long)sq.L * sq.W;
-  const long long wstride = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long it = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitems; it += wstride) {
-    int i = (int)(it / sq.W), w = (int)(it % sq.W);
-    int j = w * 32 + lane;
-    float p = (j < sq.L && j <= i) ? __ldg(Ph + (size_t)i * sq.L + j) : 0.0f;
-    uint32_t word = __ballot_sync(0xFFFFFFFFu, p >= pstar);
-    if (lane == 0) M[(size_t)i * sq.W + w] = word;
-  }
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (i < sq.L)
+    row_bits(M + (size_t)i * sq.W, Ph + (size_t)i * sq.L, i, sq.W, threadIdx.x & 31, [&](float p) { return p >= pstar; });
 }
 
 // Transpose of a 32 x 32 bit matrix held one row per lane: lane c returns column c (bit r = bit c of row r).
@@ -739,25 +759,15 @@ __global__ void bits_from_scores_per_map_kernel(unsigned char* blob, const float
   }
   uint32_t* M = reinterpret_cast<uint32_t*>(blob + H->off_true) + sq.true_off + (uint64_t)h * sq.L * sq.W;
   const float* Ph = P + sq.p_off + (uint64_t)h * sq.L * sq.L;
-  const int lane = threadIdx.x & 31;
-  const long long nitems = (long long)sq.L * sq.W;
-  const long long wstride = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long it = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitems; it += wstride) {
-    const int i = (int)(it / sq.W), w = (int)(it % sq.W);
-    const int j = w * 32 + lane;
-    const bool in = j < sq.L && j <= i;
-    const float x = fmaxf(in ? __ldg(Ph + (size_t)i * sq.L + j) : 0.0f, eps_f);
-    const uint32_t word = __ballot_sync(0xFFFFFFFFu, in && (double)x >= thr);
-    if (lane == 0) M[(size_t)i * sq.W + w] = word;
-  }
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (i < sq.L)
+    row_bits(M + (size_t)i * sq.W, Ph + (size_t)i * sq.L, i, sq.W, threadIdx.x & 31,
+             [&](float p) { return (double)fmaxf(p, eps_f) >= thr; });
 }
 
 cudaError_t dam_launch_bits_from_scores(const float* P, const DamBuildCtx& c, cudaStream_t st) {
   if (c.max_L == 0) return cudaSuccess;
-  long long items = (long long)c.max_L * c.max_W;
-  int bx = (int)((items + 7) / 8);
-  if (bx > 4096) bx = 4096;
-  dim3 grid(bx, c.num_seqs * c.Hq);
+  const dim3 grid((c.max_L + 7) / 8, c.num_seqs * c.Hq);      // a warp per row
   if (c.per_map) {
     // the statistics borrow the first bytes of every map's counter area, which is cleared again afterwards
     map_stats_kernel<<<c.num_seqs * c.Hq, 1024, 0, st>>>(c.blob, P, c.scratch, c.off_cnt, c.eps);
@@ -772,33 +782,75 @@ cudaError_t dam_launch_bits_from_scores(const float* P, const DamBuildCtx& c, cu
 
 // ---------------------------------------------------------------------------------------------
 // Multi-sample capture (Sec. 4.2.2): A[h][i][j] += sum over the samples b of a batch of P_b[h][i][j]
-// (i, j < L_b = min(S_b, L_max)), C[i] += #{b : L_b > i}.  One thread per cell of a row; the samples
-// of the batch are added in index order, so the fp32 sums do not depend on the launch.
+// (i, j < L_b = min(S_b, L_max)), C[i] += #{b : L_b > i}.  The samples of the batch are added in index order, so the
+// fp32 sums do not depend on the launch.
 // ---------------------------------------------------------------------------------------------
-__global__ void capture_accumulate_kernel(const float* __restrict__ P, const int32_t* __restrict__ cu, int num_seqs,
-                                          int Hq, int Lmax, float* __restrict__ A, int32_t* __restrict__ C) {
-  const int i = blockIdx.x, h = blockIdx.y;
-  unsigned long long p_off = 0;                      // fp32 elements before sample b in the score tensor
+// A warp per row; VEC: four columns per lane and read (every row of P and A starts on a 16-byte boundary).  The samples'
+// reads of a column group are requested together, eight at a time, and added in order in registers, so that A is read and
+// written once.  Bound by the read of the lower triangles of P: 8 maps of 512 x 512 x 32 heads 99 -> 40 us (one sample
+// after the other, A read and written for each, before).  A warp per 128 columns instead of per row: 58 us.
+constexpr int kCapBatch = 8;
+
+template <int VEC>
+__global__ void __launch_bounds__(256)
+capture_accumulate_kernel(const float* __restrict__ P, const int32_t* __restrict__ cu, int num_seqs,
+                          int Hq, int Lmax, float* __restrict__ A, int32_t* __restrict__ C) {
+  const int lane = threadIdx.x & 31, h = blockIdx.y;
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (i >= Lmax) return;
+  float* Ar = A + ((unsigned long long)h * Lmax + i) * Lmax;
+  unsigned long long p_off = 0;                      // fp32 elements before sample b0 in the score tensor
   int cnt = 0;
-  for (int b = 0; b < num_seqs; ++b) {
-    const int S = cu[b + 1] - cu[b];
-    const int L = S < Lmax ? S : Lmax;
-    if (i < L) {
-      ++cnt;
-      const float* Pr = P + p_off + ((unsigned long long)h * L + i) * L;
-      float* Ar = A + ((unsigned long long)h * Lmax + i) * Lmax;
-      for (int j = threadIdx.x; j <= i; j += blockDim.x) Ar[j] += __ldg(Pr + j);
+  for (int b0 = 0; b0 < num_seqs; b0 += kCapBatch) {
+    const float* row[kCapBatch];                     // a sample without row i reads A's (and is not added)
+    uint32_t has = 0u;
+#pragma unroll
+    for (int u = 0; u < kCapBatch; ++u) {
+      row[u] = Ar;
+      if (b0 + u < num_seqs) {
+        const int S = __ldg(cu + b0 + u + 1) - __ldg(cu + b0 + u);
+        const int L = S < Lmax ? S : Lmax;
+        if (i < L) { row[u] = P + p_off + ((unsigned long long)h * L + i) * L; has |= 1u << u; }
+        p_off += (unsigned long long)Hq * L * L;
+      }
     }
-    p_off += (unsigned long long)Hq * L * L;
+    cnt += __popc(has);
+    for (int j = lane * VEC; j <= i; j += 32 * VEC) {
+      if (VEC == 4 && j + 3 <= i) {
+        float4 v[kCapBatch];
+        float4 a = *reinterpret_cast<const float4*>(Ar + j);
+#pragma unroll
+        for (int u = 0; u < kCapBatch; ++u) v[u] = *reinterpret_cast<const float4*>(row[u] + j);
+#pragma unroll
+        for (int u = 0; u < kCapBatch; ++u)
+          if (has >> u & 1u) { a.x += v[u].x; a.y += v[u].y; a.z += v[u].z; a.w += v[u].w; }
+        *reinterpret_cast<float4*>(Ar + j) = a;
+      } else {
+        for (int k = j; k < j + VEC && k <= i; ++k) {
+          float a = Ar[k], v[kCapBatch];
+#pragma unroll
+          for (int u = 0; u < kCapBatch; ++u) v[u] = row[u][k];
+#pragma unroll
+          for (int u = 0; u < kCapBatch; ++u)
+            if (has >> u & 1u) a += v[u];
+          Ar[k] = a;
+        }
+      }
+    }
   }
-  if (h == 0 && threadIdx.x == 0) C[i] += cnt;
+  if (h == 0 && lane == 0) C[i] += cnt;
 }
 
 // Averaged map in the layout the rule kernels read: for every (sequence b, head h) of the target shape,
-// P_out[i][j] = A[h][i][j] / (float(C[i]) + eps) for j <= i < L_b, 0 above the diagonal (IEEE single division).
-__global__ void capture_average_kernel(const float* __restrict__ A, const int32_t* __restrict__ C, int Lmax, float eps,
-                                       const int32_t* __restrict__ cu, int num_seqs, int Hq, float* __restrict__ P_out) {
-  const int i = blockIdx.x, h = blockIdx.y;
+// P_out[i][j] = A[h][i][j] / (float(C[i]) + eps) for j <= i < L_b, 0 above the diagonal (IEEE single division).  A warp per
+// row, VEC columns per lane and access; bound by the write of the maps (32 maps of 512 x 512: 21.5 -> 12 us).
+template <int VEC>
+__global__ void __launch_bounds__(256)
+capture_average_kernel(const float* __restrict__ A, const int32_t* __restrict__ C, int Lmax, float eps,
+                       const int32_t* __restrict__ cu, int num_seqs, int Hq, float* __restrict__ P_out) {
+  const int lane = threadIdx.x & 31, h = blockIdx.y;
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (i >= Lmax) return;
   const float den = (float)C[i] + eps;
   const float* Ar = A + ((unsigned long long)h * Lmax + i) * Lmax;
   unsigned long long p_off = 0;
@@ -807,10 +859,35 @@ __global__ void capture_average_kernel(const float* __restrict__ A, const int32_
     const int L = S < Lmax ? S : Lmax;
     if (i < L) {
       float* Pr = P_out + p_off + ((unsigned long long)h * L + i) * L;
-      for (int j = threadIdx.x; j < L; j += blockDim.x) Pr[j] = j <= i ? Ar[j] / den : 0.f;
+      for (int j = lane * VEC; j < L; j += 32 * VEC) {
+        if constexpr (VEC == 4) {
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (j <= i) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(Ar + j));
+            v.x = a.x / den;
+            if (j + 1 <= i) v.y = a.y / den;
+            if (j + 2 <= i) v.z = a.z / den;
+            if (j + 3 <= i) v.w = a.w / den;
+          }
+          *reinterpret_cast<float4*>(Pr + j) = v;
+        } else {
+          Pr[j] = j <= i ? __ldg(Ar + j) / den : 0.f;
+        }
+      }
     }
     p_off += (unsigned long long)Hq * L * L;
   }
+}
+
+// Four columns per lane when every row of the maps (L floats, one behind the other) and of A (Lmax floats) starts on a
+// 16-byte boundary.
+static bool capture_vec4(const dam_shape_t* s, int Lmax, const void* P, const void* A) {
+  if (Lmax % 4 || reinterpret_cast<uintptr_t>(P) % 16 || reinterpret_cast<uintptr_t>(A) % 16) return false;
+  for (int b = 0; b < s->num_seqs; ++b) {
+    const int S = s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b];
+    if ((S < Lmax ? S : Lmax) % 4) return false;
+  }
+  return true;
 }
 
 cudaError_t dam_launch_capture_accumulate(const float* P, const dam_shape_t* s, int Lmax, float* A, int32_t* C,
@@ -822,8 +899,11 @@ cudaError_t dam_launch_capture_accumulate(const float* P, const dam_shape_t* s, 
     maxL = L > maxL ? L : maxL;
   }
   if (maxL == 0) return cudaSuccess;
-  capture_accumulate_kernel<<<dim3(maxL, s->num_q_heads), 256, 0, st>>>(P, s->cu_seqlens_dev, s->num_seqs,
-                                                                        s->num_q_heads, Lmax, A, C);
+  const dim3 grid((maxL + 7) / 8, s->num_q_heads);
+  if (capture_vec4(s, Lmax, P, A))
+    capture_accumulate_kernel<4><<<grid, 256, 0, st>>>(P, s->cu_seqlens_dev, s->num_seqs, s->num_q_heads, Lmax, A, C);
+  else
+    capture_accumulate_kernel<1><<<grid, 256, 0, st>>>(P, s->cu_seqlens_dev, s->num_seqs, s->num_q_heads, Lmax, A, C);
   return cudaGetLastError();
 }
 
@@ -836,8 +916,11 @@ cudaError_t dam_launch_capture_average(const float* A, const int32_t* C, int Lma
     maxL = L > maxL ? L : maxL;
   }
   if (maxL == 0) return cudaSuccess;
-  capture_average_kernel<<<dim3(maxL, s->num_q_heads), 256, 0, st>>>(A, C, Lmax, eps, s->cu_seqlens_dev, s->num_seqs,
-                                                                     s->num_q_heads, P_out);
+  const dim3 grid((maxL + 7) / 8, s->num_q_heads);
+  if (capture_vec4(s, Lmax, P_out, A))
+    capture_average_kernel<4><<<grid, 256, 0, st>>>(A, C, Lmax, eps, s->cu_seqlens_dev, s->num_seqs, s->num_q_heads, P_out);
+  else
+    capture_average_kernel<1><<<grid, 256, 0, st>>>(A, C, Lmax, eps, s->cu_seqlens_dev, s->num_seqs, s->num_q_heads, P_out);
   return cudaGetLastError();
 }
 

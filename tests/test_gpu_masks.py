@@ -344,6 +344,51 @@ def test_multi_sample_capture_masks_bit_exact():
     H.check_blob_against_oracle(blob, tshape, masks)
 
 
+@pytest.mark.parametrize("pcl,lengths", [
+    (1, [1, 3]),                            # one cell
+    (37, [50, 20, 37, 9]),                  # odd rows: element-wise stores and reads
+    (100, [100, 300, 60, 8]),               # rows of 16-byte but not of 32-byte multiples
+    (136, [136, 520, 72, 128, 136, 8, 200, 64, 136, 40]),        # 32-byte rows; more samples than are read together
+    (264, [264, 1000]),                     # nine 32-column words in three tiles
+])
+def test_capture_of_maps_edges(pcl, lengths):
+    """The dumped maps against a float64 softmax, their sums and averages exactly (the same fp32 additions and divisions in
+    the same order), and the true mask of the averages against the oracle, at the edges of rows and of vector accesses."""
+    Hq, Hkv, d = 4, 2, 64
+    w = synth.small_case(0, Hq, Hkv, d, max(pcl, 8), seed=50, dtype=torch.bfloat16, lengths=lengths)
+    shape = B.make_shape(w.cu_seqlens, Hq, Hkv, d, w.Q.dtype, DEV)
+    rule = B.make_rule(pcl, w.tau, w.mu)
+    dump = torch.full((sum(Hq * min(S, pcl) ** 2 for S in lengths),), float("nan"), device=DEV)
+    B.dam_build_masks(w.Q.to(DEV), w.K.to(DEV), shape, rule, scores_dump=dump)
+    P = H.split_dump(dump.cpu().numpy(), lengths, Hq, pcl)
+    want_A, want_C = np.zeros((Hq, pcl, pcl), np.float32), np.zeros(pcl, np.int32)
+    for b, S in enumerate(lengths):
+        L = min(S, pcl)
+        want_C[:L] += 1
+        for h in range(Hq):
+            q, k = (x[w.cu_seqlens[b]: w.cu_seqlens[b] + L, i].double() for x, i in ((w.Q, h), (w.K, h // 2)))
+            s = (q @ k.T / np.sqrt(d)).masked_fill(torch.ones(L, L).triu(1).bool(), -np.inf)
+            # logits of at most 12 in magnitude with fp32 sums of 64 terms: 64 * 12 * 2^-24 = 5e-5, plus the exponential
+            assert np.abs(P[b][h] - torch.softmax(s, 1).numpy()).max() <= 1e-4
+            assert not np.triu(P[b][h], 1).any()
+            want_A[h, :L, :L] += P[b][h]
+    A = torch.zeros(Hq, pcl, pcl, dtype=torch.float32, device=DEV)
+    C = torch.zeros(pcl, dtype=torch.int32, device=DEV)
+    B.dam_capture_accumulate(dump, shape, pcl, A, C)
+    assert np.array_equal(A.cpu().numpy(), want_A) and np.array_equal(C.cpu().numpy(), want_C)
+    avg = B.dam_capture_average(A, C, pcl, 1e-8, shape)
+    blob, _ = B.dam_build_masks_from_scores(avg, shape, rule)
+    mb = B.MaskBlob(blob)
+    Pa = H.split_dump(avg.cpu().numpy(), lengths, Hq, pcl)
+    for b, S in enumerate(lengths):
+        L = min(S, pcl)
+        for h in range(Hq):
+            want = want_A[h, :L, :L] / (want_C[:L, None].astype(np.float32) + np.float32(1e-8))
+            assert np.array_equal(Pa[b][h], want)
+            hm = orc.head_mask_from_probs(np.ascontiguousarray(want), S, w.tau, w.mu)
+            assert np.array_equal(mb.true_mask(b, h), hm.M)
+
+
 @pytest.mark.parametrize("transform,lam,tau", [
     ("log", 0.0, 13.0), ("sqrt", 0.0, 0.1), ("arcsinh", 0.0, 0.01), ("average", 0.0, 0.01),
     ("boxcox", 0.25, 1.5), ("boxcox", 0.0, 13.0), ("yeo_johnson", 0.5, 0.01), ("yeo_johnson", 0.0, 0.01),
