@@ -445,7 +445,6 @@ dam_status_t dam_decode_attention(const void* q, const void* K, const void* V, c
   if (scratch_bytes < 256) return DAM_ERR_BUFFER_TOO_SMALL;
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)shape->head_dim);
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(scratch, 0, 256, cs) != cudaSuccess) return DAM_ERR_CUDA;
   cudaError_t e = dam_launch_decode(q, K, V, mask, shape, positions_dev, scale, O, lse, scratch, cs);
   if (e == cudaErrorNotSupported) return DAM_ERR_UNSUPPORTED;
   return e == cudaSuccess ? DAM_OK : DAM_ERR_CUDA;

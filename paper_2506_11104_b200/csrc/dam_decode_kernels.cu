@@ -284,6 +284,8 @@ cudaError_t dam_launch_decode(const void* q, const void* K, const void* V, const
   // bf16 with a GQA group of at most 8 heads: one block per (sequence, KV head) on the tensor cores
   const cudaError_t ge = dam_launch_decode_group(q, K, V, blob, s, pos_dev, scale, O, lse, scratch, st);
   if (ge != cudaErrorNotSupported) return ge;
+  const cudaError_t ce = cudaMemsetAsync(scratch, 0, 256, st);      // (the grouped kernel writes the scratch block itself)
+  if (ce != cudaSuccess) return ce;
   const dim3 grid((unsigned)s->num_q_heads, (unsigned)s->num_seqs);
   const int group = s->num_q_heads / s->num_kv_heads;
   const float sl2 = scale * 1.4426950408889634f;

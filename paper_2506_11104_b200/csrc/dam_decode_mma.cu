@@ -11,8 +11,12 @@
 // keep gets -inf before the softmax of that head's column (probability exactly 0).  Each warp walks its own chunks
 // of 16 keys with a running softmax per head; the warps are merged through shared memory at the end.
 //
+// Few (sequence, KV head) pairs leave most SMs idle: then a cluster of two, four or eight blocks takes one, each with its
+// share of the chunks, and the partial results are merged through distributed shared memory (decode_split).
+//
 // This is a gather of a few hundred 256-byte rows per head: bound by HBM / L2 bandwidth and latency, not by the
 // tensor cores, which is why the small synchronous MMA shape serves (a 128-row tcgen05 tile would be 97 % padding).
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -26,6 +30,7 @@ constexpr int kGStages = 1;           // chunks of 16 keys a warp holds in share
 constexpr int kGMinBlocks = 4;         // resident blocks per SM the register limit is sized for
 constexpr int kGChunk = 16;           // keys per chunk (the K dimension of the P V instruction)
 constexpr int kGRoundWords = 128;     // pattern words expanded per round (at most 4096 keys)
+constexpr int kGMaxSplit = 8;         // blocks of a cluster (the largest portable size)
 constexpr int kGMaxGroup = 8;         // query heads per KV head this kernel takes (rows 0..7 of the m16 tile)
 
 __device__ __forceinline__ float g_ex2(float x) {
@@ -91,20 +96,21 @@ struct GLayout {
   static constexpr int part_bytes = kGChunk * row_bytes;            // the K (or V) rows of one chunk
   static constexpr int stage_bytes = 2 * part_bytes;
   static constexpr int stages_total = kGWarps * kGStages * stage_bytes;
-  static constexpr int merge_bytes = kGWarps * kGMaxGroup * (D + 2) * 4;   // per warp and head: O row, m, l
+  static constexpr int merge_bytes = (kGWarps + 1) * kGMaxGroup * (D + 2) * 4;   // per warp and head, and folded per head: O row, m, l
   static constexpr int work_bytes = stages_total > merge_bytes ? stages_total : merge_bytes;   // the merge reuses the stages
   static constexpr int codes_off = work_bytes;                              // u16 per listed key: round-local word * 32 + bit
   static constexpr int words_off = codes_off + kGRoundWords * 32 * 2;       // u32 [head][round-local word]: the round's pattern words
   static constexpr int total = words_off + kGMaxGroup * kGRoundWords * 4;
 };
 
-template <int D>
+// CLUSTER: the blocks of a cluster share one (sequence, KV head).
+template <int D, bool CLUSTER>
 __global__ void __launch_bounds__(kGWarps * 32, kGMinBlocks)
 decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ K,
                     const __nv_bfloat16* __restrict__ V, const unsigned char* __restrict__ blob,
                     const int32_t* __restrict__ cu, const int32_t* __restrict__ pos_dev, int num_seqs, int Hq, int G,
                     int64_t kst, int64_t ksh, int64_t vst, int64_t vsh, float scale_log2,
-                    __nv_bfloat16* __restrict__ O, float* __restrict__ lse, uint32_t* status) {
+                    __nv_bfloat16* __restrict__ O, float* __restrict__ lse, uint32_t* __restrict__ scratch) {
   using LY = GLayout<D>;
   constexpr int KS = D / 16;                 // k-steps of S = Q K^T
   constexpr int kThreads = kGWarps * 32;
@@ -112,17 +118,31 @@ decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
   __shared__ int warp_tot[kGWarps];
   unsigned short* codes = reinterpret_cast<unsigned short*>(gsm + LY::codes_off);
   uint32_t* whs = reinterpret_cast<uint32_t*>(gsm + LY::words_off);
-  const int kvh = blockIdx.x, b = blockIdx.y, h0 = kvh * G;
+  const int nsplit = CLUSTER ? (int)cooperative_groups::this_cluster().num_blocks() : 1;
+  const int split = CLUSTER ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+  const int kvh = CLUSTER ? blockIdx.x / nsplit : blockIdx.x, b = blockIdx.y, h0 = kvh * G;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, row = lane >> 2, quad = lane & 3;
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   // the header, the position and the sequence bounds are requested together (one round trip to memory, not three)
   const int pos = __ldg(pos_dev + b), cu0 = __ldg(cu + b), cu1 = __ldg(cu + b + 1);
-  const bool bad = H->magic != DAM_MAGIC || H->num_seqs != num_seqs || H->num_q_heads != Hq || pos < 0 || pos >= cu1 - cu0;
+  const bool bad_blob = H->magic != DAM_MAGIC || H->num_seqs != num_seqs || H->num_q_heads != Hq;
+  const bool bad = bad_blob || pos < 0 || pos >= cu1 - cu0;
+  if (blockIdx.x == 0 && b == 0) {
+    // the scratch block for the whole call, its status word included: this block alone looks at every sequence's position
+    bool any = bad_blob;
+    for (int x = tid; x < num_seqs; x += kThreads) {
+      const int p = __ldg(pos_dev + x);
+      any |= p < 0 || p >= __ldg(cu + x + 1) - __ldg(cu + x);
+    }
+    const int st = __syncthreads_or(any) ? (int)DAM_ERR_INVALID_ARGUMENT : 0;
+    if (tid < 64) scratch[tid] = tid == 1 ? (uint32_t)st : 0u;
+  }
   if (bad) {
-    if (tid == 0) atomicMax(status, (uint32_t)DAM_ERR_INVALID_ARGUMENT);
-    for (int t = tid; t < G * D; t += kThreads) O[((int64_t)b * Hq + h0) * D + t] = __float2bfloat16_rn(0.f);
-    if (tid < G) lse[(int64_t)b * Hq + h0 + tid] = -CUDART_INF_F;
-    return;
+    if (split == 0) {
+      for (int t = tid; t < G * D; t += kThreads) O[((int64_t)b * Hq + h0) * D + t] = __float2bfloat16_rn(0.f);
+      if (tid < G) lse[(int64_t)b * Hq + h0 + tid] = -CUDART_INF_F;
+    }
+    return;                                                  // (all blocks of a cluster)
   }
   const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[b];
   const int L = sq.L, W = sq.W;
@@ -210,6 +230,7 @@ decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
 
     // ---- chunks of 16 keys, dealt to the warps round robin; a warp copies chunk i + 1 while it works on chunk i
     const int nchunks = (total + kGChunk - 1) / kGChunk;
+    const int w_first = split * kGWarps + warp, w_step = nsplit * kGWarps;      // this warp's chunks: w_first, w_first + w_step, ...
     auto issue = [&](int c, int stage) {
       const uint32_t dstK = stage0 + stage * LY::stage_bytes, dstV = dstK + LY::part_bytes;
       constexpr int PPR = LY::row_bytes / 16;               // 16-byte pieces per row
@@ -227,13 +248,13 @@ decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
     // kGStages - 1 groups are complete" always means "this iteration's chunk has landed")
 #pragma unroll
     for (int pre = 0; pre < kGStages - 1; ++pre) {
-      if (warp + pre * kGWarps < nchunks) issue(warp + pre * kGWarps, pre);
+      if (w_first + pre * w_step < nchunks) issue(w_first + pre * w_step, pre);
       cp_async_commit();
     }
     int it = 0;
-    for (int c = warp; c < nchunks; c += kGWarps, ++it) {
+    for (int c = w_first; c < nchunks; c += w_step, ++it) {
       const int stage = it % kGStages;
-      if (c + (kGStages - 1) * kGWarps < nchunks) issue(c + (kGStages - 1) * kGWarps, (it + kGStages - 1) % kGStages);
+      if (c + (kGStages - 1) * w_step < nchunks) issue(c + (kGStages - 1) * w_step, (it + kGStages - 1) % kGStages);
       cp_async_commit();
       cp_async_wait<kGStages - 1>();
       __syncwarp();
@@ -308,6 +329,49 @@ decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
       if (row == 0) { dst[D] = m[e]; dst[D + 1] = l[e]; }
     }
   }
+  if constexpr (CLUSTER) {
+    // each block folds its own warps into one row per head, which the other blocks of the cluster read
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    float* folded = mg + kGWarps * kGMaxGroup * (D + 2);
+    __syncthreads();
+    for (int e = tid; e < G * (D + 2); e += kThreads) {
+      const int g = e / (D + 2), t = e % (D + 2);
+      float mxw = -CUDART_INF_F, acc = 0.f;
+#pragma unroll
+      for (int w = 0; w < kGWarps; ++w) mxw = fmaxf(mxw, mg[((size_t)w * kGMaxGroup + g) * (D + 2) + D]);
+#pragma unroll
+      for (int w = 0; w < kGWarps; ++w) {
+        const float* src = mg + ((size_t)w * kGMaxGroup + g) * (D + 2);
+        acc += src[D] == -CUDART_INF_F ? 0.f : src[t] * g_ex2(src[D] - mxw);
+      }
+      folded[e] = t == D ? mxw : acc;
+    }
+    cl.sync();
+    for (int e = split * kThreads + tid; e < G * D; e += nsplit * kThreads) {
+      const int g = e / D, t = e % D;
+      float mv[kGMaxSplit], lv[kGMaxSplit], ov[kGMaxSplit], mx = -CUDART_INF_F;
+#pragma unroll
+      for (int k = 0; k < kGMaxSplit; ++k) {
+        mv[k] = -CUDART_INF_F; lv[k] = ov[k] = 0.f;
+        if (k < nsplit) {
+          const float* src = cl.map_shared_rank(folded, k) + g * (D + 2);
+          mv[k] = src[D]; lv[k] = src[D + 1]; ov[k] = src[t];
+        }
+        mx = fmaxf(mx, mv[k]);
+      }
+      float lt = 0.f, ot = 0.f;
+#pragma unroll
+      for (int k = 0; k < kGMaxSplit; ++k) {
+        const float f = mv[k] == -CUDART_INF_F ? 0.f : g_ex2(mv[k] - mx);
+        lt += lv[k] * f;
+        ot += ov[k] * f;
+      }
+      O[((int64_t)b * Hq + h0 + g) * D + t] = __float2bfloat16_rn(lt > 0.f ? ot / lt : 0.f);
+      if (t == 0) lse[(int64_t)b * Hq + h0 + g] = lt > 0.f ? (mx + log2f(lt)) * 0.6931471805599453f : -CUDART_INF_F;
+    }
+    cl.sync();                                               // the folded rows stay until every block has read them
+    return;
+  }
   __syncthreads();
   for (int e = tid; e < G * D; e += kThreads) {
     const int g = e / D, t = e % D;
@@ -327,6 +391,36 @@ decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
   }
 }
 
+// Blocks per (sequence, KV head), from the number of those pairs: a block spends about 6 us before its first rows arrive
+// and then streams its list, so splitting the list pays as long as all blocks are resident at once (four per SM) and the
+// chip is not yet bound by the gather itself.  us per launch with 1 / 2 / 4 / 8 blocks (32 / 8 heads, 148 SMs):
+//   pairs    8   19.2 / 15.7 / 12.1 / 11.0      32   28.3 / 20.0 / 14.8 / 13.4      64   28.8 / 20.5 / 16.5 / 16.4
+//          128   30.0 / 22.6 / 20.0 / 28.0     192   32.6 / 25.3 / 31.6 / 39.0     384   44.9 / 38.3 / 41.9 / 63.9
+//          512   41.6 / 49.7 / 61.7 / 92.3 (longer lists)
+int decode_split(int pairs, int sm_count) {
+  if (pairs * 8 <= 3 * sm_count) return 8;
+  if (pairs <= sm_count) return 4;
+  if (pairs <= 3 * sm_count) return 2;
+  return 1;
+}
+
+template <int D>
+cudaError_t launch_group(const __nv_bfloat16* q, const __nv_bfloat16* K, const __nv_bfloat16* V, const unsigned char* blob,
+                         const dam_shape_t* s, const int32_t* pos_dev, float scale_log2, __nv_bfloat16* O, float* lse,
+                         uint32_t* scratch, int split, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(s->num_kv_heads * split), (unsigned)s->num_seqs);
+  cfg.blockDim = dim3(kGWarps * 32); cfg.dynamicSmemBytes = GLayout<D>::total; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = split > 1 ? 1 : 0;
+  const int G = s->num_q_heads / s->num_kv_heads;
+  return cudaLaunchKernelEx(&cfg, split > 1 ? decode_group_kernel<D, true> : decode_group_kernel<D, false>, q, K, V, blob,
+                            (const int32_t*)s->cu_seqlens_dev, pos_dev, (int)s->num_seqs, (int)s->num_q_heads, G, s->k_stride_tok,
+                            s->k_stride_head, s->v_stride_tok, s->v_stride_head, scale_log2, O, lse, scratch);
+}
+
 }  // namespace
 
 // bf16, head_dim 64 or 128, at most 8 query heads per KV head; cudaErrorNotSupported otherwise (the caller then
@@ -343,26 +437,20 @@ cudaError_t dam_launch_decode_group(const void* q, const void* K, const void* V,
   const int smem = s->head_dim == 128 ? GLayout<128>::total : GLayout<64>::total;
   if (di.smem_optin < smem) return cudaErrorNotSupported;
   if ((e = dam_device_table().once(dev, DAM_SETUP_DECODE_SMEM, [](void) -> cudaError_t {
-         cudaError_t r = cudaFuncSetAttribute(decode_group_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, GLayout<128>::total);
-         if (r != cudaSuccess) return r;
-         return cudaFuncSetAttribute(decode_group_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, GLayout<64>::total);
+         cudaError_t r;
+         if ((r = cudaFuncSetAttribute(decode_group_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GLayout<128>::total)) != cudaSuccess) return r;
+         if ((r = cudaFuncSetAttribute(decode_group_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GLayout<128>::total)) != cudaSuccess) return r;
+         if ((r = cudaFuncSetAttribute(decode_group_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GLayout<64>::total)) != cudaSuccess) return r;
+         return cudaFuncSetAttribute(decode_group_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GLayout<64>::total);
        })) != cudaSuccess)
     return e;
-  const dim3 grid((unsigned)s->num_kv_heads, (unsigned)s->num_seqs);
   const float sl2 = scale * 1.4426950408889634f;
-  uint32_t* status = reinterpret_cast<uint32_t*>(scratch) + 1;
+  const int split = decode_split(s->num_kv_heads * s->num_seqs, di.sm_count);
   const __nv_bfloat16 *qq = reinterpret_cast<const __nv_bfloat16*>(q), *kk = reinterpret_cast<const __nv_bfloat16*>(K),
                       *vv = reinterpret_cast<const __nv_bfloat16*>(V);
   const unsigned char* bl = reinterpret_cast<const unsigned char*>(blob);
-  if (s->head_dim == 128)
-    decode_group_kernel<128><<<grid, kGWarps * 32, smem, st>>>(qq, kk, vv, bl, s->cu_seqlens_dev, pos_dev, s->num_seqs,
-                                                               s->num_q_heads, G, s->k_stride_tok, s->k_stride_head,
-                                                               s->v_stride_tok, s->v_stride_head, sl2,
-                                                               reinterpret_cast<__nv_bfloat16*>(O), lse, status);
-  else
-    decode_group_kernel<64><<<grid, kGWarps * 32, smem, st>>>(qq, kk, vv, bl, s->cu_seqlens_dev, pos_dev, s->num_seqs,
-                                                              s->num_q_heads, G, s->k_stride_tok, s->k_stride_head,
-                                                              s->v_stride_tok, s->v_stride_head, sl2,
-                                                              reinterpret_cast<__nv_bfloat16*>(O), lse, status);
-  return cudaGetLastError();
+  __nv_bfloat16* oo = reinterpret_cast<__nv_bfloat16*>(O);
+  uint32_t* scr = reinterpret_cast<uint32_t*>(scratch);
+  return s->head_dim == 128 ? launch_group<128>(qq, kk, vv, bl, s, pos_dev, sl2, oo, lse, scr, split, st)
+                            : launch_group<64>(qq, kk, vv, bl, s, pos_dev, sl2, oo, lse, scr, split, st);
 }

@@ -86,6 +86,16 @@ def test_decode_matches_oracle(cache_lengths, build_lengths, Hq, Hkv, d, dtype, 
         _decode_and_check(w, blob, masks, [p[min(k, len(p) - 1)] for p in per_seq])
 
 
+@pytest.mark.parametrize("num_seqs,d", [(55, 64), (56, 128), (148, 64), (149, 64), (444, 64), (445, 64)])
+def test_decode_split_over_blocks(num_seqs, d):
+    """Enough (sequence, KV head) pairs for 8, 4, 2 and 1 blocks each (both sides of every boundary on 148 SMs), with key
+    lists from empty to longer than one chunk per warp."""
+    w = synth.small_case(0, 2, 1, d, 96, seed=12, dtype=torch.bfloat16, lengths=[200] * num_seqs)
+    blob, masks = _build(w, [200] * num_seqs)
+    rng = np.random.default_rng(num_seqs)
+    _decode_and_check(w, blob, masks, [int(p) for p in rng.integers(0, 200, size=num_seqs)])
+
+
 def test_decode_agrees_with_prefill_rows():
     """The same rows through the tile-list kernel and through the pattern-walking kernel."""
     w = synth.small_case(0, 8, 2, 128, 128, seed=5, dtype=torch.bfloat16, lengths=[768, 400])
