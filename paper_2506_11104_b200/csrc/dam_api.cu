@@ -15,7 +15,7 @@ struct Layout {
   size_t mask_bytes;
   size_t build_scratch_bytes;
   size_t attn_scratch_bytes;
-  uint64_t off_cnt, off_cnt_end, off_rowcnt, off_hist, off_cursor, off_items;
+  uint64_t off_cnt, off_cnt_end, off_keys, off_items;
   int max_L, max_W, max_nL, max_nq;
   uint64_t score_elems;
 };
@@ -66,6 +66,7 @@ bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) %
 void compute_layout(const dam_shape_t* s, int pcl_max, int all_ones_causal, int gather, Layout* out) {
   Layout& y = *out;
   memset(&y, 0, sizeof(y));
+  DamHeader& h = y.hdr;
   const int Hq = s->num_q_heads;
   uint64_t dv = 0, tr = 0, cnt = 0, cap = 0, causal_tiles = 0, po = 0, gath = 0;
   int total_qb = 0, total_pairs = 0;
@@ -82,6 +83,7 @@ void compute_layout(const dam_shape_t* s, int pcl_max, int all_ones_causal, int 
     gath += (uint64_t)Hq * nL;
     causal_tiles += (uint64_t)Hq * nq * (nq + 1) / 2;
     if (pcl_max > 0) {
+      h.head_tile_cap += dam_row_tile_prefix(nq, nL, L, gather);
       for (int qb = 0; qb < nq; ++qb) cap += (uint64_t)Hq * dam_row_tile_bound(qb, nL, L, gather);
     } else {
       cap += (uint64_t)Hq * (all_ones_causal ? (uint64_t)nq * (nq + 1) / 2 : (uint64_t)nq * nq);
@@ -93,7 +95,6 @@ void compute_layout(const dam_shape_t* s, int pcl_max, int all_ones_causal, int 
     if (nL > y.max_nL) y.max_nL = nL;
     if (nq > y.max_nq) y.max_nq = nq;
   }
-  DamHeader& h = y.hdr;
   h.magic = DAM_MAGIC;
   h.status = 0;
   h.version = 1;
@@ -117,13 +118,11 @@ void compute_layout(const dam_shape_t* s, int pcl_max, int all_ones_causal, int 
   h.off_tiles = dam_align(h.off_work + (uint64_t)sizeof(DamItem) * h.prows, 256);
   h.causal_tiles = causal_tiles;
   y.mask_bytes = dam_align(h.off_tiles + 4ull * cap, 256);
-  // build scratch: [0,256) status block and work counter | counts | row counts | hist | cursor | unordered items
+  // build scratch: [0,256) status block and work counter | counts | keys (listed tiles per work item) | unordered items
   y.off_cnt = 256;
   y.off_cnt_end = dam_align(y.off_cnt + 4ull * cnt, 256);
-  y.off_rowcnt = y.off_cnt_end;
-  y.off_hist = dam_align(y.off_rowcnt + 4ull * h.rows, 256);
-  y.off_cursor = y.off_hist + 4ull * DAM_HIST;
-  y.off_items = dam_align(y.off_cursor + 4ull * DAM_HIST, 256);          // work items before they are ordered
+  y.off_keys = y.off_cnt_end;
+  y.off_items = dam_align(y.off_keys + 4ull * h.prows, 256);
   y.build_scratch_bytes = dam_align(y.off_items + (uint64_t)sizeof(DamItem) * h.prows, 256);
   // attention scratch: 256-byte status block, then (gathered columns only) one K tile and one V tile of
   // 128 keys per gathered-column tile
@@ -213,10 +212,15 @@ dam_status_t fill_ctx(const dam_shape_t* s, const dam_rule_t* r, void* mask, siz
   c->pstar = c->per_map ? INFINITY : find_pstar(r);
   c->mu = r->mu; c->min_support = r->min_support;
   c->scale = r->softmax_scale > 0.f ? r->softmax_scale : 1.0f / sqrtf((float)s->head_dim);
-  c->off_cnt = y->off_cnt; c->off_cnt_end = y->off_cnt_end; c->off_rowcnt = y->off_rowcnt; c->off_items = y->off_items;
-  c->off_hist = y->off_hist; c->off_cursor = y->off_cursor;
+  c->off_cnt = y->off_cnt; c->off_cnt_end = y->off_cnt_end; c->off_keys = y->off_keys; c->off_items = y->off_items;
   c->gather = gather;
-  c->off_true = y->hdr.off_true; c->true_bytes = y->hdr.off_tile_ptr - y->hdr.off_true;
+  c->plan.h = y->hdr;
+  c->plan.nkeys = 2 * (2 * y->max_nL + 1) + 1 < DAM_HIST ? 2 * (2 * y->max_nL + 1) + 1 : DAM_HIST;
+  c->plan.nseq = s->num_seqs <= kDamTabSeqs ? s->num_seqs : 0;
+  DamSeqCursor cur = {};
+  for (int b = 0; b < c->plan.nseq; ++b)
+    c->plan.seq[b] = cur.next(s->cu_seqlens_host[b], s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b], r->pcl_max, s->num_q_heads,
+                              gather, -1);
   return DAM_OK;
 }
 
@@ -310,8 +314,8 @@ dam_status_t dam_build_masks(const void* Q, const void* K, const dam_shape_t* sh
   // thresholds from a map's own statistics need the finished map: with a dump buffer the map is written there first
   // and thresholded in a second pass; without one the caller has to go through dam_build_masks_from_scores
   if (c.per_map && !scores_dump) return DAM_ERR_UNSUPPORTED;
-  if (dam_launch_rule_prepare(c, cs) != cudaSuccess) return DAM_ERR_CUDA;
-  if (dam_launch_init_blob(shape, rule->pcl_max, y.hdr.flags, mask, y.hdr, cs) != cudaSuccess)
+  // (the status block and the counters of the rule kernels start at zero)
+  if (dam_launch_init_blob(shape, rule->pcl_max, y.hdr.flags, mask, y.hdr, scratch, y.off_cnt_end, cs) != cudaSuccess)
     return DAM_ERR_CUDA;
   cudaError_t e = cudaErrorNotSupported;
   if (sm100_shape(shape)) e = dam_launch_scores_sm100(Q, K, shape, c, scores_dump, cs);
@@ -330,8 +334,8 @@ dam_status_t dam_build_masks_from_scores(const float* P, const dam_shape_t* shap
   if (st != DAM_OK) return st;
   if (!P || !aligned(P, 4)) return DAM_ERR_INVALID_ARGUMENT;
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-  if (dam_launch_rule_prepare(c, cs) != cudaSuccess) return DAM_ERR_CUDA;
-  if (dam_launch_init_blob(shape, rule->pcl_max, y.hdr.flags, mask, y.hdr, cs) != cudaSuccess)
+  // (the status block and the counters of the rule kernels start at zero)
+  if (dam_launch_init_blob(shape, rule->pcl_max, y.hdr.flags, mask, y.hdr, scratch, y.off_cnt_end, cs) != cudaSuccess)
     return DAM_ERR_CUDA;
   if (dam_launch_bits_from_scores(P, c, cs) != cudaSuccess) return DAM_ERR_CUDA;
   if (dam_launch_rule(c, cs) != cudaSuccess) return DAM_ERR_CUDA;
@@ -366,7 +370,7 @@ dam_status_t dam_mask_all_ones(const dam_shape_t* shape, int32_t causal, void* m
   compute_layout(shape, 0, causal != 0, 0, &y);
   if (mask_capacity < y.mask_bytes) return DAM_ERR_BUFFER_TOO_SMALL;
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-  if (dam_launch_init_blob(shape, 0, y.hdr.flags, mask, y.hdr, cs) != cudaSuccess)
+  if (dam_launch_init_blob(shape, 0, y.hdr.flags, mask, y.hdr, nullptr, 0, cs) != cudaSuccess)
     return DAM_ERR_CUDA;
   if (dam_launch_all_ones(shape, causal != 0, mask, cs) != cudaSuccess) return DAM_ERR_CUDA;
   return DAM_OK;

@@ -87,6 +87,20 @@ struct DamSeq {
 };
 static_assert(sizeof(DamSeq) == 80, "DamSeq must be 80 bytes");
 
+// The layout a build call works on, handed to its kernels by value: the header as the host computed it and, for batches
+// of a few sequences, their records too.  The rule kernels are short and follow one another; every dependent read of the
+// header and of the sequence table in the blob costs each of them most of a microsecond.
+constexpr int kDamTabSeqs = 6;
+struct DamPlan {
+  DamHeader h;
+  int32_t nseq;            // sequences in seq[], 0: more than fit (the records are read from the blob)
+  int32_t nkeys;           // work items have fewer than this many listed tiles (or DAM_HIST - 1 of them and more)
+  DamSeq seq[kDamTabSeqs];
+};
+__device__ __forceinline__ DamSeq dam_plan_seq(const DamPlan& p, const unsigned char* blob, int b) {
+  return p.nseq ? p.seq[b] : reinterpret_cast<const DamSeq*>(blob + p.h.off_seq)[b];
+}
+
 // Per-(seq, head) words in the build scratch count area:
 //   cntD[L], cntV[L], prefD[W + 1], prefV[W + 1], tile_pop[nL * nL], padded to a multiple of 4.
 __host__ __device__ inline uint64_t dam_cnt_stride(int L, int W, int nL) {
@@ -119,6 +133,33 @@ __host__ __device__ inline uint64_t dam_row_tile_prefix(int qb, int nL, int L, i
   const uint64_t j = k < m ? k : m;
   return j * (j + 1) / 2 + (k - j) * m + ((uint64_t)qb - k) * m;
 }
+
+// Running offsets of the per-sequence sections: next() gives the record of one sequence after another.
+// all_ones_causal: -1 for a DAM mask, otherwise the all-ones blob's flag (cnt_off is then a tile offset per head).
+struct DamSeqCursor {
+  uint64_t dv, tr, po, co, go, tb;
+  int fq, fp;
+  __host__ __device__ inline DamSeq next(int tok0, int S, int pcl_max, int Hq, int gather, int all_ones_causal) {
+    int L = S < pcl_max ? S : pcl_max;
+    if (L < 0) L = 0;
+    const int W = L > 0 ? dam_words(L) : 0;
+    const int nL = (L + DAM_TILE - 1) / DAM_TILE, nq = (S + DAM_TILE - 1) / DAM_TILE;
+    DamSeq s;
+    s.tok_start = tok0; s.S = S; s.L = L; s.nq = nq;
+    s.first_qblock = fq; s.W = W; s.nL = nL; s.first_pair = fp;
+    s.dv_off = dv; s.true_off = tr; s.p_off = po; s.cnt_off = co; s.gath_off = go; s.tile_base = tb;
+    dv += (uint64_t)Hq * 3 * W;
+    tr += (uint64_t)Hq * L * W;
+    po += (uint64_t)Hq * L * L;
+    if (all_ones_causal < 0) co += (uint64_t)Hq * dam_cnt_stride(L, W, nL);
+    else co += all_ones_causal ? (uint64_t)nq * (nq + 1) / 2 : (uint64_t)nq * nq;
+    go += (uint64_t)Hq * nL;
+    if (all_ones_causal < 0) tb += dam_row_tile_prefix(nq, nL, L, gather);
+    fq += nq;
+    fp += (nq + 1) / 2;
+    return s;
+  }
+};
 
 // Gathered-column tiles serve the query blocks that start at or after row 2L - 1 (first multiple of 128).
 __host__ __device__ inline int dam_gather_first_qblock(int L) { return (2 * L - 1 + DAM_TILE - 1) / DAM_TILE; }
@@ -249,16 +290,16 @@ struct DamBuildCtx {
   int min_support;
   float scale;
   int gather;        // list gathered-column tiles
-  uint64_t off_cnt, off_cnt_end, off_rowcnt, off_hist, off_cursor, off_items;   // scratch sections
-  uint64_t off_true, true_bytes;                                     // true-mask section of the blob
+  uint64_t off_cnt, off_cnt_end, off_keys, off_items;   // scratch sections
+  DamPlan plan;
 };
 
+// `clear` (clear_bytes bytes, may be NULL) is filled with zeros by the same launch
 cudaError_t dam_launch_init_blob(const dam_shape_t* shape, int pcl_max, uint32_t flags, void* blob,
-                                 const DamHeader& host_hdr, cudaStream_t st);
+                                 const DamHeader& host_hdr, void* clear, size_t clear_bytes, cudaStream_t st);
 cudaError_t dam_launch_scores_ref(const void* Q, const void* K, const dam_shape_t* shape, const DamBuildCtx& c,
                                   float* scores_dump, cudaStream_t st);
 cudaError_t dam_launch_bits_from_scores(const float* P, const DamBuildCtx& c, cudaStream_t st);
-cudaError_t dam_launch_rule_prepare(const DamBuildCtx& c, cudaStream_t st);   // before the true mask is produced
 cudaError_t dam_launch_rule(const DamBuildCtx& c, cudaStream_t st);
 cudaError_t dam_launch_all_ones(const dam_shape_t* shape, int causal, void* blob, cudaStream_t st);
 cudaError_t dam_launch_expand_rows(const void* blob, int seq, int head, int row_begin, int nrows, int words,

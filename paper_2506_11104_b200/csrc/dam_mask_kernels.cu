@@ -33,48 +33,36 @@ __device__ __forceinline__ const DamSeq* blob_seqs(const unsigned char* blob, co
 
 // ---------------------------------------------------------------------------------------------
 // Header + per-sequence table + q-block table, computed on the device from cu_seqlens so that no
-// host buffer has to outlive the call.  One block.
+// host buffer has to outlive the call.  Block 0; the other blocks clear the counters of the kernels that follow.
 // ---------------------------------------------------------------------------------------------
 __global__ void init_blob_kernel(unsigned char* blob, DamHeader hdr, const int32_t* __restrict__ cu,
-                                 int pcl_max, int Hq, int all_ones_causal /* -1: DAM mask */) {
+                                 int pcl_max, int Hq, int all_ones_causal /* -1: DAM mask */, uint4* clear, uint32_t clear_vecs) {
   asm volatile("griddepcontrol.launch_dependents;");     // a kernel chained behind this one may start its prologue
+  if (blockIdx.x > 0) {
+    for (uint32_t x = (blockIdx.x - 1) * blockDim.x + threadIdx.x; x < clear_vecs; x += (gridDim.x - 1) * blockDim.x)
+      clear[x] = make_uint4(0u, 0u, 0u, 0u);
+    return;
+  }
   DamHeader* H = reinterpret_cast<DamHeader*>(blob);
   DamSeq* seqs = reinterpret_cast<DamSeq*>(blob + hdr.off_seq);
   int32_t* qbseq = reinterpret_cast<int32_t*>(blob + hdr.off_qbseq);
   uint32_t* pairtab = reinterpret_cast<uint32_t*>(blob + hdr.off_pairtab);
   if (threadIdx.x == 0) {
-    *H = hdr;
-    uint64_t dv = 0, tr = 0, po = 0, co = 0, go = 0, tb = 0;
-    int fq = 0, fp = 0;
+    DamSeqCursor cur = {};
     const int gather = (hdr.flags & DAM_FLAG_GATHER) ? 1 : 0;
+    int t0 = cu[0];
     for (int b = 0; b < hdr.num_seqs; ++b) {
-      int t0 = cu[b], S = cu[b + 1] - t0;
-      int L = S < pcl_max ? S : pcl_max;
-      if (L < 0) L = 0;
-      int W = L > 0 ? dam_words(L) : 0;
-      int nL = (L + DAM_TILE - 1) / DAM_TILE;
-      int nq = (S + DAM_TILE - 1) / DAM_TILE;
-      DamSeq s;
-      s.tok_start = t0; s.S = S; s.L = L; s.nq = nq;
-      s.first_qblock = fq; s.W = W; s.nL = nL; s.first_pair = fp;
-      s.dv_off = dv; s.true_off = tr; s.p_off = po; s.cnt_off = co; s.gath_off = go; s.tile_base = tb;
-      seqs[b] = s;
-      dv += (uint64_t)Hq * 3 * W;
-      tr += (uint64_t)Hq * L * W;
-      po += (uint64_t)Hq * L * L;
-      if (all_ones_causal < 0) co += (uint64_t)Hq * dam_cnt_stride(L, W, nL);
-      else co += all_ones_causal ? (uint64_t)nq * (nq + 1) / 2 : (uint64_t)nq * nq;   // tile base per head
-      go += (uint64_t)Hq * nL;
-      if (all_ones_causal < 0) tb += dam_row_tile_prefix(nq, nL, L, gather);
-      fq += nq;
-      fp += (nq + 1) / 2;
+      const int t1 = cu[b + 1];
+      seqs[b] = cur.next(t0, t1 - t0, pcl_max, Hq, gather, all_ones_causal);
+      t0 = t1;
     }
-    H->head_tile_cap = tb;
+    hdr.head_tile_cap = cur.tb;
     if (all_ones_causal < 0) {
       // the tile lists have a fixed place per row (see the layout notes): nothing to compact, no sizes to wait for
-      H->bytes_used = hdr.off_tiles + 4ull * Hq * tb;
-      reinterpret_cast<uint32_t*>(blob + hdr.off_tile_ptr)[hdr.rows] = (uint32_t)(Hq * tb);
+      hdr.bytes_used = hdr.off_tiles + 4ull * Hq * cur.tb;
+      reinterpret_cast<uint32_t*>(blob + hdr.off_tile_ptr)[hdr.rows] = (uint32_t)(Hq * cur.tb);
     }
+    *H = hdr;
   }
   __syncthreads();
   for (int b = 0; b < hdr.num_seqs; ++b) {
@@ -145,12 +133,12 @@ __device__ __forceinline__ uint32_t dam_transpose32(uint32_t x, int lane) {
 // and its 128 bits.  Column counts (128), diagonal counts (255) and the tile's popcount are made per warp
 // with bit-matrix transposes, summed in shared memory and flushed with integer atomics (order-independent).
 // ---------------------------------------------------------------------------------------------
-__global__ void counts_kernel(const unsigned char* blob, unsigned char* scratch, uint64_t off_cnt) {
+__global__ void counts_kernel(const unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, const __grid_constant__ DamPlan plan) {
   dam_chain_prologue();
-  const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
+  const DamHeader* H = &plan.h;
   const int sh = blockIdx.y;
   const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
-  const DamSeq sq = blob_seqs(blob, H)[b];
+  const DamSeq sq = dam_plan_seq(plan, blob, b);
   const int nL = sq.nL;
   // tile index -> (qb, kb) over the lower triangle
   int t = blockIdx.x;
@@ -226,12 +214,13 @@ __global__ void counts_kernel(const unsigned char* blob, unsigned char* scratch,
 // Match: D[r] = [cntD[r] >= mu * (L - r)], V[c] likewise (one fp32 multiply, one compare), written
 // as bit sets; Drev = D reversed; prefix popcounts per word for range queries.  Block per (seq, head).
 // ---------------------------------------------------------------------------------------------
-__global__ void match_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, float mu, int min_support) {
+__global__ void match_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, float mu, int min_support,
+                             const __grid_constant__ DamPlan plan) {
   dam_chain_prologue();
-  const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
+  const DamHeader* H = &plan.h;
   const int sh = blockIdx.x;
   const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
-  const DamSeq sq = blob_seqs(blob, H)[b];
+  const DamSeq sq = dam_plan_seq(plan, blob, b);
   if (sq.L == 0) return;
   const int L = sq.L, W = sq.W;
   uint32_t* dv = reinterpret_cast<uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * W;
@@ -352,9 +341,10 @@ __device__ __forceinline__ uint32_t classify_band(const HeadView& v, int qb, int
 }
 
 __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, uint64_t off_items,
-                                uint64_t off_keys) {
+                                uint64_t off_keys, const __grid_constant__ DamPlan bp) {
   dam_chain_prologue();
-  DamHeader* H = reinterpret_cast<DamHeader*>(blob);
+  const DamHeader* H = &bp.h;
+  DamHeader* stats = reinterpret_cast<DamHeader*>(blob);
   const int lane = threadIdx.x & 31;
   const int prow = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // one warp per (head, q-block pair)
   // block totals of the three statistics: one global atomic per block instead of one per warp on the same address
@@ -364,10 +354,14 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
   __syncthreads();
   if (prow < H->prows) {
   const int h = prow / H->total_pairs, gp = prow % H->total_pairs;
-  const uint32_t pt = reinterpret_cast<const uint32_t*>(blob + H->off_pairtab)[gp];
-  const int gqb0 = (int)(pt & 0x7FFFFFFFu), nblk = (pt >> 31) ? 2 : 1;
-  const int b = reinterpret_cast<const int32_t*>(blob + H->off_qbseq)[gqb0];
-  const DamSeq sq = blob_seqs(blob, H)[b];
+  int b = 0;
+  if (bp.nseq) {
+    while (b + 1 < bp.nseq && bp.seq[b + 1].first_pair <= gp) ++b;      // (an empty sequence has no pair of its own)
+  } else {
+    b = reinterpret_cast<const int32_t*>(blob + H->off_qbseq)[reinterpret_cast<const uint32_t*>(blob + H->off_pairtab)[gp] & 0x7FFFFFFFu];
+  }
+  const DamSeq sq = dam_plan_seq(bp, blob, b);
+  const int gqb0 = sq.first_qblock + 2 * (gp - sq.first_pair), nblk = 2 * (gp - sq.first_pair) + 1 < sq.nq ? 2 : 1;
   HeadView v;
   const uint32_t* dv = reinterpret_cast<const uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * sq.W;
   const int32_t* cnt = reinterpret_cast<const int32_t*>(scratch + off_cnt) + sq.cnt_off +
@@ -478,7 +472,7 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
     // index (pair, head): the order the pairs keep inside a bucket of the work list
     const size_t at = (size_t)gp * H->num_q_heads + h;
     reinterpret_cast<DamItem*>(scratch + off_items)[at] = it;
-    reinterpret_cast<uint32_t*>(scratch + off_keys)[at] = (uint32_t)min(pair_total, DAM_HIST - 1);
+    reinterpret_cast<uint32_t*>(scratch + off_keys)[at] = (uint32_t)min(pair_total, bp.nkeys - 1);
     atomicAdd(&s_mask_tiles, (unsigned long long)mask_tiles);
     atomicAdd(&s_total, (uint32_t)pair_total);
     atomicAdd(&s_full, (uint32_t)nfull);
@@ -486,9 +480,9 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (s_mask_tiles) atomicAdd(reinterpret_cast<unsigned long long*>(&H->mask_tiles), s_mask_tiles);
-    if (s_total) atomicAdd(&H->total_tiles, s_total);
-    if (s_full) atomicAdd(&H->full_tiles, s_full);
+    if (s_mask_tiles) atomicAdd(reinterpret_cast<unsigned long long*>(&stats->mask_tiles), s_mask_tiles);
+    if (s_total) atomicAdd(&stats->total_tiles, s_total);
+    if (s_full) atomicAdd(&stats->full_tiles, s_full);
   }
 }
 
@@ -524,18 +518,16 @@ __device__ uint32_t block_excl_scan(uint32_t x, uint32_t* total, uint32_t* sm /*
 }
 
 __global__ void __launch_bounds__(1024)
-order_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_items, uint64_t off_keys) {
+order_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_items, uint64_t off_keys, int prows, uint64_t off_work, int nkeys) {
   dam_chain_prologue();
-  DamHeader* H = reinterpret_cast<DamHeader*>(blob);
   __shared__ uint32_t sm[32];
   __shared__ uint32_t tot;
   __shared__ uint32_t start[DAM_HIST];      // pairs per key, then the first place of the key's bucket
   __shared__ uint32_t before[DAM_HIST];     // pairs per key that precede this block's share, then the running cursor
   const uint4* src = reinterpret_cast<const uint4*>(scratch + off_items);      // items in (pair, head) order
   const uint32_t* keys = reinterpret_cast<const uint32_t*>(scratch + off_keys);
-  uint4* dst = reinterpret_cast<uint4*>(blob + H->off_work);
-  const int prows = H->prows;
-  for (int k = threadIdx.x; k < DAM_HIST; k += blockDim.x) { start[k] = 0u; before[k] = 0u; }
+  uint4* dst = reinterpret_cast<uint4*>(blob + off_work);
+  for (int k = threadIdx.x; k < nkeys; k += blockDim.x) { start[k] = 0u; before[k] = 0u; }
   __syncthreads();
   // Every block places blockDim.x pairs and needs nothing from the other blocks: it counts all pairs per key
   // itself, and those that precede its share.  Inside a bucket the pairs keep the order (pair, head): the query
@@ -565,12 +557,12 @@ order_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_items, ui
   __syncthreads();
   // first place of every bucket: after all buckets with more tiles (descending order of the key)
   {
-    const int per = (DAM_HIST + blockDim.x - 1) / blockDim.x;
-    const int q0 = threadIdx.x * per, q1 = min(DAM_HIST, q0 + per);     // positions in descending-key order
+    const int per = (nkeys + blockDim.x - 1) / blockDim.x;
+    const int q0 = threadIdx.x * per, q1 = min(nkeys, q0 + per);     // positions in descending-key order
     uint32_t local = 0;
-    for (int k = q0; k < q1; ++k) local += start[DAM_HIST - 1 - k];
+    for (int k = q0; k < q1; ++k) local += start[nkeys - 1 - k];
     uint32_t e = block_excl_scan(local, &tot, sm);
-    for (int k = q0; k < q1; ++k) { const uint32_t c = start[DAM_HIST - 1 - k]; start[DAM_HIST - 1 - k] = e; e += c; }
+    for (int k = q0; k < q1; ++k) { const uint32_t c = start[nkeys - 1 - k]; start[nkeys - 1 - k] = e; e += c; }
   }
   __syncthreads();
   {
@@ -688,10 +680,13 @@ __global__ void expand_rows_kernel(const unsigned char* blob, int seq, int head,
 }  // namespace
 
 cudaError_t dam_launch_init_blob(const dam_shape_t* shape, int pcl_max, uint32_t flags, void* blob,
-                                 const DamHeader& host_hdr, cudaStream_t st) {
+                                 const DamHeader& host_hdr, void* clear, size_t clear_bytes, cudaStream_t st) {
   int mode = (flags & DAM_FLAG_ALL_ONES) ? ((flags & DAM_FLAG_CAUSAL_LIST) ? 1 : 0) : -1;
-  init_blob_kernel<<<1, 256, 0, st>>>(reinterpret_cast<unsigned char*>(blob), host_hdr, shape->cu_seqlens_dev,
-                                      pcl_max, shape->num_q_heads, mode);
+  const size_t vecs = clear_bytes / 16;                      // (the sections are multiples of 256 bytes)
+  const size_t blocks = vecs ? (vecs + 1023) / 1024 : 0;     // four 16-byte stores per thread, at most 1024 blocks
+  init_blob_kernel<<<1 + (unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st>>>(
+      reinterpret_cast<unsigned char*>(blob), host_hdr, shape->cu_seqlens_dev, pcl_max, shape->num_q_heads, mode,
+      reinterpret_cast<uint4*>(clear), (uint32_t)vecs);
   return cudaGetLastError();
 }
 
@@ -924,28 +919,20 @@ cudaError_t dam_launch_capture_average(const float* A, const int32_t* C, int Lma
   return cudaGetLastError();
 }
 
-// The counters of the rule kernels start at zero: counts + prefix + tile popcounts, row counts, histogram,
-// cursors.  Enqueued before the kernel that produces the true mask, so that the rule kernels follow it directly.
-cudaError_t dam_launch_rule_prepare(const DamBuildCtx& c, cudaStream_t st) {
-  // the sections are contiguous (status block and work counter of the scoring kernel | counts | row counts |
-  // histogram | cursors): one fill
-  return cudaMemsetAsync(c.scratch, 0, c.off_cursor + 4ull * DAM_HIST, st);
-}
-
 cudaError_t dam_launch_rule(const DamBuildCtx& c, cudaStream_t st) {
   cudaError_t e;
   if (c.max_nL > 0) {
     dim3 g(c.max_nL * (c.max_nL + 1) / 2, c.num_seqs * c.Hq);
-    if ((e = launch_chained(counts_kernel, g, dim3(DAM_TILE), st, c.blob, c.scratch, c.off_cnt)) != cudaSuccess) return e;
+    if ((e = launch_chained(counts_kernel, g, dim3(DAM_TILE), st, c.blob, c.scratch, c.off_cnt, c.plan)) != cudaSuccess) return e;
     if ((e = launch_chained(match_kernel, dim3(c.num_seqs * c.Hq), dim3(1024), st, c.blob, c.scratch, c.off_cnt, c.mu,
-                            c.min_support)) != cudaSuccess) return e;
+                            c.min_support, c.plan)) != cudaSuccess) return e;
   }
   if (c.rows > 0) {
     int blocks = (c.prows + 7) / 8;
     if ((e = launch_chained(classify_kernel, dim3(blocks), dim3(256), st, c.blob, c.scratch, c.off_cnt, c.off_items,
-                            c.off_rowcnt)) != cudaSuccess) return e;
+                            c.off_keys, c.plan)) != cudaSuccess) return e;
     if ((e = launch_chained(order_kernel, dim3((c.prows + 1023) / 1024), dim3(1024), st, c.blob, c.scratch, c.off_items,
-                            c.off_rowcnt)) != cudaSuccess)
+                            c.off_keys, c.prows, c.plan.h.off_work, c.plan.nkeys)) != cudaSuccess)
       return e;
   }
   return cudaGetLastError();

@@ -50,6 +50,7 @@ struct ScoreParams {
   int num_seqs, Hq, group, max_nL;
   int dump_vec8;              // every row of the dumped maps starts on a 32-byte boundary and is a multiple of 32 bytes
   float scale_log2, pstar;
+  DamPlan plan;
 };
 
 __device__ __forceinline__ void st_global_v8(float* p, const float* v) {
@@ -80,13 +81,13 @@ __device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1, f
 
 struct Item { int b, h, qb, valid; DamSeq sq; };
 
-__device__ __forceinline__ Item decode_item(const unsigned char* blob, const DamHeader* H, const ScoreParams& p, int w) {
+__device__ __forceinline__ Item decode_item(const unsigned char* blob, const ScoreParams& p, int w) {
   Item it;
   const int per = p.num_seqs * p.Hq;
   it.qb = p.max_nL - 1 - w / per;           // heaviest query blocks first
   const int sh = w % per;
   it.b = sh / p.Hq; it.h = sh % p.Hq;
-  it.sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[it.b];
+  it.sq = dam_plan_seq(p.plan, blob, it.b);
   it.valid = it.qb < it.sq.nL;
   return it;
 }
@@ -94,7 +95,7 @@ __device__ __forceinline__ Item decode_item(const unsigned char* blob, const Dam
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                   const ScoreParams prm) {
+                   const __grid_constant__ ScoreParams prm) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
@@ -111,7 +112,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* blob = prm.blob;
-  const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
+  const DamHeader* H = &prm.plan.h;
   const int nitems = prm.max_nL * prm.num_seqs * prm.Hq;
   // Items (heaviest query blocks first) are claimed from a global counter by the producer thread and handed
   // to the MMA thread and the eight softmax warps through a two-entry ring; a negative entry ends the loop.
@@ -138,7 +139,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   const uint32_t tmem = *tmem_slot;
   // everything above is independent of the kernel before this one; the blob it initialises is read from here on
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (blockIdx.x == 0 && tid == 0) const_cast<DamHeader*>(H)->reserved[0] = 1ull;   // the map of this blob was scored on the tensor cores
+  if (blockIdx.x == 0 && tid == 0) reinterpret_cast<DamHeader*>(blob)->reserved[0] = 1ull;   // the map of this blob was scored on the tensor cores
 
   if (warp == 0) {
     if (elect_one()) {              // (elected, not lane 0: PCL 4096 292 -> 274 us for stage 1, PCL 2048 97.6 -> 95.8 us)
@@ -155,7 +156,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         sched_items[sl] = w;
         mbar_arrive(bSchedFull + 8 * sl);
         if (w < 0) break;
-        const Item it = decode_item(blob, H, prm, w);
+        const Item it = decode_item(blob, prm, w);
         if (!it.valid) continue;
         if (!(ok = mbar_wait(bQEmpty, (ic & 1u) ^ 1u, abort_flag))) break;
         mbar_arrive_expect_tx(bQFull, DAM_TILE * D * 2);
@@ -195,7 +196,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const int w = next_item_consumer(n);
         if (w != -2) mbar_arrive(bSchedEmpty + 8 * (n & 1u));
         if (w < 0) { ok = (w == -1); break; }
-        const Item it = decode_item(blob, H, prm, w);
+        const Item it = decode_item(blob, prm, w);
         if (!it.valid) continue;
         if (!(ok = mbar_wait(bQFull, ic & 1u, abort_flag))) break;
         ++ic;
@@ -232,7 +233,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       __syncwarp();
       if (lane == 0 && w != -2) mbar_arrive(bSchedEmpty + 8 * (n & 1u));
       if (w < 0) { ok = (w == -1); break; }
-      const Item it = decode_item(blob, H, prm, w);
+      const Item it = decode_item(blob, prm, w);
       if (!it.valid) continue;
       const int L = it.sq.L, W = it.sq.W;
       const int i = it.qb * DAM_TILE + r;
@@ -430,6 +431,7 @@ cudaError_t dam_launch_scores_sm100(const void* Q, const void* K, const dam_shap
   p.num_seqs = c.num_seqs; p.Hq = c.Hq; p.group = c.Hq / c.Hkv; p.max_nL = c.max_nL;
   p.scale_log2 = c.scale * 1.4426950408889634f;
   p.pstar = c.pstar;
+  p.plan = c.plan;
   bool vec8 = dump && reinterpret_cast<uintptr_t>(dump) % 32 == 0;
   for (int b = 0; b < s->num_seqs && vec8; ++b) {
     const int S = s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b];

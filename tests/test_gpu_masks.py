@@ -344,6 +344,18 @@ def test_multi_sample_capture_masks_bit_exact():
     H.check_blob_against_oracle(blob, tshape, masks)
 
 
+@pytest.mark.parametrize("gather", GATHER)
+@pytest.mark.parametrize("lengths", [[300, 0, 129, 1, 0, 700], [0, 300, 129, 0, 1, 700, 513], [40] * 9])
+def test_more_sequences_than_the_record_table_holds(lengths, gather):
+    """Six sequences (their records travel with the launches) and more (read from the blob), empty ones among them."""
+    w = synth.small_case(0, 4, 2, 64, 160, seed=60, dtype=torch.bfloat16, lengths=lengths)
+    shape, rule = _shape(w), _rule(w, gather_columns=gather)
+    dump = torch.zeros(sum(4 * min(S, 160) ** 2 for S in lengths), dtype=torch.float32, device=DEV)
+    blob, _ = B.dam_build_masks(w.Q.to(DEV), w.K.to(DEV), shape, rule, scores_dump=dump)
+    assert B.dam_poll_status(blob) == 0
+    H.check_blob_against_oracle(blob, shape, H.oracle_masks_from_dump(w, dump.cpu().numpy()))
+
+
 @pytest.mark.parametrize("pcl,lengths", [
     (1, [1, 3]),                            # one cell
     (37, [50, 20, 37, 9]),                  # odd rows: element-wise stores and reads
