@@ -404,16 +404,16 @@ static dam_status_t sparse_attention_impl(const void* Q, const void* K, const vo
   if (scratch_bytes < 256) return DAM_ERR_BUFFER_TOO_SMALL;
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)shape->head_dim);
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-  // status word and work counter start at zero (a continuation clears the work counter only)
-  if (cudaMemsetAsync(reinterpret_cast<unsigned char*>(scratch) + (continuation ? 8 : 0), 0, continuation ? 248 : 256, cs) !=
-      cudaSuccess)
-    return DAM_ERR_CUDA;
   cudaError_t e = cudaErrorNotSupported;
   if (sm100_shape(shape))
     e = dam_launch_attn_sm100(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, scratch_bytes, ranges_dev,
                               !continuation, cs);
-  if (e == cudaErrorNotSupported)
+  if (e == cudaErrorNotSupported) {
+    if (cudaMemsetAsync(reinterpret_cast<unsigned char*>(scratch) + (continuation ? 8 : 0), 0, continuation ? 248 : 256, cs) !=
+        cudaSuccess)
+      return DAM_ERR_CUDA;
     e = dam_launch_attn_ref(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, ranges_dev, cs);
+  }
   return e == cudaSuccess ? DAM_OK : DAM_ERR_CUDA;
 }
 

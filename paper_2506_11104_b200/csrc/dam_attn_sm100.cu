@@ -715,7 +715,13 @@ __global__ void __launch_bounds__(128)
 gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat16* __restrict__ K,
                       const __nv_bfloat16* __restrict__ V, int Hq, int group, int d, int64_t kst, int64_t ksh, int64_t vst,
                       int64_t vsh, unsigned char* scratch, unsigned long long scratch_bytes) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");     // (launched under the tail of the kernel before it)
   asm volatile("griddepcontrol.launch_dependents;");     // the attention kernel behind this one may start its prologue
+  // the attention kernel's status block starts at zero
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < 64) reinterpret_cast<uint32_t*>(scratch)[threadIdx.x] = 0u;
+    __syncthreads();
+  }
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   if (!(H->flags & DAM_FLAG_GATHER)) return;
   if (H->attn_scratch_bytes > scratch_bytes) {
@@ -852,12 +858,25 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
   if (!dam_make_tmap_bf16(&tg, has_g ? reinterpret_cast<const unsigned char*>(scratch) + 256 : Q, d, 1,
                           has_g ? (int64_t)grows : DAM_TILE, d, d))
     return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
   if (has_g && run_gather) {
-    gather_columns_kernel<<<sm_count * 4, 128, 0, st>>>(
-        reinterpret_cast<const unsigned char*>(blob), reinterpret_cast<const __nv_bfloat16*>(K),
-        reinterpret_cast<const __nv_bfloat16*>(V), s->num_q_heads, s->num_q_heads / s->num_kv_heads, d, s->k_stride_tok,
-        s->k_stride_head, s->v_stride_tok, s->v_stride_head, reinterpret_cast<unsigned char*>(scratch),
-        (unsigned long long)scratch_bytes);
+    // clears the status block too
+    cfg.gridDim = dim3(sm_count * 4); cfg.blockDim = dim3(128);
+    if ((e = cudaLaunchKernelEx(&cfg, gather_columns_kernel, reinterpret_cast<const unsigned char*>(blob),
+                                reinterpret_cast<const __nv_bfloat16*>(K), reinterpret_cast<const __nv_bfloat16*>(V),
+                                (int)s->num_q_heads, (int)(s->num_q_heads / s->num_kv_heads), d, s->k_stride_tok, s->k_stride_head,
+                                s->v_stride_tok, s->v_stride_head, reinterpret_cast<unsigned char*>(scratch),
+                                (unsigned long long)scratch_bytes)) != cudaSuccess)
+      return e;
+  } else {
+    // status word and work counter start at zero (a further row range clears the work counter only)
+    if ((e = cudaMemsetAsync(reinterpret_cast<unsigned char*>(scratch) + (run_gather ? 0 : 8), 0, run_gather ? 256 : 248, st)) != cudaSuccess)
+      return e;
   }
   if (!dam_make_tmap_bf16(&to, O, d, s->num_q_heads, s->total_tokens, s->o_stride_tok, s->o_stride_head, 32) ||
       !dam_make_tmap_bf16(&tq, Q, d, s->num_q_heads, s->total_tokens, s->q_stride_tok, s->q_stride_head) ||
@@ -884,12 +903,7 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
   p.o_stride_tok = s->o_stride_tok; p.o_stride_head = s->o_stride_head;
   p.scale_log2 = scale * 1.4426950408889634f;
   const int grid = pairs < sm_count ? pairs : sm_count;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes;
   if (d == 128) {
     if (ranges) return cudaLaunchKernelEx(&cfg, attn_sm100_kernel<true, 128>, tq, tk, tv, to, tg, p);
     return cudaLaunchKernelEx(&cfg, attn_sm100_kernel<false, 128>, tq, tk, tv, to, tg, p);
