@@ -259,7 +259,8 @@ def dam_sparse_attention_rows(Q, K, V, mask, shape: Shape, row_ranges, O: torch.
     flat = [int(x) for pair in row_ranges for x in pair]
     assert len(flat) == 2 * shape.c.num_seqs
     host = (ctypes.c_int32 * len(flat))(*flat)
-    dev = torch.tensor(flat, dtype=torch.int32, device=Q.device)
+    # queued without waiting for the stream (CUDA has taken its own copy of a small pageable source when the call returns)
+    dev = torch.tensor(flat, dtype=torch.int32).to(Q.device, non_blocking=True)
     if scratch is None:
         off = _HDR.fields["attn_scratch_bytes"][1]
         need = int(mask[off: off + 8].cpu().numpy().view(np.uint64)[0]) if mask.numel() >= 256 else 256
