@@ -271,7 +271,8 @@ dam_status_t dam_decode_attention(const void* q, const void* K, const void* V, c
                                   size_t scratch_bytes, void* stream);
 
 /*
- * Counts taken from a mask blob (DEVICE): out[0] = listed tiles (what the attention kernel executes),
+ * Counts taken from a mask blob (DEVICE): out[0] = listed tiles (what the attention kernel executes; the
+ * tensor-core kernel multiplies fewer where a head's single far diagonal lies across two tiles that hold nothing else),
  * out[1] = of those, fully active ones, out[2] = total causal tiles of the shape (for densities),
  * out[3] = bytes of the blob in use (the tile lists have a fixed place per row, sized by the row's upper
  * bound, so this follows from the shapes; out[0] says how many entries are real), out[4] = 128 x 128 tiles of the masks themselves that hold an

@@ -18,6 +18,12 @@
 //               TMEM (twice: running max, then probabilities), applies the tile's mask bits where the tile
 //               is not fully active, writes P (bf16) back to TMEM, rescales O in TMEM when the running max
 //               moved by more than 2^8, and finally normalises and stores O and the log-sum-exp.
+// A head's lone diagonal (dam_internal.cuh) is served by one tile per query block that starts at the block's first key on
+// it, multiplied last, in place of the two listed tiles it lies across; the softmax of that tile is one entry per row.
+// (32k tokens 453 -> 434 us, 8k 113 -> 107, mixed-length batch 1594 -> 1461, 128k 2112 -> 1993.  The tiles of both
+// blocks in one step with two K and two V tiles, so that the streams overlap: slower by 1 - 2 %.)  The code is kept small
+// where it is not hot: the masked maximum, the rescaling of O and the epilogue are loops that are not unrolled, which by
+// itself is 2 % on the sparse lists (the loops of both streams' phases and the issuing thread share the instruction cache).
 // Only the tiles the mask lists are ever loaded or multiplied (paper Sec. 4.3: masked logits are -inf).
 // Every wait is bounded; an expired wait sets the status word in the scratch buffer and the CTA drains
 // and exits.
@@ -69,7 +75,8 @@ constexpr int kSmemBytes = SmemLayout::total + 1024;   // + slack for the 1024-b
 // walking item -> sequence record -> tile list in global memory.
 struct ItemRec {
   uint4 u, v;               // the two words of the DamItem
-  uint32_t eA, eB, pad0, pad1;
+  uint32_t eA, eB;
+  int2 lone;                // the head's lone diagonal (or -1) and the entries in front of it
   DamHeadBits hb;
 };
 static_assert(sizeof(ItemRec) == 96, "ItemRec must be 96 bytes");
@@ -112,12 +119,32 @@ __device__ __forceinline__ Item item_from_words(const uint4& u, const uint4& v) 
   return it;
 }
 
+// The lone diagonal of a head on one query block: the `n` entries from `at` on list tiles that hold its cells and nothing
+// else; they are left out, and one tile of keys from `key` on takes their place behind the list.  n = 0: nothing of the
+// kind on this block.
+struct Lone {
+  uint32_t at, n;
+  int key;
+  __device__ __forceinline__ Lone(int2 lone, uint32_t t0, int qb, int nL, int S) : at(0u), n(0u), key(0) {
+    const int i0 = qb * DAM_TILE, r = lone.x;
+    if (r >= 0 && qb >= dam_lone_first_qblock(r, nL) && i0 < S) {
+      key = i0 - r;
+      n = (uint32_t)(min(i0 + DAM_TILE, S) - 1 - r) / DAM_TILE - (uint32_t)key / DAM_TILE + 1u;
+      at = t0 + (uint32_t)lone.y;
+    }
+  }
+};
+
 // Merge of the two ascending tile lists: every step is one kv tile with the kinds it has in A and in B.
 struct Walker {
   const uint32_t* tiles;
   uint32_t ia, ea, ib, eb, ca, cb;
-  __device__ __forceinline__ void init(const uint32_t* t, const Item& it) {
+  uint32_t la, na, lb, nb;      // entries [la, la + na) and [lb, lb + nb) are left out
+  __device__ __forceinline__ void init(const uint32_t* t, const Item& it, const Lone& A, const Lone& B) {
     tiles = t; ia = it.a0; ea = it.a1; ib = it.b0; eb = it.b1;
+    la = A.at; na = A.n; lb = B.at; nb = B.n;
+    if (ia == la) ia += na;
+    if (ib == lb) ib += nb;
     ca = ia < ea ? __ldg(tiles + ia) : kNone;
     cb = ib < eb ? __ldg(tiles + ib) : kNone;
   }
@@ -134,8 +161,8 @@ struct Walker {
     kb = (int)(k & 0x0FFFFFFFu);
     kindA = (ja == k) ? (ca >> 28) : 0u;
     kindB = (jb == k) ? (cb >> 28) : 0u;
-    if (ja == k) { ++ia; ca = ia < ea ? __ldg(tiles + ia) : kNone; }
-    if (jb == k) { ++ib; cb = ib < eb ? __ldg(tiles + ib) : kNone; }
+    if (ja == k) { ++ia; if (ia == la) ia += na; ca = ia < ea ? __ldg(tiles + ia) : kNone; }
+    if (jb == k) { ++ib; if (ib == lb) ib += nb; cb = ib < eb ? __ldg(tiles + ib) : kNone; }
     return true;
   }
   __device__ __forceinline__ bool a_done() const { return ia >= ea; }
@@ -207,6 +234,29 @@ __device__ __forceinline__ float sweep_max(uint32_t tS, const uint4& bits) {
       mx0 = max3(mx0, v0, v1); mx1 = max3(mx1, v2, v3);
     }
     if (c < 3) tc_wait_ld();
+  }
+  return fmaxf(mx0, mx1);
+}
+
+// The masked maximum again, as small code: it runs on the first tile of a list and where the bound was exceeded.
+__device__ __forceinline__ float sweep_max_masked(uint32_t tS, uint4 bits) {
+  float mx0 = -CUDART_INF_F, mx1 = -CUDART_INF_F;
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    const uint32_t word = bits.x;
+    bits.x = bits.y; bits.y = bits.z; bits.z = bits.w;
+    if (!__any_sync(0xFFFFFFFFu, word != 0u)) continue;
+    uint32_t cur[32];
+    tmem_ld32(tS + c * 32, cur);
+    tc_wait_ld();
+#pragma unroll
+    for (int q = 0; q < 32; q += 4) {
+      const float v0 = ((word >> q) & 1u) ? __uint_as_float(cur[q]) : -CUDART_INF_F;
+      const float v1 = ((word >> (q + 1)) & 1u) ? __uint_as_float(cur[q + 1]) : -CUDART_INF_F;
+      const float v2 = ((word >> (q + 2)) & 1u) ? __uint_as_float(cur[q + 2]) : -CUDART_INF_F;
+      const float v3 = ((word >> (q + 3)) & 1u) ? __uint_as_float(cur[q + 3]) : -CUDART_INF_F;
+      mx0 = max3(mx0, v0, v1); mx1 = max3(mx1, v2, v3);
+    }
   }
   return fmaxf(mx0, mx1);
 }
@@ -376,6 +426,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         Item it;
         bool skip = false;
         long long gtile0 = 0;
+        int2 lone = make_int2(-1, 0);
+        int nL = 0;
         if (w >= 0) {
           const uint4* src = reinterpret_cast<const uint4*>(blob + H->off_work) + 2 * (size_t)w;
           const uint4 u = __ldg(src), v = __ldg(src + 1);
@@ -385,6 +437,9 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           rec.u = u; rec.v = v;
           if (!skip) {
             const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[it.seq];
+            nL = sq.nL;
+            if (H->off_lone) lone = __ldg(reinterpret_cast<const int2*>(blob + H->off_lone) + it.seq * H->num_q_heads + it.head);
+            rec.lone = lone;
             rec.eA = it.a0 < it.a1 ? __ldg(tiles + it.a0) : 0u;
             rec.eB = it.b0 < it.b1 ? __ldg(tiles + it.b0) : 0u;
             rec.hb = dam_head_bits(blob, H, sq, it.head);
@@ -408,12 +463,14 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         ++ic;
         const int kvh = it.head / prm.group;
-        Walker wk; wk.init(tiles, it);
+        const Lone lA(lone, it.a0, it.qb0, nL, it.S), lB(lone, it.b0, it.qb0 + 1, nL, it.S);
+        Walker wk; wk.init(tiles, it, lA, lB);
         int kb; uint32_t kA, kB;
         while (ok && wk.next(kb, kA, kB)) {
           // what the MMA thread needs to know about this step, visible to it once the step's K tile has landed
-          step_desc[step++ & 15u] = (kA ? kStepA : 0u) | (kB ? kStepB : 0u) | (kA && wk.a_done() ? kStepLastA : 0u) |
-                                    (kB && wk.b_done() ? kStepLastB : 0u) | (wk.a_done() && wk.b_done() ? 0u : kStepMore);
+          step_desc[step++ & 15u] = (kA ? kStepA : 0u) | (kB ? kStepB : 0u) | (kA && !lA.n && wk.a_done() ? kStepLastA : 0u) |
+                                    (kB && !lB.n && wk.b_done() ? kStepLastB : 0u) |
+                                    (wk.a_done() && wk.b_done() && !(lA.n | lB.n) ? 0u : kStepMore);
           if (kA == DAM_KIND_GATHERED || kB == DAM_KIND_GATHERED) {
             const int row = (int)((gtile0 + kb) * 2 * DAM_TILE);
             ok = load_tile(&tmG, 0, row);
@@ -422,6 +479,15 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             ok = load_tile(&tmK, kvh, it.tok0 + kb * DAM_TILE);
             if (ok) ok = load_tile(&tmV, kvh, it.tok0 + kb * DAM_TILE);
           }
+        }
+        // the lone diagonal's tile of each block comes last
+#pragma unroll 1
+        for (int X = 0; X < 2 && ok; ++X) {
+          if (!(X ? lB.n : lA.n)) continue;
+          step_desc[step++ & 15u] = X ? kStepB | kStepLastB : kStepA | kStepLastA | (lB.n ? kStepMore : 0u);
+          const int tok = it.tok0 + (X ? lB.key : lA.key);
+          ok = load_tile(&tmK, kvh, tok);
+          if (ok) ok = load_tile(&tmV, kvh, tok);
         }
       }
       if (!ok) {
@@ -543,11 +609,13 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       const Item it = item_from_words(rec.u, rec.v);
       const DamHeadBits hb = rec.hb;                         // (not meaningful for an item without steps)
       const uint32_t e_first = X ? rec.eB : rec.eA;
+      const int2 lone = rec.lone;
       __syncwarp();
       if (lane == 0) mbar_arrive(bSchedEmpty + 8 * (n & 1u));               // the whole warp has read the record
       if ((X == 1 && !it.hasB) || !item_active(it)) continue;
       const int qb = it.qb0 + X;
-      const uint32_t t0 = X ? it.b0 : it.a0, t1 = X ? it.b1 : it.a1;
+      const uint32_t t0 = X ? it.b0 : it.a0;
+      uint32_t t1 = X ? it.b1 : it.a1;
       const int i = qb * DAM_TILE + r;
       const bool row_valid = i < it.S;
       __nv_bfloat16* orow = prm.O + (int64_t)(it.tok0 + i) * prm.o_stride_tok + (int64_t)it.head * prm.o_stride_head;
@@ -575,15 +643,20 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         need = (kind != DAM_KIND_FULL) || (prm.causal && kb >= qb) || ((kb + 1) * DAM_TILE > it.S);
         return need ? dam_apply_bits(hb, kind, i, kb, prm.causal) : make_uint4(~0u, ~0u, ~0u, ~0u);
       };
-      uint32_t e_next = t0 + 1 < t1 ? __ldg(tiles + t0 + 1) : 0u;
+      // entries left out: entry t of what remains is entry t + ln.n of the list from ln.at on
+      const Lone ln(lone, t0, qb, (hb.L + DAM_TILE - 1) / DAM_TILE, it.S);
+      t1 -= ln.n;
+      auto entry = [&](uint32_t t) -> uint32_t { return __ldg(tiles + (t >= ln.at ? t + ln.n : t)); };
+      uint32_t e_next = t0 + 1 < t1 ? entry(t0 + 1) : 0u;
       bool need_nx = false;
-      uint4 bits_nx = tile_bits(e_first, need_nx);
+      uint4 bits_nx = make_uint4(0u, 0u, 0u, 0u);
+      if (t0 < t1) bits_nx = tile_bits(ln.n && t0 == ln.at ? entry(t0) : e_first, need_nx);
       for (uint32_t t = t0; t < t1; ++t) {
         const bool need_mask = need_nx;
         const uint4 bits = bits_nx;
         if (t + 1 < t1) {
           bits_nx = tile_bits(e_next, need_nx);
-          if (t + 2 < t1) e_next = __ldg(tiles + t + 2);
+          if (t + 2 < t1) e_next = entry(t + 2);
         }
         if (!(ok = mbar_wait(bS, cS & 1u, abort_flag))) break;
         ++cS;
@@ -599,7 +672,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           if (!need_mask) mx = mu;
           else masked_max = __any_sync(0xFFFFFFFFu, mu * prm.scale_log2 - m_ref > kRescaleThreshold);   // -inf reference: true
         }
-        if (masked_max) mx = sweep_max<true>(tS, bits);
+        if (masked_max) mx = sweep_max_masked(tS, bits);
         const float m_new = fmaxf(m_ref, mx * prm.scale_log2);
         // move the reference only on the first tile or when the max grew by more than the threshold
         bool move = (t == t0) || (m_new - m_ref > kRescaleThreshold);   // -inf reference: inf > 8 is true
@@ -618,7 +691,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         if (t > t0) {
           const bool resc = alpha != 1.f;
           if (__any_sync(0xFFFFFFFFu, resc)) {
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {
               uint32_t rr[32];
               tmem_ld32(tO + c * 32, rr);
@@ -635,6 +708,52 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         if (lane == 0) mbar_arrive(bP);
       }
       if (!ok) break;
+      if (ln.n) {
+        // ---- the lone diagonal's tile: row r needs its entry r alone, which lies in the warp's own 32-column chunk
+        if (!(ok = mbar_wait(bS, cS & 1u, abort_flag))) break;
+        ++cS;
+        tc_fence_after();
+        uint32_t v[32];
+        tmem_ld32(tS + (warp & 3) * 32, v);
+        tc_wait_ld();
+#pragma unroll
+        for (int w = 16; w >= 1; w >>= 1)
+#pragma unroll
+          for (int q = 0; q < w; ++q) v[q] = (lane & w) ? v[q + w] : v[q];
+        const float y = row_valid ? __uint_as_float(v[0]) * prm.scale_log2 : -CUDART_INF_F;
+        float alpha = 1.f;
+        if (y - m_ref > kRescaleThreshold) {                 // (-inf reference: inf > 8, unless y is -inf too: NaN)
+          alpha = (m_ref == -CUDART_INF_F) ? 0.f : ex2(m_ref - y);
+          m_ref = y;
+        }
+        const float p = row_valid ? ex2(y - m_ref) : 0.f;
+        l = l * alpha + p;
+        const __nv_bfloat16 pb = __float2bfloat16_rn(p);
+        const uint32_t pw = (uint32_t)*reinterpret_cast<const unsigned short*>(&pb) << (16 * (lane & 1));
+        // P: zeros but for that entry
+#pragma unroll
+        for (int q = 0; q < 32; ++q) v[q] = 0u;
+        tmem_st32(tS, v);
+        tmem_st32(tS + 32, v);
+        tc_wait_st();
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = q == (lane >> 1) ? pw : 0u;
+        tmem_st16(tS + (warp & 3) * 16, v);
+        if (t0 < t1 && __any_sync(0xFFFFFFFFu, alpha != 1.f)) {
+#pragma unroll 1
+          for (int c = 0; c < D / 32; ++c) {
+            tmem_ld32(tO + c * 32, v);
+            tc_wait_ld();
+#pragma unroll
+            for (int q = 0; q < 32; ++q) v[q] = __float_as_uint(__uint_as_float(v[q]) * alpha);
+            tmem_st32(tO + c * 32, v);
+          }
+        }
+        tc_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bP);
+      }
       // ---- epilogue: O / l and the log-sum-exp
       if (!(ok = mbar_wait(bO, cO & 1u, abort_flag))) break;
       ++cO;
@@ -643,7 +762,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       if ((qb + 1) * DAM_TILE <= it.S) {
         // whole tile inside the sequence: through shared memory (128-byte swizzle) and TMA stores
         const int tok = it.tok0 + qb * DAM_TILE;
-#pragma unroll
+#pragma unroll 1
         for (int half = 0; half < D / 64; ++half) {
           uint32_t pk[32];
 #pragma unroll

@@ -12,6 +12,8 @@
 //   per (seq, head) true mask    L rows x W words, bit (j % 32) of word (j / 32) = M[i][j]
 //   pair_tab[total_pairs]        first global q-block of every pair of adjacent q-blocks (2p, 2p+1) of a
 //                                sequence; bit 31 set when the second block exists
+//   lone[num_seqs * num_q_heads] int2 per (seq, head): its lone diagonal (see dam_lone_first_qblock) or -1, and how many
+//                                entries the list of a query block it is served on has in front of the diagonal's own
 //   tile_ptr[rows + 1]           start of every row's entries in tiles[], rows = head * total_qblocks + global
 //                                q-block.  Every pair of adjacent q-blocks owns a fixed range of tiles[] (the sum
 //                                of the two rows' upper bounds, known from the shapes alone): the first row's
@@ -64,7 +66,9 @@ struct DamHeader {
   uint64_t attn_scratch_bytes;   // scratch dam_sparse_attention needs for this blob
   uint64_t mask_tiles;      // 128 x 128 tiles of the masks that hold an active cell (= total_tiles unless gathered)
   uint64_t head_tile_cap;   // entries of tiles[] every head owns (sum of the row bounds of all sequences)
-  uint64_t reserved[11];    // [0]: 1 when the window map was scored by the tensor-core kernel (test hook)
+  uint64_t reserved[9];     // [0]: 1 when the window map was scored by the tensor-core kernel (test hook)
+  uint64_t off_lone;        // 0: no section (all-ones blob)
+  uint64_t exec_tiles;      // tiles the tensor-core attention kernel multiplies (total_tiles, or fewer: lone diagonals)
 };
 static_assert(sizeof(DamHeader) == 256, "DamHeader must be 256 bytes");
 
@@ -164,6 +168,16 @@ struct DamSeqCursor {
 // Gathered-column tiles serve the query blocks that start at or after row 2L - 1 (first multiple of 128).
 __host__ __device__ inline int dam_gather_first_qblock(int L) { return (2 * L - 1 + DAM_TILE - 1) / DAM_TILE; }
 __host__ __device__ inline int dam_gather_first_row(int L) { return dam_gather_first_qblock(L) * DAM_TILE; }
+
+// A lone diagonal: the largest matched diagonal r of a head, when it is at least 255 and no other is within 254 of it, so
+// that a 128 x 128 tile with a cell of it has cells of it alone (on the query blocks below).  The usual one is r = L - 1,
+// which has a single cell in the window and so matches whenever the window's last row keeps the first key: every head
+// with a sink.  Its 128 keys of a query block lie across two tiles of the grid that hold nothing else; the tensor-core
+// attention kernel multiplies one tile that starts at the block's first such key instead, of which a row needs one entry
+// (the two listed tiles were 18 % of the attention time at 8k and 32k tokens).  Query blocks from this one on: all their
+// keys on the diagonal lie beyond the tiles of the window, so no matched column meets them.
+constexpr int kLoneMin = 255;
+__host__ __device__ inline int dam_lone_first_qblock(int r, int nL) { return nL + (r + DAM_TILE - 1) / DAM_TILE; }
 
 struct DamHeadBits {
   const uint32_t* D;

@@ -221,7 +221,8 @@ __global__ void match_kernel(unsigned char* blob, unsigned char* scratch, uint64
   const int sh = blockIdx.x;
   const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
   const DamSeq sq = dam_plan_seq(plan, blob, b);
-  if (sq.L == 0) return;
+  int2* lone = reinterpret_cast<int2*>(blob + H->off_lone) + sh;
+  if (sq.L == 0) { if (threadIdx.x == 0) *lone = make_int2(-1, 0); return; }
   const int L = sq.L, W = sq.W;
   uint32_t* dv = reinterpret_cast<uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * W;
   uint32_t* Dw = dv; uint32_t* Rw = dv + W; uint32_t* Vw = dv + 2 * W;
@@ -270,6 +271,23 @@ __global__ void match_kernel(unsigned char* blob, unsigned char* scratch, uint64
       runV += __shfl_sync(0xFFFFFFFFu, iv, 31);
     }
     if (lane == 0) { prefD[W] = runD; prefV[W] = runV; }
+    // the largest matched diagonal and the largest one below it
+    int top = -1, below = -1;
+    for (int w = lane; w < W; w += 32) if (Dw[w]) top = 32 * w + 31 - __clz(Dw[w]);
+    top = __reduce_max_sync(0xFFFFFFFFu, top);
+    for (int w = lane; w < W; w += 32) {
+      const uint32_t x = Dw[w] & ~(w == top >> 5 ? 1u << (top & 31) : 0u);
+      if (x) below = 32 * w + 31 - __clz(x);
+    }
+    below = __reduce_max_sync(0xFFFFFFFFu, below);
+    // in front of it: the gathered tiles, or the window's tiles that hold a matched column
+    int front = (runV + DAM_TILE - 1) / DAM_TILE;
+    if (!(H->flags & DAM_FLAG_GATHER)) {
+      front = 0;
+      for (int g = lane; g < W / 4; g += 32) front += (Vw[4 * g] | Vw[4 * g + 1] | Vw[4 * g + 2] | Vw[4 * g + 3]) != 0u;
+      front = __reduce_add_sync(0xFFFFFFFFu, front);
+    }
+    if (lane == 0) *lone = make_int2(top >= kLoneMin && (below < 0 || top - below >= kLoneMin) ? top : -1, front);
   }
 }
 
@@ -349,8 +367,8 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
   const int prow = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // one warp per (head, q-block pair)
   // block totals of the three statistics: one global atomic per block instead of one per warp on the same address
   __shared__ unsigned long long s_mask_tiles;
-  __shared__ uint32_t s_total, s_full;
-  if (threadIdx.x == 0) { s_mask_tiles = 0ull; s_total = 0u; s_full = 0u; }
+  __shared__ uint32_t s_total, s_full, s_exec;
+  if (threadIdx.x == 0) { s_mask_tiles = 0ull; s_total = 0u; s_full = 0u; s_exec = 0u; }
   __syncthreads();
   if (prow < H->prows) {
   const int h = prow / H->total_pairs, gp = prow % H->total_pairs;
@@ -378,7 +396,8 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
   const uint32_t pair_begin = (uint32_t)(head_base + dam_row_tile_prefix(qb0, sq.nL, sq.L, gflag));
   const uint32_t pair_end = (uint32_t)(head_base + dam_row_tile_prefix(qb0 + nblk, sq.nL, sq.L, gflag));
   uint32_t base = pair_begin, a1 = pair_begin;
-  int pair_total = 0, nfull = 0, mask_tiles = 0;
+  int pair_total = 0, nfull = 0, mask_tiles = 0, saved = 0;
+  const int lone = reinterpret_cast<const int2*>(blob + H->off_lone)[b * H->num_q_heads + h].x;
   // Per query block: candidates, ascending: [0, min(qb, nL-1)] then [max(that + 1, qb - nL), qb].  From row 2L - 1
   // on (gathered columns enabled) the first range is replaced by the gathered tiles and the second range is
   // classified on the matched diagonals alone.  The tiles of the mask itself (128 x 128 grid) with an active cell
@@ -430,6 +449,10 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
     if (x == 0) a1 = base;
     pair_total += total;
     mask_tiles += plan[x].gathered ? nat : total;
+    if (lone >= 0 && plan[x].qb >= dam_lone_first_qblock(lone, sq.nL)) {      // one tile in place of those with a cell of the lone diagonal
+      const int i0 = plan[x].qb * DAM_TILE, i1 = min(i0 + DAM_TILE, sq.S);
+      saved += (i1 - 1 - lone) / DAM_TILE - (i0 - lone) / DAM_TILE;
+    }
     total = 0; nat = 0;
   };
   const int span0 = max(plan[0].ncand, plan[0].nmask), span1 = max(plan[1].ncand, plan[1].nmask);
@@ -475,6 +498,7 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
     reinterpret_cast<uint32_t*>(scratch + off_keys)[at] = (uint32_t)min(pair_total, bp.nkeys - 1);
     atomicAdd(&s_mask_tiles, (unsigned long long)mask_tiles);
     atomicAdd(&s_total, (uint32_t)pair_total);
+    atomicAdd(&s_exec, (uint32_t)(pair_total - saved));
     atomicAdd(&s_full, (uint32_t)nfull);
   }
   }
@@ -482,6 +506,7 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
   if (threadIdx.x == 0) {
     if (s_mask_tiles) atomicAdd(reinterpret_cast<unsigned long long*>(&stats->mask_tiles), s_mask_tiles);
     if (s_total) atomicAdd(&stats->total_tiles, s_total);
+    if (s_exec) atomicAdd(reinterpret_cast<unsigned long long*>(&stats->exec_tiles), (unsigned long long)s_exec);
     if (s_full) atomicAdd(&stats->full_tiles, s_full);
   }
 }
@@ -616,6 +641,7 @@ __global__ void all_ones_kernel(unsigned char* blob, int causal) {
       H->total_tiles = tot;
       H->full_tiles = tot;
       H->mask_tiles = tot;
+      H->exec_tiles = tot;
       H->bytes_used = H->off_tiles + 4ull * tot;
     }
   }

@@ -125,6 +125,25 @@ def test_masked_small_cases_every_row(lengths, pcl, Hq, Hkv, d, dtype, gather):
     _masked_case(w, _all_rows, gather=gather)
 
 
+@pytest.mark.parametrize("gather", [False, True])
+@pytest.mark.parametrize("lengths,pcl,Hq,Hkv,d", [
+    ([1700], 384, 4, 2, 128),                # the lone diagonal crosses two tiles of every block
+    ([1283, 1153, 900], 500, 4, 1, 64),      # window not a multiple of the tile; last blocks of 3 and 1 rows; one without such blocks
+    ([1664], 385, 2, 2, 128),                # r = 384: whole tiles of the grid
+])
+def test_lone_diagonal_every_row(lengths, pcl, Hq, Hkv, d, gather):
+    """Heads whose window keeps the first key in its last row: the diagonal r = L - 1 stands alone and is served by a
+    tile that starts at its first key.  Head 0 attends to the first key only (a block whose list has nothing else)."""
+    w = synth.small_case(0, Hq, Hkv, d, pcl, seed=23, dtype=torch.bfloat16, lengths=lengths)
+    plans = [[synth.HeadPlan(sink=True, band_m=0 if h == 0 else (8, 16, 24)[h % 3], stripes=[] if h == 0 else [5, pcl // 2])
+              for h in range(Hq)] for _ in lengths]
+    parts = [synth.make_sequence(S, Hq, Hkv, d, min(S, pcl), plans[b], 8.0, [23, b], "cpu") for b, S in enumerate(lengths)]
+    w.Q, w.K, w.V = (torch.cat([p[k] for p in parts]).to(torch.bfloat16) for k in range(3))
+    blob, shape, masks, _, _, _ = _masked_case(w, _all_rows, gather=gather, sentinel=True)
+    st = B.dam_mask_stats(blob, shape)
+    assert st["executed_tiles"] < st["tiles"] if pcl != 385 else st["executed_tiles"] == st["tiles"]
+
+
 def test_empty_rows_and_no_patterns():
     """mu > 1: nothing matches, every row below the window is empty."""
     w = synth.small_case(0, 4, 2, 128, 128, seed=5, lengths=[600])
