@@ -241,7 +241,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       uint32_t* Mrow = reinterpret_cast<uint32_t*>(blob + H->off_true) + it.sq.true_off + (uint64_t)it.h * L * W + (size_t)i * W;
       float* Prow = prm.dump ? prm.dump + it.sq.p_off + (uint64_t)it.h * L * L + (size_t)i * L : nullptr;
       const int nk = it.qb + 1;
-      float m = -CUDART_INF_F, l = 0.f, inv_l = 0.f, thr_raw = 0.f;
+      float m = -CUDART_INF_F, l = 0.f, inv_l = 0.f, thr_raw = 0.f, margin = 0.f;
       for (int t = 0; t < 2 * nk; ++t, ++g) {
         if (t == nk) {
           // all groups have finished sweep A: merge their (max, sum) per row through shared memory
@@ -261,7 +261,8 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           }
           m = mn; l = ls;
           inv_l = l > 0.f ? 1.0f / l : 0.f;
-          thr_raw = (log2f(prm.pstar * l) - 0.03125f + m) / prm.scale_log2;   // the same bound on the raw dot product
+          thr_raw = (log2f(prm.pstar * l) + m) / prm.scale_log2;              // the raw dot product at which p = p*
+          margin = (0.000244140625f + fabsf(m) * 7.62939453125e-6f) / prm.scale_log2;      // 2^-12 + |m| 2^-17
         }
         if ((g & 3u) != (uint32_t)G) continue;
         const int kb = t % nk;
@@ -333,23 +334,25 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
               }
             }
           } else {
-            // only the decision p >= p* is needed.  p = 2^(x scale - m) / l, so an entry whose x scale - m lies
-            // more than 2^-5 below log2(p* l) cannot reach p* (the margin is five orders of magnitude above the
-            // rounding of the fast exponential and of the comparison on the raw value); groups of 8 columns with
-            // no candidate in the whole warp skip the special-function unit.  Candidates are evaluated exactly
-            // as in the branch above.
+            // only the decision p >= p* is needed, p = 2^(x scale - m) / l.  It is the sign of x - thr, thr being the raw
+            // product at which p reaches p*, except where x lies within `margin` of it: a chunk with such an entry is
+            // evaluated exactly as in the branch above.  (Rounding of thr and of p is below 2^-17 + |m| 2^-22 in log2
+            // units, the margin is 32 times that.)  The special-function unit is not needed otherwise: with a candidate
+            // test and the exact form for every candidate, rows of noise were candidates throughout.
             uint32_t word = 0u;
+            float near = CUDART_INF_F;
 #pragma unroll
-            for (int q8 = 0; q8 < 32; q8 += 8) {
-              bool any = false;
+            for (int q = 31; q >= 0; --q) {
+              const float dlt = thr_raw - x[q];                            // negative: p > p*
+              near = fminf(near, fabsf(dlt));
+              word = __funnelshift_l(__float_as_uint(dlt), word, 1);       // its sign bit becomes the lowest bit
+            }
+            if (__any_sync(0xFFFFFFFFu, near <= margin)) {
+              word = 0u;
 #pragma unroll
-              for (int u = 0; u < 8; ++u) any |= x[q8 + u] > thr_raw;
-              if (__any_sync(0xFFFFFFFFu, any)) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                  const float p = ex2(fmaf(x[q8 + u], prm.scale_log2, -m)) * inv_l;
-                  word |= (p >= prm.pstar ? 1u : 0u) << (q8 + u);
-                }
+              for (int q = 0; q < 32; ++q) {
+                const float p = ex2(fmaf(x[q], prm.scale_log2, -m)) * inv_l;
+                word |= (p >= prm.pstar ? 1u : 0u) << q;
               }
             }
             if (c == 0) words.x = word; else if (c == 1) words.y = word; else if (c == 2) words.z = word; else words.w = word;
