@@ -402,7 +402,9 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
   // on (gathered columns enabled) the first range is replaced by the gathered tiles and the second range is
   // classified on the matched diagonals alone.  The tiles of the mask itself (128 x 128 grid) with an active cell
   // are counted in the same sweep: they equal the listed tiles unless the row is served by gathered tiles.
-  struct BlockPlan { int qb, gathered, n1, lo2, ncand, m1, l2, nmask; };
+  // On a gathered row whose band lies beyond the window's tiles (`apart`) they are the window's tiles with a matched
+  // column and the listed band tiles: the band is not classified a second time for the count.
+  struct BlockPlan { int qb, gathered, n1, lo2, ncand, m1, l2, nmask, apart; };
   const int nV = (gflag && sq.L > 0) ? v.prefV[sq.W] : 0;        // matched columns of the head
   BlockPlan plan[2];
 #pragma unroll
@@ -415,7 +417,8 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
     p.ncand = x < nblk ? p.n1 + max(0, p.qb - p.lo2 + 1) : 0;
     p.m1 = min(p.qb, sq.nL - 1) + 1;
     p.l2 = max(p.m1, p.qb - sq.nL);
-    p.nmask = (x < nblk && p.gathered) ? p.m1 + max(0, p.qb - p.l2 + 1) : 0;
+    p.apart = p.gathered && p.qb - sq.nL >= sq.nL;
+    p.nmask = (x < nblk && p.gathered) ? (p.apart ? sq.nL : p.m1 + max(0, p.qb - p.l2 + 1)) : 0;
   }
   // one candidate per lane: list entry (kind 0: not listed) and whether the mask tile has an active cell
   auto eval = [&](const BlockPlan& p, int idx, uint32_t& kind, uint32_t& entry, bool& act) {
@@ -430,7 +433,8 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
         entry = (uint32_t)kb | (kind << 28);
       }
     }
-    act = idx < p.nmask && classify_tile(v, p.qb, idx < p.m1 ? idx : p.l2 + (idx - p.m1)) != 0u;
+    act = idx < p.nmask && (p.apart ? cnt_range(v.Vw, v.prefV, idx * DAM_TILE, min(idx * DAM_TILE + DAM_TILE, v.L) - 1) > 0
+                                    : classify_tile(v, p.qb, idx < p.m1 ? idx : p.l2 + (idx - p.m1)) != 0u);
   };
   int total = 0, nat = 0;
   auto consume = [&](uint32_t kind, uint32_t entry, bool act) {
@@ -448,7 +452,7 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
     base += total;
     if (x == 0) a1 = base;
     pair_total += total;
-    mask_tiles += plan[x].gathered ? nat : total;
+    mask_tiles += plan[x].apart ? nat + total - plan[x].n1 : plan[x].gathered ? nat : total;
     if (lone >= 0 && plan[x].qb >= dam_lone_first_qblock(lone, sq.nL)) {      // one tile in place of those with a cell of the lone diagonal
       const int i0 = plan[x].qb * DAM_TILE, i1 = min(i0 + DAM_TILE, sq.S);
       saved += (i1 - 1 - lone) / DAM_TILE - (i0 - lone) / DAM_TILE;
