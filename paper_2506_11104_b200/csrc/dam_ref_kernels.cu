@@ -53,6 +53,18 @@ __device__ __forceinline__ void load_stage(float* dst, int pitch, const T* __res
   }
 }
 
+// The same for fp32 rows with asynchronous copies: the caller commits and waits.
+__device__ __forceinline__ void load_stage_async(float* dst, int pitch, const float* __restrict__ src, int64_t st, int j0, int n, int d) {
+  const int ppr = d >> 2;                                       // 16-byte pieces per row
+  for (int x = threadIdx.x; x < kStageKeys * ppr; x += blockDim.x) {
+    const int r = x / ppr, piece = x % ppr;
+    const uint32_t to = static_cast<uint32_t>(__cvta_generic_to_shared(dst + r * pitch + piece * 4));
+    const bool in = j0 + r < n;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(src + (int64_t)(in ? j0 + r : 0) * st + piece * 4),
+                 "r"(in ? 16 : 0) : "memory");                  // (0 source bytes: zeros)
+  }
+}
+
 // Dot products of R query rows (fp32, shared memory, d floats apart) with the keys of rows k0 and k1: one fused
 // multiply-add per dimension in ascending order.
 template <int R>
@@ -89,6 +101,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 // Two sweeps over the keys of a row (max / sum, then probabilities); the fp32 probability that is
 // compared with p* is the very value written to the dump.
 // ---------------------------------------------------------------------------------------------
+// `nbuf` stages of K fit in shared memory: a block that needs no more loads them all at once, before the first sweep, and
+// neither sweep waits again (512 tokens, PCL 128: 12.4 -> 11.3 us).  Otherwise a stage is loaded when it is due.
 // Bound by latency at the sizes this path serves.  A block takes 8 R adjacent rows (R per warp) of one map and walks
 // the keys in stages of 64 held in shared memory, so that a key row is read from memory once per block and not once per
 // row.  R = 1 while that leaves SMs idle, 4 otherwise (a stage then feeds four times the multiply-adds).
@@ -96,8 +110,8 @@ template <typename T, int R>
 __global__ void __launch_bounds__(256)
 scores_ref_kernel(unsigned char* blob, const T* __restrict__ Q, const T* __restrict__ K,
                   int Hq, int group, int d, int64_t qst, int64_t qsh, int64_t kst, int64_t ksh,
-                  float scale, float pstar, float* __restrict__ dump) {
-  extern __shared__ float smem[];
+                  float scale, float pstar, float* __restrict__ dump, int nbuf) {
+  extern __shared__ __align__(16) float smem[];
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   const int sh = blockIdx.y;
   const int b = sh / Hq, h = sh % Hq;
@@ -107,13 +121,18 @@ scores_ref_kernel(unsigned char* blob, const T* __restrict__ Q, const T* __restr
   if (i_block >= sq.L) return;
   const int i_end = min(i_block + nw * R, sq.L);                // keys 0 .. i_end - 1 matter to the block
   const int i0 = i_block + warp * R;
+  const int stage = kStageKeys * k_pitch(d);
   float* k_s = smem;
-  float* q_s = smem + kStageKeys * k_pitch(d) + warp * R * d;
+  float* q_s = smem + nbuf * stage + warp * R * d;
+  const int nstage = (i_end + kStageKeys - 1) / kStageKeys;
+  const bool resident = nstage <= nbuf;
+  const T* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
+  if (resident) for (int t = 0; t < nstage; ++t) load_stage<T>(k_s + t * stage, k_pitch(d), Kh, kst, t * kStageKeys, sq.L, d);
   for (int x = lane; x < R * d; x += 32) {
     const int i = i0 + x / d;
     q_s[x] = i < sq.L ? Ld8<T>::one(Q + (int64_t)(sq.tok_start + i) * qst + (int64_t)h * qsh + x % d) : 0.f;
   }
-  const T* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
+  if (resident) __syncthreads();
   uint32_t* M = reinterpret_cast<uint32_t*>(blob + H->off_true) + sq.true_off + (uint64_t)h * sq.L * sq.W;
   float* Ph = dump ? dump + sq.p_off + (uint64_t)h * sq.L * sq.L : nullptr;
   float m[R], l[R], mw[R];
@@ -121,17 +140,17 @@ scores_ref_kernel(unsigned char* blob, const T* __restrict__ Q, const T* __restr
   for (int r = 0; r < R; ++r) { m[r] = -CUDART_INF_F; l[r] = 0.f; mw[r] = 0.f; }
   const float* k0 = k_s + lane * k_pitch(d);
   const float* k1 = k0 + 32 * k_pitch(d);
-  const int nstage = (i_end + kStageKeys - 1) / kStageKeys;
   for (int sweep = 0; sweep < 2; ++sweep) {
     for (int t = 0; t < nstage; ++t) {
       const int j0 = t * kStageKeys;
-      if (nstage > 1 || sweep == 0) {                           // a single stage is still there in the second sweep
+      if (!resident) {
         __syncthreads();
         load_stage<T>(k_s, k_pitch(d), Kh, kst, j0, sq.L, d);
         __syncthreads();
       }
       float s[R][2];
-      dot_rows<R>(q_s, k0, k1, d, s);
+      const int at = resident ? t * stage : 0;
+      dot_rows<R>(q_s, k0 + at, k1 + at, d, s);
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const int j = j0 + c * 32 + lane;
@@ -176,15 +195,17 @@ scores_ref_kernel(unsigned char* blob, const T* __restrict__ Q, const T* __restr
 // (head, q-block) row of the tile list and walks its tiles in stages of 64 keys whose K and V rows sit in shared memory;
 // a stage without an active cell in the block's rows is not loaded.  The lanes of a warp are keys for the scores and
 // dimensions for the output.  Latency bound at the sizes this path serves: R = 1 while that leaves SMs idle, 4 otherwise.
+// PIPE (fp32, two stages fit in shared memory): the next stage with an active cell is looked for and its copies are
+// started before this one is worked on (512 tokens, 2 heads: 28.5 -> 21.7 us; leaving out the keys no row keeps inside a stage: no change).
 // ---------------------------------------------------------------------------------------------
-template <typename T, int R, int ND>
+template <typename T, int R, int ND, bool PIPE>
 __global__ void __launch_bounds__(256)
 attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __restrict__ K,
                 const T* __restrict__ V, int Hq, int group, int d, int64_t qst, int64_t qsh,
                 int64_t kst, int64_t ksh, int64_t vst, int64_t vsh, int64_t ost, int64_t osh,
                 int causal, float scale, T* __restrict__ O, float* __restrict__ lse, int total_tokens,
                 const int32_t* __restrict__ ranges) {
-  extern __shared__ float smem[];
+  extern __shared__ __align__(16) float smem[];
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   const int row = blockIdx.x;
   const int h = row / H->total_qblocks, gqb = row % H->total_qblocks;
@@ -204,18 +225,17 @@ attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __r
   const uint32_t t0 = tile_ptr[row], t1 = tile_ptr[row + 1];
   const DamHeadBits hb = dam_head_bits(blob, H, sq, h);
   const int pitch = k_pitch(d);
+  const int stage = kStageKeys * (pitch + d);
   float* k_s = smem;
   float* v_s = k_s + kStageKeys * pitch;
-  float* q_s = v_s + kStageKeys * d + warp * R * d;
-  float* p_s = v_s + kStageKeys * d + nw * R * d + warp * R * kStageKeys;       // the warp's probabilities of a stage
+  float* q_s = smem + (PIPE ? 2 : 1) * stage + warp * R * d;
+  float* p_s = smem + (PIPE ? 2 : 1) * stage + nw * R * d + warp * R * kStageKeys;       // the warp's probabilities of a stage
   for (int x = lane; x < R * d; x += 32) {
     const int i = i0 + x / d;
     q_s[x] = i < sq.S ? Ld8<T>::one(Q + (int64_t)(sq.tok_start + i) * qst + (int64_t)h * qsh + x % d) : 0.f;
   }
   const T* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
   const T* Vh = V + (int64_t)sq.tok_start * vst + (int64_t)(h / group) * vsh;
-  const float* k0 = k_s + lane * pitch;
-  const float* k1 = k0 + 32 * pitch;
   float acc[R][ND], m[R], l[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -223,63 +243,102 @@ attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __r
 #pragma unroll
     for (int u = 0; u < ND; ++u) acc[r][u] = 0.f;
   }
-  for (uint32_t t = t0; t < t1; ++t) {
-    const uint32_t e = __ldg(tiles + t);
-    if ((e >> 28) == 0u) continue;                      // padding behind the row's entries
-    const int kb = (int)(e & 0x0FFFFFFFu);
-    uint4 bits[R];
+  // the stages of the row's tiles that hold an active cell of the block's rows, in order
+  struct Stage { uint32_t w0[R], w1[R], any; int j0; bool valid; };
+  uint32_t t = t0;
+  int half = 2, kb = 0;
+  uint4 bits[R];
+  auto find = [&](Stage& g) {
+    while (true) {
+      if (half == 2) {
+        uint32_t e = 0u;
+        while (t < t1 && ((e = __ldg(tiles + t)) >> 28) == 0u) ++t;     // padding behind the row's entries
+        if (t >= t1) { g.valid = false; return; }
+        ++t;
+        kb = (int)(e & 0x0FFFFFFFu);
 #pragma unroll
-    for (int r = 0; r < R; ++r) bits[r] = dam_apply_bits(hb, e >> 28, i0 + r, kb, causal);
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t any = 0u;
-#pragma unroll
-      for (int r = 0; r < R; ++r) any |= half ? (bits[r].z | bits[r].w) : (bits[r].x | bits[r].y);
-      if (!__syncthreads_or(any != 0u)) continue;       // (the previous stage is no longer read)
-      const int j0 = kb * DAM_TILE + half * kStageKeys;
-      load_stage<T>(k_s, pitch, Kh, kst, j0, sq.S, d);
-      load_stage<T>(v_s, d, Vh, vst, j0, sq.S, d);
-      __syncthreads();
-      if (!any) continue;                               // (the same in all lanes: the words are the row's)
-      float s[R][2];
-      dot_rows<R>(q_s, k0, k1, d, s);
+        for (int r = 0; r < R; ++r) bits[r] = dam_apply_bits(hb, e >> 28, i0 + r, kb, causal);
+        half = 0;
+      }
+      g.any = 0u;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const uint32_t w0 = half ? bits[r].z : bits[r].x, w1 = half ? bits[r].w : bits[r].y;
-        const bool a0 = (w0 >> lane) & 1u, a1 = (w1 >> lane) & 1u;
-        const float x0 = a0 ? s[r][0] * scale : -CUDART_INF_F, x1 = a1 ? s[r][1] * scale : -CUDART_INF_F;
-        const float mn = fmaxf(m[r], warp_max(fmaxf(x0, x1)));
-        const float corr = (m[r] == -CUDART_INF_F) ? 0.f : expf(m[r] - mn);
-        const float p0 = a0 ? expf(x0 - mn) : 0.f, p1 = a1 ? expf(x1 - mn) : 0.f;
-        l[r] = l[r] * corr + warp_sum(p0 + p1);
-        m[r] = mn;
-#pragma unroll
-        for (int u = 0; u < ND; ++u) acc[r][u] *= corr;
-        p_s[r * kStageKeys + lane] = p0;
-        p_s[r * kStageKeys + 32 + lane] = p1;
+        g.w0[r] = half ? bits[r].z : bits[r].x;
+        g.w1[r] = half ? bits[r].w : bits[r].y;
+        g.any |= g.w0[r] | g.w1[r];
       }
-      __syncwarp();
+      g.j0 = kb * DAM_TILE + half * kStageKeys;
+      ++half;
+      if (__syncthreads_or(g.any != 0u)) { g.valid = true; return; }    // (a barrier: the stage before the last is no longer read)
+    }
+  };
+  auto work = [&](const Stage& g, const float* k_b, const float* v_b) {
+    if (!g.any) return;                                 // (the same in all lanes: the words are the row's)
+    float s[R][2];
+    dot_rows<R>(q_s, k_b + lane * pitch, k_b + (32 + lane) * pitch, d, s);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const bool a0 = (g.w0[r] >> lane) & 1u, a1 = (g.w1[r] >> lane) & 1u;
+      const float x0 = a0 ? s[r][0] * scale : -CUDART_INF_F, x1 = a1 ? s[r][1] * scale : -CUDART_INF_F;
+      const float mn = fmaxf(m[r], warp_max(fmaxf(x0, x1)));
+      const float corr = (m[r] == -CUDART_INF_F) ? 0.f : expf(m[r] - mn);
+      const float p0 = a0 ? expf(x0 - mn) : 0.f, p1 = a1 ? expf(x1 - mn) : 0.f;
+      l[r] = l[r] * corr + warp_sum(p0 + p1);
+      m[r] = mn;
+#pragma unroll
+      for (int u = 0; u < ND; ++u) acc[r][u] *= corr;
+      p_s[r * kStageKeys + lane] = p0;
+      p_s[r * kStageKeys + 32 + lane] = p1;
+    }
+    __syncwarp();
 #pragma unroll 2
-      for (int k = 0; k < kStageKeys; k += 4) {
-        float4 p[R];
+    for (int k = 0; k < kStageKeys; k += 4) {
+      float4 p[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) p[r] = *reinterpret_cast<const float4*>(p_s + r * kStageKeys + k);
+      for (int r = 0; r < R; ++r) p[r] = *reinterpret_cast<const float4*>(p_s + r * kStageKeys + k);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < 4; ++q) {
 #pragma unroll
-          for (int u = 0; u < ND; ++u) {
-            const int t_ = lane + 32 * u;
-            const float v = t_ < d ? v_s[(k + q) * d + t_] : 0.f;
+        for (int u = 0; u < ND; ++u) {
+          const int t_ = lane + 32 * u;
+          const float v = t_ < d ? v_b[(k + q) * d + t_] : 0.f;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-              // (a key the row does not keep is left out, whatever its V row holds)
-              const float pk = q == 0 ? p[r].x : q == 1 ? p[r].y : q == 2 ? p[r].z : p[r].w;
-              if (pk != 0.f) acc[r][u] = fmaf(pk, v, acc[r][u]);
-            }
+          for (int r = 0; r < R; ++r) {
+            // (a key the row does not keep is left out, whatever its V row holds)
+            const float pk = q == 0 ? p[r].x : q == 1 ? p[r].y : q == 2 ? p[r].z : p[r].w;
+            if (pk != 0.f) acc[r][u] = fmaf(pk, v, acc[r][u]);
           }
         }
       }
-      __syncwarp();
+    }
+    __syncwarp();
+  };
+  if constexpr (PIPE) {
+    auto start = [&](const Stage& g, int buf) {
+      if (g.valid) {
+        load_stage_async(k_s + buf * stage, pitch, reinterpret_cast<const float*>(Kh), kst, g.j0, sq.S, d);
+        load_stage_async(v_s + buf * stage, d, reinterpret_cast<const float*>(Vh), vst, g.j0, sq.S, d);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    Stage cur, nxt;
+    find(cur);
+    start(cur, 0);
+    for (int buf = 0; cur.valid; buf ^= 1) {
+      find(nxt);
+      start(nxt, buf ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncthreads();
+      work(cur, k_s + buf * stage, v_s + buf * stage);
+      cur = nxt;
+    }
+  } else {
+    Stage cur;
+    for (find(cur); cur.valid; find(cur)) {
+      load_stage<T>(k_s, pitch, Kh, kst, cur.j0, sq.S, d);
+      load_stage<T>(v_s, d, Vh, vst, cur.j0, sq.S, d);
+      __syncthreads();
+      work(cur, k_s, v_s);
     }
   }
 #pragma unroll
@@ -302,31 +361,44 @@ attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __r
 constexpr int kRefWarps = 8;
 inline bool four_rows(long long rows, int sm_count) { return rows >= (long long)sm_count * kRefWarps * 4; }
 
-size_t score_smem(int d, int R) { return ((size_t)kStageKeys * k_pitch(d) + (size_t)kRefWarps * R * d) * sizeof(float); }
-size_t attn_smem(int d, int R) {
-  return ((size_t)kStageKeys * (k_pitch(d) + d) + (size_t)kRefWarps * R * (d + kStageKeys)) * sizeof(float);
+size_t score_smem(int d, int R, int nbuf) { return ((size_t)nbuf * kStageKeys * k_pitch(d) + (size_t)kRefWarps * R * d) * sizeof(float); }
+size_t attn_smem(int d, int R, int nbuf) {
+  return ((size_t)nbuf * kStageKeys * (k_pitch(d) + d) + (size_t)kRefWarps * R * (d + kStageKeys)) * sizeof(float);
+}
+
+// (48 KB of dynamic shared memory need no opt-in)
+template <typename F>
+cudaError_t allow_smem(F* kernel, size_t bytes) {
+  return bytes <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 template <typename T, int R>
-cudaError_t launch_scores(const void* Q, const void* K, const dam_shape_t* s, const DamBuildCtx& c, float* dump, cudaStream_t st) {
-  const size_t sm = score_smem(c.d, R);
-  cudaError_t e = cudaFuncSetAttribute(scores_ref_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_scores(const void* Q, const void* K, const dam_shape_t* s, const DamBuildCtx& c, float* dump, int sm_count,
+                          int smem_max, cudaStream_t st) {
   const dim3 grid((c.max_L + kRefWarps * R - 1) / (kRefWarps * R), c.num_seqs * c.Hq);
+  // all stages at once while every block has an SM of its own anyway (a block's shared memory then costs no occupancy)
+  const int nstage = (c.max_L + kStageKeys - 1) / kStageKeys;
+  const int nbuf = (long long)grid.x * grid.y <= sm_count && score_smem(c.d, R, nstage) <= (size_t)smem_max ? nstage : 1;
+  const size_t sm = score_smem(c.d, R, nbuf);
+  cudaError_t e = allow_smem(scores_ref_kernel<T, R>, sm);
+  if (e != cudaSuccess) return e;
   scores_ref_kernel<T, R><<<grid, kRefWarps * 32, sm, st>>>(c.blob, (const T*)Q, (const T*)K, c.Hq, c.Hq / c.Hkv, c.d, s->q_stride_tok,
                                                             s->q_stride_head, s->k_stride_tok, s->k_stride_head, c.scale,
-                                                            c.pstar, dump);
+                                                            c.pstar, dump, nbuf);
   return cudaGetLastError();
 }
 
 template <typename T, int R, int ND>
 cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
-                        float scale, void* O, float* lse, const int32_t* ranges, int rows, cudaStream_t st) {
-  const size_t sm = attn_smem(s->head_dim, R);
-  cudaError_t e = cudaFuncSetAttribute(attn_ref_kernel<T, R, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                        float scale, void* O, float* lse, const int32_t* ranges, int rows, int smem_max, cudaStream_t st) {
+  const bool pipe = sizeof(T) == 4 && attn_smem(s->head_dim, R, 2) <= (size_t)smem_max;
+  const size_t sm = attn_smem(s->head_dim, R, pipe ? 2 : 1);
+  auto kernel = attn_ref_kernel<T, R, ND, false>;
+  if constexpr (sizeof(T) == 4) { if (pipe) kernel = attn_ref_kernel<T, R, ND, true>; }
+  cudaError_t e = allow_smem(kernel, sm);
   if (e != cudaSuccess) return e;
   const dim3 grid(rows, DAM_TILE / (kRefWarps * R));
-  attn_ref_kernel<T, R, ND><<<grid, kRefWarps * 32, sm, st>>>(
+  kernel<<<grid, kRefWarps * 32, sm, st>>>(
       (const unsigned char*)blob, (const T*)Q, (const T*)K, (const T*)V, s->num_q_heads, s->num_q_heads / s->num_kv_heads, s->head_dim,
       s->q_stride_tok, s->q_stride_head, s->k_stride_tok, s->k_stride_head, s->v_stride_tok, s->v_stride_head, s->o_stride_tok,
       s->o_stride_head, causal, scale, (T*)O, lse, s->total_tokens, ranges);
@@ -335,11 +407,11 @@ cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void*
 
 template <typename T, int R>
 cudaError_t launch_attn_dims(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
-                             float scale, void* O, float* lse, const int32_t* ranges, int rows, cudaStream_t st) {
+                             float scale, void* O, float* lse, const int32_t* ranges, int rows, int smem_max, cudaStream_t st) {
   const int nd = (s->head_dim + 31) / 32;
-  if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
-  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
-  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
+  if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, smem_max, st);
+  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, smem_max, st);
+  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, smem_max, st);
 }
 
 }  // namespace
@@ -353,8 +425,8 @@ cudaError_t dam_launch_scores_ref(const void* Q, const void* K, const dam_shape_
   if (e != cudaSuccess) return e;
   const bool four = four_rows((long long)c.max_L * c.num_seqs * c.Hq, di.sm_count);
   if (c.dtype == DAM_F32)
-    return four ? launch_scores<float, 4>(Q, K, s, c, dump, st) : launch_scores<float, 1>(Q, K, s, c, dump, st);
-  return four ? launch_scores<__nv_bfloat16, 4>(Q, K, s, c, dump, st) : launch_scores<__nv_bfloat16, 1>(Q, K, s, c, dump, st);
+    return four ? launch_scores<float, 4>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st) : launch_scores<float, 1>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st);
+  return four ? launch_scores<__nv_bfloat16, 4>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st) : launch_scores<__nv_bfloat16, 1>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st);
 }
 
 cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s,
@@ -372,8 +444,8 @@ cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, con
   if (e != cudaSuccess) return e;
   const bool four = four_rows((long long)rows * DAM_TILE, di.sm_count);
   if (s->dtype == DAM_F32)
-    return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st)
-                : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
-  return four ? launch_attn_dims<__nv_bfloat16, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st)
-              : launch_attn_dims<__nv_bfloat16, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, st);
+    return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, di.smem_optin, st)
+                : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, di.smem_optin, st);
+  return four ? launch_attn_dims<__nv_bfloat16, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, di.smem_optin, st)
+              : launch_attn_dims<__nv_bfloat16, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rows, di.smem_optin, st);
 }

@@ -125,6 +125,19 @@ def test_masked_small_cases_every_row(lengths, pcl, Hq, Hkv, d, dtype, gather):
     _masked_case(w, _all_rows, gather=gather)
 
 
+@pytest.mark.parametrize("S,pcl,d,dtype", [
+    (300, 150, 8, torch.float32), (300, 150, 160, torch.float32),        # one and two staged buffers' largest head_dim range
+    (260, 130, 256, torch.float32), (260, 130, 256, torch.bfloat16),      # two buffers do not fit with four rows per warp
+    (1300, 700, 64, torch.float32), (5000, 130, 40, torch.float32),       # four rows per warp; a window of more stages than fit
+])
+def test_cuda_core_kernels_every_row(S, pcl, d, dtype):
+    w = synth.small_case(S, 2, 1, d, pcl, seed=14, dtype=dtype) if d >= 16 else None
+    if w is None:                                                        # too narrow for planted structure: noise alone
+        w = synth.small_case(S, 2, 1, 16, pcl, seed=14, dtype=dtype)
+        w.Q, w.K, w.V = (x[..., -d:].contiguous() for x in (w.Q, w.K, w.V))
+    _masked_case(w, _sample_rows(pcl) if S > 2000 else _all_rows)
+
+
 @pytest.mark.parametrize("gather", [False, True])
 @pytest.mark.parametrize("lengths,pcl,Hq,Hkv,d", [
     ([1700], 384, 4, 2, 128),                # the lone diagonal crosses two tiles of every block
