@@ -830,6 +830,10 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 // Copies the K and V rows of the matched columns of every (sequence, head) into dense tiles of 128 keys in
 // the scratch buffer (K tile at rows (2T) * 128, V tile at rows (2T + 1) * 128 of a [rows][head_dim] bf16 array;
 // T = gath_off + head * nL + g).  Rows past the last matched column are zero.  One block per tile, grid-stride.
+// Bound by latency: a chain of header, column index, row.  The indices are read from the list that stands beside the
+// ordering of the work list; found here instead, from the V words by prefix counts and a search per place, they took
+// another 1-1.5 us of every call (a 2048-row chunk against a 2048-token window 66.4 us, now 64.9; 1024 tokens with a
+// 256-token window 59.3, now 58.6; 8192 tokens 151.2, now 149.7).
 __global__ void __launch_bounds__(128)
 gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat16* __restrict__ K,
                       const __nv_bfloat16* __restrict__ V, int Hq, int group, int d, int64_t kst, int64_t ksh, int64_t vst,
@@ -847,52 +851,23 @@ gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat1
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(reinterpret_cast<uint32_t*>(scratch) + 1, (uint32_t)DAM_ERR_BUFFER_TOO_SMALL);
     return;
   }
-  __shared__ int pref[1025];
   __shared__ int col[DAM_TILE];
   uint4* out = reinterpret_cast<uint4*>(scratch + 256);
+  const unsigned short* cols = reinterpret_cast<const unsigned short*>(blob + H->off_cols);
   const DamSeq* seqs = reinterpret_cast<const DamSeq*>(blob + H->off_seq);
   const int tid = threadIdx.x;
   for (long long T = blockIdx.x; T < (long long)H->gath_tiles; T += gridDim.x) {
+    const int c_mine = __ldg(cols + T * DAM_TILE + tid);
     int b = 0;
     while (b + 1 < H->num_seqs && (long long)seqs[b + 1].gath_off <= T) ++b;
     const DamSeq sq = seqs[b];
     if (sq.nL == 0) continue;
     const int h = (int)((T - (long long)sq.gath_off) / sq.nL), g = (int)((T - (long long)sq.gath_off) % sq.nL);
     if (h >= Hq) continue;
-    const uint32_t* Vw = reinterpret_cast<const uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * sq.W + 2 * sq.W;
-    // exclusive prefix popcounts of the V words (W <= 1024 words, i.e. windows up to 32768 tokens)
-    const int W = min(sq.W, 1024);
     __syncthreads();
-    if (tid < 32) {                                              // warp 0: 32 words per step
-      int run = 0;
-      for (int w0 = 0; w0 < W; w0 += 32) {
-        const int w = w0 + tid;
-        const int pc = w < W ? __popc(__ldg(Vw + w)) : 0;
-        int inc = pc;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-          if (tid >= o) inc += y;
-        }
-        if (w < W) pref[w] = run + inc - pc;
-        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
-      }
-      if (tid == 0) pref[W] = run;
-    }
+    col[tid] = c_mine == 0xFFFF ? -1 : c_mine;
     __syncthreads();
-    const int nV = pref[W];
-    if (g * DAM_TILE >= nV) continue;                         // capacity tile that no row list refers to
-    {
-      const int rank = g * DAM_TILE + tid;
-      int c = -1;
-      if (rank < nV) {
-        int lo = 0, hi = W;                                     // last word with pref <= rank
-        while (hi - lo > 1) { int mid = (lo + hi) >> 1; if (pref[mid] <= rank) lo = mid; else hi = mid; }
-        c = lo * 32 + (int)__fns(Vw[lo], 0, rank - pref[lo] + 1);
-      }
-      col[tid] = c;
-    }
-    __syncthreads();
+    if (col[0] < 0) continue;                                 // capacity tile that no row list refers to
     const __nv_bfloat16* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
     const __nv_bfloat16* Vh = V + (int64_t)sq.tok_start * vst + (int64_t)(h / group) * vsh;
     const int ppr = d >> 3;                                      // 16-byte pieces per row (16 at head_dim 128, 8 at 64)

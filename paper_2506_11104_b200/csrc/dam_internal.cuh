@@ -14,6 +14,8 @@
 //                                sequence; bit 31 set when the second block exists
 //   lone[num_seqs * num_q_heads] int2 per (seq, head): its lone diagonal (see dam_lone_first_qblock) or -1, and how many
 //                                entries the list of a query block it is served on has in front of the diagonal's own
+//   cols (gathered columns only) u16 per place of every gathered-column tile of every (seq, head): the head's matched
+//                                columns in ascending order, 0xFFFF behind the last one
 //   tile_ptr[rows + 1]           start of every row's entries in tiles[], rows = head * total_qblocks + global
 //                                q-block.  Every pair of adjacent q-blocks owns a fixed range of tiles[] (the sum
 //                                of the two rows' upper bounds, known from the shapes alone): the first row's
@@ -66,7 +68,8 @@ struct DamHeader {
   uint64_t attn_scratch_bytes;   // scratch dam_sparse_attention needs for this blob
   uint64_t mask_tiles;      // 128 x 128 tiles of the masks that hold an active cell (= total_tiles unless gathered)
   uint64_t head_tile_cap;   // entries of tiles[] every head owns (sum of the row bounds of all sequences)
-  uint64_t reserved[9];     // [0]: 1 when the window map was scored by the tensor-core kernel (test hook)
+  uint64_t reserved[8];     // [0]: 1 when the window map was scored by the tensor-core kernel (test hook)
+  uint64_t off_cols;        // 0: no section (all-ones blob, or no gathered columns)
   uint64_t off_lone;        // 0: no section (all-ones blob)
   uint64_t exec_tiles;      // tiles the tensor-core attention kernel multiplies (total_tiles, or fewer: lone diagonals)
 };

@@ -546,9 +546,36 @@ __device__ uint32_t block_excl_scan(uint32_t x, uint32_t* total, uint32_t* sm /*
   return r;
 }
 
+// The matched columns of one (sequence, head) in ascending order: one 16-bit index per place of the head's
+// gathered-column tiles, 0xFFFF behind the last one.  In blocks of its own beside the ordering: at the end of the
+// matching kernel, whose one block per head everything behind it waits for, it gave back what the gather kernel gains.
+__device__ __forceinline__ void list_columns(unsigned char* blob, const unsigned char* scratch, uint64_t off_cnt,
+                                             const DamPlan& plan, int sh) {
+  const DamHeader* H = &plan.h;
+  const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
+  const DamSeq sq = dam_plan_seq(plan, blob, b);
+  if (sq.L == 0) return;
+  const uint32_t* Vw = reinterpret_cast<const uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * sq.W + 2 * sq.W;
+  const int32_t* prefV = reinterpret_cast<const int32_t*>(scratch + off_cnt) + sq.cnt_off +
+                         (uint64_t)h * dam_cnt_stride(sq.L, sq.W, sq.nL) + 2 * sq.L + sq.W + 1;
+  unsigned short* cols = reinterpret_cast<unsigned short*>(blob + H->off_cols) + (sq.gath_off + (uint64_t)h * sq.nL) * DAM_TILE;
+  const int nV = prefV[sq.W];
+  for (int k = threadIdx.x; k < sq.nL * DAM_TILE; k += blockDim.x) {
+    const uint32_t vw = k < sq.L ? Vw[k >> 5] : 0u;
+    if ((vw >> (k & 31)) & 1u) cols[prefV[k >> 5] + __popc(vw & ((1u << (k & 31)) - 1u))] = (unsigned short)k;
+    if (k >= nV) cols[k] = 0xFFFFu;
+  }
+}
+
+// The first `nshares` blocks order the work list; the blocks behind them (gathered columns only), one per
+// (sequence, head), list the matched columns beside them.
 __global__ void __launch_bounds__(1024)
-order_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_items, uint64_t off_keys, int prows, uint64_t off_work, int nkeys) {
+order_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, uint64_t off_items, uint64_t off_keys, int prows,
+             int nshares, const __grid_constant__ DamPlan plan) {
   dam_chain_prologue();
+  if ((int)blockIdx.x >= nshares) { list_columns(blob, scratch, off_cnt, plan, (int)blockIdx.x - nshares); return; }
+  const uint64_t off_work = plan.h.off_work;
+  const int nkeys = plan.nkeys;
   __shared__ uint32_t sm[32];
   __shared__ uint32_t tot;
   __shared__ uint32_t start[DAM_HIST];      // pairs per key, then the first place of the key's bucket
@@ -961,8 +988,9 @@ cudaError_t dam_launch_rule(const DamBuildCtx& c, cudaStream_t st) {
     int blocks = (c.prows + 7) / 8;
     if ((e = launch_chained(classify_kernel, dim3(blocks), dim3(256), st, c.blob, c.scratch, c.off_cnt, c.off_items,
                             c.off_keys, c.plan)) != cudaSuccess) return e;
-    if ((e = launch_chained(order_kernel, dim3((c.prows + 1023) / 1024), dim3(1024), st, c.blob, c.scratch, c.off_items,
-                            c.off_keys, c.prows, c.plan.h.off_work, c.plan.nkeys)) != cudaSuccess)
+    const int nshares = (c.prows + 1023) / 1024;
+    if ((e = launch_chained(order_kernel, dim3(nshares + (c.plan.h.off_cols ? c.num_seqs * c.Hq : 0)), dim3(1024), st, c.blob,
+                            c.scratch, c.off_cnt, c.off_items, c.off_keys, c.prows, nshares, c.plan)) != cudaSuccess)
       return e;
   }
   return cudaGetLastError();

@@ -356,6 +356,38 @@ def test_more_sequences_than_the_record_table_holds(lengths, gather):
     H.check_blob_against_oracle(blob, shape, H.oracle_masks_from_dump(w, dump.cpu().numpy()))
 
 
+@pytest.mark.parametrize("L,counts", [
+    (1, [0, 1, 1, 0]),
+    (128, [128, 0, 127, 1]),
+    (300, [129, 300, 31, 256]),             # a second place range, every column, an odd remainder, two full tiles
+])
+def test_matched_columns_are_listed_in_order(L, counts):
+    """The gathered columns of a head: the indices of its matched columns, ascending, 0xFFFF behind the last one."""
+    rng = np.random.default_rng(70)
+    lengths = [L + 700, 0, L]
+    P = []
+    for S in lengths:
+        maps = []
+        for n in counts:
+            p = np.zeros((min(S, L), min(S, L)), np.float32)
+            p[:, rng.permutation(L)[:n] if S else []] = 1.0
+            maps.append(np.tril(p))
+        P.append(maps)
+    cu = np.concatenate([[0], np.cumsum(lengths)]).tolist()
+    shape = B.make_shape(cu, 4, 4, 64, torch.bfloat16, DEV)
+    flat = np.concatenate([p.reshape(-1) for per in P for p in per])
+    blob, _ = B.dam_build_masks_from_scores(torch.from_numpy(flat).to(DEV), shape, B.make_rule(L, 0.3, 0.8, gather_columns=True))
+    mb = B.MaskBlob(blob)
+    for b in (0, 2):
+        s = mb.seqs[b]
+        for h, n in enumerate(counts):
+            V = np.flatnonzero(orc.head_mask_from_probs(np.ascontiguousarray(P[b][h]), lengths[b], 0.3, 0.8).V)
+            assert len(V) >= n
+            k = int(s["nL"]) * 128
+            got = np.frombuffer(mb.raw, dtype="<u2", count=k, offset=int(mb.hdr["off_cols"]) + 2 * 128 * (int(s["gath_off"]) + h * int(s["nL"])))
+            assert got.tolist() == V.tolist() + [0xFFFF] * (k - len(V))
+
+
 @pytest.mark.parametrize("pcl,lengths", [
     (1, [1, 3]),                            # one cell
     (37, [50, 20, 37, 9]),                  # odd rows: element-wise stores and reads
