@@ -412,12 +412,8 @@ static dam_status_t sparse_attention_impl(const void* Q, const void* K, const vo
   if (sm100_shape(shape))
     e = dam_launch_attn_sm100(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, scratch_bytes, ranges_dev,
                               !continuation, cs);
-  if (e == cudaErrorNotSupported) {
-    if (cudaMemsetAsync(reinterpret_cast<unsigned char*>(scratch) + (continuation ? 8 : 0), 0, continuation ? 248 : 256, cs) !=
-        cudaSuccess)
-      return DAM_ERR_CUDA;
-    e = dam_launch_attn_ref(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, ranges_dev, cs);
-  }
+  if (e == cudaErrorNotSupported)
+    e = dam_launch_attn_ref(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, continuation, ranges_dev, cs);
   return e == cudaSuccess ? DAM_OK : DAM_ERR_CUDA;
 }
 

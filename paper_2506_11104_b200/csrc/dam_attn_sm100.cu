@@ -832,8 +832,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 // T = gath_off + head * nL + g).  Rows past the last matched column are zero.  One block per tile, grid-stride.
 // Bound by latency: a chain of header, column index, row.  The indices are read from the list that stands beside the
 // ordering of the work list; found here instead, from the V words by prefix counts and a search per place, they took
-// another 1-1.5 us of every call (a 2048-row chunk against a 2048-token window 66.4 us, now 64.9; 1024 tokens with a
-// 256-token window 59.3, now 58.6; 8192 tokens 151.2, now 149.7).
+// another 1-1.5 us of every call (a 2048-row chunk against a 2048-token window 66.4 us, now 64.9; 1237 tokens with a
+// 512-token window 59.3, now 58.6; 8192 tokens 151.2, now 149.7).
 __global__ void __launch_bounds__(128)
 gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat16* __restrict__ K,
                       const __nv_bfloat16* __restrict__ V, int Hq, int group, int d, int64_t kst, int64_t ksh, int64_t vst,
@@ -896,6 +896,13 @@ gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat1
       }
     }
   }
+}
+
+// The status block of a call without a gather kernel in front: a kernel, so that the chain of launches is not broken.
+__global__ void clear_status_kernel(uint32_t* scratch, int keep) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");     // (late, as in the gather kernel)
+  if ((int)threadIdx.x >= keep) scratch[threadIdx.x] = 0u;
 }
 
 // Self-test of the bounded wait every kernel in this library uses: waits on an mbarrier that nothing ever
@@ -969,7 +976,8 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
       return e;
   } else {
     // status word and work counter start at zero (a further row range clears the work counter only)
-    if ((e = cudaMemsetAsync(reinterpret_cast<unsigned char*>(scratch) + (run_gather ? 0 : 8), 0, run_gather ? 256 : 248, st)) != cudaSuccess)
+    if ((e = dam_launch_chained(clear_status_kernel, dim3(1), dim3(64), 0, st, reinterpret_cast<uint32_t*>(scratch),
+                                run_gather ? 0 : 2)) != cudaSuccess)
       return e;
   }
   if (!dam_make_tmap_bf16(&to, O, d, s->num_q_heads, s->total_tokens, s->o_stride_tok, s->o_stride_head, 32) ||

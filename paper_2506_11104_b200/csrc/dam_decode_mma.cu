@@ -111,6 +111,7 @@ decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
                     const int32_t* __restrict__ cu, const int32_t* __restrict__ pos_dev, int num_seqs, int Hq, int G,
                     int64_t kst, int64_t ksh, int64_t vst, int64_t vsh, float scale_log2,
                     __nv_bfloat16* __restrict__ O, float* __restrict__ lse, uint32_t* __restrict__ scratch) {
+  dam_chain_prologue();
   using LY = GLayout<D>;
   constexpr int KS = D / 16;                 // k-steps of S = Q K^T
   constexpr int kThreads = kGWarps * 32;
@@ -411,10 +412,12 @@ cudaError_t launch_group(const __nv_bfloat16* q, const __nv_bfloat16* K, const _
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(s->num_kv_heads * split), (unsigned)s->num_seqs);
   cfg.blockDim = dim3(kGWarps * 32); cfg.dynamicSmemBytes = GLayout<D>::total; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = split > 1 ? 1 : 0;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = split > 1 ? 2 : 1;
   const int G = s->num_q_heads / s->num_kv_heads;
   return cudaLaunchKernelEx(&cfg, split > 1 ? decode_group_kernel<D, true> : decode_group_kernel<D, false>, q, K, V, blob,
                             (const int32_t*)s->cu_seqlens_dev, pos_dev, (int)s->num_seqs, (int)s->num_q_heads, G, s->k_stride_tok,

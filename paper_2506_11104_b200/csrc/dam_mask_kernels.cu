@@ -7,26 +7,6 @@
 
 namespace {
 
-// The rule kernels form a chain of short, dependent launches.  Each lets the next launch begin as soon as all
-// of its own blocks are running (programmatic dependent launch) and then waits for the kernel before it to
-// have completed with its memory visible: the launch latency of every link is hidden under its predecessor.
-// Both instructions do nothing in a kernel that was launched the ordinary way.
-__device__ __forceinline__ void dam_chain_prologue() {
-  asm volatile("griddepcontrol.launch_dependents;");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = 0; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 __device__ __forceinline__ const DamSeq* blob_seqs(const unsigned char* blob, const DamHeader* h) {
   return reinterpret_cast<const DamSeq*>(blob + h->off_seq);
 }
@@ -37,7 +17,7 @@ __device__ __forceinline__ const DamSeq* blob_seqs(const unsigned char* blob, co
 // ---------------------------------------------------------------------------------------------
 __global__ void init_blob_kernel(unsigned char* blob, DamHeader hdr, const int32_t* __restrict__ cu,
                                  int pcl_max, int Hq, int all_ones_causal /* -1: DAM mask */, uint4* clear, uint32_t clear_vecs) {
-  asm volatile("griddepcontrol.launch_dependents;");     // a kernel chained behind this one may start its prologue
+  dam_chain_prologue();
   if (blockIdx.x > 0) {
     for (uint32_t x = (blockIdx.x - 1) * blockDim.x + threadIdx.x; x < clear_vecs; x += (gridDim.x - 1) * blockDim.x)
       clear[x] = make_uint4(0u, 0u, 0u, 0u);
@@ -106,6 +86,7 @@ __device__ __forceinline__ void row_bits(uint32_t* __restrict__ Mrow, const floa
 }
 
 __global__ void bits_from_scores_kernel(unsigned char* blob, const float* __restrict__ P, float pstar) {
+  dam_chain_prologue();
   const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
   const int sh = blockIdx.y;
   const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
@@ -741,10 +722,9 @@ cudaError_t dam_launch_init_blob(const dam_shape_t* shape, int pcl_max, uint32_t
   int mode = (flags & DAM_FLAG_ALL_ONES) ? ((flags & DAM_FLAG_CAUSAL_LIST) ? 1 : 0) : -1;
   const size_t vecs = clear_bytes / 16;                      // (the sections are multiples of 256 bytes)
   const size_t blocks = vecs ? (vecs + 1023) / 1024 : 0;     // four 16-byte stores per thread, at most 1024 blocks
-  init_blob_kernel<<<1 + (unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st>>>(
-      reinterpret_cast<unsigned char*>(blob), host_hdr, shape->cu_seqlens_dev, pcl_max, shape->num_q_heads, mode,
-      reinterpret_cast<uint4*>(clear), (uint32_t)vecs);
-  return cudaGetLastError();
+  return dam_launch_chained(init_blob_kernel, dim3(1 + (unsigned)(blocks < 1024 ? blocks : 1024)), dim3(256), 0, st,
+                            reinterpret_cast<unsigned char*>(blob), host_hdr, shape->cu_seqlens_dev, pcl_max, shape->num_q_heads,
+                            mode, reinterpret_cast<uint4*>(clear), (uint32_t)vecs);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -828,8 +808,7 @@ cudaError_t dam_launch_bits_from_scores(const float* P, const DamBuildCtx& c, cu
     if (e != cudaSuccess) return e;
     return cudaMemsetAsync(c.scratch + c.off_cnt, 0, c.off_cnt_end - c.off_cnt, st);
   }
-  bits_from_scores_kernel<<<grid, 256, 0, st>>>(c.blob, P, c.pstar);
-  return cudaGetLastError();
+  return dam_launch_chained(bits_from_scores_kernel, grid, dim3(256), 0, st, c.blob, P, c.pstar);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -980,16 +959,16 @@ cudaError_t dam_launch_rule(const DamBuildCtx& c, cudaStream_t st) {
   cudaError_t e;
   if (c.max_nL > 0) {
     dim3 g(c.max_nL * (c.max_nL + 1) / 2, c.num_seqs * c.Hq);
-    if ((e = launch_chained(counts_kernel, g, dim3(DAM_TILE), st, c.blob, c.scratch, c.off_cnt, c.plan)) != cudaSuccess) return e;
-    if ((e = launch_chained(match_kernel, dim3(c.num_seqs * c.Hq), dim3(1024), st, c.blob, c.scratch, c.off_cnt, c.mu,
+    if ((e = dam_launch_chained(counts_kernel, g, dim3(DAM_TILE), 0, st, c.blob, c.scratch, c.off_cnt, c.plan)) != cudaSuccess) return e;
+    if ((e = dam_launch_chained(match_kernel, dim3(c.num_seqs * c.Hq), dim3(1024), 0, st, c.blob, c.scratch, c.off_cnt, c.mu,
                             c.min_support, c.plan)) != cudaSuccess) return e;
   }
   if (c.rows > 0) {
     int blocks = (c.prows + 7) / 8;
-    if ((e = launch_chained(classify_kernel, dim3(blocks), dim3(256), st, c.blob, c.scratch, c.off_cnt, c.off_items,
+    if ((e = dam_launch_chained(classify_kernel, dim3(blocks), dim3(256), 0, st, c.blob, c.scratch, c.off_cnt, c.off_items,
                             c.off_keys, c.plan)) != cudaSuccess) return e;
     const int nshares = (c.prows + 1023) / 1024;
-    if ((e = launch_chained(order_kernel, dim3(nshares + (c.plan.h.off_cols ? c.num_seqs * c.Hq : 0)), dim3(1024), st, c.blob,
+    if ((e = dam_launch_chained(order_kernel, dim3(nshares + (c.plan.h.off_cols ? c.num_seqs * c.Hq : 0)), dim3(1024), 0, st, c.blob,
                             c.scratch, c.off_cnt, c.off_items, c.off_keys, c.prows, nshares, c.plan)) != cudaSuccess)
       return e;
   }
