@@ -830,8 +830,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 // Copies the K and V rows of the matched columns of every (sequence, head) into dense tiles of 128 keys in
 // the scratch buffer (K tile at rows (2T) * 128, V tile at rows (2T + 1) * 128 of a [rows][head_dim] bf16 array;
 // T = gath_off + head * nL + g).  Rows past the last matched column are zero.  One block per tile, grid-stride.
-// Bound by latency: a chain of header, column index, row.  The indices are read from the list that stands beside the
-// ordering of the work list; found here instead, from the V words by prefix counts and a search per place, they took
+// Bound by latency: a chain of header, column index, row.  The indices are read from the list that the classification
+// leaves; found here instead, from the V words by prefix counts and a search per place, they took
 // another 1-1.5 us of every call (a 2048-row chunk against a 2048-token window 66.4 us, now 64.9; 1237 tokens with a
 // 512-token window 59.3, now 58.6; 8192 tokens 151.2, now 149.7).
 __global__ void __launch_bounds__(128)

@@ -7,6 +7,8 @@
 
 namespace {
 
+constexpr int kClassifyWarps = 16;       // (8 or 32: 1237 tokens 55.7 us a pass instead of 55.0)
+
 __device__ __forceinline__ const DamSeq* blob_seqs(const unsigned char* blob, const DamHeader* h) {
   return reinterpret_cast<const DamSeq*>(blob + h->off_seq);
 }
@@ -193,25 +195,13 @@ __global__ void counts_kernel(const unsigned char* blob, unsigned char* scratch,
 
 // ---------------------------------------------------------------------------------------------
 // Match: D[r] = [cntD[r] >= mu * (L - r)], V[c] likewise (one fp32 multiply, one compare), written
-// as bit sets; Drev = D reversed; prefix popcounts per word for range queries.  Block per (seq, head).
+// as bit sets; Drev = D reversed; prefix popcounts per word for range queries.  By one block; Dw, Rw, Vw, prefD, prefV
+// in shared memory, or in global memory where they do not fit.
 // ---------------------------------------------------------------------------------------------
-__global__ void match_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, float mu, int min_support,
-                             const __grid_constant__ DamPlan plan) {
-  dam_chain_prologue();
-  const DamHeader* H = &plan.h;
-  const int sh = blockIdx.x;
-  const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
-  const DamSeq sq = dam_plan_seq(plan, blob, b);
-  int2* lone = reinterpret_cast<int2*>(blob + H->off_lone) + sh;
-  if (sq.L == 0) { if (threadIdx.x == 0) *lone = make_int2(-1, 0); return; }
+__device__ __forceinline__ void match_head(const DamSeq& sq, bool gather, float mu, int min_support, const int32_t* cntD,
+                                           const int32_t* cntV, uint32_t* Dw, uint32_t* Rw, uint32_t* Vw, int32_t* prefD,
+                                           int32_t* prefV, int2* lone) {
   const int L = sq.L, W = sq.W;
-  uint32_t* dv = reinterpret_cast<uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * W;
-  uint32_t* Dw = dv; uint32_t* Rw = dv + W; uint32_t* Vw = dv + 2 * W;
-  int32_t* cnt = reinterpret_cast<int32_t*>(scratch + off_cnt) + sq.cnt_off + (uint64_t)h * dam_cnt_stride(L, W, sq.nL);
-  const int32_t* cntD = cnt;
-  const int32_t* cntV = cnt + L;
-  int32_t* prefD = cnt + 2 * L;
-  int32_t* prefV = prefD + (W + 1);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int w = warp; w < W; w += nw) {
     int k = w * 32 + lane;
@@ -263,7 +253,7 @@ __global__ void match_kernel(unsigned char* blob, unsigned char* scratch, uint64
     below = __reduce_max_sync(0xFFFFFFFFu, below);
     // in front of it: the gathered tiles, or the window's tiles that hold a matched column
     int front = (runV + DAM_TILE - 1) / DAM_TILE;
-    if (!(H->flags & DAM_FLAG_GATHER)) {
+    if (!gather) {
       front = 0;
       for (int g = lane; g < W / 4; g += 32) front += (Vw[4 * g] | Vw[4 * g + 1] | Vw[4 * g + 2] | Vw[4 * g + 3]) != 0u;
       front = __reduce_add_sync(0xFFFFFFFFu, front);
@@ -273,8 +263,8 @@ __global__ void match_kernel(unsigned char* blob, unsigned char* scratch, uint64
 }
 
 // ---------------------------------------------------------------------------------------------
-// Tile classification.  One warp per row = (head, global q-block); lanes test candidate kv tiles in
-// ascending order and writes the kept ones into the pair's fixed range of tiles[] (one pass: nothing is counted
+// Tile classification.  One warp per pair of query blocks of a head; its lanes test candidate kv tiles in
+// ascending order and write the kept ones into the pair's fixed range of tiles[] (one pass: nothing is counted
 // first, nothing is compacted afterwards).
 // ---------------------------------------------------------------------------------------------
 struct HeadView {
@@ -339,35 +329,18 @@ __device__ __forceinline__ uint32_t classify_band(const HeadView& v, int qb, int
   return (whole && n == 2 * DAM_TILE - 1) ? DAM_KIND_FULL : DAM_KIND_PARTIAL;
 }
 
-__global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, uint64_t off_items,
-                                uint64_t off_keys, const __grid_constant__ DamPlan bp) {
-  dam_chain_prologue();
-  const DamHeader* H = &bp.h;
-  DamHeader* stats = reinterpret_cast<DamHeader*>(blob);
+// Tile statistics of a block's pairs: one global atomic per block and statistic instead of one per warp on the same address.
+struct TileStats {
+  unsigned long long mask_tiles;
+  uint32_t total, full, exec;
+};
+
+// Lists the tiles of one pair of query blocks of a (sequence, head), and leaves its work item and its key: one warp.
+__device__ __forceinline__ void classify_pair(unsigned char* blob, unsigned char* scratch, uint64_t off_items, uint64_t off_keys,
+                                              const DamHeader* H, int nkeys, const DamSeq& sq, int b, int h, int gp,
+                                              const HeadView& v, int lone, TileStats& st) {
   const int lane = threadIdx.x & 31;
-  const int prow = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // one warp per (head, q-block pair)
-  // block totals of the three statistics: one global atomic per block instead of one per warp on the same address
-  __shared__ unsigned long long s_mask_tiles;
-  __shared__ uint32_t s_total, s_full, s_exec;
-  if (threadIdx.x == 0) { s_mask_tiles = 0ull; s_total = 0u; s_full = 0u; s_exec = 0u; }
-  __syncthreads();
-  if (prow < H->prows) {
-  const int h = prow / H->total_pairs, gp = prow % H->total_pairs;
-  int b = 0;
-  if (bp.nseq) {
-    while (b + 1 < bp.nseq && bp.seq[b + 1].first_pair <= gp) ++b;      // (an empty sequence has no pair of its own)
-  } else {
-    b = reinterpret_cast<const int32_t*>(blob + H->off_qbseq)[reinterpret_cast<const uint32_t*>(blob + H->off_pairtab)[gp] & 0x7FFFFFFFu];
-  }
-  const DamSeq sq = dam_plan_seq(bp, blob, b);
   const int gqb0 = sq.first_qblock + 2 * (gp - sq.first_pair), nblk = 2 * (gp - sq.first_pair) + 1 < sq.nq ? 2 : 1;
-  HeadView v;
-  const uint32_t* dv = reinterpret_cast<const uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * sq.W;
-  const int32_t* cnt = reinterpret_cast<const int32_t*>(scratch + off_cnt) + sq.cnt_off +
-                       (uint64_t)h * dam_cnt_stride(sq.L, sq.W, sq.nL);
-  v.Dw = dv; v.Vw = dv + 2 * sq.W;
-  v.prefD = cnt + 2 * sq.L; v.prefV = v.prefD + (sq.W + 1); v.tile_pop = v.prefV + (sq.W + 1);
-  v.L = sq.L; v.W = sq.W; v.nL = sq.nL; v.S = sq.S;
   uint32_t* tile_ptr = reinterpret_cast<uint32_t*>(blob + H->off_tile_ptr);
   uint32_t* tiles = reinterpret_cast<uint32_t*>(blob + H->off_tiles);
   const int gflag = (H->flags & DAM_FLAG_GATHER) ? 1 : 0;
@@ -378,7 +351,6 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
   const uint32_t pair_end = (uint32_t)(head_base + dam_row_tile_prefix(qb0 + nblk, sq.nL, sq.L, gflag));
   uint32_t base = pair_begin, a1 = pair_begin;
   int pair_total = 0, nfull = 0, mask_tiles = 0, saved = 0;
-  const int lone = reinterpret_cast<const int2*>(blob + H->off_lone)[b * H->num_q_heads + h].x;
   // Per query block: candidates, ascending: [0, min(qb, nL-1)] then [max(that + 1, qb - nL), qb].  From row 2L - 1
   // on (gathered columns enabled) the first range is replaced by the gathered tiles and the second range is
   // classified on the matched diagonals alone.  The tiles of the mask itself (128 x 128 grid) with an active cell
@@ -480,20 +452,83 @@ __global__ void classify_kernel(unsigned char* blob, unsigned char* scratch, uin
     // index (pair, head): the order the pairs keep inside a bucket of the work list
     const size_t at = (size_t)gp * H->num_q_heads + h;
     reinterpret_cast<DamItem*>(scratch + off_items)[at] = it;
-    reinterpret_cast<uint32_t*>(scratch + off_keys)[at] = (uint32_t)min(pair_total, bp.nkeys - 1);
-    atomicAdd(&s_mask_tiles, (unsigned long long)mask_tiles);
-    atomicAdd(&s_total, (uint32_t)pair_total);
-    atomicAdd(&s_exec, (uint32_t)(pair_total - saved));
-    atomicAdd(&s_full, (uint32_t)nfull);
+    reinterpret_cast<uint32_t*>(scratch + off_keys)[at] = (uint32_t)min(pair_total, nkeys - 1);
+    atomicAdd(&st.mask_tiles, (unsigned long long)mask_tiles);
+    atomicAdd(&st.total, (uint32_t)pair_total);
+    atomicAdd(&st.exec, (uint32_t)(pair_total - saved));
+    atomicAdd(&st.full, (uint32_t)nfull);
   }
+}
+
+__device__ __forceinline__ void flush_stats(unsigned char* blob, const TileStats& st) {
+  DamHeader* H = reinterpret_cast<DamHeader*>(blob);
+  if (st.mask_tiles) atomicAdd(reinterpret_cast<unsigned long long*>(&H->mask_tiles), st.mask_tiles);
+  if (st.total) atomicAdd(&H->total_tiles, st.total);
+  if (st.exec) atomicAdd(reinterpret_cast<unsigned long long*>(&H->exec_tiles), (unsigned long long)st.exec);
+  if (st.full) atomicAdd(&H->full_tiles, st.full);
+}
+
+// The matched columns of one (sequence, head) in ascending order: one 16-bit index per place of the head's
+// gathered-column tiles, 0xFFFF behind the last one.
+__device__ __forceinline__ void list_columns(unsigned char* blob, const DamHeader* H, const DamSeq& sq, int h, const uint32_t* Vw,
+                                             const int32_t* prefV) {
+  if (sq.L == 0) return;
+  unsigned short* cols = reinterpret_cast<unsigned short*>(blob + H->off_cols) + (sq.gath_off + (uint64_t)h * sq.nL) * DAM_TILE;
+  const int nV = prefV[sq.W];
+  for (int k = threadIdx.x; k < sq.nL * DAM_TILE; k += blockDim.x) {
+    const uint32_t vw = k < sq.L ? Vw[k >> 5] : 0u;
+    if ((vw >> (k & 31)) & 1u) cols[prefV[k >> 5] + __popc(vw & ((1u << (k & 31)) - 1u))] = (unsigned short)k;
+    if (k >= nV) cols[k] = 0xFFFFu;
+  }
+}
+
+// Match and classification of one (sequence, head): blockIdx.y; its pairs of query blocks are dealt over the warps of
+// up to gridDim.x blocks, each of which matches the head's patterns for itself and keeps them in shared memory.  Latency
+// bound, like all kernels here: a matching kernel of one block per head in front of this one took another 4.5 - 9.5 us of
+// the chain (5 alone at a 512-token window), the match repeated by every block 1 - 2.  Stage 1: fp32, 512 tokens 23.6 ->
+// 22.3 us, 1237 tokens 26.9 -> 26.0, 16001 tokens 34.7 -> 33.8, 32768 tokens 82.6 -> 80.5, 131072 tokens 258 -> 253.
+__global__ void __launch_bounds__(kClassifyWarps * 32, 2)
+classify_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, uint64_t off_items, uint64_t off_keys, float mu,
+                int min_support, int in_smem, const __grid_constant__ DamPlan bp) {
+  dam_chain_prologue();
+  extern __shared__ int32_t csm[];
+  __shared__ TileStats st;
+  __shared__ int2 lone;
+  const DamHeader* H = &bp.h;
+  const int sh = blockIdx.y, b = sh / H->num_q_heads, h = sh % H->num_q_heads;
+  const DamSeq sq = dam_plan_seq(bp, blob, b);
+  const int npairs = (sq.nq + 1) / 2, warp = threadIdx.x >> 5;
+  const int nblk = max(1, min((int)gridDim.x, (npairs + kClassifyWarps - 1) / kClassifyWarps));
+  if ((int)blockIdx.x >= nblk) return;
+  const bool last = (int)blockIdx.x == nblk - 1;         // (the one with the fewest pairs: it writes the head's sections)
+  const int L = sq.L, W = sq.W;
+  uint32_t* dv = reinterpret_cast<uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * W;
+  int32_t* cnt = reinterpret_cast<int32_t*>(scratch + off_cnt) + sq.cnt_off + (uint64_t)h * dam_cnt_stride(L, W, sq.nL);
+  // (windows whose patterns do not fit shared memory: in place, every block writes the same words)
+  uint32_t* bits = in_smem ? reinterpret_cast<uint32_t*>(csm) : dv;
+  int32_t* prefD = in_smem ? csm + 3 * W : cnt + 2 * L;
+  int32_t* prefV = prefD + (W + 1);
+  if (threadIdx.x == 0) { st = TileStats{0ull, 0u, 0u, 0u}; lone = make_int2(-1, 0); }
+  __syncthreads();
+  if (L > 0) {
+    match_head(sq, (H->flags & DAM_FLAG_GATHER) != 0, mu, min_support, cnt, cnt + L, bits, bits + W, bits + 2 * W, prefD, prefV,
+               &lone);
+    __threadfence_block();
+    __syncthreads();
+  }
+  HeadView v;
+  v.Dw = bits; v.Vw = bits + 2 * W; v.prefD = prefD; v.prefV = prefV; v.tile_pop = cnt + 2 * L + 2 * (W + 1);
+  v.L = L; v.W = W; v.nL = sq.nL; v.S = sq.S;
+  for (int p = blockIdx.x * kClassifyWarps + warp; p < npairs; p += nblk * kClassifyWarps)
+    classify_pair(blob, scratch, off_items, off_keys, H, bp.nkeys, sq, b, h, sq.first_pair + p, v, lone.x, st);
+  if (last) {
+    if (in_smem)
+      for (int w = threadIdx.x; w < 3 * W; w += blockDim.x) dv[w] = bits[w];
+    if (threadIdx.x == 0) reinterpret_cast<int2*>(blob + H->off_lone)[sh] = lone;
+    if (H->off_cols) list_columns(blob, H, sq, h, bits + 2 * W, prefV);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (s_mask_tiles) atomicAdd(reinterpret_cast<unsigned long long*>(&stats->mask_tiles), s_mask_tiles);
-    if (s_total) atomicAdd(&stats->total_tiles, s_total);
-    if (s_exec) atomicAdd(reinterpret_cast<unsigned long long*>(&stats->exec_tiles), (unsigned long long)s_exec);
-    if (s_full) atomicAdd(&stats->full_tiles, s_full);
-  }
+  if (threadIdx.x == 0) flush_stats(blob, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -527,36 +562,9 @@ __device__ uint32_t block_excl_scan(uint32_t x, uint32_t* total, uint32_t* sm /*
   return r;
 }
 
-// The matched columns of one (sequence, head) in ascending order: one 16-bit index per place of the head's
-// gathered-column tiles, 0xFFFF behind the last one.  In blocks of its own beside the ordering: at the end of the
-// matching kernel, whose one block per head everything behind it waits for, it gave back what the gather kernel gains.
-__device__ __forceinline__ void list_columns(unsigned char* blob, const unsigned char* scratch, uint64_t off_cnt,
-                                             const DamPlan& plan, int sh) {
-  const DamHeader* H = &plan.h;
-  const int b = sh / H->num_q_heads, h = sh % H->num_q_heads;
-  const DamSeq sq = dam_plan_seq(plan, blob, b);
-  if (sq.L == 0) return;
-  const uint32_t* Vw = reinterpret_cast<const uint32_t*>(blob + H->off_dv) + sq.dv_off + (uint64_t)h * 3 * sq.W + 2 * sq.W;
-  const int32_t* prefV = reinterpret_cast<const int32_t*>(scratch + off_cnt) + sq.cnt_off +
-                         (uint64_t)h * dam_cnt_stride(sq.L, sq.W, sq.nL) + 2 * sq.L + sq.W + 1;
-  unsigned short* cols = reinterpret_cast<unsigned short*>(blob + H->off_cols) + (sq.gath_off + (uint64_t)h * sq.nL) * DAM_TILE;
-  const int nV = prefV[sq.W];
-  for (int k = threadIdx.x; k < sq.nL * DAM_TILE; k += blockDim.x) {
-    const uint32_t vw = k < sq.L ? Vw[k >> 5] : 0u;
-    if ((vw >> (k & 31)) & 1u) cols[prefV[k >> 5] + __popc(vw & ((1u << (k & 31)) - 1u))] = (unsigned short)k;
-    if (k >= nV) cols[k] = 0xFFFFu;
-  }
-}
-
-// The first `nshares` blocks order the work list; the blocks behind them (gathered columns only), one per
-// (sequence, head), list the matched columns beside them.
 __global__ void __launch_bounds__(1024)
-order_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, uint64_t off_items, uint64_t off_keys, int prows,
-             int nshares, const __grid_constant__ DamPlan plan) {
+order_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_items, uint64_t off_keys, int prows, uint64_t off_work, int nkeys) {
   dam_chain_prologue();
-  if ((int)blockIdx.x >= nshares) { list_columns(blob, scratch, off_cnt, plan, (int)blockIdx.x - nshares); return; }
-  const uint64_t off_work = plan.h.off_work;
-  const int nkeys = plan.nkeys;
   __shared__ uint32_t sm[32];
   __shared__ uint32_t tot;
   __shared__ uint32_t start[DAM_HIST];      // pairs per key, then the first place of the key's bucket
@@ -960,16 +968,20 @@ cudaError_t dam_launch_rule(const DamBuildCtx& c, cudaStream_t st) {
   if (c.max_nL > 0) {
     dim3 g(c.max_nL * (c.max_nL + 1) / 2, c.num_seqs * c.Hq);
     if ((e = dam_launch_chained(counts_kernel, g, dim3(DAM_TILE), 0, st, c.blob, c.scratch, c.off_cnt, c.plan)) != cudaSuccess) return e;
-    if ((e = dam_launch_chained(match_kernel, dim3(c.num_seqs * c.Hq), dim3(1024), 0, st, c.blob, c.scratch, c.off_cnt, c.mu,
-                            c.min_support, c.plan)) != cudaSuccess) return e;
   }
   if (c.rows > 0) {
-    int blocks = (c.prows + 7) / 8;
-    if ((e = dam_launch_chained(classify_kernel, dim3(blocks), dim3(256), 0, st, c.blob, c.scratch, c.off_cnt, c.off_items,
-                            c.off_keys, c.plan)) != cudaSuccess) return e;
-    const int nshares = (c.prows + 1023) / 1024;
-    if ((e = dam_launch_chained(order_kernel, dim3(nshares + (c.plan.h.off_cols ? c.num_seqs * c.Hq : 0)), dim3(1024), 0, st, c.blob,
-                            c.scratch, c.off_cnt, c.off_items, c.off_keys, c.prows, nshares, c.plan)) != cudaSuccess)
+    // A pair per warp, but at most eight blocks per head: beyond that the repeated match costs more than the second to
+    // fourth pair of a warp (stage 1 of 131072 tokens, 512 pairs per head: 262 us with nine blocks per head, 260 with
+    // eight, 278 with 32; mixed lengths, 192 heads of up to 256 pairs: 178 with one, 147 with eight, 151 with sixteen).
+    const int heads = c.num_seqs * c.Hq, want = ((c.max_nq + 1) / 2 + kClassifyWarps - 1) / kClassifyWarps;
+    const int per_head = want < 8 ? want : 8;
+    const size_t smem = 4 * (size_t)(5 * c.max_W + 2);
+    const int in_smem = smem <= 46 * 1024;
+    if ((e = dam_launch_chained(classify_kernel, dim3(per_head, heads), dim3(kClassifyWarps * 32), in_smem ? smem : 0, st, c.blob,
+                                c.scratch, c.off_cnt, c.off_items, c.off_keys, c.mu, c.min_support, in_smem, c.plan)) != cudaSuccess)
+      return e;
+    if ((e = dam_launch_chained(order_kernel, dim3((c.prows + 1023) / 1024), dim3(1024), 0, st, c.blob, c.scratch, c.off_items,
+                                c.off_keys, c.prows, c.plan.h.off_work, c.plan.nkeys)) != cudaSuccess)
       return e;
   }
   return cudaGetLastError();
