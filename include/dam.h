@@ -240,7 +240,8 @@ dam_status_t dam_capture_average(const float* A, const int32_t* C, int32_t pcl_m
  * without saying how they arrive); the arithmetic per row is exactly that of dam_sparse_attention.
  * Work is dealt in pairs of 128-row query blocks, so every begin must be a multiple of 256 and every end a
  * multiple of 256 or the sequence length (INVALID_ARGUMENT otherwise); an empty range skips the sequence.
- *   row_ranges_host : HOST, int32[2 * num_seqs] (validated);  row_ranges_dev : DEVICE, the same values.
+ *   row_ranges_host : HOST, int32[2 * num_seqs] (validated);  row_ranges_dev : DEVICE, the same values (not NULL, but
+ *   not read for batches of up to 16 sequences, whose ranges travel with the launch).
  * Everything else as dam_sparse_attention.
  */
 dam_status_t dam_sparse_attention_rows(const void* Q, const void* K, const void* V, const void* mask,

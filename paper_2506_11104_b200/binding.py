@@ -276,15 +276,20 @@ def dam_sparse_attention_rows(Q, K, V, mask, shape: Shape, row_ranges, O: torch.
     flat = [int(x) for pair in row_ranges for x in pair]
     assert len(flat) == 2 * shape.c.num_seqs
     host = (ctypes.c_int32 * len(flat))(*flat)
-    # queued without waiting for the stream (CUDA has taken its own copy of a small pageable source when the call returns)
-    dev = torch.tensor(flat, dtype=torch.int32).to(Q.device, non_blocking=True)
+    # up to 16 sequences the library hands the ranges to the kernel itself; beyond, a copy on the device, queued without
+    # waiting for the stream (CUDA has taken its own copy of a small pageable source when the call returns)
+    if shape.c.num_seqs <= 16:
+        dev = shape.c.cu_seqlens_dev
+    else:
+        dev_copy = torch.tensor(flat, dtype=torch.int32).to(Q.device, non_blocking=True)
+        dev = dev_copy.data_ptr()
     if scratch is None:
         off = _HDR.fields["attn_scratch_bytes"][1]
         need = int(mask[off: off + 8].cpu().numpy().view(np.uint64)[0]) if mask.numel() >= 256 else 256
         scratch = _alloc(max(256, need), Q.device)
     rc = lib().dam_sparse_attention_rows(_ptr(Q), _ptr(K), _ptr(V), _ptr(mask), shape.ref, int(causal),
                                          shape.c.num_q_heads // shape.c.num_kv_heads, softmax_scale,
-                                         _ptr(O), _ptr(lse), host, _ptr(dev), _ptr(scratch),
+                                         _ptr(O), _ptr(lse), host, dev, _ptr(scratch),
                                          scratch.numel(), _stream(Q.device))
     _check(rc, "dam_sparse_attention_rows")
     return scratch

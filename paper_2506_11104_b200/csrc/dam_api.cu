@@ -411,9 +411,9 @@ static dam_status_t sparse_attention_impl(const void* Q, const void* K, const vo
   cudaError_t e = cudaErrorNotSupported;
   if (sm100_shape(shape))
     e = dam_launch_attn_sm100(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, scratch_bytes, ranges_dev,
-                              !continuation, cs);
+                              ranges_host, !continuation, cs);
   if (e == cudaErrorNotSupported)
-    e = dam_launch_attn_ref(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, continuation, ranges_dev, cs);
+    e = dam_launch_attn_ref(Q, K, V, mask, shape, causal != 0, scale, O, lse, scratch, continuation, ranges_dev, ranges_host, cs);
   return e == cudaSuccess ? DAM_OK : DAM_ERR_CUDA;
 }
 

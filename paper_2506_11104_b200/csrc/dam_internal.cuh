@@ -267,6 +267,22 @@ __device__ __forceinline__ uint4 dam_apply_bits(const DamHeadBits& hb, uint32_t 
   return dam_low_ones128(n);
 }
 
+// Row ranges of a chunked call, handed to the kernel by value for batches of a few sequences (n = 0: read from memory).
+constexpr int kRangeSeqs = 16;
+struct DamRowRanges {
+  int n;
+  int2 r[kRangeSeqs];
+  DamRowRanges(const int32_t* host, int num_seqs) : n(host && num_seqs <= kRangeSeqs ? num_seqs : 0) {
+    for (int b = 0; b < kRangeSeqs; ++b) r[b] = b < n ? make_int2(host[2 * b], host[2 * b + 1]) : make_int2(0, 0);
+  }
+  // whether the pair of query blocks that starts with block qb0 of sequence `seq` is inside
+  __device__ __forceinline__ bool holds(const int32_t* __restrict__ ranges, int seq, int qb0) const {
+    const int r0 = qb0 * DAM_TILE;
+    if (n) return r0 >= r[seq].x && r0 < r[seq].y;
+    return r0 >= __ldg(ranges + 2 * seq) && r0 < __ldg(ranges + 2 * seq + 1);
+  }
+};
+
 // ---- launches that follow one another ----------------------------------------------------------
 // Most kernels here form a chain of short, dependent launches.  Each lets the next launch begin as soon as all
 // of its own blocks are running (programmatic dependent launch) and then waits for the kernel before it to
@@ -346,15 +362,16 @@ cudaError_t dam_launch_all_ones(const dam_shape_t* shape, int causal, void* blob
 cudaError_t dam_launch_expand_rows(const void* blob, int seq, int head, int row_begin, int nrows, int words,
                                    int causal, uint32_t* out, cudaStream_t st);
 cudaError_t dam_launch_active_elems(const void* blob, int num_seqs, int Hq, unsigned long long* out, cudaStream_t st);
-// `ranges` (device, int32[2 * num_seqs], or NULL): only the pairs of query blocks whose first row lies in
+// `ranges` (device, int32[2 * num_seqs], or NULL; `ranges_host`: the same values): only the pairs of query blocks whose first row lies in
 // [ranges[2b], ranges[2b+1]) of sequence b are computed
 cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, const void* blob,
                                 const dam_shape_t* shape, int causal, float scale, void* O, float* lse,
-                                void* scratch, bool keep_status, const int32_t* ranges, cudaStream_t st);
+                                void* scratch, bool keep_status, const int32_t* ranges, const int32_t* ranges_host, cudaStream_t st);
 // tensor-core paths (bf16, d = 128); return cudaErrorNotSupported when the shape does not qualify
 cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, const void* blob,
                                   const dam_shape_t* shape, int causal, float scale, void* O, float* lse,
-                                  void* scratch, size_t scratch_bytes, const int32_t* ranges, bool run_gather, cudaStream_t st);
+                                  void* scratch, size_t scratch_bytes, const int32_t* ranges, const int32_t* ranges_host,
+                                  bool run_gather, cudaStream_t st);
 cudaError_t dam_launch_scores_sm100(const void* Q, const void* K, const dam_shape_t* shape, const DamBuildCtx& c,
                                     float* scores_dump, cudaStream_t st);
 

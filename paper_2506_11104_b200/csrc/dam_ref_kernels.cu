@@ -205,7 +205,7 @@ attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __r
                 const T* __restrict__ V, int Hq, int group, int d, int64_t qst, int64_t qsh,
                 int64_t kst, int64_t ksh, int64_t vst, int64_t vsh, int64_t ost, int64_t osh,
                 int causal, float scale, T* __restrict__ O, float* __restrict__ lse, int total_tokens,
-                const int32_t* __restrict__ ranges, uint32_t* scratch, int keep) {
+                const int32_t* __restrict__ ranges, const __grid_constant__ DamRowRanges rr, uint32_t* scratch, int keep) {
   // the status block starts at zero (its first `keep` words stay: a further row range of the same layer)
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x >= keep && threadIdx.x < 64) scratch[threadIdx.x] = 0u;
   extern __shared__ __align__(16) float smem[];
@@ -215,10 +215,7 @@ attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __r
   const int b = reinterpret_cast<const int32_t*>(blob + H->off_qbseq)[gqb];
   const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[b];
   const int qb = gqb - sq.first_qblock;
-  if (ranges) {                                 // row ranges: whole pairs of query blocks, chosen by the pair's first row
-    const int r0 = (qb & ~1) * DAM_TILE;
-    if (r0 < ranges[2 * b] || r0 >= ranges[2 * b + 1]) return;
-  }
+  if (ranges && !rr.holds(ranges, b, qb & ~1)) return;         // row ranges: whole pairs of query blocks
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int i_block = qb * DAM_TILE + blockIdx.y * nw * R;
   if (i_block >= sq.S) return;
@@ -392,7 +389,7 @@ cudaError_t launch_scores(const void* Q, const void* K, const dam_shape_t* s, co
 
 template <typename T, int R, int ND>
 cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
-                        float scale, void* O, float* lse, const int32_t* ranges, uint32_t* scratch, int keep, int rows, int smem_max, cudaStream_t st) {
+                        float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int smem_max, cudaStream_t st) {
   const bool pipe = sizeof(T) == 4 && attn_smem(s->head_dim, R, 2) <= (size_t)smem_max;
   const size_t sm = attn_smem(s->head_dim, R, pipe ? 2 : 1);
   auto kernel = attn_ref_kernel<T, R, ND, false>;
@@ -405,17 +402,17 @@ cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void*
   kernel<<<grid, kRefWarps * 32, sm, st>>>(
       (const unsigned char*)blob, (const T*)Q, (const T*)K, (const T*)V, s->num_q_heads, s->num_q_heads / s->num_kv_heads, s->head_dim,
       s->q_stride_tok, s->q_stride_head, s->k_stride_tok, s->k_stride_head, s->v_stride_tok, s->v_stride_head, s->o_stride_tok,
-      s->o_stride_head, causal, scale, (T*)O, lse, s->total_tokens, ranges, scratch, keep);
+      s->o_stride_head, causal, scale, (T*)O, lse, s->total_tokens, ranges, rr, scratch, keep);
   return cudaGetLastError();
 }
 
 template <typename T, int R>
 cudaError_t launch_attn_dims(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
-                             float scale, void* O, float* lse, const int32_t* ranges, uint32_t* scratch, int keep, int rows, int smem_max, cudaStream_t st) {
+                             float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int smem_max, cudaStream_t st) {
   const int nd = (s->head_dim + 31) / 32;
-  if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, scratch, keep, rows, smem_max, st);
-  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, scratch, keep, rows, smem_max, st);
-  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, scratch, keep, rows, smem_max, st);
+  if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, smem_max, st);
+  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, smem_max, st);
+  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, smem_max, st);
 }
 
 }  // namespace
@@ -435,12 +432,13 @@ cudaError_t dam_launch_scores_ref(const void* Q, const void* K, const dam_shape_
 
 cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s,
                                 int causal, float scale, void* O, float* lse, void* scratch, bool keep_status,
-                                const int32_t* ranges, cudaStream_t st) {
+                                const int32_t* ranges, const int32_t* ranges_host, cudaStream_t st) {
   int rows = 0;
   for (int b = 0; b < s->num_seqs; ++b)
     rows += (s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b] + DAM_TILE - 1) / DAM_TILE;
   rows *= s->num_q_heads;
   uint32_t* scr = reinterpret_cast<uint32_t*>(scratch);
+  const DamRowRanges rr(ranges ? ranges_host : nullptr, s->num_seqs);
   const int keep = keep_status ? 2 : 0;
   if (rows == 0) return cudaMemsetAsync(scr + keep, 0, 256 - 4 * keep, st);
   int dev = 0;
@@ -449,8 +447,8 @@ cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, con
   if (e != cudaSuccess) return e;
   const bool four = four_rows((long long)rows * DAM_TILE, di.sm_count);
   if (s->dtype == DAM_F32)
-    return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, scr, keep, rows, di.smem_optin, st)
-                : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, scr, keep, rows, di.smem_optin, st);
-  return four ? launch_attn_dims<__nv_bfloat16, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, scr, keep, rows, di.smem_optin, st)
-              : launch_attn_dims<__nv_bfloat16, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, scr, keep, rows, di.smem_optin, st);
+    return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st)
+                : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st);
+  return four ? launch_attn_dims<__nv_bfloat16, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st)
+              : launch_attn_dims<__nv_bfloat16, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st);
 }

@@ -301,6 +301,31 @@ def test_chunked_prefill_equals_one_call(lengths, Hq, Hkv, d, dtype, gather):
     assert torch.equal(lse, lse_ref)
 
 
+@pytest.mark.parametrize("lengths,Hq,ranges", [
+    ([600] * 16, 4, [(256, 600)] * 16),                          # the last batch whose ranges travel with the launch
+    ([600, 0, 256] * 5 + [700, 40], 4, [(0, 512), (0, 0), (0, 256)] * 5 + [(512, 700), (0, 40)]),      # one sequence more
+    ([32700], 128, [(20480, 20992)]),                            # 16384 items, as many as a CTA marks
+    ([33000], 128, [(20480, 20992)]),                            # 16512: claimed one after the other
+])
+def test_row_ranges_of_long_lists_and_many_sequences(lengths, Hq, ranges):
+    """Rows of the single call, bit for bit, and no others."""
+    torch.manual_seed(23)
+    cu = np.concatenate([[0], np.cumsum(lengths)]).tolist()
+    Q = torch.randn(cu[-1], Hq, 64, dtype=torch.bfloat16, device=DEV)
+    K, V = (torch.randn(cu[-1], 2, 64, dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    shape = B.make_shape(cu, Hq, 2, 64, torch.bfloat16, DEV)
+    blob, _ = B.dam_build_masks(Q, K, shape, B.make_rule(64, 0.1, 0.5, gather_columns=True))
+    O_ref, lse_ref, _ = B.dam_sparse_attention(Q, K, V, blob, shape, causal=True)
+    O, lse = torch.full_like(O_ref, 7.0), torch.full_like(lse_ref, 7.0)
+    scratch = B.dam_sparse_attention_rows(Q, K, V, blob, shape, ranges, O, lse)
+    assert B.dam_poll_status(scratch) == 0
+    inside = torch.zeros(cu[-1], dtype=torch.bool, device=DEV)
+    for t0, (r0, r1) in zip(cu, ranges):
+        inside[t0 + r0: t0 + r1] = True
+    assert torch.equal(O[inside], O_ref[inside]) and torch.equal(lse[:, inside], lse_ref[:, inside])
+    assert (O[~inside] == 7.0).all() and (lse[:, ~inside] == 7.0).all()
+
+
 def test_row_ranges_leave_other_rows_alone_and_reject_odd_bounds():
     w = synth.small_case(0, 4, 2, 128, 128, seed=22, dtype=torch.bfloat16, lengths=[768, 512])
     shape = _shape(w)
