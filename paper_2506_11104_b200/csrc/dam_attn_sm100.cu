@@ -874,7 +874,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 // leaves; found here instead, from the V words by prefix counts and a search per place, they took
 // another 1-1.5 us of every call (a 2048-row chunk against a 2048-token window 66.4 us, now 64.9; 1237 tokens with a
 // 512-token window 59.3, now 58.6; 8192 tokens 151.2, now 149.7).
-__global__ void __launch_bounds__(128)
+constexpr int kGatherThreads = 256;
+__global__ void __launch_bounds__(kGatherThreads)
 gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat16* __restrict__ K,
                       const __nv_bfloat16* __restrict__ V, int Hq, int group, int d, int64_t kst, int64_t ksh, int64_t vst,
                       int64_t vsh, unsigned char* scratch, unsigned long long scratch_bytes) {
@@ -897,7 +898,7 @@ gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat1
   const DamSeq* seqs = reinterpret_cast<const DamSeq*>(blob + H->off_seq);
   const int tid = threadIdx.x;
   for (long long T = blockIdx.x; T < (long long)H->gath_tiles; T += gridDim.x) {
-    const int c_mine = __ldg(cols + T * DAM_TILE + tid);
+    const int c_mine = tid < DAM_TILE ? __ldg(cols + T * DAM_TILE + tid) : 0;
     int b = 0;
     while (b + 1 < H->num_seqs && (long long)seqs[b + 1].gath_off <= T) ++b;
     const DamSeq sq = seqs[b];
@@ -905,15 +906,16 @@ gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat1
     const int h = (int)((T - (long long)sq.gath_off) / sq.nL), g = (int)((T - (long long)sq.gath_off) % sq.nL);
     if (h >= Hq) continue;
     __syncthreads();
-    col[tid] = c_mine == 0xFFFF ? -1 : c_mine;
+    if (tid < DAM_TILE) col[tid] = c_mine == 0xFFFF ? -1 : c_mine;
     __syncthreads();
     if (col[0] < 0) continue;                                 // capacity tile that no row list refers to
     const __nv_bfloat16* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
     const __nv_bfloat16* Vh = V + (int64_t)sq.tok_start * vst + (int64_t)(h / group) * vsh;
     const int ppr = d >> 3;                                      // 16-byte pieces per row (16 at head_dim 128, 8 at 64)
-    const int part = tid % ppr, r0 = tid / ppr, step = 128 / ppr;
+    const int part = tid % ppr, r0 = tid / ppr, step = kGatherThreads / ppr;
     // eight rows of K and of V per thread are requested before the first is stored (the block is one dependent
-    // chain of loads as it is; one round trip per row would be most of its time)
+    // chain of loads as it is; one round trip per row would be most of its time), so 256 threads request the whole tile
+    // at once (128 threads, two round trips: the call at 8192 tokens 105.4 us, now 104.0)
     for (int rb = r0; rb < DAM_TILE; rb += 8 * step) {
       uint4 kv[8], vv[8];
 #pragma unroll
@@ -1008,7 +1010,7 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
   cfg.attrs = attr; cfg.numAttrs = 1;
   if (has_g && run_gather) {
     // clears the status block too
-    cfg.gridDim = dim3(sm_count * 4); cfg.blockDim = dim3(128);
+    cfg.gridDim = dim3(sm_count * 4); cfg.blockDim = dim3(kGatherThreads);
     if ((e = cudaLaunchKernelEx(&cfg, gather_columns_kernel, reinterpret_cast<const unsigned char*>(blob),
                                 reinterpret_cast<const __nv_bfloat16*>(K), reinterpret_cast<const __nv_bfloat16*>(V),
                                 (int)s->num_q_heads, (int)(s->num_q_heads / s->num_kv_heads), d, s->k_stride_tok, s->k_stride_head,
