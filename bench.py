@@ -353,7 +353,7 @@ def run_config(cfg, steps, warmup, gather, rank, world, local_rank, dev, pk, B, 
                                      "listed_min": round(float(he.min()), 4), "listed_median": round(float(np.median(he)), 4),
                                      "listed_max": round(float(he.max()), 4)},
            "roofline": roof, "clocks": clocks, "distinct_layers": n_layers,
-           "gpu_launches": (8 if gather else 7) * steps}      # init, score, counts, match, classify, order, [gather], attention
+           "gpu_launches": 7 * steps}      # init, score, counts, classify, order, gather (or the status block's clearing), attention
     if want_dense and rank == 0:
         # the build's own dense causal attention at the same length (all tiles listed as fully active)
         dmb, _, _ = B.dam_mask_sizes(shape, None, True)
