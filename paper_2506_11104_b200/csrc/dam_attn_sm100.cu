@@ -128,9 +128,9 @@ __device__ __forceinline__ Item item_from_words(const uint4& u, const uint4& v) 
 struct Lone {
   uint32_t at, n;
   int key;
-  __device__ __forceinline__ Lone(int2 lone, uint32_t t0, int qb, int nL, int S) : at(0u), n(0u), key(0) {
+  __device__ __forceinline__ Lone(int2 lone, uint32_t t0, int qb, int L, bool gather, int S) : at(0u), n(0u), key(0) {
     const int i0 = qb * DAM_TILE, r = lone.x;
-    if (r >= 0 && qb >= dam_lone_first_qblock(r, nL) && i0 < S) {
+    if (r >= 0 && qb >= dam_lone_first_qblock(r, L, gather) && i0 < S) {
       key = i0 - r;
       n = (uint32_t)(min(i0 + DAM_TILE, S) - 1 - r) / DAM_TILE - (uint32_t)key / DAM_TILE + 1u;
       at = t0 + (uint32_t)lone.y;
@@ -364,6 +364,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   // Dynamic scheduling: the work list is sorted longest first; the producer thread takes positions from a
   // global counter (the first one is the CTA index) and hands each to the other roles through a two-entry
   // ring in shared memory.  A negative position ends the loop.
+  const bool gather = (H->flags & DAM_FLAG_GATHER) != 0;
   const bool row_list = RANGED && nitems <= 32 * kRowBitWords;
   uint32_t* row_bits = reinterpret_cast<uint32_t*>(smem + SmemLayout::row_bits);
   auto item_active = [&](const Item& it) -> bool { return !RANGED || row_list || rows.holds(prm.ranges, it.seq, it.qb0); };
@@ -467,7 +468,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         bool skip = false;
         long long gtile0 = 0;
         int2 lone = make_int2(-1, 0);
-        int nL = 0;
+        int L = 0;
         if (w >= 0) {
           const uint4* src = reinterpret_cast<const uint4*>(blob + H->off_work) + 2 * (size_t)w;
           const uint4 u = __ldg(src), v = __ldg(src + 1);
@@ -477,7 +478,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           rec.u = u; rec.v = v;
           if (!skip) {
             const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[it.seq];
-            nL = sq.nL;
+            L = sq.L;
             if (H->off_lone) lone = __ldg(reinterpret_cast<const int2*>(blob + H->off_lone) + it.seq * H->num_q_heads + it.head);
             rec.lone = lone;
             rec.eA = it.a0 < it.a1 ? __ldg(tiles + it.a0) : 0u;
@@ -503,7 +504,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         ++ic;
         const int kvh = it.head / prm.group;
-        const Lone lA(lone, it.a0, it.qb0, nL, it.S), lB(lone, it.b0, it.qb0 + 1, nL, it.S);
+        const Lone lA(lone, it.a0, it.qb0, L, gather, it.S), lB(lone, it.b0, it.qb0 + 1, L, gather, it.S);
         Walker wk; wk.init(tiles, it, lA, lB);
         int kb; uint32_t kA, kB;
         while (ok && wk.next(kb, kA, kB)) {
@@ -684,7 +685,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         return need ? dam_apply_bits(hb, kind, i, kb, prm.causal) : make_uint4(~0u, ~0u, ~0u, ~0u);
       };
       // entries left out: entry t of what remains is entry t + ln.n of the list from ln.at on
-      const Lone ln(lone, t0, qb, (hb.L + DAM_TILE - 1) / DAM_TILE, it.S);
+      const Lone ln(lone, t0, qb, hb.L, gather, it.S);
       t1 -= ln.n;
       auto entry = [&](uint32_t t) -> uint32_t { return __ldg(tiles + (t >= ln.at ? t + ln.n : t)); };
       uint32_t e_next = t0 + 1 < t1 ? entry(t0 + 1) : 0u;

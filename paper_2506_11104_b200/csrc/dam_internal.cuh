@@ -178,9 +178,15 @@ __host__ __device__ inline int dam_gather_first_row(int L) { return dam_gather_f
 // with a sink.  Its 128 keys of a query block lie across two tiles of the grid that hold nothing else; the tensor-core
 // attention kernel multiplies one tile that starts at the block's first such key instead, of which a row needs one entry
 // (the two listed tiles were 18 % of the attention time at 8k and 32k tokens).  Query blocks from this one on: all their
-// keys on the diagonal lie beyond the tiles of the window, so no matched column meets them.
+// keys on the diagonal lie beyond the tiles of the window, so no matched column meets them, and their lists have the same
+// number of entries in front of the diagonal's.  With gathered columns that holds from the first block that lists them:
+// the blocks before it list window tiles instead, one per tile with a matched column (L = 1024, columns 10, 200 and 900:
+// three entries, where the blocks after it have one).
 constexpr int kLoneMin = 255;
-__host__ __device__ inline int dam_lone_first_qblock(int r, int nL) { return nL + (r + DAM_TILE - 1) / DAM_TILE; }
+__host__ __device__ inline int dam_lone_first_qblock(int r, int L, bool gather) {
+  const int beyond = (L + DAM_TILE - 1) / DAM_TILE + (r + DAM_TILE - 1) / DAM_TILE, gathered = gather ? dam_gather_first_qblock(L) : 0;
+  return beyond > gathered ? beyond : gathered;
+}
 
 struct DamHeadBits {
   const uint32_t* D;

@@ -406,7 +406,7 @@ __device__ __forceinline__ void classify_pair(unsigned char* blob, unsigned char
     if (x == 0) a1 = base;
     pair_total += total;
     mask_tiles += plan[x].apart ? nat + total - plan[x].n1 : plan[x].gathered ? nat : total;
-    if (lone >= 0 && plan[x].qb >= dam_lone_first_qblock(lone, sq.nL)) {      // one tile in place of those with a cell of the lone diagonal
+    if (lone >= 0 && plan[x].qb >= dam_lone_first_qblock(lone, sq.L, gflag != 0)) {      // one tile in place of those with a cell of the lone diagonal
       const int i0 = plan[x].qb * DAM_TILE, i1 = min(i0 + DAM_TILE, sq.S);
       saved += (i1 - 1 - lone) / DAM_TILE - (i0 - lone) / DAM_TILE;
     }

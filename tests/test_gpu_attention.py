@@ -157,6 +157,33 @@ def test_lone_diagonal_every_row(lengths, pcl, Hq, Hkv, d, gather):
     assert st["executed_tiles"] < st["tiles"] if pcl != 385 else st["executed_tiles"] == st["tiles"]
 
 
+@pytest.mark.parametrize("gather", [False, True])
+@pytest.mark.parametrize("L,d", [(512, 128), (1000, 64)])
+def test_lone_diagonal_at_any_distance(L, d, gather):
+    """A lone diagonal far below L - 1 (a head that attends at a fixed lag), one head per distance, with matched columns
+    that lie in more window tiles than they would fill as gathered columns.  The blocks between the first one beyond the
+    diagonal's reach into the window and the first one with gathered columns list the window's tiles."""
+    distances = [255, 300, L - 129, L - 128, L - 1]
+    Hq = len(distances)
+    w = synth.small_case(0, Hq, 1, d, L, seed=29, dtype=torch.bfloat16, lengths=[3 * L + 77])
+    i = np.arange(L)
+    maps = np.zeros((Hq, L, L), np.float32)
+    for h, r in enumerate(distances):
+        for lag in (0, 1, r):
+            maps[h, i[lag:], i[:L - lag]] = 0.5
+        for c in (5, L // 3, L - 100):
+            maps[h, c:, c] = 0.5
+    shape = _shape(w)
+    rule = B.make_rule(L, w.tau, w.mu, w.lam, w.eps, gather_columns=gather)
+    blob, _ = B.dam_build_masks_from_scores(torch.from_numpy(maps).to(DEV), shape, rule)
+    masks = H.oracle_masks_from_dump(w, maps.reshape(-1))
+    assert [int(np.flatnonzero(m.D)[-1]) for m in masks[0]] == distances
+    O, lse = _run(w, blob, shape, sentinel=True)
+    _check(w, O, lse, masks, _all_rows)
+    st = B.dam_mask_stats(blob, shape)
+    assert st["executed_tiles"] < st["tiles"]
+
+
 def test_empty_rows_and_no_patterns():
     """mu > 1: nothing matches, every row below the window is empty."""
     w = synth.small_case(0, 4, 2, 128, 128, seed=5, lengths=[600])
