@@ -116,3 +116,31 @@ def test_per_device_table_keeps_one_record_per_ordinal():
     for t in ts:
         t.join()
     assert len(results) == 8 and all(r[0] == 0 and r[2] == (2, 2) for r in results)
+
+
+def test_host_tensors_are_refused_before_the_library_is_called():
+    """Host tensors in every entry point that takes device tensors: an exception from the binding."""
+    for device in (torch.device("cpu"), "cpu", "meta"):
+        with pytest.raises(ValueError):
+            B._stream(device)
+    shape = B.make_shape([0, 256], 2, 2, 64, torch.bfloat16, "cpu")
+    rule = B.make_rule(128, 0.3, 0.8)
+    x = torch.zeros(256, 2, 64, dtype=torch.bfloat16)
+    buf = torch.zeros(1 << 20, dtype=torch.uint8)
+    lse, f = torch.zeros(2, 256), torch.zeros(2, 128, 128)
+    n = torch.zeros(128, dtype=torch.int32)
+    for call in (lambda: B.dam_build_masks(x, x, shape, rule, buf, buf),
+                 lambda: B.dam_build_masks_static(x, x, shape, rule, buf),
+                 lambda: B.dam_build_masks_from_scores(f, shape, rule, buf, buf),
+                 lambda: B.dam_mask_all_ones(shape, True, "cpu", buf),
+                 lambda: B.dam_sparse_attention(x, x, x, buf, shape, True, 0.0, x, lse, buf),
+                 lambda: B.dam_sparse_attention_rows(x, x, x, buf, shape, [(0, 256)], x, lse, scratch=buf),
+                 lambda: B.dam_decode_attention(x[:1], x, x, buf, shape, n[:1], 0.0, x[:1], lse[:1, :2], buf),
+                 lambda: B.dam_capture_accumulate(f, shape, 128, f, n),
+                 lambda: B.dam_capture_average(f, n, 128, 1e-8, shape),
+                 lambda: B.dam_mask_stats(buf, shape), lambda: B.dam_poll_status(buf),
+                 lambda: B.dam_mask_expand_rows(buf, shape, 0, 0, 0, 1),
+                 lambda: B.dam_selftest_bounded_wait("cpu"),
+                 lambda: B.dam_prefill_host(x, x, x, shape, rule, x, lse, buf, "cpu")):
+        with pytest.raises(ValueError):
+            call()
