@@ -356,8 +356,11 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   const int nitems = H->prows;
   const uint32_t* tiles = reinterpret_cast<const uint32_t*>(blob + H->off_tiles);
   // a blob with gathered-column tiles needs the larger scratch: nothing is computed without it, and the status
-  // word says why (the gather kernel is not even launched when the scratch holds no tile at all)
+  // word says why (the gather kernel is not even launched when the scratch holds no tile at all).  The kernel in front
+  // clears that word: the error is written, and the CTA ends, only after it.  (The blob itself may be read before: the
+  // kernel in front lets this one begin after its own wait for the kernels that wrote the blob.)
   if ((H->flags & DAM_FLAG_GATHER) && H->attn_scratch_bytes > prm.scratch_bytes) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (blockIdx.x == 0 && tid == 0) atomicMax(prm.status, (uint32_t)DAM_ERR_BUFFER_TOO_SMALL);
     return;
   }

@@ -244,6 +244,23 @@ def test_gathered_blob_with_small_scratch_reports_error():
         assert (O == 7.0).all()
 
 
+@pytest.mark.parametrize("d", [128, 64])
+def test_small_scratch_is_reported_by_every_chunk(d):
+    """The kernel that clears the status word runs right before the one that writes the error: the error stays, call
+    after call, and no row is written."""
+    w = synth.small_case(0, 4, 2, d, 128, seed=4, lengths=[900])
+    shape = _shape(w)
+    Q, K, V = w.Q.to(DEV), w.K.to(DEV), w.V.to(DEV)
+    blob, _ = B.dam_build_masks(Q, K, shape, B.make_rule(w.pcl_max, w.tau, w.mu, gather_columns=True))
+    O, lse = torch.full_like(Q, 7.0), torch.full((4, 900), 7.0, device=DEV)
+    for nbytes in (256, 256 + 65536):
+        small = torch.zeros(256 + 70000, dtype=torch.uint8, device=DEV)[:nbytes]
+        for k in range(20):
+            B.dam_sparse_attention_rows(Q, K, V, blob, shape, [(256 * (k % 3), 256 * (k % 3) + 256)], O, lse, scratch=small)
+            assert B.dam_poll_status(small) == 3
+    assert (O == 7.0).all() and (lse == 7.0).all()
+
+
 def test_bounded_wait_times_out_cleanly():
     """A wait that nothing satisfies gives up after its limit, the status word says so, and the device keeps
     working (the next kernel runs and is correct)."""
