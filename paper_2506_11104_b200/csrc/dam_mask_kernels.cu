@@ -332,13 +332,13 @@ __device__ __forceinline__ uint32_t classify_band(const HeadView& v, int qb, int
 // Tile statistics of a block's pairs: one global atomic per block and statistic instead of one per warp on the same address.
 struct TileStats {
   unsigned long long mask_tiles;
-  uint32_t total, full, exec;
+  uint32_t total, full, saved;      // saved: listed, but not multiplied (lone diagonals)
 };
 
 // Lists the tiles of one pair of query blocks of a (sequence, head), and leaves its work item and its key: one warp.
 __device__ __forceinline__ void classify_pair(unsigned char* blob, unsigned char* scratch, uint64_t off_items, uint64_t off_keys,
                                               const DamHeader* H, int nkeys, const DamSeq& sq, int b, int h, int gp,
-                                              const HeadView& v, int lone, TileStats& st) {
+                                              const HeadView& v, TileStats& st) {
   const int lane = threadIdx.x & 31;
   const int gqb0 = sq.first_qblock + 2 * (gp - sq.first_pair), nblk = 2 * (gp - sq.first_pair) + 1 < sq.nq ? 2 : 1;
   uint32_t* tile_ptr = reinterpret_cast<uint32_t*>(blob + H->off_tile_ptr);
@@ -350,7 +350,7 @@ __device__ __forceinline__ void classify_pair(unsigned char* blob, unsigned char
   const uint32_t pair_begin = (uint32_t)(head_base + dam_row_tile_prefix(qb0, sq.nL, sq.L, gflag));
   const uint32_t pair_end = (uint32_t)(head_base + dam_row_tile_prefix(qb0 + nblk, sq.nL, sq.L, gflag));
   uint32_t base = pair_begin, a1 = pair_begin;
-  int pair_total = 0, nfull = 0, mask_tiles = 0, saved = 0;
+  int pair_total = 0, nfull = 0, mask_tiles = 0;
   // Per query block: candidates, ascending: [0, min(qb, nL-1)] then [max(that + 1, qb - nL), qb].  From row 2L - 1
   // on (gathered columns enabled) the first range is replaced by the gathered tiles and the second range is
   // classified on the matched diagonals alone.  The tiles of the mask itself (128 x 128 grid) with an active cell
@@ -406,10 +406,6 @@ __device__ __forceinline__ void classify_pair(unsigned char* blob, unsigned char
     if (x == 0) a1 = base;
     pair_total += total;
     mask_tiles += plan[x].apart ? nat + total - plan[x].n1 : plan[x].gathered ? nat : total;
-    if (lone >= 0 && plan[x].qb >= dam_lone_first_qblock(lone, sq.L, gflag != 0)) {      // one tile in place of those with a cell of the lone diagonal
-      const int i0 = plan[x].qb * DAM_TILE, i1 = min(i0 + DAM_TILE, sq.S);
-      saved += (i1 - 1 - lone) / DAM_TILE - (i0 - lone) / DAM_TILE;
-    }
     total = 0; nat = 0;
   };
   const int span0 = max(plan[0].ncand, plan[0].nmask), span1 = max(plan[1].ncand, plan[1].nmask);
@@ -455,16 +451,26 @@ __device__ __forceinline__ void classify_pair(unsigned char* blob, unsigned char
     reinterpret_cast<uint32_t*>(scratch + off_keys)[at] = (uint32_t)min(pair_total, nkeys - 1);
     atomicAdd(&st.mask_tiles, (unsigned long long)mask_tiles);
     atomicAdd(&st.total, (uint32_t)pair_total);
-    atomicAdd(&st.exec, (uint32_t)(pair_total - saved));
     atomicAdd(&st.full, (uint32_t)nfull);
   }
+}
+
+// Listed tiles of a head that its lone diagonal r makes superfluous: on every block it is served on, one tile takes the place
+// of the one or two with a cell of it.  (Once per head: counted block by block in classify_pair, the same lines cost every
+// pass 0.4 us.)
+__device__ __forceinline__ uint32_t lone_saved_tiles(const DamSeq& sq, int r, bool gather) {
+  const int first = dam_lone_first_qblock(r, sq.L, gather), whole = sq.S / DAM_TILE;
+  int saved = r % DAM_TILE ? max(0, whole - first) : 0;
+  if (whole < sq.nq && whole >= first) saved += (sq.S - 1 - r) / DAM_TILE - (whole * DAM_TILE - r) / DAM_TILE;
+  return (uint32_t)saved;
 }
 
 __device__ __forceinline__ void flush_stats(unsigned char* blob, const TileStats& st) {
   DamHeader* H = reinterpret_cast<DamHeader*>(blob);
   if (st.mask_tiles) atomicAdd(reinterpret_cast<unsigned long long*>(&H->mask_tiles), st.mask_tiles);
   if (st.total) atomicAdd(&H->total_tiles, st.total);
-  if (st.exec) atomicAdd(reinterpret_cast<unsigned long long*>(&H->exec_tiles), (unsigned long long)st.exec);
+  if (st.total != st.saved)                                // (modulo 2^64: a block may leave out more than it lists)
+    atomicAdd(reinterpret_cast<unsigned long long*>(&H->exec_tiles), (unsigned long long)st.total - st.saved);
   if (st.full) atomicAdd(&H->full_tiles, st.full);
 }
 
@@ -520,11 +526,14 @@ classify_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, u
   v.Dw = bits; v.Vw = bits + 2 * W; v.prefD = prefD; v.prefV = prefV; v.tile_pop = cnt + 2 * L + 2 * (W + 1);
   v.L = L; v.W = W; v.nL = sq.nL; v.S = sq.S;
   for (int p = blockIdx.x * kClassifyWarps + warp; p < npairs; p += nblk * kClassifyWarps)
-    classify_pair(blob, scratch, off_items, off_keys, H, bp.nkeys, sq, b, h, sq.first_pair + p, v, lone.x, st);
+    classify_pair(blob, scratch, off_items, off_keys, H, bp.nkeys, sq, b, h, sq.first_pair + p, v, st);
   if (last) {
     if (in_smem)
       for (int w = threadIdx.x; w < 3 * W; w += blockDim.x) dv[w] = bits[w];
-    if (threadIdx.x == 0) reinterpret_cast<int2*>(blob + H->off_lone)[sh] = lone;
+    if (threadIdx.x == 0) {
+      reinterpret_cast<int2*>(blob + H->off_lone)[sh] = lone;
+      if (lone.x >= 0) st.saved = lone_saved_tiles(sq, lone.x, (H->flags & DAM_FLAG_GATHER) != 0);
+    }
     if (H->off_cols) list_columns(blob, H, sq, h, bits + 2 * W, prefV);
   }
   __syncthreads();
