@@ -404,8 +404,8 @@ _HDR = np.dtype([("magic", "<u4"), ("status", "<u4"), ("version", "<u4"), ("flag
                  ("off_seq", "<u8"), ("off_qbseq", "<u8"), ("off_dv", "<u8"), ("off_true", "<u8"),
                  ("off_tile_ptr", "<u8"), ("off_work", "<u8"), ("off_tiles", "<u8"), ("bytes_used", "<u8"),
                  ("causal_tiles", "<u8"), ("off_pairtab", "<u8"), ("total_pairs", "<i4"), ("prows", "<i4"),
-                 ("gath_tiles", "<u8"), ("attn_scratch_bytes", "<u8"), ("mask_tiles", "<u8"), ("head_tile_cap", "<u8"), ("reserved", "<u8", (8,)),
-                 ("off_cols", "<u8"), ("off_lone", "<u8"), ("exec_tiles", "<u8")])
+                 ("gath_tiles", "<u8"), ("attn_scratch_bytes", "<u8"), ("mask_tiles", "<u8"), ("head_tile_cap", "<u8"), ("reserved", "<u8", (7,)),
+                 ("off_lone", "<u8"), ("off_cols", "<u8"), ("off_lone2", "<u8"), ("exec_tiles", "<u8")])
 _SEQ = np.dtype([("tok_start", "<i4"), ("S", "<i4"), ("L", "<i4"), ("nq", "<i4"), ("first_qblock", "<i4"),
                  ("W", "<i4"), ("nL", "<i4"), ("first_pair", "<i4"), ("dv_off", "<u8"), ("true_off", "<u8"),
                  ("p_off", "<u8"), ("cnt_off", "<u8"), ("gath_off", "<u8"), ("tile_base", "<u8")])

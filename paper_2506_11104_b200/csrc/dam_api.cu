@@ -113,7 +113,7 @@ void compute_layout(const dam_shape_t* s, int pcl_max, int all_ones_causal, int 
   h.off_pairtab = dam_align(h.off_qbseq + 4ull * total_qb, 256);
   const uint64_t lone = dam_align(h.off_pairtab + 4ull * total_pairs, 256);
   h.off_lone = pcl_max > 0 ? lone : 0;
-  const uint64_t cols = pcl_max > 0 ? dam_align(lone + 8ull * s->num_seqs * Hq, 256) : lone;
+  const uint64_t cols = pcl_max > 0 ? dam_align(lone + 16ull * s->num_seqs * Hq, 256) : lone;
   h.off_cols = pcl_max > 0 && gather ? cols : 0;
   h.off_dv = h.off_cols ? dam_align(cols + 2ull * DAM_TILE * gath, 256) : cols;
   h.off_true = dam_align(h.off_dv + 4ull * dv, 256);

@@ -65,7 +65,7 @@ struct SmemLayout {
   static constexpr int sched_items = bars + 8 * n_bars;     // int[2]: work-list positions handed to the consumers
   static constexpr int step_desc = sched_items + 8;         // u32[16]: what the producer found at each step (kStep*)
   static constexpr int item_rec = (step_desc + 64 + 15) & ~15;   // ItemRec[2] (16-byte aligned): what the softmax warps need to start an item
-  static constexpr int tmem_slot = item_rec + 2 * 96;
+  static constexpr int tmem_slot = item_rec + 2 * 112;
   static constexpr int abort_flag = tmem_slot + 4;
   static constexpr int row_bits = abort_flag + 4;           // u32[kRowBitWords]: the work list's items inside the row ranges
   static constexpr int total = row_bits + 4 * kRowBitWords;
@@ -76,13 +76,14 @@ constexpr int kSmemBytes = SmemLayout::total;          // (the array is declared
 // What the producer hands to the softmax warps with every work-list position: the item record, the first tile
 // entry of each stream and the head's bit-set pointers, so that their set-up reads shared memory instead of
 // walking item -> sequence record -> tile list in global memory.
-struct ItemRec {
+struct alignas(16) ItemRec {
   uint4 u, v;               // the two words of the DamItem
   uint32_t eA, eB;
-  int2 lone;                // the head's lone diagonal (or -1) and the entries in front of it
+  int2 lone;                // the head's lone diagonal and the entries in front of it
   DamHeadBits hb;
+  int lone_from;            // the first query block it is served on
 };
-static_assert(sizeof(ItemRec) == 96, "ItemRec must be 96 bytes");
+static_assert(sizeof(ItemRec) == 112, "ItemRec must be 112 bytes");
 
 struct AttnParams {
   const unsigned char* blob;
@@ -128,9 +129,9 @@ __device__ __forceinline__ Item item_from_words(const uint4& u, const uint4& v) 
 struct Lone {
   uint32_t at, n;
   int key;
-  __device__ __forceinline__ Lone(int2 lone, uint32_t t0, int qb, int L, bool gather, int S) : at(0u), n(0u), key(0) {
+  __device__ __forceinline__ Lone(int2 lone, int from, uint32_t t0, int qb, int S) : at(0u), n(0u), key(0) {
     const int i0 = qb * DAM_TILE, r = lone.x;
-    if (r >= 0 && qb >= dam_lone_first_qblock(r, L, gather) && i0 < S) {
+    if (qb >= from && i0 < S) {
       key = i0 - r;
       n = (uint32_t)(min(i0 + DAM_TILE, S) - 1 - r) / DAM_TILE - (uint32_t)key / DAM_TILE + 1u;
       at = t0 + (uint32_t)lone.y;
@@ -367,7 +368,6 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   // Dynamic scheduling: the work list is sorted longest first; the producer thread takes positions from a
   // global counter (the first one is the CTA index) and hands each to the other roles through a two-entry
   // ring in shared memory.  A negative position ends the loop.
-  const bool gather = (H->flags & DAM_FLAG_GATHER) != 0;
   const bool row_list = RANGED && nitems <= 32 * kRowBitWords;
   uint32_t* row_bits = reinterpret_cast<uint32_t*>(smem + SmemLayout::row_bits);
   auto item_active = [&](const Item& it) -> bool { return !RANGED || row_list || rows.holds(prm.ranges, it.seq, it.qb0); };
@@ -471,7 +471,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         bool skip = false;
         long long gtile0 = 0;
         int2 lone = make_int2(-1, 0);
-        int L = 0;
+        int lone_from = 0x7FFFFFFF;
         if (w >= 0) {
           const uint4* src = reinterpret_cast<const uint4*>(blob + H->off_work) + 2 * (size_t)w;
           const uint4 u = __ldg(src), v = __ldg(src + 1);
@@ -481,8 +481,13 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           rec.u = u; rec.v = v;
           if (!skip) {
             const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[it.seq];
-            L = sq.L;
-            if (H->off_lone) lone = __ldg(reinterpret_cast<const int2*>(blob + H->off_lone) + it.seq * H->num_q_heads + it.head);
+            if (H->off_lone) {
+              // (in two pieces: as one 16-byte read the row-range kernel spills more, a 2048-row chunk 51.6 -> 52.5 us)
+              const int2* lr = reinterpret_cast<const int2*>(blob + H->off_lone) + 2 * (it.seq * H->num_q_heads + it.head);
+              lone = __ldg(lr);
+              lone_from = __ldg(&lr[1].x);
+            }
+            rec.lone_from = lone_from;
             rec.lone = lone;
             rec.eA = it.a0 < it.a1 ? __ldg(tiles + it.a0) : 0u;
             rec.eB = it.b0 < it.b1 ? __ldg(tiles + it.b0) : 0u;
@@ -507,7 +512,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         ++ic;
         const int kvh = it.head / prm.group;
-        const Lone lA(lone, it.a0, it.qb0, L, gather, it.S), lB(lone, it.b0, it.qb0 + 1, L, gather, it.S);
+        const Lone lA(lone, lone_from, it.a0, it.qb0, it.S), lB(lone, lone_from, it.b0, it.qb0 + 1, it.S);
         Walker wk; wk.init(tiles, it, lA, lB);
         int kb; uint32_t kA, kB;
         while (ok && wk.next(kb, kA, kB)) {
@@ -654,6 +659,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       const DamHeadBits hb = rec.hb;                         // (not meaningful for an item without steps)
       const uint32_t e_first = X ? rec.eB : rec.eA;
       const int2 lone = rec.lone;
+      const int lone_from = rec.lone_from;
       __syncwarp();
       if (lane == 0) mbar_arrive(bSchedEmpty + 8 * (n & 1u));               // the whole warp has read the record
       if ((X == 1 && !it.hasB) || !item_active(it)) continue;
@@ -688,7 +694,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         return need ? dam_apply_bits(hb, kind, i, kb, prm.causal) : make_uint4(~0u, ~0u, ~0u, ~0u);
       };
       // entries left out: entry t of what remains is entry t + ln.n of the list from ln.at on
-      const Lone ln(lone, t0, qb, hb.L, gather, it.S);
+      const Lone ln(lone, lone_from, t0, qb, it.S);
       t1 -= ln.n;
       auto entry = [&](uint32_t t) -> uint32_t { return __ldg(tiles + (t >= ln.at ? t + ln.n : t)); };
       uint32_t e_next = t0 + 1 < t1 ? entry(t0 + 1) : 0u;

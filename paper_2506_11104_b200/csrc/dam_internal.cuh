@@ -12,8 +12,9 @@
 //   per (seq, head) true mask    L rows x W words, bit (j % 32) of word (j / 32) = M[i][j]
 //   pair_tab[total_pairs]        first global q-block of every pair of adjacent q-blocks (2p, 2p+1) of a
 //                                sequence; bit 31 set when the second block exists
-//   lone[num_seqs * num_q_heads] int2 per (seq, head): its lone diagonal (see dam_lone_first_qblock) or -1, and how many
-//                                entries the list of a query block it is served on has in front of the diagonal's own
+//   lone[num_seqs * num_q_heads] int4 per (seq, head): its lone diagonal (see dam_lone_first_qblock) or -1, how many
+//                                entries the list of a query block it is served on has in front of the diagonal's own,
+//                                and the first such block
 //   cols (gathered columns only) u16 per place of every gathered-column tile of every (seq, head): the head's matched
 //                                columns in ascending order, 0xFFFF behind the last one
 //   tile_ptr[rows + 1]           start of every row's entries in tiles[], rows = head * total_qblocks + global
@@ -68,9 +69,10 @@ struct DamHeader {
   uint64_t attn_scratch_bytes;   // scratch dam_sparse_attention needs for this blob
   uint64_t mask_tiles;      // 128 x 128 tiles of the masks that hold an active cell (= total_tiles unless gathered)
   uint64_t head_tile_cap;   // entries of tiles[] every head owns (sum of the row bounds of all sequences)
-  uint64_t reserved[8];     // [0]: 1 when the window map was scored by the tensor-core kernel (test hook)
-  uint64_t off_cols;        // 0: no section (all-ones blob, or no gathered columns)
+  uint64_t reserved[7];     // [0]: 1 when the window map was scored by the tensor-core kernel (test hook)
   uint64_t off_lone;        // 0: no section (all-ones blob)
+  uint64_t off_cols;        // 0: no section (all-ones blob, or no gathered columns)
+  uint64_t off_lone2;       // (0; blobs of an earlier build have 8-byte records of the lone diagonals here, which are not read)
   uint64_t exec_tiles;      // tiles the tensor-core attention kernel multiplies (total_tiles, or fewer: lone diagonals)
 };
 static_assert(sizeof(DamHeader) == 256, "DamHeader must be 256 bytes");

@@ -200,7 +200,7 @@ __global__ void counts_kernel(const unsigned char* blob, unsigned char* scratch,
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void match_head(const DamSeq& sq, bool gather, float mu, int min_support, const int32_t* cntD,
                                            const int32_t* cntV, uint32_t* Dw, uint32_t* Rw, uint32_t* Vw, int32_t* prefD,
-                                           int32_t* prefV, int2* lone) {
+                                           int32_t* prefV, int4* lone) {
   const int L = sq.L, W = sq.W;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int w = warp; w < W; w += nw) {
@@ -258,7 +258,8 @@ __device__ __forceinline__ void match_head(const DamSeq& sq, bool gather, float 
       for (int g = lane; g < W / 4; g += 32) front += (Vw[4 * g] | Vw[4 * g + 1] | Vw[4 * g + 2] | Vw[4 * g + 3]) != 0u;
       front = __reduce_add_sync(0xFFFFFFFFu, front);
     }
-    if (lane == 0) *lone = make_int2(top >= kLoneMin && (below < 0 || top - below >= kLoneMin) ? top : -1, front);
+    if (lane == 0 && top >= kLoneMin && (below < 0 || top - below >= kLoneMin))
+      *lone = make_int4(top, front, dam_lone_first_qblock(top, L, gather), 0);
   }
 }
 
@@ -458,8 +459,8 @@ __device__ __forceinline__ void classify_pair(unsigned char* blob, unsigned char
 // Listed tiles of a head that its lone diagonal r makes superfluous: on every block it is served on, one tile takes the place
 // of the one or two with a cell of it.  (Once per head: counted block by block in classify_pair, the same lines cost every
 // pass 0.4 us.)
-__device__ __forceinline__ uint32_t lone_saved_tiles(const DamSeq& sq, int r, bool gather) {
-  const int first = dam_lone_first_qblock(r, sq.L, gather), whole = sq.S / DAM_TILE;
+__device__ __forceinline__ uint32_t lone_saved_tiles(const DamSeq& sq, int r, int first) {
+  const int whole = sq.S / DAM_TILE;
   int saved = r % DAM_TILE ? max(0, whole - first) : 0;
   if (whole < sq.nq && whole >= first) saved += (sq.S - 1 - r) / DAM_TILE - (whole * DAM_TILE - r) / DAM_TILE;
   return (uint32_t)saved;
@@ -499,7 +500,7 @@ classify_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, u
   dam_chain_prologue();
   extern __shared__ int32_t csm[];
   __shared__ TileStats st;
-  __shared__ int2 lone;
+  __shared__ int4 lone;
   const DamHeader* H = &bp.h;
   const int sh = blockIdx.y, b = sh / H->num_q_heads, h = sh % H->num_q_heads;
   const DamSeq sq = dam_plan_seq(bp, blob, b);
@@ -514,7 +515,7 @@ classify_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, u
   uint32_t* bits = in_smem ? reinterpret_cast<uint32_t*>(csm) : dv;
   int32_t* prefD = in_smem ? csm + 3 * W : cnt + 2 * L;
   int32_t* prefV = prefD + (W + 1);
-  if (threadIdx.x == 0) { st = TileStats{0ull, 0u, 0u, 0u}; lone = make_int2(-1, 0); }
+  if (threadIdx.x == 0) { st = TileStats{0ull, 0u, 0u, 0u}; lone = make_int4(-1, 0, 0x7FFFFFFF, 0); }
   __syncthreads();
   if (L > 0) {
     match_head(sq, (H->flags & DAM_FLAG_GATHER) != 0, mu, min_support, cnt, cnt + L, bits, bits + W, bits + 2 * W, prefD, prefV,
@@ -531,8 +532,8 @@ classify_kernel(unsigned char* blob, unsigned char* scratch, uint64_t off_cnt, u
     if (in_smem)
       for (int w = threadIdx.x; w < 3 * W; w += blockDim.x) dv[w] = bits[w];
     if (threadIdx.x == 0) {
-      reinterpret_cast<int2*>(blob + H->off_lone)[sh] = lone;
-      if (lone.x >= 0) st.saved = lone_saved_tiles(sq, lone.x, (H->flags & DAM_FLAG_GATHER) != 0);
+      reinterpret_cast<int4*>(blob + H->off_lone)[sh] = lone;
+      if (lone.x >= 0) st.saved = lone_saved_tiles(sq, lone.x, lone.z);
     }
     if (H->off_cols) list_columns(blob, H, sq, h, bits + 2 * W, prefV);
   }

@@ -166,6 +166,9 @@ def test_lone_diagonal_at_any_distance(L, d, gather):
     distances = [255, 300, L - 129, L - 128, L - 1]
     Hq = len(distances)
     w = synth.small_case(0, Hq, 1, d, L, seed=29, dtype=torch.bfloat16, lengths=[3 * L + 77])
+    # a row keeps a handful of keys, so O reaches the largest |V|, about 5: half a bf16 step there is 2^-6, and P's rounding
+    # adds 2^-9 of |V|: 0.026, over the tolerance.  With V halved (exactly) both are halved: 0.013.
+    w.V = w.V * 0.5
     i = np.arange(L)
     maps = np.zeros((Hq, L, L), np.float32)
     for h, r in enumerate(distances):
