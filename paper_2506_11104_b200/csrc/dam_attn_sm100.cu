@@ -79,7 +79,8 @@ constexpr int kSmemBytes = SmemLayout::total;          // (the array is declared
 struct alignas(16) ItemRec {
   uint4 u, v;               // the two words of the DamItem
   uint32_t eA, eB;
-  int2 lone;                // the head's lone diagonal and the entries in front of it
+  int2 lone;                // the head's lone diagonal and the entries in front of it (with the next as one int4 the row-range
+                            // kernel spills more: a 2048-row chunk 51.6 -> 52.5 us)
   DamHeadBits hb;
   int lone_from;            // the first query block it is served on
 };
@@ -482,10 +483,9 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           if (!skip) {
             const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[it.seq];
             if (H->off_lone) {
-              // (in two pieces: as one 16-byte read the row-range kernel spills more, a 2048-row chunk 51.6 -> 52.5 us)
-              const int2* lr = reinterpret_cast<const int2*>(blob + H->off_lone) + 2 * (it.seq * H->num_q_heads + it.head);
-              lone = __ldg(lr);
-              lone_from = __ldg(&lr[1].x);
+              const int4 lr = __ldg(reinterpret_cast<const int4*>(blob + H->off_lone) + it.seq * H->num_q_heads + it.head);
+              lone = make_int2(lr.x, lr.y);
+              lone_from = lr.z;
             }
             rec.lone_from = lone_from;
             rec.lone = lone;
