@@ -102,18 +102,22 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 # the handle without the Stream object that torch.cuda.current_stream makes (0.1 us instead of 2.3), where torch has it
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+# indices of the CUDA devices asked for so far (device.type makes a string by way of a C++ stream: 4 us of a first pass)
+_cuda_index = {}
 
 
 def _stream(device) -> int:
     """Handle of the device's current stream; ValueError for a device that is not a GPU (every entry point asks for the
     stream of its first tensor's device: host memory never reaches a kernel by that argument)."""
-    d = torch.device(device) if isinstance(device, str) else device
-    if isinstance(d, torch.device):
-        if d.type != "cuda":
+    index = _cuda_index.get(device)
+    if index is None:
+        d = torch.device(device) if isinstance(device, str) else device
+        if isinstance(d, torch.device) and d.type != "cuda":
             raise ValueError(f"expected tensors on a CUDA device, got {d}")
-        if d.index is not None and _raw_stream is not None:
-            return _raw_stream(d.index)
-    return torch.cuda.current_stream(device).cuda_stream
+        if not isinstance(d, torch.device) or d.index is None or _raw_stream is None:
+            return torch.cuda.current_stream(device).cuda_stream
+        index = _cuda_index[device] = d.index
+    return _raw_stream(index)
 
 
 @dataclass
