@@ -990,7 +990,8 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
                                   cudaStream_t st) {
   const int d = s->head_dim;
   if (s->dtype != DAM_BF16 || (d != 128 && d != 64)) return cudaErrorNotSupported;
-  if (s->total_tokens == 0) return cudaSuccess;
+  if (s->total_tokens == 0)                              // nothing to compute: the status block starts at zero all the same
+    return dam_launch_chained(clear_status_kernel, dim3(1), dim3(64), 0, st, reinterpret_cast<uint32_t*>(scratch), run_gather ? 0 : 2);
   int dev = 0;
   DamDeviceInfo di;
   cudaError_t e;

@@ -268,6 +268,21 @@ def test_small_scratch_is_reported_by_every_chunk(d):
     assert (O == 7.0).all() and (lse == 7.0).all()
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("ranges", [None, [(0, 0), (0, 0)]])
+def test_empty_batch_clears_the_status_block(dtype, ranges):
+    """A call with no tokens leaves a clean status block, whatever the buffer held."""
+    shape = B.make_shape([0, 0, 0], 2, 1, 128, dtype, DEV)
+    x, lse = torch.zeros(8, 2, 128, dtype=dtype, device=DEV), torch.zeros(2, 8, device=DEV)
+    blob = torch.zeros(4096, dtype=torch.uint8, device=DEV)
+    scratch = torch.full((256,), 3, dtype=torch.uint8, device=DEV)
+    if ranges is None:
+        B.dam_sparse_attention(x, x, x, blob, shape, O=x, lse=lse, scratch=scratch)
+    else:
+        B.dam_sparse_attention_rows(x, x, x, blob, shape, ranges, x, lse, scratch=scratch)
+    assert B.dam_poll_status(scratch) == 0 and not scratch.any()
+
+
 def test_bounded_wait_times_out_cleanly():
     """A wait that nothing satisfies gives up after its limit, the status word says so, and the device keeps
     working (the next kernel runs and is correct)."""
