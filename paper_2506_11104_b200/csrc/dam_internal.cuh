@@ -327,7 +327,7 @@ typedef cudaError_t (*dam_device_setup_fn)(void);
 class DamDeviceTable {
  public:
   static constexpr int kMaxDevices = 64;
-  static constexpr int kMaxSetups = 8;
+  static constexpr int kMaxSetups = 32;
   // The record of `device`, filled by `query` the first time the ordinal is seen.
   cudaError_t info(int device, dam_device_query_fn query, DamDeviceInfo* out);
   // Runs `fn` (with `device` current) unless set-up step `key` already succeeded on that device.
@@ -336,7 +336,8 @@ class DamDeviceTable {
   struct Slot { bool filled; DamDeviceInfo info; bool done[kMaxSetups]; };
   Slot slots_[kMaxDevices] = {};
 };
-enum { DAM_SETUP_ATTN_SMEM = 0, DAM_SETUP_SCORE_SMEM = 1, DAM_SETUP_DECODE_SMEM = 2 };
+// (from DAM_SETUP_REF_SMEM on: one step per instance of the CUDA-core kernels)
+enum { DAM_SETUP_ATTN_SMEM = 0, DAM_SETUP_SCORE_SMEM = 1, DAM_SETUP_DECODE_SMEM = 2, DAM_SETUP_REF_SMEM = 3 };
 
 DamDeviceTable& dam_device_table();                                       // the library's own table
 cudaError_t dam_current_device(int* device, DamDeviceInfo* info);         // ordinal and record of the current device

@@ -366,21 +366,41 @@ size_t attn_smem(int d, int R, int nbuf) {
   return ((size_t)nbuf * kStageKeys * (k_pitch(d) + d) + (size_t)kRefWarps * R * (d + kStageKeys)) * sizeof(float);
 }
 
-// (48 KB of dynamic shared memory need no opt-in)
-template <typename F>
-cudaError_t allow_smem(F* kernel, size_t bytes) {
-  return bytes <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// Opt-in of one kernel instance to all the shared memory a block may have, once per device: the limit belongs to the
+// instance, and its calls differ in what they use (head_dim, stages), so a limit set to the need of each call could be
+// lowered by one thread between another's setting and launch.  (48 KB need no opt-in.)
+template <typename K>
+cudaError_t allow_all_smem(K* kernel) {
+  int dev = 0, bytes = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) : e;
+}
+template <typename T, int R>
+cudaError_t opt_in_scores(int dev, size_t bytes) {
+  constexpr int key = DAM_SETUP_REF_SMEM + 2 * (sizeof(T) == 4) + (R == 4);
+  return bytes <= 48 * 1024 ? cudaSuccess
+                            : dam_device_table().once(dev, key, []() -> cudaError_t { return allow_all_smem(scores_ref_kernel<T, R>); });
+}
+template <typename T, int R, int ND, bool PIPE>
+cudaError_t opt_in_attn(int dev, size_t bytes) {
+  constexpr int dims = ND == 2 ? 0 : ND == 4 ? 1 : 2, type = PIPE ? 2 : sizeof(T) == 4;
+  constexpr int key = DAM_SETUP_REF_SMEM + 4 + (3 * type + dims) * 2 + (R == 4);
+  static_assert(key < DamDeviceTable::kMaxSetups, "a set-up step per instance");
+  return bytes <= 48 * 1024
+             ? cudaSuccess
+             : dam_device_table().once(dev, key, []() -> cudaError_t { return allow_all_smem(attn_ref_kernel<T, R, ND, PIPE>); });
 }
 
 template <typename T, int R>
-cudaError_t launch_scores(const void* Q, const void* K, const dam_shape_t* s, const DamBuildCtx& c, float* dump, int sm_count,
-                          int smem_max, cudaStream_t st) {
+cudaError_t launch_scores(const void* Q, const void* K, const dam_shape_t* s, const DamBuildCtx& c, float* dump, int dev,
+                          const DamDeviceInfo& di, cudaStream_t st) {
   const dim3 grid((c.max_L + kRefWarps * R - 1) / (kRefWarps * R), c.num_seqs * c.Hq);
   // all stages at once while every block has an SM of its own anyway (a block's shared memory then costs no occupancy)
   const int nstage = (c.max_L + kStageKeys - 1) / kStageKeys;
-  const int nbuf = (long long)grid.x * grid.y <= sm_count && score_smem(c.d, R, nstage) <= (size_t)smem_max ? nstage : 1;
+  const int nbuf = (long long)grid.x * grid.y <= di.sm_count && score_smem(c.d, R, nstage) <= (size_t)di.smem_optin ? nstage : 1;
   const size_t sm = score_smem(c.d, R, nbuf);
-  cudaError_t e = allow_smem(scores_ref_kernel<T, R>, sm);
+  cudaError_t e = opt_in_scores<T, R>(dev, sm);
   if (e != cudaSuccess) return e;
   return dam_launch_chained(scores_ref_kernel<T, R>, grid, dim3(kRefWarps * 32), sm, st, c.blob, (const T*)Q, (const T*)K, c.Hq,
                             c.Hq / c.Hkv, c.d, s->q_stride_tok, s->q_stride_head, s->k_stride_tok, s->k_stride_head, c.scale,
@@ -389,12 +409,16 @@ cudaError_t launch_scores(const void* Q, const void* K, const dam_shape_t* s, co
 
 template <typename T, int R, int ND>
 cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
-                        float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int smem_max, cudaStream_t st) {
+                        float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int dev, int smem_max, cudaStream_t st) {
   const bool pipe = sizeof(T) == 4 && attn_smem(s->head_dim, R, 2) <= (size_t)smem_max;
   const size_t sm = attn_smem(s->head_dim, R, pipe ? 2 : 1);
   auto kernel = attn_ref_kernel<T, R, ND, false>;
-  if constexpr (sizeof(T) == 4) { if (pipe) kernel = attn_ref_kernel<T, R, ND, true>; }
-  cudaError_t e = allow_smem(kernel, sm);
+  cudaError_t e;
+  if (sizeof(T) == 4 && pipe) {
+    if constexpr (sizeof(T) == 4) { kernel = attn_ref_kernel<T, R, ND, true>; e = opt_in_attn<T, R, ND, true>(dev, sm); }
+  } else {
+    e = opt_in_attn<T, R, ND, false>(dev, sm);
+  }
   if (e != cudaSuccess) return e;
   const dim3 grid(rows, DAM_TILE / (kRefWarps * R));
   // (an ordinary launch: as a link of the chain its blocks are placed while the ordering kernel still holds SMs, several to
@@ -408,11 +432,11 @@ cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void*
 
 template <typename T, int R>
 cudaError_t launch_attn_dims(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
-                             float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int smem_max, cudaStream_t st) {
+                             float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int dev, int smem_max, cudaStream_t st) {
   const int nd = (s->head_dim + 31) / 32;
-  if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, smem_max, st);
-  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, smem_max, st);
-  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, smem_max, st);
+  if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
+  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
+  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
 }
 
 }  // namespace
@@ -426,8 +450,8 @@ cudaError_t dam_launch_scores_ref(const void* Q, const void* K, const dam_shape_
   if (e != cudaSuccess) return e;
   const bool four = four_rows((long long)c.max_L * c.num_seqs * c.Hq, di.sm_count);
   if (c.dtype == DAM_F32)
-    return four ? launch_scores<float, 4>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st) : launch_scores<float, 1>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st);
-  return four ? launch_scores<__nv_bfloat16, 4>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st) : launch_scores<__nv_bfloat16, 1>(Q, K, s, c, dump, di.sm_count, di.smem_optin, st);
+    return four ? launch_scores<float, 4>(Q, K, s, c, dump, dev, di, st) : launch_scores<float, 1>(Q, K, s, c, dump, dev, di, st);
+  return four ? launch_scores<__nv_bfloat16, 4>(Q, K, s, c, dump, dev, di, st) : launch_scores<__nv_bfloat16, 1>(Q, K, s, c, dump, dev, di, st);
 }
 
 cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s,
@@ -447,8 +471,8 @@ cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, con
   if (e != cudaSuccess) return e;
   const bool four = four_rows((long long)rows * DAM_TILE, di.sm_count);
   if (s->dtype == DAM_F32)
-    return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st)
-                : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st);
-  return four ? launch_attn_dims<__nv_bfloat16, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st)
-              : launch_attn_dims<__nv_bfloat16, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, di.smem_optin, st);
+    return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st)
+                : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st);
+  return four ? launch_attn_dims<__nv_bfloat16, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st)
+              : launch_attn_dims<__nv_bfloat16, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st);
 }

@@ -283,6 +283,39 @@ def test_empty_batch_clears_the_status_block(dtype, ranges):
     assert B.dam_poll_status(scratch) == 0 and not scratch.any()
 
 
+def test_threads_with_different_shared_memory_sizes():
+    """Threads on streams of their own whose calls share a kernel instance but not the amount of shared memory it is
+    launched with (fp32: head_dim 136 and 160 for the attention, windows of one and six stages for the scores)."""
+    import threading
+    failures = []
+
+    def work(d, S):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            w = synth.small_case(S, 2, 1, d, S, seed=6, dtype=torch.float32)
+            shape = _shape(w)
+            rule = B.make_rule(S, 0.1, 0.8)
+            Q, K, V = w.Q.to(DEV), w.K.to(DEV), w.V.to(DEV)
+            blob, build = B.dam_build_masks(Q, K, shape, rule)
+            O, lse, scratch = B.dam_sparse_attention(Q, K, V, blob, shape)
+            first = O.clone()
+            try:
+                for _ in range(1500):
+                    B.dam_build_masks(Q, K, shape, rule, blob, build)
+                    B.dam_sparse_attention(Q, K, V, blob, shape, O=O, lse=lse, scratch=scratch)
+                stream.synchronize()
+                assert torch.equal(O, first)
+            except Exception as e:                           # (an assertion in a thread would be lost)
+                failures.append((d, S, repr(e)))
+
+    threads = [threading.Thread(target=work, args=a) for a in ((160, 64), (136, 64), (160, 384), (136, 384))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures
+
+
 def test_bounded_wait_times_out_cleanly():
     """A wait that nothing satisfies gives up after its limit, the status word says so, and the device keeps
     working (the next kernel runs and is correct)."""
