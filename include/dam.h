@@ -241,9 +241,11 @@ dam_status_t dam_capture_average(const float* A, const int32_t* C, int32_t pcl_m
  * Work is dealt in pairs of 128-row query blocks, so every begin must be a multiple of 256 and every end a
  * multiple of 256 or the sequence length (INVALID_ARGUMENT otherwise); an empty range skips the sequence.
  *   row_ranges_host : HOST, int32[2 * num_seqs] (validated);  row_ranges_dev : DEVICE, the same values (not NULL, but
- *   not read for batches of up to 16 sequences, whose ranges travel with the launch).
+ *   not read for batches of up to DAM_ROW_RANGES_BY_VALUE sequences, whose ranges travel with the launch: a captured
+ *   call keeps the ranges it was captured with).
  * Everything else as dam_sparse_attention.
  */
+#define DAM_ROW_RANGES_BY_VALUE 16
 dam_status_t dam_sparse_attention_rows(const void* Q, const void* K, const void* V, const void* mask,
                                        const dam_shape_t* shape, int32_t causal, int32_t gqa_group,
                                        float softmax_scale, void* O, float* lse,

@@ -159,6 +159,7 @@ def make_shape(cu_seqlens: Sequence[int], Hq: int, Hkv: int, d: int, dtype: torc
 
 
 DAM_RULE_GATHER_COLUMNS = 1
+DAM_ROW_RANGES_BY_VALUE = 16
 
 
 def make_rule(pcl_max: int, tau: float, mu: float, lam: float = 0.5, eps: float = 1e-8,
@@ -290,9 +291,9 @@ def dam_sparse_attention_rows(Q, K, V, mask, shape: Shape, row_ranges, O: torch.
     flat = [int(x) for pair in row_ranges for x in pair]
     assert len(flat) == 2 * shape.c.num_seqs
     host = (ctypes.c_int32 * len(flat))(*flat)
-    # up to 16 sequences the library hands the ranges to the kernel itself; beyond, a copy on the device, queued without
+    # so many sequences' ranges the library hands to the kernel itself; beyond, a copy on the device, queued without
     # waiting for the stream (CUDA has taken its own copy of a small pageable source when the call returns)
-    if shape.c.num_seqs <= 16:
+    if shape.c.num_seqs <= DAM_ROW_RANGES_BY_VALUE:
         dev = shape.c.cu_seqlens_dev
     else:
         dev_copy = torch.tensor(flat, dtype=torch.int32).to(Q.device, non_blocking=True)

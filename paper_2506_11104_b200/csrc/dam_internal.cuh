@@ -276,7 +276,7 @@ __device__ __forceinline__ uint4 dam_apply_bits(const DamHeadBits& hb, uint32_t 
 }
 
 // Row ranges of a chunked call, handed to the kernel by value for batches of a few sequences (n = 0: read from memory).
-constexpr int kRangeSeqs = 16;
+constexpr int kRangeSeqs = DAM_ROW_RANGES_BY_VALUE;
 struct DamRowRanges {
   int n;
   int2 r[kRangeSeqs];

@@ -28,6 +28,12 @@ def test_exports_match_header():
         assert hasattr(lib, name), name
 
 
+def test_constants_match_header():
+    text = open(os.path.join(ROOT, "include", "dam.h")).read()
+    for name in ("DAM_RULE_GATHER_COLUMNS", "DAM_ROW_RANGES_BY_VALUE"):
+        assert int(re.search(r"#define %s (\d+)u?\b" % name, text).group(1)) == getattr(B, name)
+
+
 def test_version_and_status_strings():
     assert B.dam_version() >= 1000
     assert B.dam_status_string(0) == "ok"
