@@ -296,6 +296,9 @@ def dam_sparse_attention_rows(Q, K, V, mask, shape: Shape, row_ranges, O: torch.
     if shape.c.num_seqs <= DAM_ROW_RANGES_BY_VALUE:
         dev = shape.c.cu_seqlens_dev
     else:
+        with torch.cuda.device(Q.device):
+            if torch.cuda.is_current_stream_capturing():     # (a replay would copy from host memory that is long gone)
+                raise RuntimeError("the row ranges of more than %d sequences cannot be captured" % DAM_ROW_RANGES_BY_VALUE)
         dev_copy = torch.tensor(flat, dtype=torch.int32).to(Q.device, non_blocking=True)
         dev = dev_copy.data_ptr()
     if scratch is None:

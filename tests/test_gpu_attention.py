@@ -425,6 +425,37 @@ def test_row_ranges_of_long_lists_and_many_sequences(lengths, Hq, ranges):
     assert (O[~inside] == 7.0).all() and (lse[:, ~inside] == 7.0).all()
 
 
+def test_row_ranges_under_stream_capture():
+    """Ranges that travel with the launch are captured with it; a batch whose ranges would be copied from host memory at
+    every replay is refused, and the capture around the refused call stays valid."""
+    def case(n):
+        torch.manual_seed(31)
+        Q = torch.randn(300 * n, 2, 64, dtype=torch.bfloat16, device=DEV)
+        K, V = (torch.randn(300 * n, 1, 64, dtype=torch.bfloat16, device=DEV) for _ in range(2))
+        shape = B.make_shape([300 * b for b in range(n + 1)], 2, 1, 64, torch.bfloat16, DEV)
+        rule = B.make_rule(64, 0.1, 0.5, gather_columns=True)
+        blob, _ = B.dam_build_masks(Q, K, shape, rule)
+        scratch = torch.zeros(B.dam_mask_sizes(shape, rule)[2], dtype=torch.uint8, device=DEV)
+        return Q, K, V, blob, shape, [(256, 300)] * n, torch.zeros_like(Q), torch.zeros(2, 300 * n, device=DEV), scratch
+
+    few, many = case(16), case(17)
+    B.dam_sparse_attention_rows(*many[:8], scratch=many[8])                   # (a first call outside of the capture)
+    B.dam_sparse_attention_rows(*few[:8], scratch=few[8])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.dam_sparse_attention_rows(*few[:8], scratch=few[8])
+        with pytest.raises(RuntimeError):
+            B.dam_sparse_attention_rows(*many[:8], scratch=many[8])
+    few[0].neg_()
+    want = few[6].clone()
+    B.dam_sparse_attention_rows(*few[:6], want, few[7], scratch=few[8])
+    few[6].zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    inside = (torch.arange(300 * 16, device=DEV) % 300) >= 256
+    assert torch.equal(few[6][inside], want[inside]) and not few[6][~inside].any() and want[inside].any()
+
+
 def test_row_ranges_leave_other_rows_alone_and_reject_odd_bounds():
     w = synth.small_case(0, 4, 2, 128, 128, seed=22, dtype=torch.bfloat16, lengths=[768, 512])
     shape = _shape(w)
