@@ -1040,14 +1040,18 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
       !dam_make_tmap_bf16(&tv, V, d, s->num_kv_heads, s->total_tokens, s->v_stride_tok, s->v_stride_head))
     return cudaErrorInvalidValue;
   const DamRowRanges rows(ranges ? ranges_host : nullptr, s->num_seqs);
-  int pairs = 0;                                         // (of the row ranges: whole pairs, as the caller has checked)
+  int pairs = 0, all = 0;                                // (of the row ranges: whole pairs, as the caller has checked)
   for (int b = 0; b < s->num_seqs; ++b) {
     const int S = s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b];
     const int r0 = ranges ? ranges_host[2 * b] : 0, r1 = ranges ? ranges_host[2 * b + 1] : S;
     pairs += (r1 - r0 + 2 * DAM_TILE - 1) / (2 * DAM_TILE);
+    all += (S + 2 * DAM_TILE - 1) / (2 * DAM_TILE);
   }
-  pairs *= s->num_q_heads;
+  pairs *= s->num_q_heads; all *= s->num_q_heads;
   if (pairs == 0) return cudaSuccess;
+  // a CTA for every pair to compute, but where the list is too long to be marked the CTAs walk all of it, and the walk is
+  // what takes the time: 256 rows of 204800 tokens, 32 pairs of 25600, 32 CTAs 565 us, 148 CTAs 134
+  if (all > 32 * kRowBitWords) pairs = all;
   AttnParams p;
   p.blob = reinterpret_cast<const unsigned char*>(blob);
   p.O = reinterpret_cast<__nv_bfloat16*>(O);
