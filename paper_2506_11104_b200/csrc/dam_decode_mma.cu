@@ -393,15 +393,25 @@ decode_group_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __
 }
 
 // Blocks per (sequence, KV head), from the number of those pairs: a block spends about 6 us before its first rows arrive
-// and then streams its list, so splitting the list pays as long as all blocks are resident at once (four per SM) and the
-// chip is not yet bound by the gather itself.  us per launch with 1 / 2 / 4 / 8 blocks (32 / 8 heads, 148 SMs):
-//   pairs    8   19.2 / 15.7 / 12.1 / 11.0      32   28.3 / 20.0 / 14.8 / 13.4      64   28.8 / 20.5 / 16.5 / 16.4
-//          128   30.0 / 22.6 / 20.0 / 28.0     192   32.6 / 25.3 / 31.6 / 39.0     384   44.9 / 38.3 / 41.9 / 63.9
-//          512   41.6 / 49.7 / 61.7 / 92.3 (longer lists)
+// and then streams its list, so splitting the list pays as long as all blocks are resident at once (four per SM); a second
+// round of blocks costs more than the split gains, the more the longer the lists.  Clusters of two fill the chip (296 on 148
+// SMs), of four not quite (142: the SMs of a GPC are not a multiple), of eight 71.  us a call, calls back to back, with
+// 1 / 2 / 4 / 8 blocks (32 / 8 heads, head_dim 128, 148 SMs):
+//   window    512                          2048                         8192
+//   pairs   8   15.1 / 12.5 / 10.6 /  9.8    25.9 / 17.8 / 13.2 / 10.6    35.7 / 26.9 / 22.1 / 19.1
+//          32   16.7 / 13.3 / 12.0 / 11.4    28.4 / 19.5 / 14.9 / 12.6    37.3 / 28.4 / 24.5 / 21.8
+//         128   18.7 / 16.5 / 14.4 / 22.8    31.5 / 23.4 / 18.3 / 26.4    42.7 / 33.8 / 27.8 / 43.9
+//         140   18.6 / 16.1 / 14.8 / 26.8    31.8 / 23.0 / 18.8 / 29.5    42.8 / 33.5 / 29.9 / 52.7
+//         144   18.6 / 15.9 / 21.3 / 29.5    31.8 / 22.9 / 25.6 / 32.3    42.0 / 32.9 / 44.8 / 59.3
+//         296   30.6 / 23.9 / 33.2 / 50.7    33.9 / 28.9 / 40.6 / 57.3    43.0 / 38.5 / 70.6 /  102
+//         320   31.1 / 26.9 / 34.3 /  -      37.0 / 39.0 / 42.8 /  -      47.8 / 60.7 / 73.0 /  -
+//         440   32.9 / 35.6 / 44.7 /  -      38.9 / 46.8 / 54.7 /  -      50.8 / 68.7 / 96.2 /  -
+// The split deals the chunks to other warps, so that O differs in the last bits of P's rounding; against float64 it is no
+// further off (relative error of O 1.749e-3, one block 1.771e-3, for one sequence of 8000 tokens and a window of 1024).
 int decode_split(int pairs, int sm_count) {
   if (pairs * 8 <= 3 * sm_count) return 8;
-  if (pairs <= sm_count) return 4;
-  if (pairs <= 3 * sm_count) return 2;
+  if (pairs * 16 <= 15 * sm_count) return 4;
+  if (pairs <= 2 * sm_count) return 2;
   return 1;
 }
 

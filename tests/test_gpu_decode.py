@@ -86,7 +86,8 @@ def test_decode_matches_oracle(cache_lengths, build_lengths, Hq, Hkv, d, dtype, 
         _decode_and_check(w, blob, masks, [p[min(k, len(p) - 1)] for p in per_seq])
 
 
-@pytest.mark.parametrize("num_seqs,d", [(55, 64), (56, 128), (148, 64), (149, 64), (444, 64), (445, 64)])
+@pytest.mark.parametrize("num_seqs,d", [(55, 64), (56, 128), (148, 64), (149, 64), (444, 64), (445, 64),
+                                        (138, 128), (139, 64), (296, 64), (297, 64)])
 def test_decode_split_over_blocks(num_seqs, d):
     """Enough (sequence, KV head) pairs for 8, 4, 2 and 1 blocks each (both sides of every boundary on 148 SMs), with key
     lists from empty to longer than one chunk per warp."""
