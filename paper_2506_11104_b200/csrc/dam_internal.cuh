@@ -97,15 +97,19 @@ struct DamSeq {
 static_assert(sizeof(DamSeq) == 80, "DamSeq must be 80 bytes");
 
 // The layout a build call works on, handed to its kernels by value: the header as the host computed it and, for batches
-// of a few sequences, their records too.  The rule kernels are short and follow one another; every dependent read of the
-// header and of the sequence table in the blob costs each of them most of a microsecond.
-constexpr int kDamTabSeqs = 6;
+// of up to 32 sequences, their records too.  The rule kernels are short and follow one another; every dependent read of the
+// header and of the sequence table in the blob costs each of them most of a microsecond.  32 records are what 4 KB of launch
+// parameters hold beside the tensor maps (rounded down to a power of two); unused ones cost nothing (one sequence of 8192
+// tokens, room for 6 / 16 / 32: 40.2 / 40.2 / 40.2 us of stage 1), used ones save up to a microsecond or two (8 x 8000
+// tokens, 6 or 16: 171.2 / 170.3 us; 32 x 1000, 16 or 32: 219.7 / 218.1).
+constexpr int kDamTabSeqs = 32;
 struct DamPlan {
   DamHeader h;
   int32_t nseq;            // sequences in seq[], 0: more than fit (the records are read from the blob)
   int32_t nkeys;           // work items have fewer than this many listed tiles (or DAM_HIST - 1 of them and more)
   DamSeq seq[kDamTabSeqs];
 };
+static_assert(sizeof(DamPlan) <= 4096 - 1024, "the plan travels in the launch parameters");
 __device__ __forceinline__ DamSeq dam_plan_seq(const DamPlan& p, const unsigned char* blob, int b) {
   return p.nseq ? p.seq[b] : reinterpret_cast<const DamSeq*>(blob + p.h.off_seq)[b];
 }

@@ -345,9 +345,10 @@ def test_multi_sample_capture_masks_bit_exact():
 
 
 @pytest.mark.parametrize("gather", GATHER)
-@pytest.mark.parametrize("lengths", [[300, 0, 129, 1, 0, 700], [0, 300, 129, 0, 1, 700, 513], [40] * 9])
+@pytest.mark.parametrize("lengths", [[300, 0, 129, 1, 0, 700], [0, 300, 129, 0, 1, 700, 513], [40] * 9,
+                                     [150, 0, 1, 257] * 8, [40] * 32 + [130]])
 def test_more_sequences_than_the_record_table_holds(lengths, gather):
-    """Six sequences (their records travel with the launches) and more (read from the blob), empty ones among them."""
+    """Up to 32 sequences (their records travel with the launches) and more (read from the blob), empty ones among them."""
     w = synth.small_case(0, 4, 2, 64, 160, seed=60, dtype=torch.bfloat16, lengths=lengths)
     shape, rule = _shape(w), _rule(w, gather_columns=gather)
     dump = torch.zeros(sum(4 * min(S, 160) ** 2 for S in lengths), dtype=torch.float32, device=DEV)
