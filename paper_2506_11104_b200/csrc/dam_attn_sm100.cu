@@ -877,6 +877,19 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
+// The n-th matched column of a head, counted off its pattern words (0xFFFF: it has no more), for the blobs of an earlier
+// build, which have no list.  Out of line: the hot path is a short chain of loads.
+__device__ __noinline__ int nth_column(const unsigned char* dv, const DamSeq& sq, int h, int n) {
+  const uint32_t* Vw = reinterpret_cast<const uint32_t*>(dv) + sq.dv_off + (uint64_t)h * 3 * sq.W + 2 * sq.W;
+  for (int w = 0; w < sq.W; ++w) {
+    const uint32_t word = __ldg(Vw + w);
+    const int c = __popc(word);
+    if (n < c) return 32 * w + (int)__fns(word, 0, n + 1);
+    n -= c;
+  }
+  return 0xFFFF;
+}
+
 // Copies the K and V rows of the matched columns of every (sequence, head) into dense tiles of 128 keys in
 // the scratch buffer (K tile at rows (2T) * 128, V tile at rows (2T + 1) * 128 of a [rows][head_dim] bf16 array;
 // T = gath_off + head * nL + g).  Rows past the last matched column are zero.  One block per tile, grid-stride.
@@ -904,17 +917,20 @@ gather_columns_kernel(const unsigned char* __restrict__ blob, const __nv_bfloat1
   }
   __shared__ int col[DAM_TILE];
   uint4* out = reinterpret_cast<uint4*>(scratch + 256);
-  const unsigned short* cols = reinterpret_cast<const unsigned short*>(blob + H->off_cols);
+  const bool cols_missing = H->off_cols == 0;
+  // (without a list: words of the tiles' own memory, twice 128 rows of head_dim per tile, which are not used)
+  const unsigned short* cols = reinterpret_cast<const unsigned short*>(cols_missing ? scratch + 256 : blob + H->off_cols);
   const DamSeq* seqs = reinterpret_cast<const DamSeq*>(blob + H->off_seq);
   const int tid = threadIdx.x;
   for (long long T = blockIdx.x; T < (long long)H->gath_tiles; T += gridDim.x) {
-    const int c_mine = tid < DAM_TILE ? __ldg(cols + T * DAM_TILE + tid) : 0;
+    int c_mine = tid < DAM_TILE ? __ldg(cols + T * DAM_TILE + tid) : 0;
     int b = 0;
     while (b + 1 < H->num_seqs && (long long)seqs[b + 1].gath_off <= T) ++b;
     const DamSeq sq = seqs[b];
     if (sq.nL == 0) continue;
     const int h = (int)((T - (long long)sq.gath_off) / sq.nL), g = (int)((T - (long long)sq.gath_off) % sq.nL);
     if (h >= Hq) continue;
+    if (cols_missing) c_mine = nth_column(blob + H->off_dv, sq, h, g * DAM_TILE + tid);
     __syncthreads();
     if (tid < DAM_TILE) col[tid] = c_mine == 0xFFFF ? -1 : c_mine;
     __syncthreads();

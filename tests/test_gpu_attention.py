@@ -191,6 +191,34 @@ def test_lone_diagonal_at_any_distance(L, d, gather):
     assert left_out > 0 and st["executed_tiles"] == st["tiles"] - left_out
 
 
+@pytest.mark.parametrize("d", [128, 64])
+def test_gathered_blob_of_an_earlier_build(d):
+    """A blob whose header has neither the list of matched columns nor the records of lone diagonals (both offsets zero, as
+    in a blob that was saved before these sections existed), and one with the older records where they used to be."""
+    w = synth.small_case(0, 4, 2, d, 300, seed=8, dtype=torch.bfloat16, lengths=[1500, 900])
+    shape = _shape(w)
+    dump = torch.zeros(2 * 4 * 300 * 300, device=DEV)
+    blob, _ = B.dam_build_masks(w.Q.to(DEV), w.K.to(DEV), shape, B.make_rule(w.pcl_max, w.tau, w.mu, gather_columns=True), scores_dump=dump)
+    masks = H.oracle_masks_from_dump(w, dump.cpu().numpy())
+    assert any(m.V.sum() > 0 for seq in masks for m in seq)
+    O, lse = _run(w, blob, shape)
+
+    def word(name, value=None):
+        at = B._HDR.fields[name][1]
+        if value is not None:
+            blob[at:at + 8] = torch.from_numpy(np.array([value], np.uint64).view(np.uint8)).to(DEV)
+        return int(blob[at:at + 8].cpu().numpy().view(np.uint64)[0])
+
+    lone = word("off_lone")
+    word("off_lone", 0)
+    word("off_lone2", lone)
+    _check(w, *_run(w, blob, shape, sentinel=True), masks, _all_rows)
+    word("off_lone2", 0)
+    word("off_cols", 0)
+    O_old, lse_old = _run(w, blob, shape, sentinel=True)
+    _check(w, O_old, lse_old, masks, _all_rows)
+
+
 def test_empty_rows_and_no_patterns():
     """mu > 1: nothing matches, every row below the window is empty."""
     w = synth.small_case(0, 4, 2, 128, 128, seed=5, lengths=[600])
