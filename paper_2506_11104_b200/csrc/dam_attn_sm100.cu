@@ -772,11 +772,12 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           for (int q = 0; q < w; ++q) v[q] = (lane & w) ? v[q + w] : v[q];
         const float y = row_valid ? __uint_as_float(v[0]) * prm.scale_log2 : -CUDART_INF_F;
         float alpha = 1.f;
-        if (y - m_ref > kRescaleThreshold) {                 // (-inf reference: inf > 8, unless y is -inf too: NaN)
+        if (y - m_ref > kRescaleThreshold) {                 // (-inf reference: inf > 8; NaN when y is -inf too)
           alpha = (m_ref == -CUDART_INF_F) ? 0.f : ex2(m_ref - y);
           m_ref = y;
         }
-        const float p = row_valid ? ex2(y - m_ref) : 0.f;
+        // (as in the sweeps: an infinite reference counts as zero, so that a logit of -inf gives zero and not a NaN)
+        const float p = row_valid ? ex2(y - (m_ref == -CUDART_INF_F ? 0.f : m_ref)) : 0.f;
         l = l * alpha + p;
         const __nv_bfloat16 pb = __float2bfloat16_rn(p);
         const uint32_t pw = (uint32_t)*reinterpret_cast<const unsigned short*>(&pb) << (16 * (lane & 1));

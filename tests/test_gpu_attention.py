@@ -219,6 +219,38 @@ def test_gathered_blob_of_an_earlier_build(d):
     _check(w, O_old, lse_old, masks, _all_rows)
 
 
+@pytest.mark.parametrize("gather", [False, True])
+def test_lone_diagonal_with_logits_of_minus_infinity(gather):
+    """Rows whose key on the lone diagonal has a logit that overflows to -inf, alone (head 0: O = 0 and LSE = -inf) and
+    beside a key of a column (head 1): as without the record of the lone diagonal, and the rows beside them as ever."""
+    L, S, r = 512, 1500, 300
+    i = np.arange(L)
+    maps = np.zeros((2, L, L), np.float32)
+    maps[:, i[r:], i[:L - r]] = 0.5
+    maps[1, :, 0] = 0.5
+    torch.manual_seed(37)
+    Q, K, V = (torch.randn(S, h, 64, device=DEV).to(torch.bfloat16) for h in (2, 1, 1))
+    Q[:, :, 0] = 1e30
+    K[:, 0, 0] = 0.0
+    K[3::3, 0, 0] = -1e30                                                   # product below the smallest float
+    shape = B.make_shape([0, S], 2, 1, 64, torch.bfloat16, DEV)
+    blob, _ = B.dam_build_masks_from_scores(torch.from_numpy(maps).to(DEV), shape, B.make_rule(L, 0.1, 0.8, gather_columns=gather))
+    O, lse, _ = B.dam_sparse_attention(Q, K, V, blob, shape)
+    at = B._HDR.fields["off_lone"][1]
+    blob[at:at + 8] = 0
+    O_plain, lse_plain, _ = B.dam_sparse_attention(Q, K, V, blob, shape)
+    first = 1024 if gather else 896                                         # the blocks the diagonal is served on
+    rows = torch.arange(first, S, device=DEV)
+    overflown = (rows - r) % 3 == 0
+    assert not torch.isnan(O).any() and not torch.isnan(lse).any()
+    assert torch.equal(torch.isneginf(lse[0, first:]), overflown) and torch.equal(torch.isneginf(lse_plain[0, first:]), overflown)
+    assert (O[first:, 0][overflown] == 0).all()
+    # (one key: O is its V row either way, and LSE the logit)
+    fin = rows[~overflown]
+    assert torch.equal(O[fin, 0], O_plain[fin, 0]) and (lse[0, fin] - lse_plain[0, fin]).abs().max() <= TOL[torch.bfloat16][2]
+    assert (O[:, 1].float() - O_plain[:, 1].float()).abs().max() <= 2e-2 and (lse[1] - lse_plain[1]).abs().max() <= 1e-3
+
+
 def test_empty_rows_and_no_patterns():
     """mu > 1: nothing matches, every row below the window is empty."""
     w = synth.small_case(0, 4, 2, 128, 128, seed=5, lengths=[600])
