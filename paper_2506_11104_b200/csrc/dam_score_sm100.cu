@@ -261,7 +261,8 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           }
           m = mn; l = ls;
           inv_l = l > 0.f ? 1.0f / l : 0.f;
-          thr_raw = (log2f(prm.pstar * l) + m) / prm.scale_log2;              // the raw dot product at which p = p*
+          // the raw dot product at which p = p* (below 2^-126 the exponential is zero, and so is p)
+          thr_raw = (fmaxf(log2f(prm.pstar * l), -126.f) + m) / prm.scale_log2;
           margin = (0.000244140625f + fabsf(m) * 7.62939453125e-6f) / prm.scale_log2;      // 2^-12 + |m| 2^-17
         }
         if ((g & 3u) != (uint32_t)G) continue;

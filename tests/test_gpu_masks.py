@@ -147,6 +147,26 @@ def _build_and_check(w, qblocks=None, gather=False):
     return blob, shape, masks, dump
 
 
+@pytest.mark.parametrize("d", [128, 64])
+def test_tiny_threshold_without_a_dump(d):
+    """p* far below the smallest normal float: probabilities whose exponential is flushed to zero stay inactive, whether or
+    not the map is written out (the decisions are those on the written map)."""
+    torch.manual_seed(41)
+    L, Hq = 300, 2
+    Q, K = ((torch.randn(L, h, d, device=DEV) * 7).to(torch.bfloat16) for h in (Hq, 1))
+    shape = B.make_shape([0, L], Hq, 1, d, torch.bfloat16, DEV)
+    rule = B.make_rule(L, 1e-42, 0.8, eps=1e-44, transform="average")
+    dump = torch.zeros(Hq * L * L, device=DEV)
+    with_dump, _ = B.dam_build_masks(Q, K, shape, rule, scores_dump=dump)
+    without, _ = B.dam_build_masks(Q, K, shape, rule)
+    active = (dump.view(Hq, L, L) > 0).cpu().numpy()
+    below = np.tril(np.ones((L, L), bool))
+    assert 0.1 < active[:, below].mean() < 0.9                # both sides of the flush are met
+    a, b = B.MaskBlob(with_dump), B.MaskBlob(without)
+    for h in range(Hq):
+        assert np.array_equal(a.true_mask(0, h), b.true_mask(0, h)), h
+
+
 def _score_closeness(w, dump, masks, heads):
     """GPU fp32 map vs the float64 map; every cell whose decision differs must sit within 2 % of p*."""
     Q, K, _ = H.host_qkv(w)
