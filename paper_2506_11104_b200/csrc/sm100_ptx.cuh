@@ -43,22 +43,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: gives up after `limit_ns` of wall time (checked every 256 polls), records the fact
-// in *abort_flag (shared memory, also polled so that one expired wait releases every other waiter)
-// and returns false.  No wait in these kernels can spin forever.
+// Bounded wait: gives up after `limit_ns` of wall time, records the fact in *abort_flag (shared memory, also polled so that
+// one expired wait releases every other waiter) and returns false.  No wait in these kernels can spin forever.  The poll loop
+// is short: it is inlined wherever a role waits, and the attention kernel's code is larger than the instruction cache (70 KB
+// with a loop that looked at the clock every 256 polls, 64 now: 8192 tokens 100.3 -> 98.5 us of attention, 32768 tokens 391.8 ->
+// 388.8, head_dim 64 127.8 -> 126.5).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                           uint64_t limit_ns = 2000000000ull) {
   if (mbar_try_wait(bar, parity)) return true;
-  uint64_t t0 = 0;
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255u) == 0) {
-      if (*abort_flag) return false;
-      uint64_t now = globaltimer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) { *abort_flag = 1u; return false; }
-    }
+  const uint64_t t0 = globaltimer_ns();
+#pragma unroll 1
+  while (!mbar_try_wait(bar, parity)) {
+    if (globaltimer_ns() - t0 > limit_ns) *abort_flag = 1u;
+    if (*abort_flag) return false;
   }
+  return true;
 }
 
 // ---- TMA ----------------------------------------------------------------------------------------
