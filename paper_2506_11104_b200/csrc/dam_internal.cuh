@@ -259,13 +259,13 @@ __device__ __forceinline__ uint4 dam_tile_row_bits(const DamHeadBits& hb, int i,
 
 // ones for t in [0, n), n clipped to [0, 128]
 __device__ __forceinline__ uint4 dam_low_ones128(int n) {
-  uint4 r;
-  auto w = [](int k) -> uint32_t { return k >= 32 ? 0xFFFFFFFFu : (k <= 0 ? 0u : ((1u << k) - 1u)); };
-  r.x = w(n);
-  r.y = w(n - 32);
-  r.z = w(n - 64);
-  r.w = w(n - 96);
-  return r;
+  // (the PTX shift gives zero for a count of 32 and more, and zero minus one is all ones)
+  auto w = [](int k) -> uint32_t {
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(max(k, 0)));
+    return r - 1u;
+  };
+  return make_uint4(w(n), w(n - 32), w(n - 64), w(n - 96));
 }
 
 // Final 128 bits the attention kernels apply for row i against tile kb.  The bits of a PARTIAL tile have no key beyond

@@ -412,6 +412,30 @@ def test_strided_qkv_views():
         _check(w, O, lse, masks, _all_rows)
 
 
+@pytest.mark.parametrize("offset,row_pad,head_pad", [(0, 8, 0), (8, 0, 0), (0, 0, 8), (16, 32, 16)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_output_rows_of_any_alignment(d, offset, row_pad, head_pad):
+    """O is written 32 bytes at a time where its rows start on 32-byte boundaries, 16 bytes otherwise: the same values
+    either way, and nothing between the rows."""
+    Hq, Hkv = 4, 2
+    w = synth.small_case(0, Hq, Hkv, d, 128, seed=13, lengths=[700, 131])
+    Q, K, V = w.Q.to(DEV), w.K.to(DEV), w.V.to(DEV)
+    rule = B.make_rule(w.pcl_max, w.tau, w.mu, gather_columns=True)
+    shape = _shape(w)
+    blob, _ = B.dam_build_masks(Q, K, shape, rule)
+    O_ref, lse_ref = _run(w, blob, shape, sentinel=True)
+    T, hs = Q.shape[0], d + head_pad
+    ts = Hq * hs + row_pad
+    buf = torch.full((offset + T * ts,), 7.0, dtype=torch.bfloat16, device=DEV)
+    O = buf[offset:].as_strided((T, Hq, d), (ts, hs, 1))
+    padded = B.make_shape(w.cu_seqlens, Hq, Hkv, d, torch.bfloat16, DEV, o_strides=(ts, hs))
+    _, lse, scr = B.dam_sparse_attention(Q, K, V, blob, padded, O=O)
+    assert B.dam_poll_status(scr) == 0 and B.attention_ran_on_tensor_cores(scr)
+    assert torch.equal(O, O_ref) and torch.equal(lse, lse_ref)
+    O.fill_(7.0)
+    assert (buf == 7.0).all()
+
+
 @pytest.mark.parametrize("gather", [False, True])
 def test_degenerate_lengths(gather):
     """Empty and one-token sequences inside a packed batch, a sequence shorter than a tile, MHA (group 1)."""
