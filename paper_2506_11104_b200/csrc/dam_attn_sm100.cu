@@ -203,20 +203,28 @@ __device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1, f
 
 // 2^y for a pair of values on the FMA / ALU pipes instead of the special-function unit: split y into its
 // nearest integer (added to the exponent field) and a remainder in [-0.5, 0.5] (degree-3 minimax polynomial,
-// relative error 7.6e-5, far below the bf16 rounding of P).  y is clamped at -125 so that the exponent stays
-// in range; that turns an underflowing probability into 2^-125 instead of 0.
-__device__ __forceinline__ void ex2_poly2(float y0, float y1, float& p0, float& p1) {
-  const float kMagic = 12582912.f;    // 1.5 * 2^23: adding it leaves round(y) in the low mantissa bits
-  y0 = fmaxf(y0, -125.f); y1 = fmaxf(y1, -125.f);
+// relative error 7.6e-5, far below the bf16 rounding of P).  y comes as z = (y + 125) / 250, saturated to [0, 1] by the multiply-add
+// that makes it: so the exponent stays in range without a comparison (an underflowing probability is 2^-125 instead of 0).
+__device__ __forceinline__ void ex2_poly2(float z0, float z1, float& p0, float& p1) {
+  const float kMagic = 12582912.f - 125.f;    // 1.5 * 2^23 - 125: 250 z added to it leaves round(y) in the low mantissa bits
   float r0, r1, i0, i1, f0, f1, q0, q1;
-  add2(r0, r1, y0, y1, kMagic, kMagic);
-  add2(i0, i1, r0, r1, -kMagic, -kMagic);
-  add2(f0, f1, y0, y1, -i0, -i1);
+  fma2(r0, r1, z0, z1, 250.f, 250.f, kMagic, kMagic);
+  add2(i0, i1, r0, r1, -kMagic, -kMagic);     // round(y) + 125
+  fma2(f0, f1, z0, z1, 250.f, 250.f, -i0, -i1);
   fma2(q0, q1, f0, f1, 0.05520550534129143f, 0.05520550534129143f, 0.24261397123336792f, 0.24261397123336792f);
   fma2(q0, q1, q0, q1, f0, f1, 0.6932547688484192f, 0.6932547688484192f);
   fma2(q0, q1, q0, q1, f0, f1, 0.9999276995658875f, 0.9999276995658875f);
-  p0 = __int_as_float(__float_as_int(q0) + (__float_as_int(r0) << 23));
-  p1 = __int_as_float(__float_as_int(q1) + (__float_as_int(r1) << 23));
+  // (a multiply-add for shift and add; of the magic number nothing is left in the upper bits)
+  int b0, b1;
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(b0) : "r"(__float_as_int(r0)), "r"(__float_as_int(q0)));
+  asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(b1) : "r"(__float_as_int(r1)), "r"(__float_as_int(q1)));
+  p0 = __int_as_float(b0);
+  p1 = __int_as_float(b1);
+}
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {
+  float r;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
 
 // Sweep 1 over one S row held in TMEM (4 chunks of 32 columns, next chunk in flight while one is reduced).
@@ -274,23 +282,22 @@ __device__ __forceinline__ float sweep_max_masked(uint32_t tS, uint4 bits) {
 
 // 32 probabilities p = 2^(s * scale + neg_m), zero where the mask bit is clear, packed to bf16; their sums are taken in fp32,
 // before the bf16 rounding.  Of every 8, 6 go through the special-function unit and 2 through the polynomial.
-template <bool MASKED>
-__device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, float scale, float neg_m, uint32_t* pk,
+__device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, float scale, float neg_m, float scale_z, float neg_z, uint32_t* pk,
                                           float& s0, float& s1, float& s2, float& s3) {
 #pragma unroll
   for (int q = 0; q < 32; q += 8) {
     float y[8], p[8];
+    constexpr int kEx2 = 8 - kPolyPer8;
 #pragma unroll
-    for (int u = 0; u < 8; u += 2)
+    for (int u = 0; u < kEx2; u += 2)
       fma2(y[u], y[u + 1], __uint_as_float(cur[q + u]), __uint_as_float(cur[q + u + 1]), scale, scale, neg_m, neg_m);
 #pragma unroll
-    for (int u = 0; u < 8 - kPolyPer8; ++u) p[u] = ex2(y[u]);
-    if (kPolyPer8 >= 2) ex2_poly2(y[6], y[7], p[6], p[7]);
-    if (kPolyPer8 >= 4) ex2_poly2(y[4], y[5], p[4], p[5]);
-    if (MASKED) {
+    for (int u = 0; u < kEx2; ++u) p[u] = ex2(y[u]);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) p[u] = ((word >> (q + u)) & 1u) ? p[u] : 0.f;
-    }
+    for (int u = kEx2; u < 8; u += 2)
+      ex2_poly2(fma_sat(__uint_as_float(cur[q + u]), scale_z, neg_z), fma_sat(__uint_as_float(cur[q + u + 1]), scale_z, neg_z), p[u], p[u + 1]);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) p[u] = ((word >> (q + u)) & 1u) ? p[u] : 0.f;
     add2(s0, s1, s0, s1, p[0], p[1]);
     add2(s2, s3, s2, s3, p[2], p[3]);
     add2(s0, s1, s0, s1, p[4], p[5]);
@@ -308,21 +315,24 @@ __device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, fl
 // warp is zero.  Bound by the latency of its chains: a half is one block of straight code without votes or branches, so that
 // the arithmetic of one chunk runs under the exponentials of the other.  With a vote per chunk of 32 columns, to skip
 // the inactive ones, a masked tile took 1584 cycles in a warp alone on its scheduler and 2334 beside another, now 1230 and
-// 1988, about what an unmasked one takes (attention: 1237 tokens 28.3 -> 26.6 us, 8192 tokens 98.3 -> 96.3, 32768 tokens 389 -> 379).
-template <bool MASKED>
+// 1988; an unmasked one takes 1190 and 1940.  So tiles that are active throughout go the same way: a copy without the selects is
+// 4 KB of code that the other roles' has to share the instruction cache with (8192 tokens 87.2 -> 83.8 us, 32768 tokens
+// 347 -> 340, 131072 tokens 1670 -> 1637, head_dim 64 117 -> 112; a list of active tiles alone 511 -> 519, 512 with the
+// polynomial as it is now).
 __device__ __forceinline__ float sweep_exp(uint32_t tS, const uint4& bits, int lo, int hi, float scale, float neg_m) {
   float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+  const float scale_z = scale * 0.004f, neg_z = fmaf(neg_m, 0.004f, 0.5f);      // (y + 125) / 250
 #pragma unroll 1
   for (int h = lo; h < hi; ++h) {
     uint32_t ra[32], rb[32], pk[32];
     tmem_ld32(tS + 64 * h, ra);
     tmem_ld32(tS + 64 * h + 32, rb);
     tc_wait_ld();
-    exp_chunk<MASKED>(ra, h ? bits.z : bits.x, scale, neg_m, pk, s0, s1, s2, s3);
-    exp_chunk<MASKED>(rb, h ? bits.w : bits.y, scale, neg_m, pk + 16, s0, s1, s2, s3);
+    exp_chunk(ra, h ? bits.z : bits.x, scale, neg_m, scale_z, neg_z, pk, s0, s1, s2, s3);
+    exp_chunk(rb, h ? bits.w : bits.y, scale, neg_m, scale_z, neg_z, pk + 16, s0, s1, s2, s3);
     tmem_st32(tS + 32 * h, pk);
   }
-  if (MASKED && hi - lo < 2) {
+  if (hi - lo < 2) {
     uint32_t z[32];
 #pragma unroll
     for (int q = 0; q < 32; ++q) z[q] = 0u;
@@ -489,7 +499,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         uint32_t dummy = 0;
 #pragma unroll 1
         for (uint32_t k = sc < kSlots ? 0u : sc - kSlots; k < sc; ++k)
-          mbar_wait(bSlotFull + 8 * (k % kSlots), (k / kSlots) & 1u, &dummy, 20000000ull);
+          mbar_wait(bSlotFull + 8 * (k % kSlots), (k / kSlots) & 1u, &dummy, kDrainPolls);
       }
     }
   } else if (warp == 1) {
@@ -654,7 +664,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // drain: copies already issued still write into shared memory; wait for them (bounded)
         uint32_t dummy = 0;
 #pragma unroll 1
-        for (int X = 0; X < 2; ++X) mbar_wait(bQFull + 8 * X, ((q_ph >> X) & 1u) ^ 1u, &dummy, 20000000ull);
+        for (int X = 0; X < 2; ++X) mbar_wait(bQFull + 8 * X, ((q_ph >> X) & 1u) ^ 1u, &dummy, kDrainPolls);
       }
     }
   }
@@ -765,8 +775,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         const float mm = (m_ref == -CUDART_INF_F) ? 0.f : m_ref;
         // ---- sweep 2: probabilities against the reference max, packed to bf16 into the first half of S
-        const float tsum = need_mask ? sweep_exp<true>(tS, bits, lo, hi, prm.scale_log2, -mm)
-                                     : sweep_exp<false>(tS, bits, 0, 2, prm.scale_log2, -mm);
+        const float tsum = sweep_exp(tS, bits, lo, hi, prm.scale_log2, -mm);
         l = l * alpha + tsum;
         // ---- O is complete up to the previous tile of this stream (its MMAs precede S of this tile)
         if (t > t0) {
@@ -1016,7 +1025,8 @@ __global__ void clear_status_kernel(uint32_t* scratch, int keep) {
 }
 
 // Self-test of the bounded wait every kernel in this library uses: waits on an mbarrier that nothing ever
-// arrives on, with the given limit; the wait gives up, the status word is set and the kernel returns normally.
+// arrives on, twenty thousand polls at a time, until the given limit is over; every wait gives up, the status word is set and the
+// kernel returns normally.
 __global__ void bounded_wait_selftest_kernel(uint32_t* status, unsigned long long limit_ns, unsigned long long* waited_ns) {
   __shared__ uint64_t bar;
   __shared__ uint32_t abort_flag;
@@ -1024,13 +1034,12 @@ __global__ void bounded_wait_selftest_kernel(uint32_t* status, unsigned long lon
     mbar_init(smem_u32(&bar), 1);
     abort_flag = 0u;
     mbar_fence_init();
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
     const uint64_t t0 = globaltimer_ns();
-    const bool ok = mbar_wait(smem_u32(&bar), 0u, &abort_flag, limit_ns);
+    bool ok;
+    do ok = mbar_wait(smem_u32(&bar), 0u, &abort_flag, 20000u);
+    while (!ok && globaltimer_ns() - t0 < limit_ns);
     *waited_ns = globaltimer_ns() - t0;
-    if (!ok) atomicMax(status, (uint32_t)DAM_ERR_DEVICE_TIMEOUT);
+    if (!ok && abort_flag) atomicMax(status, (uint32_t)DAM_ERR_DEVICE_TIMEOUT);
   }
 }
 

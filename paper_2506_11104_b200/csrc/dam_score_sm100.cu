@@ -118,7 +118,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   // to the MMA thread and the eight softmax warps through a two-entry ring; a negative entry ends the loop.
   auto next_item_consumer = [&](uint32_t n) -> int {
     const uint32_t slot = n & 1u;
-    if (!mbar_wait(bSchedFull + 8 * slot, (n >> 1) & 1u, abort_flag)) return -2;
+    if (!mbar_wait_slow(bSchedFull + 8 * slot, (n >> 1) & 1u, abort_flag)) return -2;
     return sched_items[slot];
   };
 
@@ -150,7 +150,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       bool ok = true;
       for (uint32_t n = 0; ok; ++n) {
         const uint32_t sl = n & 1u;
-        if (!(ok = mbar_wait(bSchedEmpty + 8 * sl, ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
+        if (!(ok = mbar_wait_slow(bSchedEmpty + 8 * sl, ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         int w = n == 0 ? (int)blockIdx.x : (int)(gridDim.x + atomicAdd(prm.work_counter, 1u));
         if (w >= nitems) w = -1;
         sched_items[sl] = w;
@@ -158,7 +158,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         if (w < 0) break;
         const Item it = decode_item(blob, prm, w);
         if (!it.valid) continue;
-        if (!(ok = mbar_wait(bQEmpty, (ic & 1u) ^ 1u, abort_flag))) break;
+        if (!(ok = mbar_wait_slow(bQEmpty, (ic & 1u) ^ 1u, abort_flag))) break;
         mbar_arrive_expect_tx(bQFull, DAM_TILE * D * 2);
         const int tokq = it.sq.tok_start + it.qb * DAM_TILE;
         tma_load_3d(sQ, &tmQ, bQFull, 0, it.h, tokq);
@@ -169,7 +169,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         for (int t = 0; t < ntile && ok; ++t) {
           const int kb = t % (it.qb + 1);
           const uint32_t s = sc % kSlots, ph = (sc / kSlots) & 1u;
-          if (!(ok = mbar_wait(bSlotEmpty + 8 * s, ph ^ 1u, abort_flag))) break;
+          if (!(ok = mbar_wait_slow(bSlotEmpty + 8 * s, ph ^ 1u, abort_flag))) break;
           const uint32_t dst = sSlots + s * kSlotBytes, bar = bSlotFull + 8 * s;
           mbar_arrive_expect_tx(bar, DAM_TILE * D * 2);
           tma_load_3d(dst, &tmK, bar, 0, kvh, it.sq.tok_start + kb * DAM_TILE);
@@ -181,8 +181,8 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       if (!ok) {
         uint32_t dummy = 0;
         for (int s = 0; s < kSlots; ++s)
-          if (armed[s] != 2u) mbar_wait(bSlotFull + 8 * s, armed[s], &dummy, 20000000ull);
-        mbar_wait(bQFull, (ic + 1u) & 1u, &dummy, 20000000ull);
+          if (armed[s] != 2u) mbar_wait_slow(bSlotFull + 8 * s, armed[s], &dummy, 20000000ull);
+        mbar_wait_slow(bQFull, (ic + 1u) & 1u, &dummy, 20000000ull);
       }
     }
   } else if (warp == 1) {
@@ -198,13 +198,13 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         if (w < 0) { ok = (w == -1); break; }
         const Item it = decode_item(blob, prm, w);
         if (!it.valid) continue;
-        if (!(ok = mbar_wait(bQFull, ic & 1u, abort_flag))) break;
+        if (!(ok = mbar_wait_slow(bQFull, ic & 1u, abort_flag))) break;
         ++ic;
         const int ntile = 2 * (it.qb + 1);
         for (int t = 0; t < ntile && ok; ++t, ++g, ++sc) {
           const uint32_t buf = g & 3u, s = sc % kSlots;
-          if (!(ok = mbar_wait(bSEmpty + 8 * buf, ((g >> 2) & 1u) ^ 1u, abort_flag))) break;
-          if (!(ok = mbar_wait(bSlotFull + 8 * s, (sc / kSlots) & 1u, abort_flag))) break;
+          if (!(ok = mbar_wait_slow(bSEmpty + 8 * buf, ((g >> 2) & 1u) ^ 1u, abort_flag))) break;
+          if (!(ok = mbar_wait_slow(bSlotFull + 8 * s, (sc / kSlots) & 1u, abort_flag))) break;
           tc_fence_after();
           const uint32_t b0 = dK_lo + s * (kSlotBytes >> 4);
 #pragma unroll
@@ -249,7 +249,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           base[G * DAM_TILE + r] = make_float2(m, l);
           __syncwarp();
           if (lane == 0) mbar_arrive(bStat);                       // release: the warp's 32 rows are written
-          if (!(ok = mbar_wait(bStat, nitem & 1u, abort_flag))) break;
+          if (!(ok = mbar_wait_slow(bStat, nitem & 1u, abort_flag))) break;
           float mn = m;
 #pragma unroll
           for (int q = 0; q < 4; ++q) mn = fmaxf(mn, base[q * DAM_TILE + r].x);
@@ -270,7 +270,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const bool sweepB = t >= nk;
         const uint32_t buf = (uint32_t)G;
         const uint32_t tS = tS0 + buf * 128;
-        if (!(ok = mbar_wait(bSFull + 8 * buf, cG & 1u, abort_flag))) break;
+        if (!(ok = mbar_wait_slow(bSFull + 8 * buf, cG & 1u, abort_flag))) break;
         ++cG;
         tc_fence_after();
         // keys beyond the causal limit (and beyond the window, which the limit implies) do not exist

@@ -43,13 +43,22 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: gives up after `limit_ns` of wall time, records the fact in *abort_flag (shared memory, also polled so that
-// one expired wait releases every other waiter) and returns false.  No wait in these kernels can spin forever.  The poll loop
-// is short: it is inlined wherever a role waits, and the attention kernel's code is larger than the instruction cache (70 KB
-// with a loop that looked at the clock every 256 polls, 64 now: 8192 tokens 100.3 -> 98.5 us of attention, 32768 tokens 391.8 ->
-// 388.8, head_dim 64 127.8 -> 126.5).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
-                                          uint64_t limit_ns = 2000000000ull) {
+// Bounded wait: gives up after `polls` looks at the barrier, records the fact in *abort_flag (shared memory) and returns false.
+// No wait in these kernels can spin forever; a role whose partner has given up waits for it in vain and gives up in its turn.
+// A look takes 43 cycles and more (measured on a barrier that nothing arrives on, a warp per scheduler polling), so the
+// default is a second or so.  The loop is as short as it can be: it is inlined wherever a role waits, all of the attention
+// kernel's code is executed for every work item, and the instruction cache holds about 64 KB of it (with a look at the
+// wall clock every 256 polls 70 KB, at every poll 64; that kernel as it is now: 55.6 KB with the wall clock, 51.8 with the
+// cycle counter, 51 with a count).
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t polls = 40000000u) {
+#pragma unroll 1
+  while (!mbar_try_wait(bar, parity))
+    if (--polls == 0u) { *abort_flag = 1u; return false; }
+  return true;
+}
+// The same with the wall clock between two looks, for a kernel with many waiting warps beside working ones (the scoring kernel:
+// with the bare loop stage 1 takes 40.7 us instead of 40.2 at 8192 tokens, 35.5 instead of 34.8 at head_dim 64).
+__device__ __forceinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint64_t limit_ns = 2000000000ull) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = globaltimer_ns();
 #pragma unroll 1
@@ -59,6 +68,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
   return true;
 }
+constexpr uint32_t kDrainPolls = 1000000u;      // 20 ms and more: a copy that has been issued lands
 
 // ---- TMA ----------------------------------------------------------------------------------------
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {
