@@ -3,14 +3,14 @@
 //
 // For every (sequence, query head) the causal softmax map over the first L tokens is computed tile by
 // tile and thresholded straight into the bit-packed true mask (paper Sec. 4.2.1 - 4.2.3); the map itself
-// is never stored unless the caller asks for the fp32 dump.  Four S buffers in TMEM let the MMA warp run two
-// tiles ahead of each softmax group.  A work item is one 128-row query block of
+// is never stored unless the caller asks for the fp32 dump.  An S buffer per softmax group in TMEM lets the MMA warp run ahead
+// of them.  A work item is one 128-row query block of
 // one (sequence, head).  Two sweeps over its kv tiles kb = 0 .. qb:
 //   sweep A  S = Q K^T (tcgen05, accumulator in TMEM) -> per-row running max and sum;
 //   sweep B  S again -> p = exp2(x - max) / sum in fp32 -> bit = [p >= p*] -> one 16-byte store of the
 //            row's 128 bits per tile (and the optional dump of p).
-// Warp roles: warp 0 TMA producer, warp 1 MMA issuer, warps 2-17 four groups of one thread per query row;
-// group G owns TMEM buffer G, i.e. every fourth kv tile, and the groups merge their row statistics through
+// Warp roles: warp 0 TMA producer, warp 1 MMA issuer, then two or four groups of one thread per query row;
+// group G owns TMEM buffer G, i.e. every second or fourth kv tile, and the groups merge their row statistics through
 // shared memory between the sweeps.  Every wait is bounded.
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -22,25 +22,25 @@ using namespace sm100;
 
 namespace {
 
-constexpr int kSlots = 5;
 constexpr int kSlotBytes = 32768;
-constexpr int kThreads = 576;              // producer warp, MMA warp, four softmax groups of four warps
-constexpr uint32_t kTmemCols = 512;       // four S buffers: tile g uses buffer g & 3, which softmax group g & 3 owns
 
+// kGroups: softmax groups of four warps, each with an S buffer (tile g uses buffer g % kGroups).
+template <int kGroups>
 struct SmemLayout {
+  static constexpr int kSlots = kGroups == 4 ? 5 : 2;
+  static constexpr int kThreads = 64 + 128 * kGroups;      // producer warp, MMA warp, softmax warps
   static constexpr int q = 0;
   static constexpr int slots = kSlotBytes;
   static constexpr int bars = kSlotBytes * (1 + kSlots);
-  // q_full, q_empty, slot_full[kSlots], slot_empty[kSlots], s_full[4], s_empty[4], stat_ready,
+  // q_full, q_empty, slot_full[kSlots], slot_empty[kSlots], s_full[kGroups], s_empty[kGroups], stat_ready,
   // sched_full[2], sched_empty[2]
-  static constexpr int n_bars = 2 + 2 * kSlots + 13;
+  static constexpr int n_bars = 2 + 2 * kSlots + 2 * kGroups + 5;
   static constexpr int sched_items = bars + 8 * n_bars;     // int[2]
-  static constexpr int stat = sched_items + 8;              // float2 [2][4][128]
-  static constexpr int tmem_slot = stat + 2 * 4 * 128 * 8;
+  static constexpr int stat = sched_items + 8;              // float2 [2][kGroups][128]
+  static constexpr int tmem_slot = stat + 2 * kGroups * 128 * 8;
   static constexpr int abort_flag = tmem_slot + 4;
-  static constexpr int total = abort_flag + 4;
+  static constexpr int total = abort_flag + 4 + 1024;
 };
-constexpr int kSmemBytes = SmemLayout::total + 1024;
 
 struct ScoreParams {
   unsigned char* blob;
@@ -92,30 +92,32 @@ __device__ __forceinline__ Item decode_item(const unsigned char* blob, const Sco
   return it;
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int D, int kGroups>
+__global__ void __launch_bounds__(SmemLayout<kGroups>::kThreads, 4 / kGroups)
 score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ ScoreParams prm) {
+  using Smem = SmemLayout<kGroups>;
+  constexpr uint32_t kSlots = Smem::kSlots, kTmemCols = 128 * kGroups;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
-  const uint32_t sQ = sbase + SmemLayout::q;
-  const uint32_t sSlots = sbase + SmemLayout::slots;
-  const uint32_t bar0 = sbase + SmemLayout::bars;
+  const uint32_t sQ = sbase + Smem::q;
+  const uint32_t sSlots = sbase + Smem::slots;
+  const uint32_t bar0 = sbase + Smem::bars;
   const uint32_t bQFull = bar0, bQEmpty = bar0 + 8;
   const uint32_t bSlotFull = bar0 + 16, bSlotEmpty = bSlotFull + 8 * kSlots;
-  const uint32_t bSFull = bSlotEmpty + 8 * kSlots, bSEmpty = bSFull + 32, bStat = bSEmpty + 32;
+  const uint32_t bSFull = bSlotEmpty + 8 * kSlots, bSEmpty = bSFull + 8 * kGroups, bStat = bSEmpty + 8 * kGroups;
   const uint32_t bSchedFull = bStat + 8, bSchedEmpty = bSchedFull + 16;
-  volatile int* sched_items = reinterpret_cast<volatile int*>(smem + SmemLayout::sched_items);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + SmemLayout::tmem_slot);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + SmemLayout::abort_flag);
+  volatile int* sched_items = reinterpret_cast<volatile int*>(smem + Smem::sched_items);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + Smem::tmem_slot);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + Smem::abort_flag);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* blob = prm.blob;
   const DamHeader* H = &prm.plan.h;
   const int nitems = prm.max_nL * prm.num_seqs * prm.Hq;
   // Items (heaviest query blocks first) are claimed from a global counter by the producer thread and handed
-  // to the MMA thread and the eight softmax warps through a two-entry ring; a negative entry ends the loop.
+  // to the MMA thread and the softmax warps through a two-entry ring; a negative entry ends the loop.
   auto next_item_consumer = [&](uint32_t n) -> int {
     const uint32_t slot = n & 1u;
     if (!mbar_wait_slow(bSchedFull + 8 * slot, (n >> 1) & 1u, abort_flag)) return -2;
@@ -125,9 +127,9 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   if (tid == 0) {
     mbar_init(bQFull, 1); mbar_init(bQEmpty, 1);
     for (int s = 0; s < kSlots; ++s) { mbar_init(bSlotFull + 8 * s, 1); mbar_init(bSlotEmpty + 8 * s, 1); }
-    for (int s = 0; s < 4; ++s) { mbar_init(bSFull + 8 * s, 1); mbar_init(bSEmpty + 8 * s, 4); }
-    mbar_init(bStat, 16);
-    for (int s = 0; s < 2; ++s) { mbar_init(bSchedFull + 8 * s, 1); mbar_init(bSchedEmpty + 8 * s, 17); }   // MMA thread + 16 softmax warps
+    for (int s = 0; s < kGroups; ++s) { mbar_init(bSFull + 8 * s, 1); mbar_init(bSEmpty + 8 * s, 4); }
+    mbar_init(bStat, 4 * kGroups);
+    for (int s = 0; s < 2; ++s) { mbar_init(bSchedFull + 8 * s, 1); mbar_init(bSchedEmpty + 8 * s, 1 + 4 * kGroups); }   // MMA thread + softmax warps
     *abort_flag = 0u;
     mbar_fence_init();
     tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK);
@@ -202,8 +204,8 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         ++ic;
         const int ntile = 2 * (it.qb + 1);
         for (int t = 0; t < ntile && ok; ++t, ++g, ++sc) {
-          const uint32_t buf = g & 3u, s = sc % kSlots;
-          if (!(ok = mbar_wait_slow(bSEmpty + 8 * buf, ((g >> 2) & 1u) ^ 1u, abort_flag))) break;
+          const uint32_t buf = g % kGroups, s = sc % kSlots;
+          if (!(ok = mbar_wait_slow(bSEmpty + 8 * buf, ((g / kGroups) & 1u) ^ 1u, abort_flag))) break;
           if (!(ok = mbar_wait_slow(bSlotFull + 8 * s, (sc / kSlots) & 1u, abort_flag))) break;
           tc_fence_after();
           const uint32_t b0 = dK_lo + s * (kSlotBytes >> 4);
@@ -220,12 +222,12 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     }
   } else {
     // ---------------------------------------------------------------- row statistics and thresholding
-    // Two groups of four warps; group G owns the S buffer G, i.e. every other kv tile of the item.
+    // Groups of four warps; group G owns the S buffer G, i.e. every kGroups-th kv tile of the item.
     const int G = (warp - 2) >> 2;
     const int r = (warp & 3) * 32 + lane;
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t tS0 = tmem + lane_addr;
-    float2* stat = reinterpret_cast<float2*>(smem + SmemLayout::stat);      // [2 item parities][2 groups][128 rows]
+    float2* stat = reinterpret_cast<float2*>(smem + Smem::stat);      // [2 item parities][kGroups][128 rows]
     uint32_t g = 0, cG = 0, nitem = 0;      // g: tiles issued so far (all groups); cG: tiles this group consumed
     bool ok = true;
     for (uint32_t n = 0; ok; ++n) {
@@ -245,17 +247,17 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       for (int t = 0; t < 2 * nk; ++t, ++g) {
         if (t == nk) {
           // all groups have finished sweep A: merge their (max, sum) per row through shared memory
-          float2* base = stat + (nitem & 1u) * 4 * DAM_TILE;
+          float2* base = stat + (nitem & 1u) * kGroups * DAM_TILE;
           base[G * DAM_TILE + r] = make_float2(m, l);
           __syncwarp();
           if (lane == 0) mbar_arrive(bStat);                       // release: the warp's 32 rows are written
           if (!(ok = mbar_wait_slow(bStat, nitem & 1u, abort_flag))) break;
           float mn = m;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) mn = fmaxf(mn, base[q * DAM_TILE + r].x);
+          for (int q = 0; q < kGroups; ++q) mn = fmaxf(mn, base[q * DAM_TILE + r].x);
           float ls = 0.f;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < kGroups; ++q) {
             const float2 o = base[q * DAM_TILE + r];
             ls += (o.x == -CUDART_INF_F) ? 0.f : o.y * ex2(o.x - mn);
           }
@@ -265,7 +267,7 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           thr_raw = (fmaxf(log2f(prm.pstar * l), -126.f) + m) / prm.scale_log2;
           margin = (0.000244140625f + fabsf(m) * 7.62939453125e-6f) / prm.scale_log2;      // 2^-12 + |m| 2^-17
         }
-        if ((g & 3u) != (uint32_t)G) continue;
+        if (g % kGroups != (uint32_t)G) continue;
         const int kb = t % nk;
         const bool sweepB = t >= nk;
         const uint32_t buf = (uint32_t)G;
@@ -381,9 +383,9 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         for (int kb = it.qb + 1; kb * 4 < W; ++kb) *reinterpret_cast<uint4*>(Mrow + kb * 4) = make_uint4(0u, 0u, 0u, 0u);
       }
       if (prm.dump) {
-        // the warp's rows one after the other, a row's zeros by all lanes; the four groups take eight rows each
+        // the warp's rows one after the other, a row's zeros by all lanes; the groups share them out
         float* P0 = prm.dump + it.sq.p_off + (uint64_t)it.h * L * L;
-        for (int rr = 8 * G; rr < 8 * G + 8; ++rr) {
+        for (int rr = 32 / kGroups * G; rr < 32 / kGroups * (G + 1); ++rr) {
           const int ir = it.qb * DAM_TILE + (warp & 3) * 32 + rr;
           if (ir >= L) break;
           float* Pr = P0 + (size_t)ir * L;
@@ -414,11 +416,13 @@ cudaError_t dam_launch_scores_sm100(const void* Q, const void* K, const dam_shap
   DamDeviceInfo di;
   cudaError_t e;
   if ((e = dam_current_device(&dev, &di)) != cudaSuccess) return e;
-  if (di.cc_major != 10 || di.smem_optin < kSmemBytes) return cudaErrorNotSupported;
+  if (di.cc_major != 10 || di.smem_optin < SmemLayout<4>::total) return cudaErrorNotSupported;
   if ((e = dam_device_table().once(dev, DAM_SETUP_SCORE_SMEM, [](void) -> cudaError_t {
-         cudaError_t r = cudaFuncSetAttribute(score_sm100_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-         if (r != cudaSuccess) return r;
-         return cudaFuncSetAttribute(score_sm100_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+         cudaError_t r;
+         if ((r = cudaFuncSetAttribute(score_sm100_kernel<128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<4>::total)) != cudaSuccess) return r;
+         if ((r = cudaFuncSetAttribute(score_sm100_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<2>::total)) != cudaSuccess) return r;
+         if ((r = cudaFuncSetAttribute(score_sm100_kernel<64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<4>::total)) != cudaSuccess) return r;
+         return cudaFuncSetAttribute(score_sm100_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<2>::total);
        })) != cudaSuccess)
     return e;
   const int sm_count = di.sm_count;
@@ -443,15 +447,23 @@ cudaError_t dam_launch_scores_sm100(const void* Q, const void* K, const dam_shap
   }
   p.dump_vec8 = vec8 ? 1 : 0;
   const int items = c.max_nL * c.num_seqs * c.Hq;
-  const int grid = items < sm_count ? items : sm_count;
+  // Two CTAs per SM with two softmax groups each, from three items per SM on; below that one CTA with four.  The four groups of
+  // a CTA are in the same sweep of the same item: first they all want the special-function unit, then the integer pipe, then
+  // all wait at the merge or for the next query tile; two items side by side fill each other's gaps, but an item takes
+  // longer.  Stage 1, one and two CTAs per SM: 256 items of up to 8 tiles (8192 tokens) 40.5 and 47.8 us, 256 of 16 tiles 53.9
+  // and 70.5, 384 67.8 and 70.5, 512 (32768 tokens) 79.8 and 76.9, 1024 of up to 32 (131072 tokens) 232 and 217, 1536 (mixed
+  // lengths) 140 and 126, 1024 of 4 with the map written 112 and 106.
+  const bool two = items >= 3 * sm_count;
+  const int ctas = two ? 2 * sm_count : sm_count, grid = items < ctas ? items : ctas;
   // launched as a programmatic dependent of the kernel that initialises the blob: its launch latency and its
   // prologue (barriers, TMEM, descriptors) hide under that kernel; it waits before it reads the blob
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = st;
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(two ? SmemLayout<2>::kThreads : SmemLayout<4>::kThreads);
+  cfg.dynamicSmemBytes = two ? SmemLayout<2>::total : SmemLayout<4>::total; cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  if (d == 128) return cudaLaunchKernelEx(&cfg, score_sm100_kernel<128>, tq, tk, p);
-  return cudaLaunchKernelEx(&cfg, score_sm100_kernel<64>, tq, tk, p);
+  if (d == 128) return two ? cudaLaunchKernelEx(&cfg, score_sm100_kernel<128, 2>, tq, tk, p) : cudaLaunchKernelEx(&cfg, score_sm100_kernel<128, 4>, tq, tk, p);
+  return two ? cudaLaunchKernelEx(&cfg, score_sm100_kernel<64, 2>, tq, tk, p) : cudaLaunchKernelEx(&cfg, score_sm100_kernel<64, 4>, tq, tk, p);
 }

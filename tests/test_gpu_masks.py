@@ -214,6 +214,16 @@ def test_small_cases_scored_on_gpu(lengths, pcl, Hq, Hkv, d, dtype, gather):
     assert flipped <= 2e-3 * total
 
 
+@pytest.mark.parametrize("seqs", [9, 10])
+@pytest.mark.parametrize("d", [128, 64])
+def test_scoring_with_one_and_two_blocks_per_multiprocessor(d, seqs):
+    """432 and 480 query blocks to score: on either side of three per multiprocessor, from where two blocks share one."""
+    w = synth.small_case(0, 16, 8, d, 300, seed=seqs, lengths=[700, 300, 257, 299, 513, 301, 640, 258, 290, 400][:seqs])
+    blob, shape, masks, dump = _build_and_check(w, gather=True)
+    flipped, total = _score_closeness(w, dump, masks, range(0, 16, 5))
+    assert flipped <= 2e-3 * total
+
+
 @pytest.mark.parametrize("gather", GATHER)
 def test_config1_full_size_masks(gather):
     """Llama-3-8B-shaped layer, 8192 tokens, PCL 1024: every head's D, V and true mask, sampled q-blocks."""
