@@ -452,8 +452,9 @@ cudaError_t dam_launch_scores_sm100(const void* Q, const void* K, const dam_shap
   // all wait at the merge or for the next query tile; two items side by side fill each other's gaps, but an item takes
   // longer.  Stage 1, one and two CTAs per SM: 256 items of up to 8 tiles (8192 tokens) 40.5 and 47.8 us, 256 of 16 tiles 53.9
   // and 70.5, 384 67.8 and 70.5, 512 (32768 tokens) 79.8 and 76.9, 1024 of up to 32 (131072 tokens) 232 and 217, 1536 (mixed
-  // lengths) 140 and 126, 1024 of 4 with the map written 112 and 106.
-  const bool two = items >= 3 * sm_count;
+  // lengths) 140 and 126, 1024 of 4 with the map written 112 and 106.  Windows of more than 16 tiles want four items per SM
+  // (512 of up to 32 tiles 125.6 and 129.2, 768 169 and 156).
+  const bool two = items >= (c.max_nL <= 16 ? 3 : 4) * sm_count;
   const int ctas = two ? 2 * sm_count : sm_count, grid = items < ctas ? items : ctas;
   // launched as a programmatic dependent of the kernel that initialises the blob: its launch latency and its
   // prologue (barriers, TMEM, descriptors) hide under that kernel; it waits before it reads the blob
