@@ -8,6 +8,9 @@
 
 namespace {
 
+constexpr int kRefWarps = 8;          // warps of a block
+constexpr int kFewRows = 8, kFewKeys = 8;      // attn_ref_few_kernel: rows of a block, keys of a warp in a stage
+
 template <typename T> struct Ld8;
 template <> struct Ld8<float> {
   static __device__ __forceinline__ void load(const float* p, float* o) {
@@ -195,9 +198,9 @@ scores_ref_kernel(unsigned char* blob, const T* __restrict__ Q, const T* __restr
 // Masked attention over the listed tiles, online softmax in fp32.  A block takes 8 R adjacent rows (R per warp) of one
 // (head, q-block) row of the tile list and walks its tiles in stages of 64 keys whose K and V rows sit in shared memory;
 // a stage without an active cell in the block's rows is not loaded.  The lanes of a warp are keys for the scores and
-// dimensions for the output.  Latency bound at the sizes this path serves: R = 1 while that leaves SMs idle, 4 otherwise.
+// dimensions for the output.  For many rows (R = 4; attn_ref_few_kernel serves few).
 // PIPE (fp32, two stages fit in shared memory): the next stage with an active cell is looked for and its copies are
-// started before this one is worked on (512 tokens, 2 heads: 28.5 -> 21.7 us; leaving out the keys no row keeps inside a stage: no change).
+// started before this one is worked on (512 tokens, 2 heads, a row per warp: 28.5 -> 21.7 us; leaving out the keys no row keeps inside a stage: no change).
 // ---------------------------------------------------------------------------------------------
 template <typename T, int R, int ND, bool PIPE>
 __global__ void __launch_bounds__(256)
@@ -356,13 +359,215 @@ attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __r
   }
 }
 
-// R rows per warp: 4 where that still gives every SM a block of 8 warps, otherwise 1 (so that a short prompt's rows are
-// spread over the whole chip).
-constexpr int kRefWarps = 8;
-inline bool four_rows(long long rows, int sm_count) { return rows >= (long long)sm_count * kRefWarps * 4; }
+// The same for few rows: a block of eight warps takes eight adjacent rows, and a warp takes eight of the 64 keys of every stage
+// for all of them.  Lane 4 r + c scores row r against keys c and c + 4; for the output a lane holds 2 dimensions (of every 64) of all
+// eight rows.  Every warp has a running softmax of its own over its keys, merged at the end.  A warp per row reads all 64
+// keys of a stage from shared memory for each row, 2300 cycles of its bandwidth; here a key is read once per block.
+// What is left is latency: a stage's two barriers and chains, and what the first one waits for (header, records, list, mask
+// words, rows).  fp32, 2 heads of 64: 512 tokens 21.6 -> 17.2 us (19.2 without the mask words asked for a tile ahead), 1100 tokens
+// 27.6 -> 21.3, 4 heads, 700 tokens 45.3 -> 33.5.  Three blocks to an SM (1500 tokens 29.3 -> 25.4).
+template <typename T, int ND, bool PIPE>
+__global__ void __launch_bounds__(256, ND == 1 ? 3 : 1)
+attn_ref_few_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __restrict__ K,
+                    const T* __restrict__ V, int Hq, int group, int d, int64_t qst, int64_t qsh,
+                    int64_t kst, int64_t ksh, int64_t vst, int64_t vsh, int64_t ost, int64_t osh,
+                    int causal, float scale, T* __restrict__ O, float* __restrict__ lse, int total_tokens,
+                    const int32_t* __restrict__ ranges, const __grid_constant__ DamRowRanges rr, uint32_t* scratch, int keep) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x >= keep && threadIdx.x < 64) scratch[threadIdx.x] = 0u;
+  extern __shared__ __align__(16) float smem[];
+  const DamHeader* H = reinterpret_cast<const DamHeader*>(blob);
+  const int row = blockIdx.x;
+  const int h = row / H->total_qblocks, gqb = row % H->total_qblocks;
+  const int b = reinterpret_cast<const int32_t*>(blob + H->off_qbseq)[gqb];
+  const DamSeq sq = reinterpret_cast<const DamSeq*>(blob + H->off_seq)[b];
+  const int qb = gqb - sq.first_qblock;
+  if (ranges && !rr.holds(ranges, b, qb & ~1)) return;         // row ranges: whole pairs of query blocks
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i0 = qb * DAM_TILE + blockIdx.y * kFewRows;
+  if (i0 >= sq.S) return;
+  const uint32_t* tile_ptr = reinterpret_cast<const uint32_t*>(blob + H->off_tile_ptr);
+  const uint32_t* tiles = reinterpret_cast<const uint32_t*>(blob + H->off_tiles);
+  const uint32_t t0 = tile_ptr[row], t1 = tile_ptr[row + 1];
+  const DamHeadBits hb = dam_head_bits(blob, H, sq, h);
+  const int pitch = k_pitch(d);
+  const int stage = kStageKeys * (pitch + d);
+  float* k_s = smem;
+  float* v_s = k_s + kStageKeys * pitch;
+  float* q_s = smem + (PIPE ? 2 : 1) * stage;                                  // kFewRows rows, `pitch` apart
+  float* p_s = q_s + kFewRows * pitch + warp * (kFewKeys + 1) * kFewRows;      // the warp's probabilities, a row per key; corrections
+  for (int x = threadIdx.x; x < kFewRows * d; x += blockDim.x) {
+    const int r = x / d, c = x % d;
+    q_s[r * pitch + c] = i0 + r < sq.S ? Ld8<T>::one(Q + (int64_t)(sq.tok_start + i0 + r) * qst + (int64_t)h * qsh + c) : 0.f;
+  }
+  const T* Kh = K + (int64_t)sq.tok_start * kst + (int64_t)(h / group) * ksh;
+  const T* Vh = V + (int64_t)sq.tok_start * vst + (int64_t)(h / group) * vsh;
+  const int my_row = lane >> 2, my_key = warp * kFewKeys + (lane & 3);          // and my_key + 4
+  float acc[kFewRows][2 * ND], m = -CUDART_INF_F, l = 0.f;
+#pragma unroll
+  for (int r = 0; r < kFewRows; ++r)
+#pragma unroll
+    for (int u = 0; u < 2 * ND; ++u) acc[r][u] = 0.f;
+  // the stages of the tiles that hold an active cell of the block's rows, in order
+  struct Stage { uint32_t mine; int j0; bool valid; };                         // mine: bits 0 and 4: the lane's two cells
+  // (the mask words of a tile are asked for one tile ahead, its entry two: a stage would wait for both in turn)
+  uint32_t t = t0, e_next = t < t1 ? __ldg(tiles + t) : 0u;
+  int half = 2, kb = 0, kb_next = 0;
+  uint4 bits = make_uint4(0u, 0u, 0u, 0u), bits_next = bits;
+  bool more = false;
+  auto ask = [&]() {
+    more = (e_next >> 28) != 0u;                                // (zero entries are padding behind the row's)
+    if (!more) return;
+    kb_next = (int)(e_next & 0x0FFFFFFFu);
+    bits_next = dam_apply_bits(hb, e_next >> 28, i0 + my_row, kb_next, causal);
+    ++t;
+    e_next = t < t1 ? __ldg(tiles + t) : 0u;
+  };
+  ask();
+  auto find = [&](Stage& g) {
+    while (true) {
+      if (half == 2) {
+        if (!more) { g.valid = false; return; }
+        kb = kb_next;
+        bits = bits_next;
+        ask();
+        half = 0;
+      }
+      const uint32_t w0 = half ? bits.z : bits.x, w1 = half ? bits.w : bits.y;
+      g.mine = ((my_key & 32) ? w1 : w0) >> (my_key & 31);
+      g.j0 = kb * DAM_TILE + half * kStageKeys;
+      ++half;
+      if (__syncthreads_or((w0 | w1) != 0u)) { g.valid = true; return; }     // (a barrier: the stage before the last is no longer read)
+    }
+  };
+  auto work = [&](const Stage& g, const float* k_b, const float* v_b) {
+    const bool a0 = g.mine & 1u, a1 = (g.mine >> 4) & 1u;
+    if (!__any_sync(0xFFFFFFFFu, a0 || a1)) return;
+    float s0 = 0.f, s1 = 0.f;
+    const float *k0 = k_b + my_key * pitch, *k1 = k0 + 4 * pitch, *q = q_s + my_row * pitch;
+#pragma unroll 4
+    for (int c = 0; c < d; c += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(q + c), y = *reinterpret_cast<const float4*>(k0 + c),
+                   z = *reinterpret_cast<const float4*>(k1 + c);
+      s0 = fmaf(x.x, y.x, s0); s1 = fmaf(x.x, z.x, s1);
+      s0 = fmaf(x.y, y.y, s0); s1 = fmaf(x.y, z.y, s1);
+      s0 = fmaf(x.z, y.z, s0); s1 = fmaf(x.z, z.z, s1);
+      s0 = fmaf(x.w, y.w, s0); s1 = fmaf(x.w, z.w, s1);
+    }
+    const float x0 = a0 ? s0 * scale : -CUDART_INF_F, x1 = a1 ? s1 * scale : -CUDART_INF_F;
+    float mn = fmaxf(x0, x1);
+    mn = fmaxf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, 1));
+    mn = fmaxf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, 2));
+    mn = fmaxf(m, mn);
+    // (an infinite maximum counts as zero: a row without a key so far, or whose logits are all -inf)
+    const float at = mn == -CUDART_INF_F ? 0.f : mn, corr = expf(m - at);
+    const float p0 = a0 ? expf(x0 - at) : 0.f, p1 = a1 ? expf(x1 - at) : 0.f;
+    l = l * corr + (p0 + p1);
+    m = mn;
+    p_s[(lane & 3) * kFewRows + my_row] = p0;
+    p_s[((lane & 3) + 4) * kFewRows + my_row] = p1;
+    p_s[kFewKeys * kFewRows + my_row] = corr;
+    __syncwarp();
+    if (__any_sync(0xFFFFFFFFu, corr != 1.f)) {
+#pragma unroll
+      for (int r = 0; r < kFewRows; ++r) {
+        const float f = p_s[kFewKeys * kFewRows + r];
+#pragma unroll
+        for (int u = 0; u < 2 * ND; ++u) acc[r][u] *= f;
+      }
+    }
+#pragma unroll 4
+    for (int k = 0; k < kFewKeys; ++k) {
+      const float4 pa = *reinterpret_cast<const float4*>(p_s + k * kFewRows), pb = *reinterpret_cast<const float4*>(p_s + k * kFewRows + 4);
+      const float pk[kFewRows] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+#pragma unroll
+      for (int u = 0; u < ND; ++u) {
+        const int c = 2 * lane + 64 * u;
+        const float2 v = c < d ? *reinterpret_cast<const float2*>(v_b + (warp * kFewKeys + k) * d + c) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < kFewRows; ++r)
+          if (pk[r] != 0.f) {                          // (a key the row does not keep is left out, whatever its V row holds)
+            acc[r][2 * u] = fmaf(pk[r], v.x, acc[r][2 * u]);
+            acc[r][2 * u + 1] = fmaf(pk[r], v.y, acc[r][2 * u + 1]);
+          }
+      }
+    }
+    __syncwarp();
+  };
+  if constexpr (PIPE) {
+    auto start = [&](const Stage& g, int buf) {
+      if (g.valid) {
+        load_stage_async(k_s + buf * stage, pitch, reinterpret_cast<const float*>(Kh), kst, g.j0, sq.S, d);
+        load_stage_async(v_s + buf * stage, d, reinterpret_cast<const float*>(Vh), vst, g.j0, sq.S, d);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    Stage cur, nxt;
+    find(cur);
+    start(cur, 0);
+    for (int buf = 0; cur.valid; buf ^= 1) {
+      find(nxt);
+      start(nxt, buf ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncthreads();
+      work(cur, k_s + buf * stage, v_s + buf * stage);
+      cur = nxt;
+    }
+  } else {
+    Stage cur;
+    for (find(cur); cur.valid; find(cur)) {
+      load_stage<T>(k_s, pitch, Kh, kst, cur.j0, sq.S, d);
+      load_stage<T>(v_s, d, Vh, vst, cur.j0, sq.S, d);
+      __syncthreads();
+      work(cur, k_s, v_s);
+    }
+  }
+  // merge of the eight warps: their references and sums, then their outputs, in the memory of the stages
+  l += __shfl_xor_sync(0xFFFFFFFFu, l, 1);
+  l += __shfl_xor_sync(0xFFFFFFFFu, l, 2);
+  __syncthreads();
+  float2* ml = reinterpret_cast<float2*>(q_s);                                 // [warp][row]
+  if ((lane & 3) == 0) ml[warp * kFewRows + my_row] = make_float2(m, l);
+#pragma unroll
+  for (int r = 0; r < kFewRows; ++r)
+#pragma unroll
+    for (int u = 0; u < ND; ++u) {
+      const int c = 2 * lane + 64 * u;
+      if (c < d) *reinterpret_cast<float2*>(smem + (warp * kFewRows + r) * d + c) = make_float2(acc[r][2 * u], acc[r][2 * u + 1]);
+    }
+  __syncthreads();
+  const int r = warp, i = i0 + r;                                              // a row per warp
+  if (i >= sq.S) return;
+  float M = -CUDART_INF_F, f[kRefWarps], sum = 0.f;
+#pragma unroll
+  for (int w = 0; w < kRefWarps; ++w) M = fmaxf(M, ml[w * kFewRows + r].x);
+#pragma unroll
+  for (int w = 0; w < kRefWarps; ++w) {
+    const float2 x = ml[w * kFewRows + r];
+    f[w] = x.x == -CUDART_INF_F ? 0.f : expf(x.x - M);
+    sum += x.y * f[w];
+  }
+  const float inv = sum > 0.f ? 1.0f / sum : 0.f;
+  T* orow = O + (int64_t)(sq.tok_start + i) * ost + (int64_t)h * osh;
+  for (int c = lane; c < d; c += 32) {
+    float o = 0.f;
+#pragma unroll
+    for (int w = 0; w < kRefWarps; ++w)
+      if (f[w] != 0.f) o = fmaf(f[w], smem[(w * kFewRows + r) * d + c], o);
+    Ld8<T>::store(orow + c, o * inv);
+  }
+  if (lane == 0) lse[(int64_t)h * total_tokens + sq.tok_start + i] = sum > 0.f ? M + logf(sum) : -CUDART_INF_F;
+}
+
+// Whether a call has many rows: `per` for every warp of a block of eight on every SM.  Scoring takes four rows per warp from
+// there on and one below, so that a short prompt's rows are spread over the whole chip (per = 4).  Attention has
+// attn_ref_few_kernel below per = 5 (fp32, head_dim 64, a warp per row, four rows per warp and it: 1400 rows 45.3, -, 33.5
+// us; 4000 54, -, 40; 4800 -, 62, 50; 6000 -, 62.4, 60.8; 8000 -, 62.5, 74.5).
+inline bool many_rows(long long rows, int sm_count, int per) { return rows >= (long long)sm_count * kRefWarps * per; }
 
 size_t score_smem(int d, int R, int nbuf) { return ((size_t)nbuf * kStageKeys * k_pitch(d) + (size_t)kRefWarps * R * d) * sizeof(float); }
 size_t attn_smem(int d, int R, int nbuf) {
+  if (R == 1)
+    return ((size_t)nbuf * kStageKeys * (k_pitch(d) + d) + (size_t)kFewRows * k_pitch(d) + kRefWarps * (kFewKeys + 1) * kFewRows) * sizeof(float);
   return ((size_t)nbuf * kStageKeys * (k_pitch(d) + d) + (size_t)kRefWarps * R * (d + kStageKeys)) * sizeof(float);
 }
 
@@ -383,13 +588,18 @@ cudaError_t opt_in_scores(int dev, size_t bytes) {
                             : dam_device_table().once(dev, key, []() -> cudaError_t { return allow_all_smem(scores_ref_kernel<T, R>); });
 }
 template <typename T, int R, int ND, bool PIPE>
+constexpr auto attn_kernel() {
+  if constexpr (R == 1) return attn_ref_few_kernel<T, ND, PIPE>;
+  else return attn_ref_kernel<T, R, 2 * ND, PIPE>;
+}
+template <typename T, int R, int ND, bool PIPE>
 cudaError_t opt_in_attn(int dev, size_t bytes) {
-  constexpr int dims = ND == 2 ? 0 : ND == 4 ? 1 : 2, type = PIPE ? 2 : sizeof(T) == 4;
+  constexpr int dims = ND == 1 ? 0 : ND == 2 ? 1 : 2, type = PIPE ? 2 : sizeof(T) == 4;
   constexpr int key = DAM_SETUP_REF_SMEM + 4 + (3 * type + dims) * 2 + (R == 4);
   static_assert(key < DamDeviceTable::kMaxSetups, "a set-up step per instance");
   return bytes <= 48 * 1024
              ? cudaSuccess
-             : dam_device_table().once(dev, key, []() -> cudaError_t { return allow_all_smem(attn_ref_kernel<T, R, ND, PIPE>); });
+             : dam_device_table().once(dev, key, []() -> cudaError_t { return allow_all_smem(attn_kernel<T, R, ND, PIPE>()); });
 }
 
 template <typename T, int R>
@@ -412,10 +622,10 @@ cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void*
                         float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int dev, int smem_max, cudaStream_t st) {
   const bool pipe = sizeof(T) == 4 && attn_smem(s->head_dim, R, 2) <= (size_t)smem_max;
   const size_t sm = attn_smem(s->head_dim, R, pipe ? 2 : 1);
-  auto kernel = attn_ref_kernel<T, R, ND, false>;
+  auto kernel = attn_kernel<T, R, ND, false>();
   cudaError_t e;
   if (sizeof(T) == 4 && pipe) {
-    if constexpr (sizeof(T) == 4) { kernel = attn_ref_kernel<T, R, ND, true>; e = opt_in_attn<T, R, ND, true>(dev, sm); }
+    if constexpr (sizeof(T) == 4) { kernel = attn_kernel<T, R, ND, true>(); e = opt_in_attn<T, R, ND, true>(dev, sm); }
   } else {
     e = opt_in_attn<T, R, ND, false>(dev, sm);
   }
@@ -433,10 +643,10 @@ cudaError_t launch_attn(const void* Q, const void* K, const void* V, const void*
 template <typename T, int R>
 cudaError_t launch_attn_dims(const void* Q, const void* K, const void* V, const void* blob, const dam_shape_t* s, int causal,
                              float scale, void* O, float* lse, const int32_t* ranges, const DamRowRanges& rr, uint32_t* scratch, int keep, int rows, int dev, int smem_max, cudaStream_t st) {
-  const int nd = (s->head_dim + 31) / 32;
+  const int nd = (s->head_dim + 63) / 64;
+  if (nd <= 1) return launch_attn<T, R, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
   if (nd <= 2) return launch_attn<T, R, 2>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
-  if (nd <= 4) return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
-  return launch_attn<T, R, 8>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
+  return launch_attn<T, R, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scratch, keep, rows, dev, smem_max, st);
 }
 
 }  // namespace
@@ -448,7 +658,7 @@ cudaError_t dam_launch_scores_ref(const void* Q, const void* K, const dam_shape_
   DamDeviceInfo di;
   cudaError_t e = dam_current_device(&dev, &di);
   if (e != cudaSuccess) return e;
-  const bool four = four_rows((long long)c.max_L * c.num_seqs * c.Hq, di.sm_count);
+  const bool four = many_rows((long long)c.max_L * c.num_seqs * c.Hq, di.sm_count, 4);
   if (c.dtype == DAM_F32)
     return four ? launch_scores<float, 4>(Q, K, s, c, dump, dev, di, st) : launch_scores<float, 1>(Q, K, s, c, dump, dev, di, st);
   return four ? launch_scores<__nv_bfloat16, 4>(Q, K, s, c, dump, dev, di, st) : launch_scores<__nv_bfloat16, 1>(Q, K, s, c, dump, dev, di, st);
@@ -469,7 +679,7 @@ cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, con
   DamDeviceInfo di;
   cudaError_t e = dam_current_device(&dev, &di);
   if (e != cudaSuccess) return e;
-  const bool four = four_rows((long long)rows * DAM_TILE, di.sm_count);
+  const bool four = many_rows((long long)rows * DAM_TILE, di.sm_count, 5);
   if (s->dtype == DAM_F32)
     return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st)
                 : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st);

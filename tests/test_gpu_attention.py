@@ -138,6 +138,17 @@ def test_cuda_core_kernels_every_row(S, pcl, d, dtype):
     _masked_case(w, _sample_rows(pcl) if S > 2000 else _all_rows)
 
 
+@pytest.mark.parametrize("lengths,pcl,d,dtype", [
+    ([9], 9, 64, torch.float32), ([77, 1, 130], 40, 72, torch.bfloat16), ([200, 500], 64, 200, torch.float32),
+    ([2900], 100, 24, torch.float32), ([3000], 100, 24, torch.float32),   # 5888 and 6144 rows: on either side of the line
+])
+def test_cuda_core_attention_of_few_rows(lengths, pcl, d, dtype):
+    """Eight rows per block, the keys of a stage dealt over its warps: remainders of rows, keys and dimensions, keys that no
+    row of a warp keeps, and the sizes around the change to four rows per warp."""
+    w = synth.small_case(0, 2, 1, d, pcl, seed=15, dtype=dtype, lengths=lengths)
+    _masked_case(w, _sample_rows(pcl) if max(lengths) > 2000 else _all_rows)
+
+
 @pytest.mark.parametrize("gather", [False, True])
 @pytest.mark.parametrize("lengths,pcl,Hq,Hkv,d", [
     ([1700], 384, 4, 2, 128),                # the lone diagonal crosses two tiles of every block
