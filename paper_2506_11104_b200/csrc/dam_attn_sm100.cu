@@ -532,9 +532,12 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           sc += (d & kStepDual) ? 2u : 1u;
         }
         sk = sc;
-        const bool early = mbar_try_wait(bSlotFull + 8 * (sk % kSlots), (sk / kSlots) & 1u);
-        if (early) dn = step_desc[step & 15u];
-        if (d && !(ok = slot_wait(sv))) break;
+        // K is waited for only when no P V is left to issue (d = 0): behind an item's last step its K may come from a
+        // record that the output warps free, and they wait for that step's P V of either stream.  A step whose next K is
+        // late is a trip of its own (dn = 0), and S of the next one another (d = 0).
+        bool have = mbar_try_wait(bSlotFull + 8 * (sk % kSlots), (sk / kSlots) & 1u);
+        if (d ? !(ok = slot_wait(sv)) : !have && !(ok = have = slot_wait(sk))) break;
+        dn = have ? step_desc[step & 15u] : 0u;
 #pragma unroll
         for (int X = 0; X < 2; ++X) {
           const uint32_t dx = d >> X, bX = 8 * X;
@@ -556,12 +559,14 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (dx & kStepLast) tc_commit(bOFinal + bX);
           }
           if (X == 0) {
-            if (!early) {
-              if (!(ok = slot_wait(sk))) break;
+            if (!have && !(d & 2u * kStepLast)) {
+              if (!(ok = have = slot_wait(sk))) break;
               dn = step_desc[step & 15u];
             }
-            ++step;
-            sc += (dn & kStepDual) ? 2u : 1u;
+            if (have) {
+              ++step;
+              sc += (dn & kStepDual) ? 2u : 1u;
+            }
           }
           const uint32_t nx = dn >> X, k = X && (dn & kStepDual) ? sk + 1u : sk;
           if (X && (dn & kStepDual) && !(ok = slot_wait(k))) break;
@@ -581,7 +586,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (nx & kStepLast) tc_commit(bQEmpty + bX);
           }
           if (X ? d != 0u : (d & kStepDual) != 0u) slot_free(v);
-          if (X ? !(dn & kStepEnd) : (dn & kStepDual) != 0u) slot_free(k);
+          if (X ? have && !(dn & kStepEnd) : (dn & kStepDual) != 0u) slot_free(k);
         }
         if (!ok || (dn & kStepEnd)) break;
         d = dn;

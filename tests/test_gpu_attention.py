@@ -448,6 +448,23 @@ def test_output_rows_of_any_alignment(d, offset, row_pad, head_pad):
 
 
 @pytest.mark.parametrize("gather", [False, True])
+@pytest.mark.parametrize("d", [64, 128])
+def test_empty_items_behind_an_item_with_tiles(d, gather):
+    """No pattern matches: 16 items with tiles in both blocks, then more than eight empty ones per multiprocessor, so the next
+    key tile (or the end of the list) comes three records or more behind a last step.  Every row is written, over the whole
+    batch and over row ranges."""
+    S = 20000
+    w = synth.small_case(0, 16, 4, d, 256, seed=23, lengths=[S], mu=1.5)
+    blob, shape, masks, O, lse, _ = _masked_case(w, _sample_rows(256, 64, 2), heads=[0, 7, 15], gather=gather, sentinel=True)
+    assert torch.isneginf(lse[:, 256:]).all() and torch.isfinite(lse[:, 0]).all()
+    Q, K, V = w.Q.to(DEV), w.K.to(DEV), w.V.to(DEV)
+    Or, lr = torch.full_like(O, float("nan")), torch.full_like(lse, float("nan"))
+    for r in [(0, 9984), (9984, S)]:
+        assert B.dam_poll_status(B.dam_sparse_attention_rows(Q, K, V, blob, shape, [r], Or, lr)) == 0
+    assert torch.equal(Or, O) and torch.equal(lr, lse)
+
+
+@pytest.mark.parametrize("gather", [False, True])
 def test_degenerate_lengths(gather):
     """Empty and one-token sequences inside a packed batch, a sequence shorter than a tile, MHA (group 1)."""
     w = synth.small_case(0, 4, 4, 128, 64, seed=17, lengths=[0, 1, 5, 0, 257, 128])
