@@ -532,9 +532,9 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
           sc += (d & kStepDual) ? 2u : 1u;
         }
         sk = sc;
-        // K is waited for only when no P V is left to issue (d = 0): behind an item's last step its K may come from a
-        // record that the output warps free, and they wait for that step's P V of either stream.  A step whose next K is
-        // late is a trip of its own (dn = 0), and S of the next one another (d = 0).
+        // K that is late is waited for between the P V of A and of B, but not behind B's last tile: the next K may then come
+        // from a record that the output warps free, and they wait for that P V.  Such a step is a trip of its own (dn = 0),
+        // S of the next one another (d = 0).  Never waiting there costs 8192 tokens 84.3 -> 86.6 us.
         bool have = mbar_try_wait(bSlotFull + 8 * (sk % kSlots), (sk / kSlots) & 1u);
         if (d ? !(ok = slot_wait(sv)) : !have && !(ok = have = slot_wait(sk))) break;
         dn = have ? step_desc[step & 15u] : 0u;
