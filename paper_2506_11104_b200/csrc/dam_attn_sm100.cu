@@ -203,14 +203,16 @@ __device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1, f
 
 // 2^y for a pair of values on the FMA / ALU pipes instead of the special-function unit: split y into its
 // nearest integer (added to the exponent field) and a remainder in [-0.5, 0.5] (degree-3 minimax polynomial,
-// relative error 7.6e-5, far below the bf16 rounding of P).  y comes as z = (y + 125) / 250, saturated to [0, 1] by the multiply-add
-// that makes it: so the exponent stays in range without a comparison (an underflowing probability is 2^-125 instead of 0).
-__device__ __forceinline__ void ex2_poly2(float z0, float z1, float& p0, float& p1) {
-  const float kMagic = 12582912.f - 125.f;    // 1.5 * 2^23 - 125: 250 z added to it leaves round(y) in the low mantissa bits
+// relative error 7.6e-5, far below the bf16 rounding of P).  y is the fp32 argument the special-function unit gets, rounded
+// once, however large the logits are.  It is clamped at -125 so that the exponent stays in range; that turns an underflowing
+// probability into 2^-125 instead of 0.
+__device__ __forceinline__ void ex2_poly2(float y0, float y1, float& p0, float& p1) {
+  const float kMagic = 12582912.f;    // 1.5 * 2^23: adding it leaves round(y) in the low mantissa bits
+  y0 = fmaxf(y0, -125.f); y1 = fmaxf(y1, -125.f);
   float r0, r1, i0, i1, f0, f1, q0, q1;
-  fma2(r0, r1, z0, z1, 250.f, 250.f, kMagic, kMagic);
-  add2(i0, i1, r0, r1, -kMagic, -kMagic);     // round(y) + 125
-  fma2(f0, f1, z0, z1, 250.f, 250.f, -i0, -i1);
+  add2(r0, r1, y0, y1, kMagic, kMagic);
+  add2(i0, i1, r0, r1, -kMagic, -kMagic);
+  add2(f0, f1, y0, y1, -i0, -i1);
   fma2(q0, q1, f0, f1, 0.05520550534129143f, 0.05520550534129143f, 0.24261397123336792f, 0.24261397123336792f);
   fma2(q0, q1, q0, q1, f0, f1, 0.6932547688484192f, 0.6932547688484192f);
   fma2(q0, q1, q0, q1, f0, f1, 0.9999276995658875f, 0.9999276995658875f);
@@ -220,11 +222,6 @@ __device__ __forceinline__ void ex2_poly2(float z0, float z1, float& p0, float& 
   asm("mad.lo.s32 %0, %1, 8388608, %2;" : "=r"(b1) : "r"(__float_as_int(r1)), "r"(__float_as_int(q1)));
   p0 = __int_as_float(b0);
   p1 = __int_as_float(b1);
-}
-__device__ __forceinline__ float fma_sat(float a, float b, float c) {
-  float r;
-  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
 }
 
 // Sweep 1 over one S row held in TMEM (4 chunks of 32 columns, next chunk in flight while one is reduced).
@@ -282,20 +279,19 @@ __device__ __forceinline__ float sweep_max_masked(uint32_t tS, uint4 bits) {
 
 // 32 probabilities p = 2^(s * scale + neg_m), zero where the mask bit is clear, packed to bf16; their sums are taken in fp32,
 // before the bf16 rounding.  Of every 8, 6 go through the special-function unit and 2 through the polynomial.
-__device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, float scale, float neg_m, float scale_z, float neg_z, uint32_t* pk,
+__device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, float scale, float neg_m, uint32_t* pk,
                                           float& s0, float& s1, float& s2, float& s3) {
 #pragma unroll
   for (int q = 0; q < 32; q += 8) {
     float y[8], p[8];
     constexpr int kEx2 = 8 - kPolyPer8;
 #pragma unroll
-    for (int u = 0; u < kEx2; u += 2)
+    for (int u = 0; u < 8; u += 2)
       fma2(y[u], y[u + 1], __uint_as_float(cur[q + u]), __uint_as_float(cur[q + u + 1]), scale, scale, neg_m, neg_m);
 #pragma unroll
     for (int u = 0; u < kEx2; ++u) p[u] = ex2(y[u]);
 #pragma unroll
-    for (int u = kEx2; u < 8; u += 2)
-      ex2_poly2(fma_sat(__uint_as_float(cur[q + u]), scale_z, neg_z), fma_sat(__uint_as_float(cur[q + u + 1]), scale_z, neg_z), p[u], p[u + 1]);
+    for (int u = kEx2; u < 8; u += 2) ex2_poly2(y[u], y[u + 1], p[u], p[u + 1]);
 #pragma unroll
     for (int u = 0; u < 8; ++u) p[u] = ((word >> (q + u)) & 1u) ? p[u] : 0.f;
     add2(s0, s1, s0, s1, p[0], p[1]);
@@ -321,15 +317,14 @@ __device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, fl
 // polynomial as it is now).
 __device__ __forceinline__ float sweep_exp(uint32_t tS, const uint4& bits, int lo, int hi, float scale, float neg_m) {
   float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-  const float scale_z = scale * 0.004f, neg_z = fmaf(neg_m, 0.004f, 0.5f);      // (y + 125) / 250
 #pragma unroll 1
   for (int h = lo; h < hi; ++h) {
     uint32_t ra[32], rb[32], pk[32];
     tmem_ld32(tS + 64 * h, ra);
     tmem_ld32(tS + 64 * h + 32, rb);
     tc_wait_ld();
-    exp_chunk(ra, h ? bits.z : bits.x, scale, neg_m, scale_z, neg_z, pk, s0, s1, s2, s3);
-    exp_chunk(rb, h ? bits.w : bits.y, scale, neg_m, scale_z, neg_z, pk + 16, s0, s1, s2, s3);
+    exp_chunk(ra, h ? bits.z : bits.x, scale, neg_m, pk, s0, s1, s2, s3);
+    exp_chunk(rb, h ? bits.w : bits.y, scale, neg_m, pk + 16, s0, s1, s2, s3);
     tmem_st32(tS + 32 * h, pk);
   }
   if (hi - lo < 2) {

@@ -105,6 +105,31 @@ def _masked_case(w, rows_for, heads=None, gather=False, sentinel=False):
     return blob, shape, masks, O, lse, worst
 
 
+@pytest.mark.parametrize("d", [64, 128])
+def test_every_column_has_the_same_scale_at_large_logits(d):
+    """Eight adjacent keys share a logit, V sets one of the eight against the others: O is zero unless some columns of a tile
+    get other probabilities than their neighbours.  Logits reach 11700 in log2 units, where an argument that is not rounded
+    once, in fp32, is off by a share of that.  Bound: 7 / 8 of the polynomial's 7.6e-5, and 8192 roundings of P to bf16 (rms
+    1.1e-3 each), averaged: 2.7 * 1.1e-3 / sqrt(8192) = 3.3e-5."""
+    n = 8192
+    rng = np.random.default_rng(3)
+    Q = torch.zeros(n, 1, d)
+    Q[:, 0, 0] = torch.arange(n) % 255
+    Q[:, 0, 1:3] = 1.0
+    K = torch.zeros(n, 1, d)
+    K[:, 0, 0] = 256.0                                                  # every product and sum of a logit is exact
+    K[:, 0, 1] = -torch.from_numpy(np.repeat(rng.integers(0, 128, n // 8), 8)) / 8.0
+    K[:, 0, 2] = -torch.from_numpy(np.repeat(rng.integers(0, 16, n // 8), 8)) / 128.0
+    V = torch.zeros(n, 1, d)
+    V[:, 0, :8] = -1.0
+    V[torch.arange(n), 0, torch.arange(n) % 8] = 7.0
+    Q, K, V = (x.to(torch.bfloat16).to(DEV) for x in (Q, K, V))
+    shape = B.make_shape([0, n], 1, 1, d, torch.bfloat16, DEV)
+    O, lse, scr = B.dam_sparse_attention(Q, K, V, B.dam_mask_all_ones(shape, False, DEV), shape, causal=False, softmax_scale=0.125)
+    assert B.dam_poll_status(scr) == 0 and B.attention_ran_on_tensor_cores(scr)
+    assert O.float().abs().max() <= 1e-4
+
+
 def test_config0_every_row():
     w = synth.config0()
     blob, shape, masks, O, lse, worst = _masked_case(w, _all_rows)
