@@ -921,10 +921,9 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     }
   }
 
-  if (*abort_flag && tid == 64) atomicMax(prm.status, (uint32_t)DAM_ERR_DEVICE_TIMEOUT);
   if (blockIdx.x == 0 && tid == 64) prm.status[3] = 1u;      // word 4 of the scratch block: which kernel served the call
   tc_fence_before();
-  __syncthreads();
+  report_expired_wait(abort_flag, prm.status, DAM_ERR_DEVICE_TIMEOUT);
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
@@ -1025,8 +1024,9 @@ __global__ void clear_status_kernel(uint32_t* scratch, int keep) {
 }
 
 // Self-test of the bounded wait every kernel in this library uses: waits on an mbarrier that nothing ever
-// arrives on, twenty thousand polls at a time, until the given limit is over; every wait gives up, the status word is set and the
-// kernel returns normally.
+// arrives on, twenty thousand polls at a time, until the given limit is over; every wait gives up, the status word is set the way
+// those kernels set it and the kernel returns normally.  The waiting thread is in the second warp; the first one, whose thread
+// writes the status word, has nothing to do.
 __global__ void bounded_wait_selftest_kernel(uint32_t* status, unsigned long long limit_ns, unsigned long long* waited_ns) {
   __shared__ uint64_t bar;
   __shared__ uint32_t abort_flag;
@@ -1034,19 +1034,22 @@ __global__ void bounded_wait_selftest_kernel(uint32_t* status, unsigned long lon
     mbar_init(smem_u32(&bar), 1);
     abort_flag = 0u;
     mbar_fence_init();
+  }
+  __syncthreads();
+  if (threadIdx.x == 32) {
     const uint64_t t0 = globaltimer_ns();
     bool ok;
     do ok = mbar_wait(smem_u32(&bar), 0u, &abort_flag, 20000u);
     while (!ok && globaltimer_ns() - t0 < limit_ns);
     *waited_ns = globaltimer_ns() - t0;
-    if (!ok && abort_flag) atomicMax(status, (uint32_t)DAM_ERR_DEVICE_TIMEOUT);
   }
+  report_expired_wait(&abort_flag, status, DAM_ERR_DEVICE_TIMEOUT);
 }
 
 }  // namespace
 
 cudaError_t dam_launch_bounded_wait_selftest(void* scratch, unsigned long long limit_ns, cudaStream_t st) {
-  bounded_wait_selftest_kernel<<<1, 32, 0, st>>>(reinterpret_cast<uint32_t*>(scratch) + 1, limit_ns,
+  bounded_wait_selftest_kernel<<<1, 64, 0, st>>>(reinterpret_cast<uint32_t*>(scratch) + 1, limit_ns,
                                                   reinterpret_cast<unsigned long long*>(scratch) + 1);
   return cudaGetLastError();
 }

@@ -399,9 +399,8 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     }
   }
 
-  if (*abort_flag && tid == 64) atomicMax(prm.status, (uint32_t)DAM_ERR_DEVICE_TIMEOUT);
   tc_fence_before();
-  __syncthreads();
+  report_expired_wait(abort_flag, prm.status, DAM_ERR_DEVICE_TIMEOUT);
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 

@@ -71,6 +71,12 @@ __device__ __forceinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, vo
     }
   }
 }
+// The end of a kernel with bounded waits, by all threads of the CTA.  The flag is read when every role has left: one role may wait,
+// and give up, long after another has done its part.
+__device__ __forceinline__ void report_expired_wait(const volatile uint32_t* abort_flag, uint32_t* status, uint32_t code) {
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) atomicMax(status, code);
+}
 constexpr uint32_t kDrainPolls = 1000000u;      // 20 ms and more: a copy that has been issued lands
 
 // ---- TMA ----------------------------------------------------------------------------------------

@@ -413,8 +413,8 @@ def test_threads_with_different_shared_memory_sizes():
 
 
 def test_bounded_wait_times_out_cleanly():
-    """A wait that nothing satisfies gives up after its limit, the status word says so, and the device keeps
-    working (the next kernel runs and is correct)."""
+    """A wait that nothing satisfies gives up after its limit, the status word says so although the thread that writes it has
+    long been done, and the device keeps working (the next kernel runs and is correct)."""
     status, waited_ns = B.dam_selftest_bounded_wait(DEV, limit_us=20000)
     assert status == 5                                   # DAM_ERR_DEVICE_TIMEOUT
     assert 15e6 <= waited_ns <= 500e6
