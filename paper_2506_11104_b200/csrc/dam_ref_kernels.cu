@@ -546,7 +546,9 @@ attn_ref_few_kernel(const unsigned char* blob, const T* __restrict__ Q, const T*
     f[w] = x.x == -CUDART_INF_F ? 0.f : expf(x.x - M);
     sum += x.y * f[w];
   }
-  const float inv = sum > 0.f ? 1.0f / sum : 0.f;
+  // (zero without a key.  A NaN stays one: a warp whose only key has a NaN logit has no reference, its output is left out below, but
+  // its sum is NaN)
+  const float inv = sum > 0.f ? 1.0f / sum : sum;
   T* orow = O + (int64_t)(sq.tok_start + i) * ost + (int64_t)h * osh;
   for (int c = lane; c < d; c += 32) {
     float o = 0.f;

@@ -174,6 +174,35 @@ def test_cuda_core_attention_of_few_rows(lengths, pcl, d, dtype):
     _masked_case(w, _sample_rows(pcl) if max(lengths) > 2000 else _all_rows)
 
 
+def _one_odd_key(n, key, value):
+    """fp32 attention of n rows (two heads, lower-triangular) with one logit of every row replaced: Q, K, V on the device, O, LSE
+    and the float64 outputs without that key."""
+    g = torch.Generator().manual_seed(31)
+    Q, K, V = (torch.randn(n, 2, 64, generator=g) for _ in range(3))
+    Q[:, :, 0] = 1.0
+    K[key, :, 0] = value
+    Q, K, V = (x.to(DEV) for x in (Q, K, V))
+    shape = B.make_shape([0, n], 2, 2, 64, torch.float32, DEV)
+    O, lse, scr = B.dam_sparse_attention(Q, K, V, B.dam_mask_all_ones(shape, True, DEV), shape)
+    assert B.dam_poll_status(scr) == 0
+    logits = torch.einsum("ihd,jhd->hij", Q.double(), K.double()) / 8.0
+    keep = torch.ones(n, n, dtype=torch.bool, device=DEV).tril()
+    keep[:, key] = False
+    P = torch.where(keep, logits, float("-inf")).softmax(-1).nan_to_num(0.0)       # (a row without any other key)
+    return O.double(), lse, torch.einsum("hij,jhd->ihd", P, V.double())
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("key", [8, 65])
+@pytest.mark.parametrize("n", [200, 3000])        # eight rows to a block, four rows to a warp
+def test_cuda_core_attention_keeps_a_nan(n, key, value):
+    """A NaN logit, or one of +inf, makes its rows NaN, also where a warp has no other key in the row; the rows in front of it
+    are not touched."""
+    O, lse, ref = _one_odd_key(n, key, value)
+    assert torch.isnan(O[key:]).all()
+    assert (O[:key] - ref[:key]).abs().max() <= 1e-4 and torch.isfinite(lse[:, :key]).all()
+
+
 @pytest.mark.parametrize("gather", [False, True])
 @pytest.mark.parametrize("lengths,pcl,Hq,Hkv,d", [
     ([1700], 384, 4, 2, 128),                # the lone diagonal crosses two tiles of every block
