@@ -284,8 +284,9 @@ attn_ref_kernel(const unsigned char* blob, const T* __restrict__ Q, const T* __r
       const bool a0 = (g.w0[r] >> lane) & 1u, a1 = (g.w1[r] >> lane) & 1u;
       const float x0 = a0 ? s[r][0] * scale : -CUDART_INF_F, x1 = a1 ? s[r][1] * scale : -CUDART_INF_F;
       const float mn = fmaxf(m[r], warp_max(fmaxf(x0, x1)));
-      const float corr = (m[r] == -CUDART_INF_F) ? 0.f : expf(m[r] - mn);
-      const float p0 = a0 ? expf(x0 - mn) : 0.f, p1 = a1 ? expf(x1 - mn) : 0.f;
+      // (an infinite maximum counts as zero: a row without a key so far, or whose logits are all -inf)
+      const float at = mn == -CUDART_INF_F ? 0.f : mn, corr = expf(m[r] - at);
+      const float p0 = a0 ? expf(x0 - at) : 0.f, p1 = a1 ? expf(x1 - at) : 0.f;
       l[r] = l[r] * corr + warp_sum(p0 + p1);
       m[r] = mn;
 #pragma unroll

@@ -203,6 +203,15 @@ def test_cuda_core_attention_keeps_a_nan(n, key, value):
     assert (O[:key] - ref[:key]).abs().max() <= 1e-4 and torch.isfinite(lse[:, :key]).all()
 
 
+@pytest.mark.parametrize("key", [0, 8, 65])
+@pytest.mark.parametrize("n", [200, 3000])
+def test_cuda_core_attention_leaves_out_a_logit_of_minus_infinity(n, key):
+    """A logit of -inf has no weight, also where it is the first of its row or the row's only one (O = 0, LSE = -inf)."""
+    O, lse, ref = _one_odd_key(n, key, float("-inf"))
+    assert (O - ref).abs().max() <= 1e-4
+    assert torch.equal(torch.isneginf(lse), (torch.arange(n, device=DEV) == 0).expand(2, n) & (key == 0))
+
+
 @pytest.mark.parametrize("gather", [False, True])
 @pytest.mark.parametrize("lengths,pcl,Hq,Hkv,d", [
     ([1700], 384, 4, 2, 128),                # the lone diagonal crosses two tiles of every block
