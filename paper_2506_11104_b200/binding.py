@@ -455,6 +455,11 @@ class MaskBlob:
         """Test hook: the window map of this blob was computed by the tcgen05 scoring kernel."""
         return int(self.hdr["reserved"][0]) == 1
 
+    @property
+    def scoring_groups(self) -> int:
+        """Test hook: softmax groups of that kernel's CTAs, 4 (one CTA per SM) or 2 (two)."""
+        return int(self.hdr["reserved"][1])
+
     def pattern_bits(self, seq: int, head: int):
         """(D, Drev, V) as uint8 [L]."""
         s = self.seqs[seq]

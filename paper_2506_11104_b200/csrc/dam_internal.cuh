@@ -69,7 +69,7 @@ struct DamHeader {
   uint64_t attn_scratch_bytes;   // scratch dam_sparse_attention needs for this blob
   uint64_t mask_tiles;      // 128 x 128 tiles of the masks that hold an active cell (= total_tiles unless gathered)
   uint64_t head_tile_cap;   // entries of tiles[] every head owns (sum of the row bounds of all sequences)
-  uint64_t reserved[7];     // [0]: 1 when the window map was scored by the tensor-core kernel (test hook)
+  uint64_t reserved[7];     // [0]: 1 when the window map was scored by the tensor-core kernel, [1]: the softmax groups of its CTAs (test hooks)
   uint64_t off_lone;        // 0: no section (all-ones blob)
   uint64_t off_cols;        // 0: no section (all-ones blob, or no gathered columns)
   uint64_t off_lone2;       // (0; blobs of an earlier build have 8-byte records of the lone diagonals here, which are not read)

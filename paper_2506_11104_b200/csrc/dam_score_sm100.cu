@@ -141,7 +141,10 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   const uint32_t tmem = *tmem_slot;
   // everything above is independent of the kernel before this one; the blob it initialises is read from here on
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (blockIdx.x == 0 && tid == 0) reinterpret_cast<DamHeader*>(blob)->reserved[0] = 1ull;   // the map of this blob was scored on the tensor cores
+  if (blockIdx.x == 0 && tid == 0) {
+    reinterpret_cast<DamHeader*>(blob)->reserved[0] = 1ull;          // the map of this blob was scored on the tensor cores
+    reinterpret_cast<DamHeader*>(blob)->reserved[1] = kGroups;
+  }
 
   if (warp == 0) {
     if (elect_one()) {              // (elected, not lane 0: PCL 4096 292 -> 274 us for stage 1, PCL 2048 97.6 -> 95.8 us)
@@ -404,6 +407,28 @@ score_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
+// Two CTAs per SM with two softmax groups each, or one with four.  The four groups of
+// a CTA are in the same sweep of the same item: first they all want the special-function unit, then the integer pipe, then
+// all wait at the merge or for the next query tile; two items side by side fill each other's gaps, but an item takes
+// longer.  So two from three items per SM on, four for windows of more than 16 tiles.  Stage 1, one and two CTAs per SM: 256 items of up to 8 tiles (8192 tokens) 40.5 and 47.8 us, 256 of 16 tiles 53.9
+// and 70.5, 384 67.8 and 70.5, 512 (32768 tokens) 79.8 and 76.9, 1024 of up to 32 (131072 tokens) 232 and 217, 1536 (mixed
+// lengths) 140 and 126, 1024 of 4 with the map written 112 and 106; 512 of up to 32 tiles 125.6 and 129.2, 768 169 and 156.
+// In a batch of several lengths the items are counted by their tiles, in units of what an item of the longest window has on
+// average: one window of 2048 tokens and 15 prompts of 100 (8 heads, 248 items, but 142 such units) 68.0 and 86.2 us, with 9 of 1000 (704
+// items, 433 units) 85.5 and 80.4.  A place of the list without an item costs a CTA a claim, which two share: a twelfth of a
+// unit (one window of 2048 and 20 of 500: 316 units, 1920 empty places 92.6 and 88.3; 2 of 2048 and 15 of 100: 271, 1800 87.1 and
+// 91.2; 2 and 30: 284, 3600 120.4 and 114.5).
+inline bool two_ctas(const dam_shape_t* s, const DamBuildCtx& c, int sm_count) {
+  int64_t tiles = 0, items = 0;
+  for (int b = 0; b < s->num_seqs; ++b) {
+    const int64_t S = s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b], nL = ((S < c.pcl_max ? S : c.pcl_max) + DAM_TILE - 1) / DAM_TILE;
+    items += nL;
+    tiles += nL * (nL + 1) / 2;
+  }
+  const int64_t empty = ((int64_t)c.max_nL * c.num_seqs - items) * c.Hq;
+  return 24 * tiles * c.Hq / (c.max_nL + 1) + empty >= 12 * (c.max_nL <= 16 ? 3 : 4) * (int64_t)sm_count;
+}
+
 }  // namespace
 
 cudaError_t dam_launch_scores_sm100(const void* Q, const void* K, const dam_shape_t* s, const DamBuildCtx& c,
@@ -446,14 +471,7 @@ cudaError_t dam_launch_scores_sm100(const void* Q, const void* K, const dam_shap
   }
   p.dump_vec8 = vec8 ? 1 : 0;
   const int items = c.max_nL * c.num_seqs * c.Hq;
-  // Two CTAs per SM with two softmax groups each, from three items per SM on; below that one CTA with four.  The four groups of
-  // a CTA are in the same sweep of the same item: first they all want the special-function unit, then the integer pipe, then
-  // all wait at the merge or for the next query tile; two items side by side fill each other's gaps, but an item takes
-  // longer.  Stage 1, one and two CTAs per SM: 256 items of up to 8 tiles (8192 tokens) 40.5 and 47.8 us, 256 of 16 tiles 53.9
-  // and 70.5, 384 67.8 and 70.5, 512 (32768 tokens) 79.8 and 76.9, 1024 of up to 32 (131072 tokens) 232 and 217, 1536 (mixed
-  // lengths) 140 and 126, 1024 of 4 with the map written 112 and 106.  Windows of more than 16 tiles want four items per SM
-  // (512 of up to 32 tiles 125.6 and 129.2, 768 169 and 156).
-  const bool two = items >= (c.max_nL <= 16 ? 3 : 4) * sm_count;
+  const bool two = two_ctas(s, c, sm_count);
   const int ctas = two ? 2 * sm_count : sm_count, grid = items < ctas ? items : ctas;
   // launched as a programmatic dependent of the kernel that initialises the blob: its launch latency and its
   // prologue (barriers, TMEM, descriptors) hide under that kernel; it waits before it reads the blob

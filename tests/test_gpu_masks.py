@@ -224,6 +224,27 @@ def test_scoring_with_one_and_two_blocks_per_multiprocessor(d, seqs):
     assert flipped <= 2e-3 * total
 
 
+@pytest.mark.parametrize("lengths,pcl,heads,groups", [
+    ([2048] + [100] * 15, 2048, 8, 4),       # 2048 places, but the one long window is what takes the time
+    ([2048] * 3 + [100] * 15, 2048, 8, 2),
+    ([2300], 2432, 32, 4), ([2400], 2432, 32, 2),       # windows of more than 16 tiles: on either side of four items per multiprocessor
+])
+def test_scoring_blocks_follow_the_work_of_a_batch(lengths, pcl, heads, groups):
+    """How many blocks share a multiprocessor is decided by the tiles there are to score, not by the places of the work list."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the sizes are chosen for 148 multiprocessors")
+    w = synth.small_case(0, heads, heads // 4, 64, pcl, seed=len(lengths), lengths=lengths)
+    shape = _shape(w)
+    dump = torch.zeros(sum(heads * min(S, pcl) ** 2 for S in lengths), dtype=torch.float32, device=DEV)
+    blob, _ = B.dam_build_masks(w.Q.to(DEV), w.K.to(DEV), shape, _rule(w), scores_dump=dump)
+    assert B.dam_poll_status(blob) == 0
+    assert B.MaskBlob(blob).scoring_groups == groups
+    masks = H.oracle_masks_from_dump(w, dump.cpu().numpy(), heads=[0, heads - 1])
+    H.check_blob_against_oracle(blob, shape, masks, qblocks_per_head=4)
+    flipped, total = _score_closeness(w, dump, masks, [0, heads - 1])
+    assert flipped <= 2e-3 * total
+
+
 @pytest.mark.parametrize("gather", GATHER)
 def test_config1_full_size_masks(gather):
     """Llama-3-8B-shaped layer, 8192 tokens, PCL 1024: every head's D, V and true mask, sampled q-blocks."""
