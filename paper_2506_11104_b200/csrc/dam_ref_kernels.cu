@@ -561,11 +561,17 @@ attn_ref_few_kernel(const unsigned char* blob, const T* __restrict__ Q, const T*
   if (lane == 0) lse[(int64_t)h * total_tokens + sq.tok_start + i] = sum > 0.f ? M + logf(sum) : -CUDART_INF_F;
 }
 
-// Whether a call has many rows: `per` for every warp of a block of eight on every SM.  Scoring takes four rows per warp from
-// there on and one below, so that a short prompt's rows are spread over the whole chip (per = 4).  Attention has
-// attn_ref_few_kernel below per = 5 (fp32, head_dim 64, a warp per row, four rows per warp and it: 1400 rows 45.3, -, 33.5
-// us; 4000 54, -, 40; 4800 -, 62, 50; 6000 -, 62.4, 60.8; 8000 -, 62.5, 74.5).
-inline bool many_rows(long long rows, int sm_count, int per) { return rows >= (long long)sm_count * kRefWarps * per; }
+// Whether a call has many rows: `halves` / 2 for every warp of a block of eight on every SM.  Scoring takes four rows per warp
+// from there on and one below, so that a short prompt's rows are spread over the whole chip (four for every warp).
+inline bool many_rows(long long rows, int sm_count, int halves) { return 2 * rows >= (long long)sm_count * kRefWarps * halves; }
+// Attention takes four rows per warp from five rows for every warp on, attn_ref_few_kernel below (fp32, head_dim 64, a warp per
+// row, four rows per warp and it: 1400 rows 45.3, -, 33.5 us; 4000 54, -, 40; 4800 -, 62, 50; 6000 -, 62.4, 60.8; 8000 -, 62.5,
+// 74.5; bf16, head_dim 40, 5800 -, 55.6, 37.3).  With a head_dim above 64 there is a block of the latter to an SM instead of
+// three, and the line is at two and a half (2 heads, windows of 128, four rows per warp and it: 2560 rows fp32 head_dim 96 45.3 and
+// 42.5, 128 51.5 and 49.4, 192 78.1 and 67.9, 256 92.4 and 102.6, bf16 96 47.0 and 47.4, 256 92.5 and 103; 3072 rows 45.3 and 48.5,
+// 51.5 and 55.9, 78.1 and 78.1, 92.4 and 119, 46.2 and 54.3, 93.9 and 121; 4608 rows fp32 128 51.5 and 75.9, bf16 96 47.4 and 71.9;
+// 5888 rows fp32 192 148 and 129, 256 174 and 197, bf16 96 62.7 and 88.5).
+inline int attn_halves(int head_dim) { return head_dim <= 64 ? 10 : 5; }
 
 size_t score_smem(int d, int R, int nbuf) { return ((size_t)nbuf * kStageKeys * k_pitch(d) + (size_t)kRefWarps * R * d) * sizeof(float); }
 size_t attn_smem(int d, int R, int nbuf) {
@@ -661,7 +667,7 @@ cudaError_t dam_launch_scores_ref(const void* Q, const void* K, const dam_shape_
   DamDeviceInfo di;
   cudaError_t e = dam_current_device(&dev, &di);
   if (e != cudaSuccess) return e;
-  const bool four = many_rows((long long)c.max_L * c.num_seqs * c.Hq, di.sm_count, 4);
+  const bool four = many_rows((long long)c.max_L * c.num_seqs * c.Hq, di.sm_count, 8);
   if (c.dtype == DAM_F32)
     return four ? launch_scores<float, 4>(Q, K, s, c, dump, dev, di, st) : launch_scores<float, 1>(Q, K, s, c, dump, dev, di, st);
   return four ? launch_scores<__nv_bfloat16, 4>(Q, K, s, c, dump, dev, di, st) : launch_scores<__nv_bfloat16, 1>(Q, K, s, c, dump, dev, di, st);
@@ -682,7 +688,7 @@ cudaError_t dam_launch_attn_ref(const void* Q, const void* K, const void* V, con
   DamDeviceInfo di;
   cudaError_t e = dam_current_device(&dev, &di);
   if (e != cudaSuccess) return e;
-  const bool four = many_rows((long long)rows * DAM_TILE, di.sm_count, 5);
+  const bool four = many_rows((long long)rows * DAM_TILE, di.sm_count, attn_halves(s->head_dim));
   if (s->dtype == DAM_F32)
     return four ? launch_attn_dims<float, 4>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st)
                 : launch_attn_dims<float, 1>(Q, K, V, blob, s, causal, scale, O, lse, ranges, rr, scr, keep, rows, dev, di.smem_optin, st);

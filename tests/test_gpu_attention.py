@@ -166,6 +166,8 @@ def test_cuda_core_kernels_every_row(S, pcl, d, dtype):
 @pytest.mark.parametrize("lengths,pcl,d,dtype", [
     ([9], 9, 64, torch.float32), ([77, 1, 130], 40, 72, torch.bfloat16), ([200, 500], 64, 200, torch.float32),
     ([2900], 100, 24, torch.float32), ([3000], 100, 24, torch.float32),   # 5888 and 6144 rows: on either side of the line
+    ([1400], 100, 96, torch.bfloat16), ([1500], 100, 96, torch.bfloat16),   # 2816 and 3072: the line of wider heads
+    ([1400], 100, 136, torch.float32), ([1500], 100, 136, torch.float32),
 ])
 def test_cuda_core_attention_of_few_rows(lengths, pcl, d, dtype):
     """Eight rows per block, the keys of a stage dealt over its warps: remainders of rows, keys and dimensions, keys that no
