@@ -37,6 +37,8 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "dam_internal.cuh"
 #include "sm100_ptx.cuh"
 
@@ -279,6 +281,7 @@ __device__ __forceinline__ float sweep_max_masked(uint32_t tS, uint4 bits) {
 
 // 32 probabilities p = 2^(s * scale + neg_m), zero where the mask bit is clear, packed to bf16; their sums are taken in fp32,
 // before the bf16 rounding.  Of every 8, 6 go through the special-function unit and 2 through the polynomial.
+template <bool MASKED>
 __device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, float scale, float neg_m, uint32_t* pk,
                                           float& s0, float& s1, float& s2, float& s3) {
 #pragma unroll
@@ -292,8 +295,10 @@ __device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, fl
     for (int u = 0; u < kEx2; ++u) p[u] = ex2(y[u]);
 #pragma unroll
     for (int u = kEx2; u < 8; u += 2) ex2_poly2(y[u], y[u + 1], p[u], p[u + 1]);
+    if (MASKED) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) p[u] = ((word >> (q + u)) & 1u) ? p[u] : 0.f;
+      for (int u = 0; u < 8; ++u) p[u] = ((word >> (q + u)) & 1u) ? p[u] : 0.f;
+    }
     add2(s0, s1, s0, s1, p[0], p[1]);
     add2(s2, s3, s2, s3, p[2], p[3]);
     add2(s0, s1, s0, s1, p[4], p[5]);
@@ -311,10 +316,10 @@ __device__ __forceinline__ void exp_chunk(const uint32_t* cur, uint32_t word, fl
 // warp is zero.  Bound by the latency of its chains: a half is one block of straight code without votes or branches, so that
 // the arithmetic of one chunk runs under the exponentials of the other.  With a vote per chunk of 32 columns, to skip
 // the inactive ones, a masked tile took 1584 cycles in a warp alone on its scheduler and 2334 beside another, now 1230 and
-// 1988; an unmasked one takes 1190 and 1940.  So tiles that are active throughout go the same way: a copy without the selects is
-// 4 KB of code that the other roles' has to share the instruction cache with (8192 tokens 87.2 -> 83.8 us, 32768 tokens
-// 347 -> 340, 131072 tokens 1670 -> 1637, head_dim 64 117 -> 112; a list of active tiles alone 511 -> 519, 512 with the
-// polynomial as it is now).
+// 1988; an unmasked one takes 1190 and 1940.  So the tiles of a mask that are active throughout go the same way: a copy without
+// the selects is 4 KB of code that the other roles' has to share the instruction cache with (8192 tokens 87.2 -> 83.8 us, 32768 tokens
+// 347 -> 340, 131072 tokens 1670 -> 1637, head_dim 64 117 -> 112).  MASKED = false is for lists of active tiles alone.
+template <bool MASKED>
 __device__ __forceinline__ float sweep_exp(uint32_t tS, const uint4& bits, int lo, int hi, float scale, float neg_m) {
   float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll 1
@@ -323,11 +328,11 @@ __device__ __forceinline__ float sweep_exp(uint32_t tS, const uint4& bits, int l
     tmem_ld32(tS + 64 * h, ra);
     tmem_ld32(tS + 64 * h + 32, rb);
     tc_wait_ld();
-    exp_chunk(ra, h ? bits.z : bits.x, scale, neg_m, pk, s0, s1, s2, s3);
-    exp_chunk(rb, h ? bits.w : bits.y, scale, neg_m, pk + 16, s0, s1, s2, s3);
+    exp_chunk<MASKED>(ra, h ? bits.z : bits.x, scale, neg_m, pk, s0, s1, s2, s3);
+    exp_chunk<MASKED>(rb, h ? bits.w : bits.y, scale, neg_m, pk + 16, s0, s1, s2, s3);
     tmem_st32(tS + 32 * h, pk);
   }
-  if (hi - lo < 2) {
+  if (MASKED && hi - lo < 2) {
     uint32_t z[32];
 #pragma unroll
     for (int q = 0; q < 32; ++q) z[q] = 0u;
@@ -677,6 +682,10 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const uint32_t tS = tmem + lane_addr + kColS + X * 128;
     const uint32_t tO = tmem + lane_addr + kColO + X * 128;
     const uint32_t bS = bSFull + 8 * X, bP = bPFull + 8 * X;
+    // An all-ones blob has a copy of this role to itself, in which a tile without a mask goes without selects: 8192 tokens 531 ->
+    // 518 us, 32768 tokens 8.30 -> 8.08 ms.  (As a branch for each tile the copy costs the other lists 1-2 %, beside the role 0.2 %.)
+    auto softmax = [&](auto all_ones_c) {
+    constexpr bool all_ones = decltype(all_ones_c)::value;
     uint32_t cS = 0, cO = 0;
     bool ok = true;
     for (uint32_t n = 0; ok; ++n) {
@@ -775,7 +784,8 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         const float mm = (m_ref == -CUDART_INF_F) ? 0.f : m_ref;
         // ---- sweep 2: probabilities against the reference max, packed to bf16 into the first half of S
-        const float tsum = sweep_exp(tS, bits, lo, hi, prm.scale_log2, -mm);
+        const float tsum = all_ones && !need_mask ? sweep_exp<false>(tS, bits, 0, 2, prm.scale_log2, -mm)
+                                                  : sweep_exp<true>(tS, bits, lo, hi, prm.scale_log2, -mm);
         l = l * alpha + tsum;
         // ---- O is complete up to the previous tile of this stream (its MMAs precede S of this tile)
         if (t > t0) {
@@ -852,6 +862,9 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       __syncwarp();
       if (lane == 0) mbar_arrive(bRow + 8 * X);
     }
+    };
+    if (H->flags & DAM_FLAG_ALL_ONES) softmax(std::true_type());
+    else softmax(std::false_type());
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     // ------------------------------------------------------------------ output warps: O / l and the log-sum-exp
