@@ -107,7 +107,7 @@ struct AttnParams {
   uint32_t* status;         // scratch status word
   uint32_t* work_counter;   // scratch word 2, zero at launch
   unsigned long long scratch_bytes;
-  int Hq, group, total_tokens, causal;
+  int group, total_tokens, causal;
   int64_t o_stride_tok, o_stride_head;
   int o_vec8;               // every row of O starts on a 32-byte boundary
   float scale_log2;         // softmax scale * log2(e)
@@ -182,11 +182,6 @@ struct TileWalk {
   }
 };
 
-__device__ __forceinline__ uint32_t pick_word(const uint4& b, int c) {
-  return c == 0 ? b.x : (c == 1 ? b.y : (c == 2 ? b.z : b.w));
-}
-
-
 // ---- packed fp32x2 arithmetic (one instruction for two lanes of a register pair) -----------------------
 __device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b0, float b1, float c0, float c1) {
   asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
@@ -227,8 +222,7 @@ __device__ __forceinline__ void ex2_poly2(float y0, float y1, float& p0, float& 
 }
 
 // Sweep 1 over one S row held in TMEM (4 chunks of 32 columns, next chunk in flight while one is reduced).
-template <bool MASKED>
-__device__ __forceinline__ float sweep_max(uint32_t tS, const uint4& bits) {
+__device__ __forceinline__ float sweep_max(uint32_t tS) {
   uint32_t ra[32], rb[32];
   float mx0 = -CUDART_INF_F, mx1 = -CUDART_INF_F;
   tmem_ld32(tS, ra);
@@ -238,25 +232,17 @@ __device__ __forceinline__ float sweep_max(uint32_t tS, const uint4& bits) {
     uint32_t* cur = (c & 1) ? rb : ra;
     uint32_t* nxt = (c & 1) ? ra : rb;
     if (c < 3) tmem_ld32(tS + (c + 1) * 32, nxt);
-    const uint32_t word = pick_word(bits, c);
 #pragma unroll
     for (int q = 0; q < 32; q += 4) {
-      float v0 = __uint_as_float(cur[q]), v1 = __uint_as_float(cur[q + 1]);
-      float v2 = __uint_as_float(cur[q + 2]), v3 = __uint_as_float(cur[q + 3]);
-      if (MASKED) {
-        v0 = ((word >> q) & 1u) ? v0 : -CUDART_INF_F;
-        v1 = ((word >> (q + 1)) & 1u) ? v1 : -CUDART_INF_F;
-        v2 = ((word >> (q + 2)) & 1u) ? v2 : -CUDART_INF_F;
-        v3 = ((word >> (q + 3)) & 1u) ? v3 : -CUDART_INF_F;
-      }
-      mx0 = max3(mx0, v0, v1); mx1 = max3(mx1, v2, v3);
+      mx0 = max3(mx0, __uint_as_float(cur[q]), __uint_as_float(cur[q + 1]));
+      mx1 = max3(mx1, __uint_as_float(cur[q + 2]), __uint_as_float(cur[q + 3]));
     }
     if (c < 3) tc_wait_ld();
   }
   return fmaxf(mx0, mx1);
 }
 
-// The masked maximum again, as small code: it runs on the first tile of a list and where the bound was exceeded.
+// The maximum over the active entries, as small code: it runs on the first tile of a list and where the bound was exceeded.
 __device__ __forceinline__ float sweep_max_masked(uint32_t tS, uint4 bits) {
   float mx0 = -CUDART_INF_F, mx1 = -CUDART_INF_F;
 #pragma unroll 1
@@ -768,7 +754,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         bool masked_max = need_mask && (t == t0);            // the first tile sets the reference
         float mx = -CUDART_INF_F;
         if (!masked_max) {
-          const float mu = sweep_max<false>(tS, bits);
+          const float mu = sweep_max(tS);
           if (!need_mask) mx = mu;
           else masked_max = __any_sync(0xFFFFFFFFu, mu * prm.scale_log2 - m_ref > kRescaleThreshold);   // -inf reference: true
         }
@@ -1145,7 +1131,7 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
   p.work_counter = reinterpret_cast<uint32_t*>(scratch) + 2;
   p.scratch_bytes = scratch_bytes;
   p.ranges = ranges;
-  p.Hq = s->num_q_heads; p.group = s->num_q_heads / s->num_kv_heads; p.total_tokens = s->total_tokens;
+  p.group = s->num_q_heads / s->num_kv_heads; p.total_tokens = s->total_tokens;
   p.causal = causal;
   p.o_vec8 = reinterpret_cast<uintptr_t>(O) % 32 == 0 && s->o_stride_tok % 16 == 0 && s->o_stride_head % 16 == 0;
   p.o_stride_tok = s->o_stride_tok; p.o_stride_head = s->o_stride_head;

@@ -231,6 +231,8 @@ __device__ __forceinline__ uint32_t dam_window32(const uint32_t* __restrict__ bi
 // Inside the window (i < L): the true-mask words.  Below it: matched columns of this tile OR the
 // matched diagonals, key j active iff D[i - j]; with Drev[x] = D[L-1-x] the keys j0 .. j0+127 read
 // Drev bits x0 .. x0+127, x0 = L - 1 - i + j0 (ascending in j), which also excludes j > i.
+// (The CUDA-core attention and dam_mask_expand_rows.  The tensor-core attention's tile_bits says the same for the rows of a warp
+// without branches: the two have to agree.)
 __device__ __forceinline__ uint4 dam_tile_row_bits(const DamHeadBits& hb, int i, int kb) {
   uint4 r = make_uint4(0u, 0u, 0u, 0u);
   const int j0 = kb * DAM_TILE;
@@ -239,9 +241,7 @@ __device__ __forceinline__ uint4 dam_tile_row_bits(const DamHeadBits& hb, int i,
     if (j0 < hb.L) r = __ldg(reinterpret_cast<const uint4*>(hb.M + (size_t)i * hb.W + kb * 4));
   } else {
     if (j0 < hb.L && i < hb.gather_from) r = __ldg(reinterpret_cast<const uint4*>(hb.V + kb * 4));
-    // five words cover the four windows: the attention kernel's softmax warps run this for every masked tile, and its
-    // instructions compete with their exponentials (with the clipping left out below: 8k tokens 123.0 -> 120.8 us, 32k
-    // 498 -> 492, head_dim 64 133.9 -> 128.3)
+    // (five words cover the four windows)
     const int x0 = hb.L - 1 - i + j0;
     if (x0 + DAM_TILE > 0 && x0 < hb.L) {
       const int w = x0 >> 5, sh = x0 & 31;
