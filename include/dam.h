@@ -309,13 +309,15 @@ dam_status_t dam_mask_expand_rows(const void* mask, const dam_shape_t* shape, in
 dam_status_t dam_poll_status(const void* mask_or_scratch, void* stream);
 
 /*
- * Self-test of the bounded waits the kernels use (every wait on an mbarrier gives up after a time limit,
- * records DAM_ERR_DEVICE_TIMEOUT in the status word and lets the kernel return; nothing spins forever).
- * Launches one tiny kernel that waits, for at most limit_us microseconds (1 .. 1000000), on a barrier
- * nothing arrives on. Afterwards dam_poll_status(scratch, stream) returns DAM_ERR_DEVICE_TIMEOUT and the
- * device stays usable. scratch: DEVICE, >= 256 bytes, 256-byte aligned; bytes 8..15 receive the time waited
- * in nanoseconds. The paper has no counterpart; this exists so that the failure path can be exercised
- * without faulting or hanging a GPU.
+ * Self-test of the bounded waits the kernels use: every wait on an mbarrier gives up, after a number of polls that takes
+ * one to four seconds (attention) or after two seconds (scoring), records DAM_ERR_DEVICE_TIMEOUT in the status word and lets
+ * the kernel return; nothing spins forever. Launches one tiny kernel with a wait of each kind on a barrier nothing arrives on,
+ * by the clock for limit_us microseconds (1 .. 1000000), by polls for an 800th of their number. Afterwards
+ * dam_poll_status(scratch, stream) returns DAM_ERR_DEVICE_TIMEOUT and the device stays usable. scratch: DEVICE,
+ * >= 256 bytes, 256-byte aligned; in nanoseconds, bytes 8..15 receive the time waited by the clock, 16..23 the time
+ * the full number of polls would take, 24..31 that of a further wait by the clock, with a longer limit, which the expired
+ * one releases; bytes 32..39 how many of the three gave up. The paper has no counterpart; this exists so
+ * that the failure path can be exercised without faulting or hanging a GPU.
  */
 dam_status_t dam_selftest_bounded_wait(void* scratch, size_t scratch_bytes, uint32_t limit_us, void* stream);
 

@@ -383,13 +383,19 @@ def dam_poll_status(buf: torch.Tensor) -> int:
 
 
 def dam_selftest_bounded_wait(device, limit_us: int = 20000):
-    """Runs the bounded-wait self-test; returns (status read back, nanoseconds waited)."""
+    """Runs the bounded-wait self-test; returns (status read back, nanoseconds waited by the clock)."""
+    status, words = bounded_wait_words(device, limit_us)
+    return status, words[0]
+
+
+def bounded_wait_words(device, limit_us: int = 20000):
+    """The same; returns the status and what the self-test leaves behind it: nanoseconds of the wait by the clock, of a full count
+    of polls and of the wait that was released, and how many of the three gave up."""
     scr = torch.zeros(256, dtype=torch.uint8, device=device)
     rc = lib().dam_selftest_bounded_wait(_ptr(scr), 256, limit_us, _stream(device))
     _check(rc, "dam_selftest_bounded_wait")
     status = dam_poll_status(scr)
-    waited = int(scr[8:16].cpu().numpy().view(np.uint64)[0])
-    return status, waited
+    return status, [int(x) for x in scr[8:40].cpu().numpy().view(np.uint64)]
 
 
 def dam_prefill_host(Qh: torch.Tensor, Kh: torch.Tensor, Vh: torch.Tensor, shape: Shape, rule: dam_rule_t,

@@ -1022,33 +1022,41 @@ __global__ void clear_status_kernel(uint32_t* scratch, int keep) {
   if ((int)threadIdx.x >= keep) scratch[threadIdx.x] = 0u;
 }
 
-// Self-test of the bounded wait every kernel in this library uses: waits on an mbarrier that nothing ever
-// arrives on, twenty thousand polls at a time, until the given limit is over; every wait gives up, the status word is set the way
-// those kernels set it and the kernel returns normally.  The waiting thread is in the second warp; the first one, whose thread
-// writes the status word, has nothing to do.
-__global__ void bounded_wait_selftest_kernel(uint32_t* status, unsigned long long limit_ns, unsigned long long* waited_ns) {
+// Self-test of the bounded waits, on mbarriers that nothing ever arrives on, a waiting thread in a warp of its own for each:
+// the attention kernel's by a count of polls (a fixed number of them, timed), the scoring kernel's by the wall clock (the
+// given limit), and another of those that the expired one has to release long before its own limit.  The status word is written the
+// way those kernels write it, by a thread that has nothing else to do.
+// words: nanoseconds of the wait by the wall clock, of the count of polls as kWaitPolls of them would take, of the released wait;
+// how many of the three gave up.
+__global__ void bounded_wait_selftest_kernel(uint32_t* status, unsigned long long limit_ns, unsigned long long* words) {
+  constexpr uint32_t kPolls = kWaitPolls / 800;
   __shared__ uint64_t bar;
-  __shared__ uint32_t abort_flag;
+  __shared__ uint32_t flag_polls, flag_clock, gave_up;
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar), 1);
-    abort_flag = 0u;
+    flag_polls = flag_clock = gave_up = 0u;
     mbar_fence_init();
   }
   __syncthreads();
+  const uint64_t t0 = globaltimer_ns();
   if (threadIdx.x == 32) {
-    const uint64_t t0 = globaltimer_ns();
-    bool ok;
-    do ok = mbar_wait(smem_u32(&bar), 0u, &abort_flag, 20000u);
-    while (!ok && globaltimer_ns() - t0 < limit_ns);
-    *waited_ns = globaltimer_ns() - t0;
+    if (!mbar_wait_slow(smem_u32(&bar), 0u, &flag_clock, limit_ns)) atomicAdd(&gave_up, 1u);
+    words[0] = globaltimer_ns() - t0;
+  } else if (threadIdx.x == 64) {
+    if (!mbar_wait(smem_u32(&bar), 0u, &flag_polls, kPolls)) atomicAdd(&gave_up, 1u);
+    words[1] = (globaltimer_ns() - t0) * (kWaitPolls / kPolls);
+  } else if (threadIdx.x == 96) {
+    if (!mbar_wait_slow(smem_u32(&bar), 0u, &flag_clock, 2 * limit_ns + 1000000000ull)) atomicAdd(&gave_up, 1u);
+    words[2] = globaltimer_ns() - t0;
   }
-  report_expired_wait(&abort_flag, status, DAM_ERR_DEVICE_TIMEOUT);
+  report_expired_wait(&flag_clock, status, DAM_ERR_DEVICE_TIMEOUT);
+  if (threadIdx.x == 0) words[3] = flag_polls ? gave_up : 0u;
 }
 
 }  // namespace
 
 cudaError_t dam_launch_bounded_wait_selftest(void* scratch, unsigned long long limit_ns, cudaStream_t st) {
-  bounded_wait_selftest_kernel<<<1, 64, 0, st>>>(reinterpret_cast<uint32_t*>(scratch) + 1, limit_ns,
+  bounded_wait_selftest_kernel<<<1, 128, 0, st>>>(reinterpret_cast<uint32_t*>(scratch) + 1, limit_ns,
                                                   reinterpret_cast<unsigned long long*>(scratch) + 1);
   return cudaGetLastError();
 }

@@ -45,19 +45,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 
 // Bounded wait: gives up after `polls` looks at the barrier, records the fact in *abort_flag (shared memory) and returns false.
 // No wait in these kernels can spin forever; a role whose partner has given up waits for it in vain and gives up in its turn.
-// A look takes 43 cycles and more (measured on a barrier that nothing arrives on, a warp per scheduler polling), so the
-// default is a second or so.  The loop is as short as it can be: it is inlined wherever a role waits, all of the attention
-// kernel's code is executed for every work item, and the instruction cache holds about 64 KB of it (with a look at the
-// wall clock every 256 polls 70 KB, at every poll 64; that kernel as it is now: 55.6 KB with the wall clock, 51.8 with the
-// cycle counter, 51 with a count).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t polls = 40000000u) {
+// A look at a barrier that nothing arrives on takes 43 cycles with a warp per scheduler polling and 165 in the self-test,
+// so kWaitPolls are one to four seconds (the self-test, which times them: 3.4).  The loop is as short as it can be: it is inlined
+// wherever a role waits, all of the attention kernel's code is executed for every work item, and the instruction cache holds
+// about 64 KB of it (the same kernel with a look at the wall clock every 256 polls 55.6 KB, with the cycle counter 51.8, with a
+// count 51).
+constexpr uint32_t kWaitPolls = 40000000u;
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t polls = kWaitPolls) {
 #pragma unroll 1
   while (!mbar_try_wait(bar, parity))
     if (--polls == 0u) { *abort_flag = 1u; return false; }
   return true;
 }
-// The same with a limit on wall time (looked at every 256 polls), for a kernel with many waiting warps beside working ones, the
-// scoring kernel: with the bare loop stage 1 takes 40.7 us instead of 40.2 at 8192 tokens, 35.5 instead of 34.8 at head_dim 64.
+// The same with a limit on wall time, looked at every 256 polls, and with it the flag, so that a wait that has expired ends the
+// others.  For a kernel with many waiting warps beside working ones, the scoring kernel: with the bare loop stage 1 takes 40.7
+// us instead of 40.2 at 8192 tokens, 35.5 instead of 34.8 at head_dim 64.
 __device__ __forceinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint64_t limit_ns = 2000000000ull) {
   if (mbar_try_wait(bar, parity)) return true;
   uint64_t t0 = 0;

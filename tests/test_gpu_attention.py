@@ -453,11 +453,13 @@ def test_threads_with_different_shared_memory_sizes():
 
 
 def test_bounded_wait_times_out_cleanly():
-    """A wait that nothing satisfies gives up after its limit, the status word says so although the thread that writes it has
-    long been done, and the device keeps working (the next kernel runs and is correct)."""
-    status, waited_ns = B.dam_selftest_bounded_wait(DEV, limit_us=20000)
-    assert status == 5                                   # DAM_ERR_DEVICE_TIMEOUT
-    assert 15e6 <= waited_ns <= 500e6
+    """Waits of both kinds that nothing satisfies give up, the one by the clock after its limit, the one by polls after a
+    number of them that takes some seconds, and the expired one releases the other; the status word says so although the
+    thread that writes it has long been done, and the device keeps working (the next kernel runs and is correct)."""
+    status, (waited_ns, polls_ns, released_ns, gave_up) = B.bounded_wait_words(DEV, limit_us=20000)
+    assert status == 5 and gave_up == 3                  # DAM_ERR_DEVICE_TIMEOUT
+    assert 15e6 <= waited_ns <= 500e6 and released_ns <= waited_ns + 100e6
+    assert 0.3e9 <= polls_ns <= 10e9
     w = synth.small_case(0, 4, 2, 128, 128, seed=9, lengths=[300])
     shape = _shape(w)
     blob = B.dam_mask_all_ones(shape, True, DEV)
