@@ -720,8 +720,10 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // the first n: of a gathered tile, the columns it holds; of a full one, the keys that exist (and not beyond the row)
         int n = kind == DAM_KIND_GATHERED ? (int)((e >> 16) & 0xFFu) + 1 : it.S - kb * DAM_TILE;
         if (kind == DAM_KIND_FULL && prm.causal) n = min(n, i - kb * DAM_TILE + 1);
-        if (!row_valid) n = 0;
         need = __any_sync(0xFFFFFFFFu, n < DAM_TILE);
+        // rows beyond the sequence keep nothing, but do not make a tile a masked one for their warp: without a reference they would
+        // have it take the masked maximum, too, in every tile (all-ones: 1000 tokens 26.6 -> 22.4 us, 3000 tokens 116.9 -> 97.5)
+        if (!row_valid) n = 0;
         return dam_low_ones128(n);
       };
       // entries left out: entry t of what remains is entry t + ln.n of the list from ln.at on
