@@ -57,14 +57,18 @@ constexpr float kRescaleThreshold = 8.0f;
 constexpr uint32_t kStepTile = 1u, kStepFirst = 4u, kStepLast = 16u, kStepDual = 64u, kStepEnd = 128u;
 constexpr int kPolyPer8 = 2;   // of every 8 exponentials, how many use the FMA-pipe polynomial (0, 2 or 4)
 
-constexpr int kRowBitWords = 512;            // work lists of up to 16384 items
+// Work lists whose items inside the row ranges are marked: up to 3840 or 16384 items (a word for 32).
+constexpr int kRowBitWords = 120, kRowBitWordsLong = 512;
 
-template <bool RANGED, int D>
+// RANGED: 0 no row ranges, 1 row ranges, 2 row ranges and a list of more than 3840 items (head_dim 128).
+template <int RANGED, int D>
 struct SmemLayout {
   static constexpr int kSlotBytes = 256 * D;            // a Q, K or V tile
   // A step with two tiles per operand holds four slots; a fifth lets the next K tile come early (32768 tokens 388 us with four
-  // and K waited for before P V, 359 with four and after, 353 with five).  With the row bits there is room for four.
-  static constexpr int kSlots = D == 64 ? 10 : RANGED ? 4 : 5;
+  // and K waited for before P V, 359 with four and after, 353 with five; 256 rows of 30000, 8 heads, 31.9 with four and 30.7 with
+  // five, 2048 rows of 8192, 32 heads, 40.6 and 38.4).  Beside the row bits of a long list there is room for four.
+  static constexpr int kSlots = D == 64 ? 10 : RANGED == 2 ? 4 : 5;
+  static constexpr int kBitWords = RANGED == 0 ? 0 : RANGED == 1 && D == 128 ? kRowBitWords : kRowBitWordsLong;
   static constexpr int q = 0;                           // Q_A, Q_B
   static constexpr int slots = 2 * kSlotBytes;
   static constexpr int bars = kSlotBytes * (2 + kSlots);
@@ -76,8 +80,8 @@ struct SmemLayout {
   static constexpr int stat = item_rec + 2 * 112;                    // float2 [stream][128]: reference and sum of every row
   static constexpr int tmem_slot = stat + 2 * DAM_TILE * 8;
   static constexpr int abort_flag = tmem_slot + 4;
-  static constexpr int row_bits = abort_flag + 4;           // u32[kRowBitWords]: the work list's items inside the row ranges
-  static constexpr int total = row_bits + (RANGED ? 4 * kRowBitWords : 0);
+  static constexpr int row_bits = abort_flag + 4;           // u32[kBitWords]: the work list's items inside the row ranges
+  static constexpr int total = row_bits + 4 * kBitWords;
   static_assert(item_rec % 16 == 0 && bars % 8 == 0 && stat % 8 == 0, "shared-memory records must be aligned");
   static_assert(total <= 232448, "227 KB of shared memory");
 };
@@ -331,7 +335,7 @@ __device__ __forceinline__ float sweep_exp(uint32_t tS, const uint4& bits, int l
 // RANGED: only the work items whose first row lies in the row range of their sequence are processed.
 // D: head_dim, 128 or 64.  With 64 a Q / K / V tile is one 16 KB box of the tensor maps, S = Q K^T takes four MMAs instead of
 // eight and O has 64 columns.
-template <bool RANGED, int D>
+template <int RANGED, int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmG, const AttnParams prm,
@@ -369,7 +373,7 @@ attn_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   }
   // Dynamic scheduling: the work list is sorted longest first; the scheduler takes positions from a global counter (the
   // first one is the CTA index) and hands a record of each to the other roles through a two-entry ring in shared memory.
-  const bool row_list = RANGED && nitems <= 32 * kRowBitWords;
+  const bool row_list = RANGED && nitems <= 32 * Smem::kBitWords;
   uint32_t* row_bits = reinterpret_cast<uint32_t*>(smem + Smem::row_bits);
 
   if (tid == 0) {
@@ -1055,6 +1059,11 @@ __global__ void bounded_wait_selftest_kernel(uint32_t* status, unsigned long lon
   if (threadIdx.x == 0) words[3] = flag_polls ? gave_up : 0u;
 }
 
+template <int RANGED, int D>
+cudaError_t allow_smem() {
+  return cudaFuncSetAttribute(attn_sm100_kernel<RANGED, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<RANGED, D>::total);
+}
+
 }  // namespace
 
 cudaError_t dam_launch_bounded_wait_selftest(void* scratch, unsigned long long limit_ns, cudaStream_t st) {
@@ -1075,15 +1084,11 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
   DamDeviceInfo di;
   cudaError_t e;
   if ((e = dam_current_device(&dev, &di)) != cudaSuccess) return e;
-  constexpr int smem[2][2] = {{SmemLayout<false, 64>::total, SmemLayout<false, 128>::total},
-                              {SmemLayout<true, 64>::total, SmemLayout<true, 128>::total}};
   if (di.cc_major != 10 || di.smem_optin < 232448) return cudaErrorNotSupported;
   if ((e = dam_device_table().once(dev, DAM_SETUP_ATTN_SMEM, [](void) -> cudaError_t {
          cudaError_t r;
-         if ((r = cudaFuncSetAttribute(attn_sm100_kernel<false, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<false, 128>::total)) != cudaSuccess) return r;
-         if ((r = cudaFuncSetAttribute(attn_sm100_kernel<true, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<true, 128>::total)) != cudaSuccess) return r;
-         if ((r = cudaFuncSetAttribute(attn_sm100_kernel<false, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<false, 64>::total)) != cudaSuccess) return r;
-         return cudaFuncSetAttribute(attn_sm100_kernel<true, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemLayout<true, 64>::total);
+         if ((r = allow_smem<0, 128>()) != cudaSuccess || (r = allow_smem<1, 128>()) != cudaSuccess || (r = allow_smem<2, 128>()) != cudaSuccess) return r;
+         return (r = allow_smem<0, 64>()) != cudaSuccess ? r : allow_smem<1, 64>();
        })) != cudaSuccess)
     return e;
   const int sm_count = di.sm_count;
@@ -1131,7 +1136,7 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
   if (pairs == 0) return cudaSuccess;
   // a CTA for every pair to compute, but where the list is too long to be marked the CTAs walk all of it, and the walk is
   // what takes the time: 256 rows of 204800 tokens, 32 pairs of 25600, 32 CTAs 565 us, 148 CTAs 134
-  if (all > 32 * kRowBitWords) pairs = all;
+  if (all > 32 * kRowBitWordsLong) pairs = all;
   if (s->o_stride_tok >= (int64_t)1 << 39 || s->o_stride_head >= (int64_t)1 << 39) return cudaErrorInvalidValue;   // (no such memory)
   AttnParams p;
   p.blob = reinterpret_cast<const unsigned char*>(blob);
@@ -1147,11 +1152,15 @@ cudaError_t dam_launch_attn_sm100(const void* Q, const void* K, const void* V, c
   p.o_stride_tok = s->o_stride_tok; p.o_stride_head = s->o_stride_head;
   p.scale_log2 = scale * 1.4426950408889634f;
   const int grid = pairs < sm_count ? pairs : sm_count;
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem[ranges ? 1 : 0][d == 128 ? 1 : 0];
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kThreads);
+  auto launch = [&](auto* kernel, int smem) -> cudaError_t {
+    cfg.dynamicSmemBytes = smem;
+    return cudaLaunchKernelEx(&cfg, kernel, tq, tk, tv, tg, p, rows);
+  };
   if (d == 128) {
-    if (ranges) return cudaLaunchKernelEx(&cfg, attn_sm100_kernel<true, 128>, tq, tk, tv, tg, p, rows);
-    return cudaLaunchKernelEx(&cfg, attn_sm100_kernel<false, 128>, tq, tk, tv, tg, p, rows);
+    if (!ranges) return launch(attn_sm100_kernel<0, 128>, SmemLayout<0, 128>::total);
+    return all <= 32 * kRowBitWords ? launch(attn_sm100_kernel<1, 128>, SmemLayout<1, 128>::total)
+                                    : launch(attn_sm100_kernel<2, 128>, SmemLayout<2, 128>::total);
   }
-  if (ranges) return cudaLaunchKernelEx(&cfg, attn_sm100_kernel<true, 64>, tq, tk, tv, tg, p, rows);
-  return cudaLaunchKernelEx(&cfg, attn_sm100_kernel<false, 64>, tq, tk, tv, tg, p, rows);
+  return ranges ? launch(attn_sm100_kernel<1, 64>, SmemLayout<1, 64>::total) : launch(attn_sm100_kernel<0, 64>, SmemLayout<0, 64>::total);
 }

@@ -587,11 +587,21 @@ def test_chunked_prefill_equals_one_call(lengths, Hq, Hkv, d, dtype, gather):
 ])
 def test_row_ranges_of_long_lists_and_many_sequences(lengths, Hq, ranges):
     """Rows of the single call, bit for bit, and no others."""
+    _rows_as_in_the_single_call(lengths, Hq, 64, ranges)
+
+
+@pytest.mark.parametrize("S,Hq", [(30720, 32), (30976, 32), (32700, 128), (33000, 128)])      # 3840, 3872, 16384, 16512 items
+def test_row_ranges_of_long_lists_at_head_dim_128(S, Hq):
+    """The lengths of work lists at which the marks of the wanted items, and with them the slots for K and V, change."""
+    _rows_as_in_the_single_call([S], Hq, 128, [(20480, 20992)])
+
+
+def _rows_as_in_the_single_call(lengths, Hq, d, ranges):
     torch.manual_seed(23)
     cu = np.concatenate([[0], np.cumsum(lengths)]).tolist()
-    Q = torch.randn(cu[-1], Hq, 64, dtype=torch.bfloat16, device=DEV)
-    K, V = (torch.randn(cu[-1], 2, 64, dtype=torch.bfloat16, device=DEV) for _ in range(2))
-    shape = B.make_shape(cu, Hq, 2, 64, torch.bfloat16, DEV)
+    Q = torch.randn(cu[-1], Hq, d, dtype=torch.bfloat16, device=DEV)
+    K, V = (torch.randn(cu[-1], 2, d, dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    shape = B.make_shape(cu, Hq, 2, d, torch.bfloat16, DEV)
     blob, _ = B.dam_build_masks(Q, K, shape, B.make_rule(64, 0.1, 0.5, gather_columns=True))
     O_ref, lse_ref, _ = B.dam_sparse_attention(Q, K, V, blob, shape, causal=True)
     O, lse = torch.full_like(O_ref, 7.0), torch.full_like(lse_ref, 7.0)
