@@ -20,12 +20,13 @@
 //               is not fully active, writes P (bf16) back to TMEM and rescales O in TMEM when the running max
 //               moved by more than 2^8; after a block's last tile it leaves the row's reference and sum;
 //   warps 12-15 output of both streams: O / sum and the log-sum-exp, 32 bytes per thread and store.
-// What bounds it: a stream's chain from P to the next S to the next P (about 1400 cycles of P V and S, 2200 of softmax),
-// two of which share the tensor pipe.  In an earlier form the softmax warps also wrote the output, the steps were those of
+// What bounds it: a stream's chain from P to the next S to the next P (P V and S about 1400 cycles, softmax 1700 to 1950),
+// two of which share the tensor pipe.  In the form before this one the softmax warps also wrote the output, the steps were those of
 // the merged lists (in a quarter of them one stream had no tile) and the item's record and Q came when everything before was
 // done: an item of 12.5 tiles took 30300 cycles at 32768 tokens, 10500 of them between a stream's last P of an item
-// and its first of the next.  Attention then -> now: 8192 tokens 96.3 -> 87.7 us, 32768 tokens 378 -> 353, 131072 tokens
-// 1720 -> 1590, head_dim 64 126 -> 118, 2048 rows of 26624 43.5 -> 41.5, dense list 506 -> 507.
+// and its first of the next.  Attention alone, that form -> this one, timed in turn: 1237 tokens 26.5 -> 24.7 us, 8192 tokens 97.1 ->
+// 90.1, 32768 tokens 413 -> 380, 131072 tokens 1995 -> 1872, mixed lengths 1645 -> 1515, 16001 tokens at head_dim 64 124 -> 110, 2048 rows
+// of 26624 43.0 -> 38.4; all-ones 8192 tokens 524 -> 525.
 // The kernel's code is kept small: all of it is executed for every item, the instruction cache holds about 64 KB, and the
 // same roles in 78 KB were a fifth slower than in 66.  So what waits or issues is written once and looped over
 // streams, operands and chunks where it is not hot, and mask words are made at one place.
